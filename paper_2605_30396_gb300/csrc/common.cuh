@@ -133,6 +133,16 @@ __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gsrc, uint3
       : "memory");
 }
 
+// TMA load of a 2-D box at element (x, y) of the tensor map (x * element size a
+// multiple of 16 bytes); parts outside the tensor arrive as zeros.
+__device__ __forceinline__ void tma_load_2d(void* smem_dst, const void* map, int x, int y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
+          "r"(smem_u32(smem_dst)),
+      "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
+      : "memory");
+}
+
 // ---- named barrier over a subset of warps --------------------------------
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -194,6 +204,13 @@ __device__ __forceinline__ uint64_t umma_smem_desc(uint32_t saddr, uint32_t lbo,
   d |= static_cast<uint64_t>(1) << 46;  // descriptor version for tcgen05
   // base offset 0, absolute LBO mode off, layout type 0 = no swizzle
   return d;
+}
+
+// The same for an operand with the 128-byte swizzle (lines of 128 bytes, groups
+// of eight lines `sbo` apart).  K-major: a line is a row, `lbo` unused.
+// MN-major: a line is a k, `lbo` the distance between blocks of 64 rows.
+__device__ __forceinline__ uint64_t umma_smem_desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return umma_smem_desc(saddr, lbo, sbo) | (static_cast<uint64_t>(2) << 61);
 }
 
 // Instruction descriptor: FP32 accumulator, K-major A and B, dense.

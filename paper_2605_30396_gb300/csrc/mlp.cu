@@ -4,18 +4,22 @@
 // restricted to them; plain OMP (Sec. 2.1) remains the fallback.
 //
 // GPU design:
-//   gemm_kernel     tcgen05 BF16 GEMM, C = A B^T with FP32 accumulation in TMEM.
-//                   Operands are read with arbitrary row/column strides (so
-//                   transposed activations need no copies) and staged into the
-//                   canonical no-swizzle K-major layout (cp.async 16-byte copies
-//                   where a row's 8 k values are contiguous, else by the
-//                   threads); three shared-memory stages keep the loads two
-//                   k-tiles ahead of the MMAs.  Epilogues: store (split-K partials), +bias,
-//                   +bias with GELU (stores the pre-activation for backward).
-//   small kernels   input normalisation, BCE-with-logits gradient and loss,
-//                   GELU backward, bias gradients, split-K reduction, Adam.
-// Inference (the logits, or the m best atoms per signal) is one fused kernel
-// (propose.cu); the layer-by-layer forward here serves training.
+//   train_gemm_kernel  tcgen05 BF16 GEMM, C = A B^T with FP32 accumulation in
+//                   TMEM, 128 x 128 tiles.  An operand is read in place by
+//                   TMA, K-major or MN-major (the transposed activations and
+//                   weights of the backward pass need no copies).  Each epilogue
+//                   does the
+//                   element-wise work that follows the product: bias + GELU,
+//                   BCE gradient + loss + column sums, GELU backward + column
+//                   sums, or the FP32 partial of a weight gradient.
+//   weight gradients  one launch for all three layers, split over the batch
+//                   Batch 8192, K = 1024 (us of device time): logits with the
+//                   BCE work 34 + 67 -> 31, dH2 with the GELU backward 103 ->
+//                   15, weight gradients 479 -> 12, the whole gradient call 810
+//                   -> 163 of which about 95 are kernels.
+//   reduce_kernel   adds the split partials and the column sums in a fixed
+//                   order (gradients), and applies Adam in a training step
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -32,329 +36,425 @@ namespace mlp {
 constexpr int GM = 128;  // tile rows = MMA M
 constexpr int GN = 128;  // tile cols = MMA N
 constexpr int GK = 64;   // k-tile: four MMAs of K = 16
-constexpr int GT = 128;  // threads per GEMM CTA
-constexpr int NS = 3;    // operand stages (loads run NS - 1 k-tiles ahead)
-constexpr uint32_t A_STAGE = GM * GK * 2;  // 16 KB
-constexpr uint32_t B_STAGE = GN * GK * 2;  // 16 KB
+constexpr int GT = 256;  // threads per GEMM CTA (warp w: TMEM lanes of quarter w & 3, columns of half w >> 2)
+// Operand tiles in shared memory, 128 rows (M or N) x 64 k, 16 KB, as TMA
+// writes them with the 128-byte swizzle (16-byte word c of 128-byte line l sits
+// at word c ^ (l & 7)):
+//   K-major   one box: line = row, 64 k; eight-row groups 1024 bytes apart
+//   MN-major  two boxes of 64 rows: line = k, 64 rows; eight-k groups 1024
+//             bytes apart, the boxes 8 KB apart
+// (With 16-byte cp.async into the unswizzled layout each word was an L2 request
+// of its own: twice the bytes and 3 to 4 times the time of the k-loops.)
+constexpr uint32_t OPER = GM * GK * 2;
+constexpr uint32_t STAGE = 2 * OPER;
+// Operand stages NS: three where the grid gives every SM two CTAs, six where it
+// gives only one.
+constexpr uint32_t gemm_smem(int ns) { return ns * STAGE + 1024; }
 
-enum : int { EPI_STORE = 0, EPI_BIAS = 1, EPI_BIAS_GELU = 2 };
+enum : int { EPI_GELU = 0, EPI_BCE = 1, EPI_GELU_BWD = 2, EPI_PART = 3 };
 
-struct Mat {
-  const __nv_bfloat16* p;
-  long long srow, scol;  // element (r, c) at p[r * srow + c * scol]
+// One product of a launch: M x N over k [0, Kd), its tiles numbered from tile0.
+// The operands' tensor maps: K-major maps have k as the inner dimension,
+// MN-major ones the rows; what lies outside reads as zero.
+struct Prod {
+  CUtensorMap A, B;
+  int M, N, Kd, tiles_n, tile0;
+  float* C;  // FP32 output (EPI_PART: partial z at C + z * zstride), row stride ldc
+  int ldc;
 };
 
 struct GemmArgs {
-  Mat A;  // M x Kd
-  Mat B;  // N x Kd
-  int M, N, Kd;
-  int klen;            // k range per split (multiple of GK)
-  float* C;            // M x N (row stride ldc), split z at C + z * zstride
-  long long ldc, zstride;
-  const float* bias;   // N (EPI_BIAS, EPI_BIAS_GELU)
-  __nv_bfloat16* H;    // GELU output, M x N (row stride ldh)
-  long long ldh;
-  int epi;
+  Prod p[3];
+  int nprod;
+  int M;                // valid rows of the batch (all epilogues but EPI_PART)
+  int klen;             // k range per split (multiple of GK)
+  long long zstride;
+  const float* bias;    // N (EPI_GELU, EPI_BCE)
+  const float* Z;       // EPI_GELU_BWD: the layer's pre-activations, row stride HID
+  __nv_bfloat16* H;     // BF16 output (activations or dZ), row stride ldh
+  int ldh;
+  float* colpart;       // column sums of the FP32 values per 128-row tile, [tile][ldh]
+  const float* X;       // EPI_GELU with XA: the signals (A is their unit-norm BF16 form)
+  __nv_bfloat16* Xn;    // and where that form is kept for the weight gradient
+  const uint16_t* idx;  // EPI_BCE: the targets
+  const uint8_t* nnz;
+  int s;
+  float inv_bk;
+  double* loss_part;    // EPI_BCE: one loss sum per CTA
   uint32_t* status;
   long long budget;
 };
 
-// Stages rows [r0, r0+rows_tile) x k-range [k0, k0+GK) of X into the canonical
-// layout at `dst` (16-byte K-blocks: byte (kk/8) * rows_tile*16 + r*16 + (kk%8)*2).
-template <int ROWS>
-__device__ __forceinline__ void stage_tile(uint8_t* dst, const Mat& X, int r0, int nrows, int k0,
-                                           int kend) {
-  const int t = threadIdx.x;
-  const bool kvec = X.scol == 1 && (X.srow % 8) == 0 && (reinterpret_cast<uintptr_t>(X.p) % 16) == 0;
-  const bool rvec = X.srow == 1 && (X.scol % 8) == 0 && (reinterpret_cast<uintptr_t>(X.p) % 16) == 0;
-  if (kvec) {
-    // chunk = 8 consecutive k of one row; consecutive threads take consecutive rows
-    for (int c = t; c < ROWS * (GK / 8); c += GT) {
-      const int kb = c / ROWS, r = c - kb * ROWS;
-      const int row = r0 + r, k = k0 + kb * 8;
-      uint8_t* d = dst + kb * (ROWS * 16) + r * 16;
-      if (row < nrows && k + 8 <= kend) {
-        // asynchronous 16-byte copy, completed by the caller's cp.async wait
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(d)),
-                     "l"(X.p + static_cast<long long>(row) * X.srow + k)
-                     : "memory");
-      } else {
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (row < nrows && k < kend) {
-          const __nv_bfloat16* src = X.p + static_cast<long long>(row) * X.srow + k;
-          __nv_bfloat16 tmp[8];
-          for (int e = 0; e < 8; ++e) tmp[e] = (k + e < kend) ? src[e] : __float2bfloat16(0.f);
-          v = *reinterpret_cast<uint4*>(tmp);
-        }
-        *reinterpret_cast<uint4*>(d) = v;
-      }
+// 32 bytes to global memory in one store (32-byte aligned).
+__device__ __forceinline__ void st32(void* p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+// 32 consecutive FP32 / BF16 values of one row (32-byte aligned).
+__device__ __forceinline__ void store_f32(float* p, const float (&v)[32]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(v[8 * q + e]);
+    st32(p + 8 * q, w);
+  }
+}
+__device__ __forceinline__ void store_bf16(__nv_bfloat16* p, const float (&v)[32]) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const __nv_bfloat162 b = __floats2bfloat162_rn(v[16 * q + 2 * e], v[16 * q + 2 * e + 1]);
+      w[e] = *reinterpret_cast<const uint32_t*>(&b);
     }
-  } else if (rvec) {
-    // chunk = 8 consecutive rows at one k; scattered into 8 core-matrix rows
-    for (int c = t; c < (ROWS / 8) * GK; c += GT) {
-      const int kk = c / (ROWS / 8), rc = c - kk * (ROWS / 8);
-      const int row = r0 + rc * 8, k = k0 + kk;
-      __nv_bfloat16 tmp[8];
-      if (k < kend && row + 8 <= nrows) {
-        *reinterpret_cast<uint4*>(tmp) =
-            *reinterpret_cast<const uint4*>(X.p + row + static_cast<long long>(k) * X.scol);
-      } else {
-        for (int e = 0; e < 8; ++e)
-          tmp[e] = (k < kend && row + e < nrows) ? X.p[row + e + static_cast<long long>(k) * X.scol]
-                                                 : __float2bfloat16(0.f);
-      }
-      uint8_t* base = dst + (kk >> 3) * (ROWS * 16) + (kk & 7) * 2;
-      for (int e = 0; e < 8; ++e)
-        *reinterpret_cast<__nv_bfloat16*>(base + (rc * 8 + e) * 16) = tmp[e];
-    }
-  } else {
-    for (int c = t; c < ROWS * GK; c += GT) {
-      const int kk = c / ROWS, r = c - kk * ROWS;
-      const int row = r0 + r, k = k0 + kk;
-      const __nv_bfloat16 v = (row < nrows && k < kend)
-                                  ? X.p[static_cast<long long>(row) * X.srow + static_cast<long long>(k) * X.scol]
-                                  : __float2bfloat16(0.f);
-      *reinterpret_cast<__nv_bfloat16*>(dst + (kk >> 3) * (ROWS * 16) + r * 16 + (kk & 7) * 2) = v;
-    }
+    st32(p + 16 * q, w);
   }
 }
 
-__global__ void __launch_bounds__(GT) gemm_kernel(const __grid_constant__ GemmArgs g) {
+// Hardware reciprocal (about 1 ulp; 0 for infinity).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Sums of the warp's 32 rows: lane l returns the sum of v[l] over the lanes
+// (a transposing butterfly, the same order on every run).
+__device__ __forceinline__ float col_sums(float (&v)[32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int m = 32, o = 16; o > 0; m >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < m / 2; ++k) {
+      const float send = up ? v[k] : v[k + m / 2];
+      const float keep = up ? v[k + m / 2] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return v[0];
+}
+
+// C = A B^T tile by tile, and the layer's element-wise work on the result.
+// Warp 0 streams the operands by TMA, warp 1 issues the MMAs, then all eight
+// warps share the epilogue; a second CTA on the SM runs its k-loop meanwhile.
+template <int EPI, bool AMN, bool BMN, bool XA, int NS>
+__global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __grid_constant__ GemmArgs g) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  uint8_t* As = smem;                        // NS stages
-  uint8_t* Bs = smem + NS * A_STAGE;         // NS stages
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + NS * (A_STAGE + B_STAGE));
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + NS);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + NS * STAGE);  // [NS] operands landed
+  uint64_t* empty = full + NS;                                       // [NS] consumed by the MMAs
+  uint64_t* done = empty + NS;                                       // every MMA complete
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
-  const int kbeg = blockIdx.z * g.klen;
-  const int kend = kbeg + g.klen < g.Kd ? kbeg + g.klen : g.Kd;
+  int pi = 0;
+  if (EPI == EPI_PART)
+    while (pi + 1 < g.nprod && static_cast<int>(blockIdx.x) >= g.p[pi + 1].tile0) ++pi;
+  const Prod& P = g.p[pi];
+  const int tile = static_cast<int>(blockIdx.x) - P.tile0;
+  const int tm = tile / P.tiles_n;
+  const int m0 = tm * GM, n0 = (tile - tm * P.tiles_n) * GN;
+  const int kbeg = blockIdx.y * g.klen;
+  const int kend = kbeg + g.klen < P.Kd ? kbeg + g.klen : P.Kd;
   const int nkt = kend > kbeg ? (kend - kbeg + GK - 1) / GK : 0;
   if (tid == 0) {
-    for (int q = 0; q < NS; ++q) mbar_init(&bar[q], 1);
+    for (int q = 0; q < NS; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&empty[q], 1);
+    }
+    mbar_init(done, 1);
     fence_mbar_init();
   }
   if (warp == 0) {
     tmem_alloc(tslot, GN);
     tmem_relinquish();
   }
+  constexpr uint32_t idesc =
+      umma_idesc(1, 1, GM, GN) | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u);  // bits 15, 16: MN-major
+  if (XA) {
+    // A = the signals at unit norm, one k-tile (Kd = XIN = GK); warp w stages
+    // rows 16 w .. 16 w + 15
+    float x0[16], x1[16];
+#pragma unroll
+    for (int rr = 0; rr < 16; ++rr) {
+      const long long r = m0 + warp * 16 + rr;
+      x0[rr] = r < g.M ? g.X[r * DLSH_D + lane] : 0.f;
+      x1[rr] = (r < g.M && lane < DLSH_D - 32) ? g.X[r * DLSH_D + 32 + lane] : 0.f;
+    }
+#pragma unroll
+    for (int rr = 0; rr < 16; ++rr) {
+      const int row = warp * 16 + rr;
+      __nv_bfloat16 y0, y1;
+      normalise_pair(x0[rr], x1[rr], y0, y1);
+      uint8_t* d = smem + row * 128 + (lane & 7) * 2;
+      *reinterpret_cast<__nv_bfloat16*>(d + (((lane >> 3) ^ (row & 7)) << 4)) = y0;
+      *reinterpret_cast<__nv_bfloat16*>(d + (((4 + (lane >> 3)) ^ (row & 7)) << 4)) = y1;
+      if (n0 == 0 && m0 + row < g.M) {
+        g.Xn[static_cast<size_t>(m0 + row) * XIN + lane] = y0;
+        g.Xn[static_cast<size_t>(m0 + row) * XIN + 32 + lane] = y1;
+      }
+    }
+    fence_proxy_async_smem();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  constexpr uint32_t idesc = umma_idesc(1, 1, GM, GN);
-  auto stage = [&](int t) {
-    const int sl = t % NS, k0 = kbeg + t * GK;
-    stage_tile<GM>(As + sl * A_STAGE, g.A, m0, g.M, k0, kend);
-    stage_tile<GN>(Bs + sl * B_STAGE, g.B, n0, g.N, k0, kend);
-  };
-  // k-tile t lands in slot t % NS; its MMAs' completion is phase t / NS of that
-  // slot's barrier.  Loads run NS - 1 tiles ahead of the MMAs.
-  for (int t = 0; t < NS - 1; ++t) {
-    if (t < nkt) stage(t);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
   bool ok = true;
-  for (int nk = 0; nk < nkt; ++nk) {
-    const int nx = nk + NS - 1;
-    if (nx < nkt && nk >= 1) {  // the slot's previous tile (nk - 1) must be consumed
-      const int tp = nk - 1;
-      if (!mbar_wait(&bar[tp % NS], static_cast<uint32_t>((tp / NS) & 1), g.budget)) {
+  if (tid == 0) {
+    int issued = 0;
+    for (int t = 0; t < nkt; ++t) {
+      const int sl = t % NS, k0 = kbeg + t * GK;
+      if (!mbar_wait(&empty[sl], static_cast<uint32_t>((t / NS) & 1) ^ 1u, g.budget)) {
+        flag_status(g.status, ST_TIMEOUT);
+        ok = false;
+        break;
+      }
+      uint8_t* d = smem + sl * STAGE;
+      mbar_arrive_expect_tx(&full[sl], XA ? OPER : STAGE);
+      if (!XA) {
+        if (AMN) {
+          tma_load_2d(d, &P.A, m0, k0, &full[sl]);
+          tma_load_2d(d + OPER / 2, &P.A, m0 + 64, k0, &full[sl]);
+        } else {
+          tma_load_2d(d, &P.A, k0, m0, &full[sl]);
+        }
+      }
+      d += OPER;
+      if (BMN) {
+        tma_load_2d(d, &P.B, n0, k0, &full[sl]);
+        tma_load_2d(d + OPER / 2, &P.B, n0 + 64, k0, &full[sl]);
+      } else {
+        tma_load_2d(d, &P.B, k0, n0, &full[sl]);
+      }
+      issued = t + 1;
+    }
+    // every issued copy has landed before the CTA may exit
+    for (int t = issued > NS ? issued - NS : 0; t < issued; ++t)
+      if (!mbar_wait(&full[t % NS], static_cast<uint32_t>((t / NS) & 1), g.budget)) {
         flag_status(g.status, ST_TIMEOUT);
         ok = false;
       }
-    }
-    if (__syncthreads_or(!ok)) break;
-    if (nx < nkt) stage(nx);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group %0;" ::"n"(NS - 1) : "memory");  // tile nk has landed
-    fence_proxy_async_smem();
-    __syncthreads();
-    if (tid == 0) {
+  } else if (tid == 32) {
+    const uint32_t s0 = smem_u32(smem);
+    for (int t = 0; t < nkt; ++t) {
+      const int sl = t % NS;
+      if (!mbar_wait(&full[sl], static_cast<uint32_t>((t / NS) & 1), g.budget)) {
+        flag_status(g.status, ST_TIMEOUT);
+        ok = false;
+        break;
+      }
       tc_fence_after();
-      const int sl = nk % NS;
-      const uint32_t a = smem_u32(As + sl * A_STAGE), b = smem_u32(Bs + sl * B_STAGE);
+      const uint32_t a = s0 + static_cast<uint32_t>(sl) * STAGE, b = a + OPER;
 #pragma unroll
       for (int ks = 0; ks < GK / 16; ++ks) {
-        const uint64_t ad = umma_smem_desc(a + ks * 2 * (GM * 16), GM * 16, 128);
-        const uint64_t bd = umma_smem_desc(b + ks * 2 * (GN * 16), GN * 16, 128);
-        umma_bf16(tmem, ad, bd, idesc, (nk > 0 || ks > 0) ? 1u : 0u);
+        // 16 k: two words further into each line (K-major), two groups of
+        // eight lines further (MN-major)
+        const uint64_t ad = umma_smem_desc_sw128(a + ks * (AMN ? 2048u : 32u), OPER / 2, 1024);
+        const uint64_t bd = umma_smem_desc_sw128(b + ks * (BMN ? 2048u : 32u), OPER / 2, 1024);
+        umma_bf16(tmem, ad, bd, idesc, (t > 0 || ks > 0) ? 1u : 0u);
       }
-      tc_commit(&bar[sl]);
+      tc_commit(&empty[sl]);
     }
+    tc_commit(done);
   }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  // drain: the last tile's commit completes after every earlier MMA
-  if (ok && nkt > 0) {
-    const int tl = nkt - 1;
-    if (!mbar_wait(&bar[tl % NS], static_cast<uint32_t>((tl / NS) & 1), g.budget)) {
-      flag_status(g.status, ST_TIMEOUT);
-      ok = false;
-    }
+  __syncwarp();
+  if (!mbar_wait(done, 0, 2 * g.budget)) {
+    flag_status(g.status, ST_TIMEOUT);
+    ok = false;
   }
-  const int nk = nkt;
-  __syncthreads();
+  ok = !__syncthreads_or(!ok);
   tc_fence_after();
-  // Epilogue: each warp moves its 32 rows x 32 columns from TMEM through a
-  // padded shared-memory tile, so every global store writes 32 consecutive
-  // columns of one row (the operand stages are free once the MMAs are done).
-  float* stg = reinterpret_cast<float*>(smem) + warp * 32 * 33;
+  // ---- epilogue: thread = one row, 64 columns in two groups of 32 (TMEM lane
+  // quarter and column half of its warp).  A row's 32 values are whole 32-byte
+  // sectors, stored straight from the registers.
+  const int q4 = warp & 3, h = warp >> 2;
+  const int row = m0 + q4 * 32 + lane;
+  float* csum = reinterpret_cast<float*>(smem);  // [4][128] column sums of the quarters (the stages are free)
+  double* lsum = reinterpret_cast<double*>(smem + 4 * GN * 4);
   if (ok) {
-    for (int cb = 0; cb < GN; cb += 32) {
+    unsigned long long tgt = 0;  // EPI_BCE: bit c = column n0 + 64 h + c is a target of the row
+    float lh = 0.f, ll = 0.f;    // the row's loss, float-float
+    if (EPI == EPI_BCE && row < g.M) {
+      int nz = g.nnz[row];
+      nz = nz > g.s ? g.s : nz;
+#pragma unroll 4
+      for (int t = 0; t < nz; ++t) {
+        const int c = static_cast<int>(g.idx[static_cast<size_t>(row) * g.s + t]) - (n0 + 64 * h);
+        if (c >= 0 && c < 64) tgt |= 1ull << c;
+      }
+    }
+#pragma unroll 1
+    for (int cg = 0; cg < 2; ++cg) {
+      const int cb = h * 64 + cg * 32, col = n0 + cb;
       float v[32];
-      __syncwarp();
-      if (nk > 0) {
-        tmem_ld32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + cb, v);
+      if (nkt > 0) {
+        tmem_ld32(tmem + (static_cast<uint32_t>(q4 * 32) << 16) + cb, v);
       } else {
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = 0.f;
       }
+      if (EPI == EPI_PART) {
+        if (row < P.M && col < P.N)  // N is a multiple of 32
+          store_f32(P.C + blockIdx.y * g.zstride + static_cast<size_t>(row) * P.ldc + col, v);
+        continue;
+      }
+      if (EPI == EPI_GELU) {
 #pragma unroll
-      for (int k = 0; k < 32; ++k) stg[lane * 33 + k] = v[k];
-      __syncwarp();
-      const int col = n0 + cb + lane;
-      const float bcol = (g.epi != EPI_STORE && col < g.N) ? g.bias[col] : 0.f;
-      for (int r = 0; r < 32; ++r) {
-        const int row = m0 + warp * 32 + r;
-        if (row < g.M && col < g.N) {
-          const float z = add_bias(stg[r * 33 + lane], bcol);
-          if (g.C)
-            g.C[static_cast<long long>(blockIdx.z) * g.zstride + static_cast<long long>(row) * g.ldc + col] = z;
-          if (g.epi == EPI_BIAS_GELU)
-            g.H[static_cast<long long>(row) * g.ldh + col] = __float2bfloat16(gelu_f(z));
+        for (int k = 0; k < 32; ++k) v[k] = add_bias(v[k], __ldg(g.bias + col + k));
+        if (row < g.M) {
+          store_f32(P.C + static_cast<size_t>(row) * P.ldc + col, v);
+#pragma unroll
+          for (int k = 0; k < 32; ++k) v[k] = gelu_f(v[k]);
+          store_bf16(g.H + static_cast<size_t>(row) * g.ldh + col, v);
+        }
+        continue;
+      }
+      if (EPI == EPI_BCE) {
+        // BCE(z, y) = max(y ? -z : z, 0) + log(1 + e^-|z|); the group's logs are
+        // taken once, of the float-float product of its 1 + e^-|z| (at most
+        // 2^32), each 1 + e^-|z| exact as a pair.  1 / (1 + e^-z) is the
+        // hardware reciprocal after one Newton step.
+        const unsigned y32 = static_cast<unsigned>(tgt >> (32 * cg));
+        float ph = 1.f, pl = 0.f;
+        auto elem = [&](int k, float bias) {
+          const float z = add_bias(v[k], bias);
+          const bool y = (y32 >> k) & 1u;
+          const float e = expf(-z), d = fminf(1.f + e, 1e37f);
+          float r = rcp_approx(d);
+          r = fmaf(r, fmaf(-d, r, 1.f), r);
+          v[k] = (r - (y ? 1.f : 0.f)) * g.inv_bk;
+          const float q = z < 0.f ? rcp_approx(e) : e;  // e^-|z|
+          const float f = 1.f + q, fl = q - (f - 1.f);
+          const float np = ph * f;
+          pl = fmaf(pl, f, fmaf(ph, fl, fmaf(ph, f, -np)));
+          ph = np;
+          const float lz = fmaxf(y ? -z : z, 0.f);
+          const float t = lh + lz, bb = t - lh;
+          ll += (lh - (t - bb)) + (lz - bb);
+          lh = t;
+        };
+        if (row < g.M && col + 32 <= P.N) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) elem(k, __ldg(g.bias + col + k));
+        } else {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) {
+            if (row < g.M && col + k < P.N) elem(k, __ldg(g.bias + col + k));
+            else v[k] = 0.f;
+          }
+        }
+        ll += logf(ph) + __fdividef(pl, ph);
+      } else {
+        float4 z4[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          z4[k] = row < g.M ? *reinterpret_cast<const float4*>(g.Z + static_cast<size_t>(row) * HID + col + 4 * k)
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          v[4 * k + 0] *= gelu_grad_f(z4[k].x);
+          v[4 * k + 1] *= gelu_grad_f(z4[k].y);
+          v[4 * k + 2] *= gelu_grad_f(z4[k].z);
+          v[4 * k + 3] *= gelu_grad_f(z4[k].w);
         }
       }
+      if (row < g.M && col < g.ldh) store_bf16(g.H + static_cast<size_t>(row) * g.ldh + col, v);
+      csum[q4 * GN + cb + lane] = col_sums(v);
+    }
+    if (EPI == EPI_BCE) {
+      double l = static_cast<double>(lh) + static_cast<double>(ll);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (lane == 0) lsum[warp] = l;
     }
   }
   tc_fence_before();
   __syncthreads();
+  if (ok && (EPI == EPI_BCE || EPI == EPI_GELU_BWD)) {
+    if (tid < GN && n0 + tid < g.ldh)
+      g.colpart[static_cast<size_t>(tm) * g.ldh + n0 + tid] =
+          (csum[tid] + csum[GN + tid]) + (csum[2 * GN + tid] + csum[3 * GN + tid]);
+    if (EPI == EPI_BCE && tid == 0) {
+      double l = 0.0;
+      for (int w = 0; w < GT / 32; ++w) l += lsum[w];
+      g.loss_part[blockIdx.x] = l;
+    }
+  }
   if (warp == 0) {
     tc_fence_after();
     tmem_dealloc(tmem, GN);
   }
 }
 
-}  // namespace mlp
-}  // namespace dlsh
+// ---- gradients from the partials, and Adam -------------------------------------
+struct ReduceArgs {
+  const float* part;  // [splits][zstride] weight gradients at their parameter offsets
+  long long zstride;
+  int splits;
+  const float* cp1;   // column sums per 128-row tile (bias gradients): [tiles][256], [tiles][256], [tiles][ldk]
+  const float* cp2;
+  const float* cp3;
+  int tiles, ldk;
+  const double* loss_part;
+  int nloss;
+  double inv_bk;
+  float* loss;        // may be NULL
+  float* G;           // gradients out (ADAM = false)
+  Blob b;             // parameters and moments (ADAM = true)
+  Layout L;
+  float lr, beta1, beta2, eps, bc1, bc2;
+};
 
-namespace dlsh {
-namespace mlp {
-
-// ---- input: xn = x / ||x|| (0 if x = 0), padded to 64 columns, BF16 ---------
-__global__ void normalize_kernel(const float* __restrict__ X, long long n, __nv_bfloat16* __restrict__ Xn) {
-  const long long i = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (i >= n) return;
-  const float x0 = X[i * DLSH_D + lane];
-  const float x1 = lane < DLSH_D - 32 ? X[i * DLSH_D + 32 + lane] : 0.f;
-  __nv_bfloat16 y0, y1;
-  normalise_pair(x0, x1, y0, y1);
-  Xn[i * XIN + lane] = y0;
-  Xn[i * XIN + 32 + lane] = y1;
-}
-
-// ---- BCE-with-logits gradient (mean over B*K) and per-row loss ----------------
-// dZ (FP32, in place of Z) and a BF16 copy; y = 1 on the row's support atoms.
-__global__ void bce_grad_kernel(float* __restrict__ Z, __nv_bfloat16* __restrict__ dZb, int K,
-                                const uint16_t* __restrict__ idx, const uint8_t* __restrict__ nnz,
-                                int s, float inv_bk, double* __restrict__ row_loss) {
-  __shared__ double red[256];
-  __shared__ int sup[32];
-  __shared__ int nz_s;
-  const long long b = blockIdx.x;
-  if (threadIdx.x == 0) nz_s = nnz[b] > s ? s : nnz[b];
-  if (static_cast<int>(threadIdx.x) < s) sup[threadIdx.x] = idx[b * s + threadIdx.x];
-  __syncthreads();
-  const int nz = nz_s;
-  double acc = 0.0;
-  float* zr = Z + b * K;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const float z = zr[k];
-    bool y = false;
-    for (int t = 0; t < nz; ++t) y |= (sup[t] == k);
-    const float sg = 1.f / (1.f + expf(-z));
-    const float g = (sg - (y ? 1.f : 0.f)) * inv_bk;
-    acc += static_cast<double>(fmaxf(z, 0.f) - (y ? z : 0.f) + log1pf(expf(-fabsf(z))));
-    zr[k] = g;
-    dZb[b * K + k] = __float2bfloat16(g);
-  }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (static_cast<int>(threadIdx.x) < w) red[threadIdx.x] += red[threadIdx.x + w];
+template <bool ADAM>
+__global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ ReduceArgs a) {
+  if (blockIdx.x == gridDim.x - 1) {  // the last block: the mean loss, a fixed-order sum
+    __shared__ double red[256];
+    double acc = 0.0;
+    for (int q = threadIdx.x; q < a.nloss; q += 256) acc += a.loss_part[q];
+    red[threadIdx.x] = acc;
     __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if (static_cast<int>(threadIdx.x) < w) red[threadIdx.x] += red[threadIdx.x + w];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0 && a.loss) *a.loss = static_cast<float>(red[0] * a.inv_bk);
+    return;
   }
-  if (threadIdx.x == 0) row_loss[b] = red[0];
-}
-
-// mean loss = sum(row_loss) / (B K), fixed-order reduction
-__global__ void loss_kernel(const double* __restrict__ row_loss, int B, double inv_bk, float* out) {
-  __shared__ double red[1024];
-  double acc = 0.0;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) acc += row_loss[b];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if (static_cast<int>(threadIdx.x) < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
+  if (i >= a.L.n) return;
+  const float* src = a.part + i;
+  long long stride = a.zstride;
+  int n = a.splits;
+  if (i >= a.L.b3) {
+    src = a.cp3 + (i - a.L.b3);
+    stride = a.ldk;
+    n = a.tiles;
+  } else if (i >= a.L.b2 && i < a.L.W3) {
+    src = a.cp2 + (i - a.L.b2);
+    stride = HID;
+    n = a.tiles;
+  } else if (i >= a.L.b1 && i < a.L.W2) {
+    src = a.cp1 + (i - a.L.b1);
+    stride = HID;
+    n = a.tiles;
   }
-  if (threadIdx.x == 0) *out = static_cast<float>(red[0] * inv_bk);
-}
-
-// dZ = dH * gelu'(Z) (FP32 in place of dH) and a BF16 copy
-__global__ void gelu_bwd_kernel(float* __restrict__ dH, const float* __restrict__ Z,
-                                __nv_bfloat16* __restrict__ dZb, long long n) {
-  const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float g = dH[i] * gelu_grad_f(Z[i]);
-  dH[i] = g;
-  dZb[i] = __float2bfloat16(g);
-}
-
-// column sums of an R x C FP32 matrix, two levels in a fixed order
-constexpr int CS_ROWS = 256;
-__global__ void colsum_partial_kernel(const float* __restrict__ A, int R, int C,
-                                      float* __restrict__ part) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  const int r0 = blockIdx.y * CS_ROWS;
-  if (c >= C) return;
-  float acc = 0.f;
-  for (int r = r0; r < r0 + CS_ROWS && r < R; ++r) acc += A[static_cast<long long>(r) * C + c];
-  part[static_cast<long long>(blockIdx.y) * C + c] = acc;
-}
-__global__ void colsum_final_kernel(const float* __restrict__ part, int nparts, int C,
-                                    float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
-  float acc = 0.f;
-  for (int p = 0; p < nparts; ++p) acc += part[static_cast<long long>(p) * C + c];
-  out[c] = acc;
-}
-
-// out[i] = sum_z part[z][i] (split-K reduction in a fixed order)
-__global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits, long long n,
-                                     float* __restrict__ out) {
-  const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float acc = 0.f;
-  for (int z = 0; z < splits; ++z) acc += part[static_cast<long long>(z) * n + i];
-  out[i] = acc;
-}
-
-// Adam on every parameter; refreshes the BF16 mirror.
-__global__ void adam_kernel(float* __restrict__ P, float* __restrict__ m1, float* __restrict__ m2,
-                            __nv_bfloat16* __restrict__ Pb, const float* __restrict__ G, long long n,
-                            float lr, float beta1, float beta2, float eps, float bc1, float bc2) {
-  const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float g = G[i];
-  const float a = beta1 * m1[i] + (1.f - beta1) * g;
-  const float v = beta2 * m2[i] + (1.f - beta2) * g * g;
-  m1[i] = a;
-  m2[i] = v;
-  const float p = P[i] - lr * (a / bc1) / (sqrtf(v / bc2) + eps);
-  P[i] = p;
-  Pb[i] = __float2bfloat16(p);
+  float g = 0.f;
+#pragma unroll 8
+  for (int z = 0; z < n; ++z) g += src[z * stride];
+  if (!ADAM) {
+    a.G[i] = g;
+    return;
+  }
+  const float m = a.beta1 * a.b.m1[i] + (1.f - a.beta1) * g;
+  const float v = a.beta2 * a.b.m2[i] + (1.f - a.beta2) * g * g;
+  a.b.m1[i] = m;
+  a.b.m2[i] = v;
+  const float p = a.b.P[i] - a.lr * (m / a.bc1) / (sqrtf(v / a.bc2) + a.eps);
+  a.b.P[i] = p;
+  a.b.Pb[i] = __float2bfloat16(p);
 }
 
 __global__ void mirror_kernel(const float* __restrict__ P, __nv_bfloat16* __restrict__ Pb, long long n) {
@@ -371,68 +471,54 @@ __global__ void mirror_kernel(const float* __restrict__ P, __nv_bfloat16* __rest
 namespace dlsh {
 namespace mlp {
 
-constexpr int SPLIT_K = 1024;  // batch rows per split of the weight-gradient GEMMs
+// cuTensorMapEncodeTiled, taken from the driver at run time
+using PFN_encodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                     const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-static int gemm(const Mat& A, const Mat& B, int M, int N, int Kd, float* C, long long ldc, int epi,
-                const float* bias, __nv_bfloat16* H, long long ldh, int splits, long long zstride,
-                uint32_t* status, cudaStream_t st) {
-  static PerDevice<int> attr;
-  int attr_ok = 0;
-  const int arc = attr.get(&attr_ok, [](int& v) {
-    DLSH_CUDA_TRY(cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       NS * (A_STAGE + B_STAGE) + 64),
-                  "dlsh_mlp: attribute");
-    v = 1;
-    return DLSH_OK;
-  });
-  if (arc) return arc;
-  GemmArgs g;
-  g.A = A;
-  g.B = B;
-  g.M = M;
-  g.N = N;
-  g.Kd = Kd;
-  const int kt = (Kd + GK - 1) / GK;
-  const int per = (kt + splits - 1) / splits;
-  g.klen = per * GK;
-  g.C = C;
-  g.ldc = ldc;
-  g.zstride = zstride;
-  g.bias = bias;
-  g.H = H;
-  g.ldh = ldh;
-  g.epi = epi;
-  g.status = status;
-  g.budget = kWaitBudget;
-  dim3 grid((N + GN - 1) / GN, (M + GM - 1) / GM, splits);
-  gemm_kernel<<<grid, GT, NS * (A_STAGE + B_STAGE) + 64, st>>>(g);
-  count_launches(1);
-  return check_launch("dlsh_mlp: gemm");
-}
+constexpr int kSms = 152;  // SMs of a GB300
 
-// Training / forward workspace for batches of up to B rows.
+// Training workspace for batches of up to B rows.
 struct TWs {
   uint32_t* status;
-  __nv_bfloat16* Xn;   // B x 64
-  float* Z1;           // B x 256 (then dZ1)
-  float* Z2;           // B x 256 (then dZ2)
-  __nv_bfloat16* H1;   // B x 256
-  __nv_bfloat16* H2;   // B x 256
-  float* Z3;           // B x K (logits, then dZ3)
-  __nv_bfloat16* dZ3b; // B x K
-  float* dH;           // B x 256 (dH2 / dH1)
-  __nv_bfloat16* dZb;  // B x 256
-  float* part;         // split-K partials / column-sum partials
-  float* grads;        // parameter gradients
-  double* row_loss;    // B
-  float* loss;         // 1
+  __nv_bfloat16* Xn;    // B x 64
+  float* Z1;            // B x 256 pre-activations
+  float* Z2;
+  __nv_bfloat16* H1;    // B x 256 activations
+  __nv_bfloat16* H2;
+  __nv_bfloat16* dZ1;   // B x 256
+  __nv_bfloat16* dZ2;
+  __nv_bfloat16* dZ3;   // B x ldk (zeros past K)
+  float* part;          // splits x zstride weight-gradient partials
+  float* cp1;           // column sums per 128-row tile
+  float* cp2;
+  float* cp3;
+  double* loss_part;    // one per CTA of the logits product
+  int ldk;
+  int splits, klen;     // split of the batch in the weight gradients
+  int tiles_m, tiles_w;
+  long long zstride;
 };
+
+// Batch split of the weight gradients: their 128 x 128 tiles (22 at K = 1024)
+// times the splits fill two CTAs per SM once, each split at least four k-tiles
+// long (shorter ones are mostly prologue and epilogue).
+static void split_batch(int K, long long B, TWs& w) {
+  w.tiles_m = static_cast<int>((B + GM - 1) / GM);
+  w.tiles_w = ((K + GM - 1) / GM) * (HID / GN) + (HID / GM) * (HID / GN) + HID / GM;
+  const long long kt = (B + GK - 1) / GK;
+  long long splits = 2LL * kSms / w.tiles_w;
+  splits = std::max<long long>(1, std::min<long long>(splits, kt / 4));
+  const long long per = (kt + splits - 1) / splits;
+  w.klen = static_cast<int>(per * GK);
+  w.splits = static_cast<int>((kt + per - 1) / per);
+}
 
 static size_t carve_t(void* base, int K, long long B, TWs& w) {
   const Layout L = layout(K);
-  const long long splits = (B + SPLIT_K - 1) / SPLIT_K;
-  const long long part = std::max<long long>(splits * std::max<long long>(static_cast<long long>(K) * HID, HID * HID),
-                                             ((B + CS_ROWS - 1) / CS_ROWS) * std::max(K, HID));
+  split_batch(K, B, w);
+  w.ldk = (K + 63) / 64 * 64;
+  w.zstride = (L.n + 63) / 64 * 64;
   Carver c(base);
   w.status = c.take<uint32_t>(64);
   w.Xn = c.take<__nv_bfloat16>(B * XIN);
@@ -440,105 +526,223 @@ static size_t carve_t(void* base, int K, long long B, TWs& w) {
   w.Z2 = c.take<float>(B * HID);
   w.H1 = c.take<__nv_bfloat16>(B * HID);
   w.H2 = c.take<__nv_bfloat16>(B * HID);
-  w.Z3 = c.take<float>(B * K);
-  w.dZ3b = c.take<__nv_bfloat16>(B * K);
-  w.dH = c.take<float>(B * HID);
-  w.dZb = c.take<__nv_bfloat16>(B * HID);
-  w.part = c.take<float>(part);
-  w.grads = c.take<float>(L.n);
-  w.row_loss = c.take<double>(B);
-  w.loss = c.take<float>(4);
+  w.dZ1 = c.take<__nv_bfloat16>(B * HID);
+  w.dZ2 = c.take<__nv_bfloat16>(B * HID);
+  w.dZ3 = c.take<__nv_bfloat16>(B * w.ldk);
+  w.part = c.take<float>(w.zstride * w.splits);
+  w.cp1 = c.take<float>(static_cast<size_t>(w.tiles_m) * HID);
+  w.cp2 = c.take<float>(static_cast<size_t>(w.tiles_m) * HID);
+  w.cp3 = c.take<float>(static_cast<size_t>(w.tiles_m) * w.ldk);
+  w.loss_part = c.take<double>(static_cast<size_t>(w.tiles_m) * ((K + GN - 1) / GN));
   return c.size();
 }
 
-static inline Mat rowmajor(const __nv_bfloat16* p, long long ld) { return Mat{p, ld, 1}; }
-static inline Mat transposed(const __nv_bfloat16* p, long long ld) { return Mat{p, 1, ld}; }
+// A BF16 matrix of `lines` lines of `inner` elements (line stride ld elements,
+// a multiple of 8) as a 128-byte-swizzled tensor map with boxes of 64 elements
+// x box_lines lines.
+static int tensor_map(CUtensorMap* m, const __nv_bfloat16* p, int inner, int lines, int ld, int box_lines) {
+  static PerDevice<PFN_encodeTiled> entry;
+  PFN_encodeTiled enc = nullptr;
+  const int rc = entry.get(&enc, [](PFN_encodeTiled& v) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    DLSH_CUDA_TRY(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q),
+                  "dlsh_mlp: cuTensorMapEncodeTiled");
+    if (!f || q != cudaDriverEntryPointSuccess)
+      return set_error(DLSH_ERR_CUDA, "dlsh_mlp: the driver has no cuTensorMapEncodeTiled");
+    v = reinterpret_cast<PFN_encodeTiled>(f);
+    return DLSH_OK;
+  });
+  if (rc) return rc;
+  const cuuint64_t dim[2] = {static_cast<cuuint64_t>(inner), static_cast<cuuint64_t>(lines)};
+  const cuuint64_t stride[1] = {static_cast<cuuint64_t>(ld) * 2};
+  const cuuint32_t box[2] = {64, static_cast<cuuint32_t>(box_lines)};
+  const cuuint32_t one[2] = {1, 1};
+  const CUresult e = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(p), dim, stride, box, one,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (e != CUDA_SUCCESS)
+    return set_error(DLSH_ERR_CUDA, "dlsh_mlp: tensor map of %d x %d: error %d", lines, inner, static_cast<int>(e));
+  return DLSH_OK;
+}
+// rows x k operands: K-major (rows are the lines) and MN-major (k are the lines)
+static int kmajor(CUtensorMap* m, const __nv_bfloat16* p, int rows, int k, int ld) {
+  return tensor_map(m, p, k, rows, ld, GM);
+}
+static int mnmajor(CUtensorMap* m, const __nv_bfloat16* p, int rows, int k, int ld) {
+  return tensor_map(m, p, rows, k, ld, GK);
+}
 
-// Training forward through the three layers: logits in w.Z3 (B x K), hidden
-// pre-activations in w.Z1 / w.Z2 for the backward pass.
-static int forward(const Blob& b, int K, const float* X, long long B, const TWs& w, cudaStream_t st) {
+template <int EPI, bool AMN, bool BMN, bool XA, int NS>
+static int launch_gemm_ns(const GemmArgs& g, int tiles, int splits, cudaStream_t st) {
+  static PerDevice<int> attr;
+  int attr_ok = 0;
+  const int arc = attr.get(&attr_ok, [](int& v) {
+    DLSH_CUDA_TRY(cudaFuncSetAttribute(train_gemm_kernel<EPI, AMN, BMN, XA, NS>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(NS)),
+                  "dlsh_mlp: attribute");
+    v = 1;
+    return DLSH_OK;
+  });
+  if (arc) return arc;
+  train_gemm_kernel<EPI, AMN, BMN, XA, NS><<<dim3(tiles, splits), GT, gemm_smem(NS), st>>>(g);
+  count_launches(1);
+  return check_launch("dlsh_mlp: gemm");
+}
+
+template <int EPI, bool AMN, bool BMN, bool XA>
+static int launch_gemm(const GemmArgs& g, int tiles, int splits, cudaStream_t st) {
+  // one k-tile (XA) needs no depth; the logits' and the weight gradients' grids
+  // give two CTAs per SM but on the smallest batches
+  if constexpr (!XA && (EPI == EPI_GELU || EPI == EPI_GELU_BWD))
+    if (tiles <= kSms) return launch_gemm_ns<EPI, AMN, BMN, XA, 6>(g, tiles, splits, st);
+  return launch_gemm_ns<EPI, AMN, BMN, XA, 3>(g, tiles, splits, st);
+}
+
+// The products of a training step on batches of M rows in the workspace w,
+// tensor maps included: built once per call, whatever the number of steps.
+struct Plan {
+  GemmArgs l1, l2, l3, d2, d1, wg;
+};
+static int make_plan(const Blob& b, int K, int M, const TWs& w, int s, Plan& t) {
   const Layout L = layout(K);
-  normalize_kernel<<<static_cast<int>((B + 7) / 8), 256, 0, st>>>(X, B, w.Xn);
-  count_launches(1);
-  int rc = gemm(rowmajor(w.Xn, XIN), rowmajor(b.Pb + L.W1, XIN), B, HID, XIN,
-                w.Z1, HID, EPI_BIAS_GELU, b.P + L.b1, w.H1, HID, 1, 0,
-                w.status, st);
-  if (rc) return rc;
-  rc = gemm(rowmajor(w.H1, HID), rowmajor(b.Pb + L.W2, HID), B, HID, HID, w.Z2,
-            HID, EPI_BIAS_GELU, b.P + L.b2, w.H2, HID, 1, 0, w.status, st);
-  if (rc) return rc;
-  return gemm(rowmajor(w.H2, HID), rowmajor(b.Pb + L.W3, HID), B, K, HID, w.Z3, K, EPI_BIAS,
-              b.P + L.b3, nullptr, 0, 1, 0, w.status, st);
+  GemmArgs g{};
+  g.nprod = 1;
+  g.M = M;
+  g.s = s;
+  g.inv_bk = static_cast<float>(1.0 / (static_cast<double>(M) * K));
+  g.status = w.status;
+  g.budget = kWaitBudget;
+  t.l1 = t.l2 = t.l3 = t.d2 = t.d1 = t.wg = g;
+  auto prod = [&](GemmArgs& a, int q, int Mr, int N, int Kd, float* C, int ldc) {
+    Prod& p = a.p[q];
+    p.M = Mr;
+    p.N = N;
+    p.Kd = Kd;
+    p.tiles_n = (N + GN - 1) / GN;
+    p.tile0 = q ? a.p[q - 1].tile0 + (a.p[q - 1].M + GM - 1) / GM * a.p[q - 1].tiles_n : 0;
+    p.C = C;
+    p.ldc = ldc;
+    a.klen = (Kd + GK - 1) / GK * GK;
+  };
+  int rc = DLSH_OK;
+  auto map = [&](int r) { rc = rc ? rc : r; };
+  // layer 1 (A: the signals, normalised as they are staged) and layer 2
+  prod(t.l1, 0, M, HID, XIN, w.Z1, HID);
+  map(kmajor(&t.l1.p[0].B, b.Pb + L.W1, HID, XIN, XIN));
+  t.l1.Xn = w.Xn;
+  t.l1.bias = b.P + L.b1;
+  t.l1.H = w.H1;
+  t.l1.ldh = HID;
+  prod(t.l2, 0, M, HID, HID, w.Z2, HID);
+  map(kmajor(&t.l2.p[0].A, w.H1, M, HID, HID));
+  map(kmajor(&t.l2.p[0].B, b.Pb + L.W2, HID, HID, HID));
+  t.l2.bias = b.P + L.b2;
+  t.l2.H = w.H2;
+  t.l2.ldh = HID;
+  // logits -> dZ3, column sums (b3) and loss
+  prod(t.l3, 0, M, K, HID, nullptr, 0);
+  map(kmajor(&t.l3.p[0].A, w.H2, M, HID, HID));
+  map(kmajor(&t.l3.p[0].B, b.Pb + L.W3, K, HID, HID));
+  t.l3.bias = b.P + L.b3;
+  t.l3.H = w.dZ3;
+  t.l3.ldh = w.ldk;
+  t.l3.colpart = w.cp3;
+  t.l3.loss_part = w.loss_part;
+  // dZ2 = (dZ3 W3) * gelu'(Z2), dZ1 = (dZ2 W2) * gelu'(Z1); the weights are
+  // read MN-major (their rows are the k of these products)
+  prod(t.d2, 0, M, HID, K, nullptr, 0);
+  map(kmajor(&t.d2.p[0].A, w.dZ3, M, w.ldk, w.ldk));
+  map(mnmajor(&t.d2.p[0].B, b.Pb + L.W3, HID, K, HID));
+  t.d2.Z = w.Z2;
+  t.d2.H = w.dZ2;
+  t.d2.ldh = HID;
+  t.d2.colpart = w.cp2;
+  prod(t.d1, 0, M, HID, HID, nullptr, 0);
+  map(kmajor(&t.d1.p[0].A, w.dZ2, M, HID, HID));
+  map(mnmajor(&t.d1.p[0].B, b.Pb + L.W2, HID, HID, HID));
+  t.d1.Z = w.Z1;
+  t.d1.H = w.dZ1;
+  t.d1.ldh = HID;
+  t.d1.colpart = w.cp1;
+  // dW = dZ^T A_in of the three layers, both operands MN-major (k = the batch)
+  t.wg.nprod = 3;
+  prod(t.wg, 0, K, HID, M, w.part + L.W3, HID);
+  map(mnmajor(&t.wg.p[0].A, w.dZ3, w.ldk, M, w.ldk));
+  map(mnmajor(&t.wg.p[0].B, w.H2, HID, M, HID));
+  prod(t.wg, 1, HID, HID, M, w.part + L.W2, HID);
+  map(mnmajor(&t.wg.p[1].A, w.dZ2, HID, M, HID));
+  map(mnmajor(&t.wg.p[1].B, w.H1, HID, M, HID));
+  prod(t.wg, 2, HID, XIN, M, w.part + L.W1, XIN);
+  map(mnmajor(&t.wg.p[2].A, w.dZ1, HID, M, HID));
+  map(mnmajor(&t.wg.p[2].B, w.Xn, XIN, M, XIN));
+  t.wg.klen = w.klen;
+  t.wg.zstride = w.zstride;
+  return rc;
 }
 
-static int colsum(const float* A, int R, int C, float* out, float* part, cudaStream_t st) {
-  const int parts = (R + CS_ROWS - 1) / CS_ROWS;
-  colsum_partial_kernel<<<dim3((C + 255) / 256, parts), 256, 0, st>>>(A, R, C, part);
-  colsum_final_kernel<<<(C + 255) / 256, 256, 0, st>>>(part, parts, C, out);
-  count_launches(2);
-  return check_launch("dlsh_mlp: colsum");
+// Forward and backward of one batch: weight-gradient partials, column sums and
+// loss sums in the workspace.
+static int backward(Plan& t, const float* X, const uint16_t* idx, const uint8_t* nnz, const TWs& w,
+                    cudaStream_t st) {
+  t.l1.X = X;
+  t.l3.idx = idx;
+  t.l3.nnz = nnz;
+  auto tiles = [&](const GemmArgs& g) { return g.p[0].tiles_n * w.tiles_m; };
+  int rc = launch_gemm<EPI_GELU, false, false, true>(t.l1, tiles(t.l1), 1, st);
+  if (!rc) rc = launch_gemm<EPI_GELU, false, false, false>(t.l2, tiles(t.l2), 1, st);
+  if (!rc) rc = launch_gemm<EPI_BCE, false, false, false>(t.l3, tiles(t.l3), 1, st);
+  if (!rc) rc = launch_gemm<EPI_GELU_BWD, false, true, false>(t.d2, tiles(t.d2), 1, st);
+  if (!rc) rc = launch_gemm<EPI_GELU_BWD, false, true, false>(t.d1, tiles(t.d1), 1, st);
+  if (!rc) rc = launch_gemm<EPI_PART, true, true, false>(t.wg, w.tiles_w, w.splits, st);
+  return rc;
 }
 
-// dW = dZ^T A_in over the batch (split-K, reduced in a fixed order)
-static int weight_grad(const __nv_bfloat16* dZb, int Nout, const __nv_bfloat16* Ain, int Nin,
-                       long long B, float* out, float* part, uint32_t* status, cudaStream_t st) {
-  const int splits = static_cast<int>((B + SPLIT_K - 1) / SPLIT_K);
-  const long long n = static_cast<long long>(Nout) * Nin;
-  int rc = gemm(transposed(dZb, Nout), transposed(Ain, Nin), Nout, Nin, static_cast<int>(B), part,
-                Nin, EPI_STORE, nullptr, nullptr, 0, splits, n, status, st);
-  if (rc) return rc;
-  splitk_reduce_kernel<<<static_cast<int>((n + 255) / 256), 256, 0, st>>>(part, splits, n, out);
-  count_launches(1);
-  return check_launch("dlsh_mlp: split-K reduce");
+static ReduceArgs reduce_args(int K, long long B, const TWs& w, float* loss) {
+  ReduceArgs a{};
+  a.part = w.part;
+  a.zstride = w.zstride;
+  a.splits = w.splits;
+  a.cp1 = w.cp1;
+  a.cp2 = w.cp2;
+  a.cp3 = w.cp3;
+  a.tiles = w.tiles_m;
+  a.ldk = w.ldk;
+  a.loss_part = w.loss_part;
+  a.nloss = w.tiles_m * ((K + GN - 1) / GN);
+  a.inv_bk = 1.0 / (static_cast<double>(B) * K);
+  a.loss = loss;
+  a.L = layout(K);
+  return a;
 }
 
-// forward + backward: parameter gradients in w.grads, mean loss in w.loss
-static int gradients(const Blob& b, int K, const float* X, long long B, const uint16_t* idx,
-                     const uint8_t* nnz, int s, const TWs& w, cudaStream_t st) {
-  const Layout L = layout(K);
-  int rc = forward(b, K, X, B, w, st);
+// Gradients of the batch's mean loss into grads, the loss into *loss (device,
+// may be NULL).
+static int gradients(Plan& t, int K, const float* X, long long B, const uint16_t* idx, const uint8_t* nnz,
+                     const TWs& w, float* grads, float* loss, cudaStream_t st) {
+  const int rc = backward(t, X, idx, nnz, w, st);
   if (rc) return rc;
-  const float inv_bk = static_cast<float>(1.0 / (static_cast<double>(B) * K));
-  bce_grad_kernel<<<static_cast<int>(B), 256, 0, st>>>(w.Z3, w.dZ3b, K, idx, nnz, s, inv_bk,
-                                                       w.row_loss);
-  loss_kernel<<<1, 1024, 0, st>>>(w.row_loss, static_cast<int>(B), 1.0 / (static_cast<double>(B) * K),
-                                  w.loss);
-  count_launches(2);
-  // layer 3
-  rc = weight_grad(w.dZ3b, K, w.H2, HID, B, w.grads + L.W3, w.part, w.status, st);
-  if (rc) return rc;
-  rc = colsum(w.Z3, static_cast<int>(B), K, w.grads + L.b3, w.part, st);
-  if (rc) return rc;
-  rc = gemm(rowmajor(w.dZ3b, K), transposed(b.Pb + L.W3, HID), B, HID, K, w.dH, HID, EPI_STORE,
-            nullptr, nullptr, 0, 1, 0, w.status, st);
-  if (rc) return rc;
-  const long long nh = B * HID;
-  gelu_bwd_kernel<<<static_cast<int>((nh + 255) / 256), 256, 0, st>>>(w.dH, w.Z2, w.dZb, nh);
+  ReduceArgs a = reduce_args(K, B, w, loss);
+  a.G = grads;
+  reduce_kernel<false><<<static_cast<int>((a.L.n + 255) / 256) + 1, 256, 0, st>>>(a);
   count_launches(1);
-  // layer 2 (dZ2 now in w.dH / w.dZb)
-  rc = weight_grad(w.dZb, HID, w.H1, HID, B, w.grads + L.W2, w.part, w.status, st);
-  if (rc) return rc;
-  rc = colsum(w.dH, static_cast<int>(B), HID, w.grads + L.b2, w.part, st);
-  if (rc) return rc;
-  rc = gemm(rowmajor(w.dZb, HID), transposed(b.Pb + L.W2, HID), B, HID, HID, w.Z2, HID, EPI_STORE,
-            nullptr, nullptr, 0, 1, 0, w.status, st);  // dH1 into the Z2 buffer (no longer needed)
-  if (rc) return rc;
-  gelu_bwd_kernel<<<static_cast<int>((nh + 255) / 256), 256, 0, st>>>(w.Z2, w.Z1, w.dZb, nh);
-  count_launches(1);
-  // layer 1 (dZ1 now in w.Z2 / w.dZb)
-  rc = weight_grad(w.dZb, HID, w.Xn, XIN, B, w.grads + L.W1, w.part, w.status, st);
-  if (rc) return rc;
-  return colsum(w.Z2, static_cast<int>(B), HID, w.grads + L.b1, w.part, st);
+  return check_launch("dlsh_mlp: reduce");
 }
 
-static int adam(const Blob& b, int K, const float* grads, float lr, long long step,
-                cudaStream_t st) {
-  const Layout L = layout(K);
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float bc1 = static_cast<float>(1.0 - pow(0.9, static_cast<double>(step)));
-  const float bc2 = static_cast<float>(1.0 - pow(0.999, static_cast<double>(step)));
-  adam_kernel<<<static_cast<int>((L.n + 255) / 256), 256, 0, st>>>(b.P, b.m1, b.m2, b.Pb, grads, L.n, lr,
-                                                                    b1, b2, eps, bc1, bc2);
+// The same, followed by Adam's step number `step` (from 1).
+static int train_step(Plan& t, const Blob& b, int K, const float* X, long long B, const uint16_t* idx,
+                      const uint8_t* nnz, const TWs& w, float lr, long long step, float* loss, cudaStream_t st) {
+  const int rc = backward(t, X, idx, nnz, w, st);
+  if (rc) return rc;
+  ReduceArgs a = reduce_args(K, B, w, loss);
+  a.b = b;
+  a.lr = lr;
+  a.beta1 = 0.9f;
+  a.beta2 = 0.999f;
+  a.eps = 1e-8f;
+  a.bc1 = static_cast<float>(1.0 - pow(0.9, static_cast<double>(step)));
+  a.bc2 = static_cast<float>(1.0 - pow(0.999, static_cast<double>(step)));
+  reduce_kernel<true><<<static_cast<int>((a.L.n + 255) / 256) + 1, 256, 0, st>>>(a);
   count_launches(1);
   return check_launch("dlsh_mlp: adam");
 }
@@ -639,14 +843,11 @@ int dlsh_mlp_gradients(const void* mlp, int K, const float* X, int64_t B, const 
   mlp::TWs w;
   mlp::carve_t(ws, K, B, w);
   DLSH_CUDA_TRY(cudaMemsetAsync(w.status, 0, 4, st), "dlsh_mlp_gradients: reset");
-  rc = mlp::gradients(b, K, X, B, idx, nnz, s, w, st);
+  mlp::Plan plan;
+  rc = mlp::make_plan(b, K, static_cast<int>(B), w, s, plan);
   if (rc) return rc;
-  DLSH_CUDA_TRY(cudaMemcpyAsync(grads, w.grads, sizeof(float) * mlp::layout(K).n,
-                                cudaMemcpyDeviceToDevice, st),
-                "dlsh_mlp_gradients: copy");
-  if (loss)
-    DLSH_CUDA_TRY(cudaMemcpyAsync(loss, w.loss, sizeof(float), cudaMemcpyDeviceToDevice, st),
-                  "dlsh_mlp_gradients: loss");
+  rc = mlp::gradients(plan, K, X, B, idx, nnz, w, grads, loss, st);
+  if (rc) return rc;
   return finish(st, w.status, flags, "dlsh_mlp_gradients");
 }
 
@@ -665,13 +866,11 @@ int dlsh_mlp_train_step(void* mlp, int K, const float* X, int64_t B, const uint1
   mlp::TWs w;
   mlp::carve_t(ws, K, B, w);
   DLSH_CUDA_TRY(cudaMemsetAsync(w.status, 0, 4, st), "dlsh_mlp_train_step: reset");
-  rc = mlp::gradients(b, K, X, B, idx, nnz, s, w, st);
+  mlp::Plan plan;
+  rc = mlp::make_plan(b, K, static_cast<int>(B), w, s, plan);
   if (rc) return rc;
-  rc = mlp::adam(b, K, w.grads, lr, step, st);
+  rc = mlp::train_step(plan, b, K, X, B, idx, nnz, w, lr, step, loss, st);
   if (rc) return rc;
-  if (loss)
-    DLSH_CUDA_TRY(cudaMemcpyAsync(loss, w.loss, sizeof(float), cudaMemcpyDeviceToDevice, st),
-                  "dlsh_mlp_train_step: loss");
   return finish(st, w.status, flags, "dlsh_mlp_train_step");
 }
 
@@ -692,6 +891,9 @@ int dlsh_mlp_train(void* mlp, int K, const float* X, int64_t N, const uint16_t* 
   mlp::TWs w;
   mlp::carve_t(ws, K, batch, w);
   DLSH_CUDA_TRY(cudaMemsetAsync(w.status, 0, 4, st), "dlsh_mlp_train: reset");
+  mlp::Plan plan;
+  rc = mlp::make_plan(b, K, static_cast<int>(batch), w, s, plan);
+  if (rc) return rc;
   const long long per_epoch = N / batch;
   const long long total = per_epoch * epochs;
   long long step = 0;
@@ -702,14 +904,9 @@ int dlsh_mlp_train(void* mlp, int K, const float* X, int64_t N, const uint16_t* 
       const double frac = static_cast<double>(step - 1) / static_cast<double>(total);
       const float lr_t = static_cast<float>(0.5 * lr * (1.0 + cos(M_PI * frac)));
       const long long off = q * batch;
-      rc = mlp::gradients(b, K, X + off * DLSH_D, batch, idx + off * s, nnz + off, s, w, st);
+      rc = mlp::train_step(plan, b, K, X + off * DLSH_D, batch, idx + off * s, nnz + off, w, lr_t, step,
+                           loss_per_step ? loss_per_step + (step - 1) : nullptr, st);
       if (rc) return rc;
-      rc = mlp::adam(b, K, w.grads, lr_t, step, st);
-      if (rc) return rc;
-      if (loss_per_step)
-        DLSH_CUDA_TRY(cudaMemcpyAsync(loss_per_step + (step - 1), w.loss, sizeof(float),
-                                      cudaMemcpyDeviceToDevice, st),
-                      "dlsh_mlp_train: loss");
     }
   }
   return finish(st, w.status, flags, "dlsh_mlp_train");

@@ -89,6 +89,31 @@ def test_gradients_match_oracle(lib, B, K, s):
     assert np.abs(gd["W1"][:, 45:]).max() == 0.0
 
 
+@pytest.mark.parametrize("B,K,s", [(1, 8, 1), (127, 100, 3), (129, 271, 8), (300, 129, 16), (640, 1000, 5)])
+def test_gradients_ragged_shapes(lib, B, K, s):
+    """Batches around one tile of 128 rows and around the split of the weight
+    gradients (four k-tiles of 64), dictionaries that leave ragged tiles and rows
+    padded to 64 columns.  The GPU keeps activations and dZ in BF16 (2^-9
+    relative, a few roundings in a chain): 2e-2 in the norm, as above."""
+    p = _params(K, 60 + K)
+    X = synth.signals(B, synth.hidden_dictionary(max(K, 32), 61), 4, 62)
+    rng = np.random.default_rng(63)
+    idx = synth.distinct_supports(rng, B, K, s)
+    nnz = rng.integers(0, s + 1, B)
+    net = lib.MLP(K, p)
+    g, loss = net.gradients(torch.from_numpy(X), torch.from_numpy(idx.astype(np.int16)).cuda(),
+                            torch.from_numpy(nnz.astype(np.uint8)).cuda())
+    gd = lib.mlp_unpack(g, K)
+    gref, f = P.backward(_oracle_params_bf16(p), bf16(P.normalise_input(X)), P.support_targets(idx, nnz, K))
+    lref = float(P.bce_with_logits(f["z3"], P.support_targets(idx, nnz, K)).mean())
+    assert abs(loss - lref) <= 1e-3 * abs(lref)
+    for k in ("W3", "b3", "W2", "b2", "W1", "b1"):
+        got = gd[k][:, :45] if k == "W1" else gd[k]
+        rel, cos = _rel(got, gref[k])
+        assert rel < 2e-2 and cos > 0.999, (k, rel, cos)
+    assert np.abs(gd["W1"][:, 45:]).max() == 0.0
+
+
 def test_adam_step_matches_oracle(lib):
     K, B, s = 128, 512, 4
     p = _params(K, 8)
