@@ -7,17 +7,23 @@
 //
 // GPU design (deterministic, no floating-point atomics):
 //   1. count_kernel     per-tile atom histograms (integer counts)
-//   2. scan kernels     per-atom totals, atom offsets, per-(atom, tile) offsets
-//   3. scatter_kernel   one CTA per signal tile writes (signal, coef, nnz) into
-//                       the atom-major list in signal order (a counting sort)
-//   4. accum_kernel     one CTA per segment of an atom's list: row j of G
-//                       (entries k >= j; G is symmetric, and its lower
-//                       triangle is mirrored from the upper one after the
-//                       reduction) and column j of B.  Each warp owns a fixed slice, one list
-//                       entry per lane pair; sums are float-float (exact FMA
-//                       products, two-sum accumulation: about FP64 accuracy
-//                       on the FP32 pipe, since GB300's FP64 units are slow),
-//                       lanes and warps are added in a fixed order
+//   2. chunk_sum, layout, tile_offsets  per-atom totals, list offsets per
+//                       (chunk of tiles, atom) and per (tile, atom), and the
+//                       accumulation segments
+//   3. scatter_kernel   one CTA per signal tile sorts its entries by atom in
+//                       shared memory and writes (signal, coef, nnz) into the
+//                       atom-major list in signal order (a counting sort)
+//   4. accum_b_kernel, accum_g_kernel  column j of B and row j of G (entries
+//                       k >= j; G is symmetric, and its lower triangle is
+//                       mirrored from the upper one after the reduction), per
+//                       segment of an atom's list; the segments run in signal
+//                       order, so that what they gather stays in L2.  Sums are
+//                       float-float (exact FMA products, two-sum accumulation:
+//                       about FP64 accuracy on the FP32 pipe, since GB300's
+//                       FP64 units are slow), added up in a fixed order.
+//                       N = 3M, K = 1024, s = 8 (us): one kernel for both,
+//                       atom by atom, took 2326; now B 552 (L1 85 % busy,
+//                       9 TB/s of L2 reads) and G 726; sort 536 -> 250.
 //   5. mixed-precision solve of (G + lambda I) D~^T = (B + lambda D_old)^T:
 //      Jacobi scaling S = diag^-1/2 (unit diagonal); one cooperative kernel
 //      factors S (G + lambda I) S = L L^T in FP32 and inverts L on the way
@@ -41,7 +47,8 @@
 namespace dlsh {
 namespace mod {
 
-constexpr int TS = 512;        // signals per counting-sort tile (one scatter CTA each)
+constexpr int CH = 64;          // counting-sort tiles per chunk
+constexpr int SEGG = 8192;      // list entries per accumulation segment of G at most (about half on average)
 constexpr int NB = 32;         // Cholesky block
 constexpr int RW = 48;         // padded RHS width (45 used)
 constexpr int MAX_K = 4096;    // shared-memory G-row partials limit
@@ -49,13 +56,63 @@ constexpr int SMEM_LIMIT = 232448;
 constexpr double RIDGE_REL = 1e-6;
 constexpr int kRefine = 3;     // FP32 solves (two FP64 residual corrections)
 
+// The counting sort of the codes by atom, shared by both dictionary updates.
+struct Sort {
+  int* cnt;         // T x K: entries of each (tile, atom), then their list offsets
+  int* csum;        // P x K: entries of each (chunk, atom)
+  int* segtot;      // P x ceil(K / 256): first B segment of each (chunk, 256 atoms)
+  int* cstart;      // P x K: list offset of each (chunk, atom)
+  int* atom_start;  // K + 1
+  int* segb_start;  // P x K + 1: first B segment of each (chunk, atom)
+  int* segg_start;  // PG x K + 1: first G segment of each (group of gc chunks, atom)
+  uint2* list;      // N*s atom-major records: (signal | nnz << 26, coefficient bits)
+  int ts, T, P;     // signals per tile, tiles, chunks
+  int segb;         // list entries per B segment
+  int gc, PG;       // chunks per group of G segments, groups
+  int threads;      // of a scatter CTA
+  uint32_t sdiv;    // e / s = umulhi(e, sdiv) for e < 65536, s >= 2
+};
+
+inline size_t scatter_smem(int K, int s, int ts, int threads);
+
+// Tiles of 1024 signals on 16 warps where they fill the GPU and two CTAs fit an
+// SM, else 512 on 8.  (Longer tiles give longer runs of list slots per atom.)
+// B segments: enough for 32 warps on every SM, 64 to 1024 entries each.
+static void sort_shape(int K, int s, int64_t N, Sort& so) {
+  const bool big = N >= 2 * 152 * 1024 && scatter_smem(K, s, 1024, 512) <= 114 * 1024;
+  so.ts = big ? 1024 : 512;
+  so.threads = big ? 512 : 256;
+  so.T = static_cast<int>(N > 0 ? (N + so.ts - 1) / so.ts : 1);
+  so.P = (so.T + CH - 1) / CH;
+  const int64_t per = N * s / (152 * 32);
+  so.segb = static_cast<int>(per < 64 ? 64 : (per > 1024 ? 1024 : per));
+  // groups of chunks in which an atom has about SEGG / 2 entries
+  const int64_t gc = static_cast<int64_t>(SEGG / 2) * K / (static_cast<int64_t>(s) * CH * so.ts);
+  so.gc = static_cast<int>(gc < 1 ? 1 : (gc > so.P ? so.P : gc));
+  so.PG = (so.P + so.gc - 1) / so.gc;
+  so.sdiv = s >= 2 ? static_cast<uint32_t>((uint64_t(1) << 32) / static_cast<uint64_t>(s) + 1) : 0u;
+}
+static void carve_sort(Carver& c, int K, int s, int64_t N, Sort& so) {
+  sort_shape(K, s, N, so);
+  so.cnt = c.take<int>(static_cast<size_t>(K) * so.T);
+  so.csum = c.take<int>(static_cast<size_t>(K) * so.P);
+  so.segtot = c.take<int>(static_cast<size_t>((K + 255) / 256) * so.P);
+  so.cstart = c.take<int>(static_cast<size_t>(K) * so.P);
+  so.atom_start = c.take<int>(K + 1);
+  so.segb_start = c.take<int>(static_cast<size_t>(K) * so.P + 1);
+  so.segg_start = c.take<int>(static_cast<size_t>(K) * so.PG + 1);
+  so.list = c.take<uint2>(static_cast<size_t>(N) * s + 1);
+}
+inline int64_t max_segb(const Sort& so, int K, int s, int64_t N) {
+  return N * s / so.segb + static_cast<int64_t>(so.P) * K;
+}
+inline int64_t max_segg(const Sort& so, int K, int s, int64_t N) {
+  return N * s / SEGG + static_cast<int64_t>(so.PG) * K;
+}
+
 struct Ws {
   uint32_t* status;
-  int* cnt;        // K x T per-(atom, tile) counts
-  int* off;        // K x T offsets
-  int* atom_total; // K
-  int* atom_start; // K + 1
-  uint2* list;     // N*s atom-major records: (signal | nnz << 26, coefficient bits)
+  Sort so;         // the atom-major list
   double* M;       // K x K: G + lambda I (FP64, kept for the refinement residuals)
   double* Z;       // K x RW: B^T (lambda D_old is added where Z is read)
   double* lam;     // [0] lambda
@@ -69,36 +126,14 @@ struct Ws {
   float* R32;      // K x RW: current residual of the scaled system
   double* Xb;      // K x RW: D~^T = S Xs, kept up to date with Xs
   int* dead;       // K
-  int* seg_start;  // P*K + 1: first accumulation segment of each (block p, atom j), p-major
-  double* Gp;      // max_segs x K partial G rows
-  double* Bp;      // max_segs x RW partial B columns
+  double* Gp;      // G segments x K partial rows
+  double* Bp;      // B segments x RW partial columns
 };
-
-constexpr int SEG = 4096;  // list entries per accumulation segment
-// Signals per accumulation block: segments never cross a block, and the grid
-// walks the blocks in order.  Blocks of 262,144 signals (47 MB of rows, held
-// in L2 while gathered) measured slower on GB300 than whole-list segments:
-// the gathers are not the binding limit, the per-segment work is.  The value
-// here puts every atom's list in one block.
-constexpr int64_t BLK = int64_t(1) << 40;
-static_assert(BLK % TS == 0, "blocks are whole counting-sort tiles");
-
-inline int64_t n_blocks(int64_t N) { return N > 0 ? (N + BLK - 1) / BLK : 1; }
-// counting-sort tiles per block, capped at the tile count (fits an int)
-inline int tiles_per_block(int64_t T) { return static_cast<int>(BLK / TS < T ? BLK / TS : T); }
-inline int64_t max_segments(int K, int s, int64_t N) {
-  return (N * s + SEG - 1) / SEG + n_blocks(N) * K;
-}
 
 static size_t carve(void* base, int K, int s, int64_t N, Ws& w) {
   Carver c(base);
-  const int64_t T = (N + TS - 1) / TS > 0 ? (N + TS - 1) / TS : 1;
   w.status = c.take<uint32_t>(64);
-  w.cnt = c.take<int>(static_cast<size_t>(K) * T);
-  w.off = c.take<int>(static_cast<size_t>(K) * T);
-  w.atom_total = c.take<int>(K);
-  w.atom_start = c.take<int>(K + 1);
-  w.list = c.take<uint2>(static_cast<size_t>(N) * s + 1);
+  carve_sort(c, K, s, N, w.so);
   w.M = c.take<double>(static_cast<size_t>(K) * K);
   w.Z = c.take<double>(static_cast<size_t>(K) * RW);
   w.lam = c.take<double>(4);
@@ -112,270 +147,13 @@ static size_t carve(void* base, int K, int s, int64_t N, Ws& w) {
   w.R32 = c.take<float>(static_cast<size_t>(K) * RW);
   w.Xb = c.take<double>(static_cast<size_t>(K) * RW);
   w.dead = c.take<int>(K);
-  w.seg_start = c.take<int>(static_cast<size_t>(n_blocks(N)) * K + 1);
-  w.Gp = c.take<double>(static_cast<size_t>(max_segments(K, s, N)) * K);
-  w.Bp = c.take<double>(static_cast<size_t>(max_segments(K, s, N)) * RW);
+  w.Gp = c.take<double>(static_cast<size_t>(max_segg(w.so, K, s, N)) * K);
+  w.Bp = c.take<double>(static_cast<size_t>(max_segb(w.so, K, s, N)) * RW);
   return c.size();
 }
 
-// ---- float-float accumulation: (hi, lo) += a * b, product exact via FMA ------
-__device__ __forceinline__ void ff_fma(float& hi, float& lo, float a, float b) {
-  const float p = __fmul_rn(a, b);
-  const float pe = __fmaf_rn(a, b, -p);
-  const float s = __fadd_rn(hi, p);
-  const float v = __fadd_rn(s, -hi);
-  float e = __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -v)), __fadd_rn(p, -v));
-  e = __fadd_rn(e, __fadd_rn(lo, pe));
-  hi = __fadd_rn(s, e);
-  lo = __fadd_rn(e, -__fadd_rn(hi, -s));
-}
-
-// ---- 1. per-tile histograms ------------------------------------------------
-__global__ void count_kernel(const uint16_t* __restrict__ idx, const uint8_t* __restrict__ nnz,
-                             int s, int64_t N, int K, int T, int* __restrict__ cnt,
-                             uint32_t* status) {
-  extern __shared__ int hist[];
-  for (int j = threadIdx.x; j < K; j += blockDim.x) hist[j] = 0;
-  __syncthreads();
-  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * TS;
-  const int nt = static_cast<int>(N - i0 < TS ? N - i0 : TS);  // signals in this tile
-  const uint16_t* tidx = idx + i0 * s;
-  bool bad = false;
-#pragma unroll 4
-  for (int e = threadIdx.x; e < nt * s; e += blockDim.x) {
-    const int q = e / s;
-    const int t = e - q * s;
-    int nz = nnz[i0 + q];
-    if (nz > s) {
-      bad = true;
-      nz = s;
-    }
-    if (t < nz) {
-      const int j = tidx[e];
-      if (j < K)
-        atomicAdd(&hist[j], 1);
-      else
-        bad = true;
-    }
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < K; j += blockDim.x) cnt[static_cast<size_t>(j) * T + blockIdx.x] = hist[j];
-  if (bad) flag_status(status, ST_BAD_INPUT);
-}
-
-// ---- 2. offsets: per-atom totals, atom starts, per-(atom, tile) offsets -------
-__device__ __forceinline__ int block_exclusive_scan(int v, int* sm, int* total) {
-  // Hillis-Steele over blockDim.x (<= 1024) values; returns the exclusive prefix
-  const int tid = threadIdx.x;
-  sm[tid] = v;
-  __syncthreads();
-  for (int o = 1; o < static_cast<int>(blockDim.x); o <<= 1) {
-    const int u = tid >= o ? sm[tid - o] : 0;
-    __syncthreads();
-    sm[tid] += u;
-    __syncthreads();
-  }
-  const int incl = sm[tid];
-  if (total) *total = sm[blockDim.x - 1];
-  __syncthreads();
-  return incl - v;
-}
-
-__global__ void atom_total_kernel(const int* __restrict__ cnt, int T, int* __restrict__ atom_total) {
-  __shared__ int red[256];
-  const int j = blockIdx.x;
-  int acc = 0;
-  for (int b = threadIdx.x; b < T; b += blockDim.x) acc += cnt[static_cast<size_t>(j) * T + b];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (static_cast<int>(threadIdx.x) < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atom_total[j] = red[0];
-}
-
-__global__ void atom_scan_kernel(const int* __restrict__ atom_total, int K,
-                                 int* __restrict__ atom_start) {
-  __shared__ int sm[1024];
-  __shared__ int carry_s;
-  int carry = 0;
-  for (int base = 0; base < K; base += 1024) {
-    const int j = base + threadIdx.x;
-    const int v = j < K ? atom_total[j] : 0;
-    int tot = 0;
-    const int ex = block_exclusive_scan(v, sm, &tot);
-    if (j < K) atom_start[j] = carry + ex;
-    if (threadIdx.x == 0) carry_s = carry + tot;
-    __syncthreads();
-    carry = carry_s;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atom_start[K] = carry;
-}
-
-__global__ void tile_offsets_kernel(const int* __restrict__ cnt, int T,
-                                    const int* __restrict__ atom_start, int* __restrict__ off) {
-  __shared__ int sm[256];
-  const int j = blockIdx.x;
-  const int per = (T + blockDim.x - 1) / blockDim.x;
-  const int b0 = threadIdx.x * per, b1 = b0 + per < T ? b0 + per : T;
-  int sum = 0;
-  for (int b = b0; b < b1; ++b) sum += cnt[static_cast<size_t>(j) * T + b];
-  int run = atom_start[j] + block_exclusive_scan(sum, sm, nullptr);
-  for (int b = b0; b < b1; ++b) {
-    off[static_cast<size_t>(j) * T + b] = run;
-    run += cnt[static_cast<size_t>(j) * T + b];
-  }
-}
-
-// ---- 3. counting-sort scatter, one CTA of 8 warps per tile, signal order ------
-// The tile's code indices and counts are first staged in shared memory with
-// coalesced loads, so that neither pass waits on a chain of dependent global
-// loads.  Warp w owns signals [64 w, 64 w + 64) of the tile and walks their code
-// slots in order, 32 at a time.  Pass 1 counts each atom per warp (lanes with
-// the same atom found by match-any); the counts become per-warp bases; pass 2
-// gives each entry its rank among the earlier entries of its atom (warps in
-// order, then lanes in order) and writes it to the atom-major list.  A signal's
-// atoms are distinct, so within an atom the entries stay in signal order.
-// SLOT: the record's upper 6 bits hold the entry's code slot t instead of nnz.
-constexpr int SC_T = 256;
-// Shared memory of a scatter CTA: staged indices (TS s uint16, a multiple of 16
-// bytes), counts (TS bytes), then per-warp counts [8][K] and tile offsets [K].
-inline size_t scatter_smem(int K, int s) {
-  return static_cast<size_t>(TS) * s * 2 + TS + static_cast<size_t>(SC_T / 32 + 1) * K * sizeof(int);
-}
-template <bool SLOT>
-__global__ void __launch_bounds__(SC_T) scatter_kernel(const uint16_t* __restrict__ idx,
-                                                      const float* __restrict__ coef,
-                                                      const uint8_t* __restrict__ nnz, int s, int64_t N,
-                                                      int K, int T, const int* __restrict__ off,
-                                                      uint2* __restrict__ list) {
-  extern __shared__ __align__(16) uint8_t scb[];
-  uint16_t* sidx = reinterpret_cast<uint16_t*>(scb);                        // [TS * s]
-  uint8_t* snz = scb + static_cast<size_t>(TS) * s * 2;                     // [TS]
-  int* wc = reinterpret_cast<int*>(snz + TS);                               // [8][K] counts, then bases
-  int* toff = wc + static_cast<size_t>(SC_T / 32) * K;                      // [K] this tile's list offsets
-  const int b = blockIdx.x;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t t0 = static_cast<int64_t>(b) * TS;
-  const int nt = static_cast<int>(N - t0 < TS ? N - t0 : TS);  // signals in this tile
-  {
-    // 16-byte loads where the tile's index rows are 16-byte aligned (the tile
-    // starts at a multiple of TS s, so only the array's base decides), the rest
-    // element by element
-    const uint16_t* src = idx + t0 * s;
-    const int ne = nt * s;
-    int done = 0;
-    if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-      const int nv = ne / 8;
-      for (int v = tid; v < nv; v += SC_T)
-        reinterpret_cast<uint4*>(sidx)[v] = __ldg(reinterpret_cast<const uint4*>(src) + v);
-      done = nv * 8;
-    }
-    for (int e = done + tid; e < ne; e += SC_T) sidx[e] = src[e];
-    for (int q = tid; q < nt; q += SC_T) snz[q] = nnz[t0 + q];
-  }
-  for (int j = tid; j < K; j += SC_T) {
-    toff[j] = off[static_cast<size_t>(j) * T + b];
-#pragma unroll
-    for (int w = 0; w < SC_T / 32; ++w) wc[w * K + j] = 0;
-  }
-  __syncthreads();
-  constexpr int SPW = TS / (SC_T / 32);  // signals per warp (64)
-  const int q0 = warp * SPW;              // the warp's first signal in the tile
-  const int64_t i0 = t0 + q0;
-  const int qn = nt - q0 < SPW ? nt - q0 : SPW;
-  const int e_end = (qn > 0 ? qn : 0) * s;  // <= 64 * 32
-  int* mine = wc + static_cast<size_t>(warp) * K;
-  const unsigned lt = (1u << lane) - 1u;
-  // entry e of the warp: its atom j (-1 if none), coefficient c (only when
-  // with_coef), count or slot field nz and signal
-  auto entry = [&](int e, bool with_coef, int& j, float& c, int& nz, int64_t& sig) {
-    j = -1;
-    c = 0.f;
-    nz = 0;
-    sig = 0;
-    if (e < e_end) {
-      const int q = e / s;
-      sig = i0 + q;
-      const int t = e - q * s;
-      nz = snz[q0 + q];
-      nz = nz > s ? s : nz;
-      const bool live = t < nz;
-      if (SLOT) nz = t;
-      if (live) {
-        const int jj = sidx[(q0 + q) * s + t];
-        if (jj < K) {
-          j = jj;
-          if (with_coef) c = coef[sig * s + t];
-        }
-      }
-    }
-  };
-  // pass 1: counts
-  for (int e0 = 0; e0 < e_end; e0 += 32) {
-    int j, nz;
-    float c;
-    int64_t sig;
-    entry(e0 + lane, false, j, c, nz, sig);
-    const unsigned m = __match_any_sync(0xffffffffu, j);
-    if (j >= 0 && (m & lt) == 0) mine[j] += __popc(m);
-    __syncwarp();
-  }
-  __syncthreads();
-  // per-warp bases: warps in order
-  for (int j = tid; j < K; j += SC_T) {
-    int run = toff[j];
-#pragma unroll
-    for (int w = 0; w < SC_T / 32; ++w) {
-      const int cw = wc[w * K + j];
-      wc[w * K + j] = run;
-      run += cw;
-    }
-  }
-  __syncthreads();
-  // pass 2: ranks and writes
-  for (int e0 = 0; e0 < e_end; e0 += 32) {
-    int j, nz;
-    float c;
-    int64_t sig;
-    entry(e0 + lane, true, j, c, nz, sig);
-    const unsigned m = __match_any_sync(0xffffffffu, j);
-    if (j >= 0) {
-      const int pos = mine[j] + __popc(m & lt);
-      list[pos] = make_uint2(static_cast<uint32_t>(sig) | (static_cast<uint32_t>(nz) << 26), __float_as_uint(c));
-    }
-    __syncwarp();
-    if (j >= 0 && (m & lt) == 0) mine[j] += __popc(m);
-    __syncwarp();
-  }
-}
-
-// ---- 4. G row j and B column j ---------------------------------------------------
-// Entry range [lo, hi) of atom j's list that lies in signal block p (tpb
-// counting-sort tiles per block).
-__device__ __forceinline__ void block_range(const int* __restrict__ off,
-                                            const int* __restrict__ atom_start, int T, int tpb,
-                                            int j, int p, int& lo, int& hi) {
-  const int t0 = p * tpb, t1 = t0 + tpb;
-  lo = t0 < T ? off[static_cast<size_t>(j) * T + t0] : atom_start[j + 1];
-  hi = t1 < T ? off[static_cast<size_t>(j) * T + t1] : atom_start[j + 1];
-}
-
-// One CTA per accumulation segment (a slice of atom j's list inside one signal
-// block); the warps split the segment, one list entry per lane pair and 16
-// entries per step:
-//   B   each lane keeps float-float sums of its entries' a_ij x_i over half of
-//       the 45 dimensions in registers (the signal row is read straight from
-//       global memory); a butterfly of two-sums adds the lanes up at the end
-//   G   for each support slot t with atom k > j, the lanes add a_ij a_ik into
-//       the warp's row partial in shared memory (the entries k < j come from
-//       row k's segments, mirrored later); lanes that hit the same atom k are
-//       grouped (match) and their products summed in lane order by the group's
-//       first lane before its single update; the diagonal k = j stays in
-//       registers
-// Every sum runs in a fixed order, so the result does not depend on timing.
+// ---- float-float accumulation -------------------------------------------------
+// (h, l) += (p, pl), renormalised: about 48 bits.
 __device__ __forceinline__ void ff_add(float& h, float& l, float p, float pl) {
   const float s = __fadd_rn(h, p);
   const float v = __fadd_rn(s, -h);
@@ -385,205 +163,605 @@ __device__ __forceinline__ void ff_add(float& h, float& l, float p, float pl) {
   l = __fadd_rn(t, -__fadd_rn(h, -s));
 }
 
-// SMAX >= s: the support slots of a lane's entry are loaded into registers at
-// the start of each step, next to its signal row, so no load waits inside the
-// slot loop.  Two lanes share an entry (half of its dimensions and slots each),
-// which halves the registers and doubles the warps an SM can hold: five CTAs
-// per SM at s <= 8 (96 registers a thread), four at s <= 16.
-constexpr int DH = (DLSH_D + 1) / 2;  // dimensions per lane of a pair (23)
-template <int SMAX>
-__global__ void __launch_bounds__(128, SMAX <= 8 ? 5 : (SMAX <= 16 ? 4 : 3))
-    accum_kernel(const float* __restrict__ X, const uint16_t* __restrict__ idx,
-                 const float* __restrict__ coef, int s, int K, const int* __restrict__ atom_start,
-                 const int* __restrict__ off, int T, int tpb, int PK,
-                 const int* __restrict__ seg_start, const uint2* __restrict__ list,
-                 double* __restrict__ Gp, double* __restrict__ Bp) {
-  extern __shared__ __align__(16) float smf[];
+// The same on pairs of values (Blackwell's packed FP32 instructions: one issue
+// slot for two lanes' worth of work).  sub(a, b) = a - b as an FMA by -1, which
+// rounds once like the subtraction.
+struct f2 {
+  uint64_t v;
+};
+__device__ __forceinline__ f2 f2_make(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_get(f2 x, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) { return f2_fma(b, f2_make(-1.f, -1.f), a); }
+// (h, l) += a x: the product exact as p + pe, h + p by a two-sum whose error and
+// pe go to l.  l is renormalised into h by f2_norm (every few hundred steps at
+// most: l stays near 2^-24 of the partial sums, so its own rounding errors are
+// those of the renormalised form).
+__device__ __forceinline__ void f2_acc(f2& h, f2& l, f2 a, f2 na, f2 x) {
+  const f2 p = f2_mul(a, x);
+  const f2 npe = f2_fma(na, x, p);  // p - a x = -pe, exact
+  const f2 s = f2_add(h, p);
+  const f2 v = f2_sub(s, h);
+  const f2 e = f2_add(f2_sub(h, f2_sub(s, v)), f2_sub(p, v));
+  l = f2_sub(f2_add(l, e), npe);
+  h = s;
+}
+__device__ __forceinline__ void f2_norm(f2& h, f2& l) {
+  const f2 s = f2_add(h, l);
+  const f2 v = f2_sub(s, h);
+  l = f2_add(f2_sub(h, f2_sub(s, v)), f2_sub(l, v));
+  h = s;
+}
+
+// Whether two active lanes of the warp hold the same place: each has read the
+// place's value, writes its lane number there and looks whether it is still
+// there; the caller then writes the new values.  (match-any answers the same
+// but takes about a hundred cycles when the places differ.)
+template <class T>
+__device__ __forceinline__ bool any_shared(T* place, bool active, T tag) {
+  __syncwarp();
+  if (active) *place = tag;
+  __syncwarp();
+  const bool lost = active && *const_cast<volatile T*>(place) != tag;
+  return __any_sync(0xffffffffu, lost);
+}
+
+// ---- 1. per-tile histograms, cnt[tile][atom] -----------------------------------
+// Two 16-bit counters per word (a tile has fewer than 65,536 entries), integer
+// atomics in shared memory.
+__global__ void __launch_bounds__(256) count_kernel(const uint16_t* __restrict__ idx, const uint8_t* __restrict__ nnz,
+                                                   int s, uint32_t sdiv, int64_t N, int K, int ts,
+                                                   int* __restrict__ cnt, uint32_t* status) {
+  extern __shared__ unsigned hist[];  // [(K + 1) / 2]
+  const int nw = (K + 1) / 2;
+  for (int j = threadIdx.x; j < nw; j += blockDim.x) hist[j] = 0;
+  __syncthreads();
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * ts;
+  const int nt = static_cast<int>(N - i0 < ts ? N - i0 : ts);  // signals in this tile
+  const uint16_t* tidx = idx + i0 * s;
+  bool bad = false;
+  auto one = [&](int e, unsigned j) {
+    const int q = s == 1 ? e : static_cast<int>(__umulhi(static_cast<uint32_t>(e), sdiv));
+    int nz = nnz[i0 + q];
+    bad |= nz > s;
+    if (e - q * s < nz) {
+      if (j < static_cast<unsigned>(K)) atomicAdd(&hist[j >> 1], (j & 1u) ? 65536u : 1u);
+      else bad = true;
+    }
+  };
+  const int ne = nt * s;
+  int done = 0;
+  if ((reinterpret_cast<uintptr_t>(tidx) & 15u) == 0) {  // eight indices per load
+    const int nv = ne / 8;
+    for (int v = threadIdx.x; v < nv; v += blockDim.x) {
+      const uint4 w = __ldg(reinterpret_cast<const uint4*>(tidx) + v);
+      const unsigned u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        one(8 * v + 2 * k, u[k] & 0xffffu);
+        one(8 * v + 2 * k + 1, u[k] >> 16);
+      }
+    }
+    done = nv * 8;
+  }
+  for (int e = done + threadIdx.x; e < ne; e += blockDim.x) one(e, tidx[e]);
+  __syncthreads();
+  int* row = cnt + static_cast<size_t>(blockIdx.x) * K;
+  for (int j = threadIdx.x; j < K; j += blockDim.x) row[j] = (hist[j >> 1] >> (16 * (j & 1))) & 0xffffu;
+  if (bad) flag_status(status, ST_BAD_INPUT);
+}
+
+// ---- 2. offsets -------------------------------------------------------------------
+// Chunks of CH tiles, 256 atoms per CTA.  chunk_sum: entries of each (chunk,
+// atom) and how many segments of B (at most segb entries each) its 256 atoms
+// need.  layout (one CTA): atom starts, G segments (SEGG entries of one atom),
+// and the first B segment of each (chunk, 256 atoms).  tile_offsets: list offset
+// of each (tile, atom), in place of its count, and of each (chunk, atom), and
+// its first B segment.  Only what needs one CTA runs on one (everything in one
+// took 38 us at 46 chunks and 84 at 92: one SM's bandwidth).
+// Exclusive prefix over the block (whole warps) and the total; sm: 32 ints.
+__device__ __forceinline__ int block_scan(int v, int* sm, int& total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += u;
+  }
+  if (lane == 31) sm[w] = x;
+  __syncthreads();
+  int y = lane < static_cast<int>(blockDim.x >> 5) ? sm[lane] : 0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, y, o);
+    if (lane >= o) y += u;
+  }
+  total = __shfl_sync(0xffffffffu, y, 31);
+  const int before = w > 0 ? __shfl_sync(0xffffffffu, y, w - 1) : 0;
+  __syncthreads();
+  return before + x - v;
+}
+
+__global__ void __launch_bounds__(256) chunk_sum_kernel(const int* __restrict__ cnt, int T, int K, int segb,
+                                                       int* __restrict__ csum, int* __restrict__ segtot) {
+  __shared__ int sm[32];
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t0 = blockIdx.y * CH, t1 = t0 + CH < T ? t0 + CH : T;
+  int acc = 0;
+  if (j < K) {
+#pragma unroll 8
+    for (int t = t0; t < t1; ++t) acc += cnt[static_cast<size_t>(t) * K + j];
+    csum[static_cast<size_t>(blockIdx.y) * K + j] = acc;
+  }
+  int all = 0;
+  block_scan((acc + segb - 1) / segb, sm, all);
+  if (threadIdx.x == 0) segtot[blockIdx.y * gridDim.x + blockIdx.x] = all;
+}
+
+__global__ void __launch_bounds__(1024) layout_kernel(const int* __restrict__ csum, int P, int K, int gc, int PG,
+                                                      int nseg, int* __restrict__ segtot, int* __restrict__ atom_start,
+                                                      int* __restrict__ segg_start, int* __restrict__ segb_end) {
+  __shared__ int sm[32];
+  int carry = 0;
+  for (int base = 0; base < K; base += 1024) {
+    const int j = base + threadIdx.x;
+    int tot = 0;
+    if (j < K)
+      for (int pg = 0; pg < PG; ++pg) {  // entries per group of chunks, then of the atom
+        int g = 0;
+        const int p1 = (pg + 1) * gc < P ? (pg + 1) * gc : P;
+#pragma unroll 8
+        for (int p = pg * gc; p < p1; ++p) g += csum[static_cast<size_t>(p) * K + j];
+        segg_start[static_cast<size_t>(pg) * K + j] = (g + SEGG - 1) / SEGG;
+        tot += g;
+      }
+    int all = 0;
+    const int st = carry + block_scan(tot, sm, all);
+    if (j < K) atom_start[j] = st;
+    carry += all;
+  }
+  auto scan = [&](int* v, int n) {  // exclusive scan in place, the total returned
+    int c = 0;
+    __syncthreads();
+    for (int base = 0; base < n; base += 4096) {  // four consecutive per thread
+      const int q = base + 4 * threadIdx.x;
+      int x[4], tot = 0, all = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        x[u] = q + u < n ? v[q + u] : 0;
+        tot += x[u];
+      }
+      int st = c + block_scan(tot, sm, all);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (q + u < n) v[q + u] = st;
+        st += x[u];
+      }
+      c += all;
+    }
+    return c;
+  };
+  const int nb = scan(segtot, nseg);
+  const int ng = scan(segg_start, PG * K);
+  if (threadIdx.x == 0) {
+    atom_start[K] = carry;
+    segg_start[PG * K] = ng;
+    *segb_end = nb;
+  }
+}
+
+__global__ void __launch_bounds__(256) tile_offsets_kernel(int* __restrict__ cnt, int T, int K, int segb,
+                                                          const int* __restrict__ csum, const int* __restrict__ segtot,
+                                                          const int* __restrict__ atom_start, int* __restrict__ cstart,
+                                                          int* __restrict__ segb_start) {
+  __shared__ int sm[32];
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, p = blockIdx.y;
+  const int n = j < K ? csum[static_cast<size_t>(p) * K + j] : 0;
+  int all = 0;
+  const int sb = segtot[p * gridDim.x + blockIdx.x] + block_scan((n + segb - 1) / segb, sm, all);
+  if (j >= K) return;
+  int run = atom_start[j];
+#pragma unroll 8
+  for (int q = 0; q < p; ++q) run += csum[static_cast<size_t>(q) * K + j];
+  cstart[static_cast<size_t>(p) * K + j] = run;
+  segb_start[static_cast<size_t>(p) * K + j] = sb;
+  const int t0 = p * CH, t1 = t0 + CH < T ? t0 + CH : T;
+  for (int tb = t0; tb < t1; tb += 8) {  // eight loads, then their stores
+    int c[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) c[u] = tb + u < t1 ? cnt[static_cast<size_t>(tb + u) * K + j] : 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (tb + u < t1) cnt[static_cast<size_t>(tb + u) * K + j] = run;
+      run += c[u];
+    }
+  }
+}
+
+// ---- 3. counting-sort scatter, one CTA per tile, signal order ------------------
+// The tile's indices, counts and coefficients are staged in shared memory by
+// coalesced loads; its entries are sorted by atom there, and the records then
+// leave in sorted order, so that a warp's store covers a few runs of
+// consecutive list slots (written straight from signal order, every record was
+// a 32-byte L2 write of its own: 397 us at 24M entries against 190).
+// Warp w owns a contiguous range of the tile's entries.  Pass 1 counts each atom
+// per warp (integer atomics); the counts become per-warp bases in tile order;
+// pass 2 ranks each entry among the earlier ones of its atom (warps in order,
+// then lanes in order).
+// SLOT: the record's upper 6 bits hold the entry's code slot t instead of nnz.
+inline size_t scatter_smem(int K, int s, int ts, int threads) {
+  const size_t ne = static_cast<size_t>(ts) * s;
+  const size_t kp = (static_cast<size_t>(K) + 1) / 2 * 2;
+  return ne * 8 + ts + 16 + kp * 2 * (threads / 32) + static_cast<size_t>(K) * 4 + 128;
+}
+template <bool SLOT>
+__global__ void __launch_bounds__(512) scatter_kernel(const uint16_t* __restrict__ idx, const float* __restrict__ coef,
+                                                      const uint8_t* __restrict__ nnz, int s, uint32_t sdiv, int64_t N,
+                                                      int K, int ts, const int* __restrict__ off,
+                                                      uint2* __restrict__ list) {
+  extern __shared__ __align__(16) uint8_t scb[];
+  const int ncap = ts * s;
+  const int kp = (K + 1) / 2 * 2;
+  const int nthr = blockDim.x, nwarps = nthr >> 5;
+  float* scoef = reinterpret_cast<float*>(scb);                             // [ts s]
+  uint16_t* sidx = reinterpret_cast<uint16_t*>(scoef + ncap);               // [ts s] atom, 0xFFFF = no entry
+  uint16_t* sorted = sidx + ncap;                                           // [ts s] entries by atom
+  uint8_t* snz = reinterpret_cast<uint8_t*>(sorted + ncap);                 // [ts]
+  int* toff = reinterpret_cast<int*>(scb + (static_cast<size_t>(ncap) * 8 + ts + 15) / 16 * 16);  // [K] list offset - local start
+  uint16_t* wc = reinterpret_cast<uint16_t*>(toff + K);                     // [warps][kp] counts, then bases
+  __shared__ int wsum[32];
+  const int b = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t t0 = static_cast<int64_t>(b) * ts;
+  const int nt = static_cast<int>(N - t0 < ts ? N - t0 : ts);  // signals in this tile
+  const int ne = nt * s;
+  auto div_s = [&](int e) { return s == 1 ? e : static_cast<int>(__umulhi(static_cast<uint32_t>(e), sdiv)); };
+  for (int q = tid; q < nt; q += nthr) snz[q] = nnz[t0 + q];
+  for (int j = tid; j < kp / 2 * nwarps; j += nthr) reinterpret_cast<unsigned*>(wc)[j] = 0u;
+  {
+    // 16-byte loads where the tile's rows are 16-byte aligned, the rest one by one
+    const float* cs = coef + t0 * s;
+    int done = 0;
+    if ((reinterpret_cast<uintptr_t>(cs) & 15u) == 0) {
+      const int nv = ne / 4;
+      for (int v = tid; v < nv; v += nthr)
+        reinterpret_cast<float4*>(scoef)[v] = __ldg(reinterpret_cast<const float4*>(cs) + v);
+      done = nv * 4;
+    }
+    for (int e = done + tid; e < ne; e += nthr) scoef[e] = cs[e];
+  }
+  __syncthreads();
+  {
+    const uint16_t* src = idx + t0 * s;
+    auto live = [&](int e, unsigned j) -> unsigned {
+      const int q = div_s(e);
+      return (e - q * s < snz[q] && j < static_cast<unsigned>(K)) ? j : 0xffffu;
+    };
+    int done = 0;
+    if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+      const int nv = ne / 8;
+      for (int v = tid; v < nv; v += nthr) {
+        const uint4 w = __ldg(reinterpret_cast<const uint4*>(src) + v);
+        unsigned u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          u[k] = live(8 * v + 2 * k, u[k] & 0xffffu) | live(8 * v + 2 * k + 1, u[k] >> 16) << 16;
+        reinterpret_cast<uint4*>(sidx)[v] = make_uint4(u[0], u[1], u[2], u[3]);
+      }
+      done = nv * 8;
+    }
+    for (int e = done + tid; e < ne; e += nthr) sidx[e] = static_cast<uint16_t>(live(e, src[e]));
+  }
+  __syncthreads();
+  // the warp's entries, a multiple of 32 but for the last warp's
+  const int per = (ne + 32 * nwarps - 1) / (32 * nwarps) * 32;
+  const int e0 = warp * per < ne ? warp * per : ne;
+  const int e1 = e0 + per < ne ? e0 + per : ne;
+  uint16_t* mine = wc + static_cast<size_t>(warp) * kp;
+  const unsigned lt = (1u << lane) - 1u;
+  // pass 1: counts
+  for (int e = e0 + lane; e < e1; e += 32) {
+    const unsigned j = sidx[e];
+    if (j != 0xffffu) atomicAdd(reinterpret_cast<unsigned*>(mine) + (j >> 1), (j & 1u) ? 65536u : 1u);
+  }
+  __syncthreads();
+  // local starts (atoms in order) and per-warp bases (warps in order)
+  int carry = 0;
+  for (int base = 0; base < K; base += nthr) {
+    const int j = base + tid;
+    int tot = 0;
+    if (j < K)
+      for (int w = 0; w < nwarps; ++w) tot += wc[static_cast<size_t>(w) * kp + j];
+    int x = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += u;
+    }
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w < nwarps; ++w) {
+      if (w < warp) before += wsum[w];
+      all += wsum[w];
+    }
+    __syncthreads();
+    if (j < K) {
+      int run = carry + before + x - tot;
+      toff[j] = off[static_cast<size_t>(b) * K + j] - run;
+      for (int w = 0; w < nwarps; ++w) {
+        const int c = wc[static_cast<size_t>(w) * kp + j];
+        wc[static_cast<size_t>(w) * kp + j] = static_cast<uint16_t>(run);
+        run += c;
+      }
+    }
+    carry += all;
+  }
+  __syncthreads();
+  // pass 2: ranks
+  for (int eb = e0; eb < e1; eb += 32) {
+    const int e = eb + lane;
+    const unsigned j = e < e1 ? sidx[e] : 0xffffu;
+    const bool on = j != 0xffffu;
+    uint16_t* place = mine + (on ? j : 0u);
+    unsigned pos = *place;
+    bool last = true;
+    if (any_shared<uint16_t>(place, on, static_cast<uint16_t>(lane))) {
+      const unsigned m = __match_any_sync(0xffffffffu, j);
+      pos += __popc(m & lt);
+      last = (m >> lane) == 1u;
+    }
+    if (on) sorted[pos] = static_cast<uint16_t>(e);
+    __syncwarp();
+    if (on && last) *place = static_cast<uint16_t>(pos + 1);
+    __syncwarp();
+  }
+  __syncthreads();
+  // the records in sorted order
+  for (int p = tid; p < carry; p += nthr) {
+    const int e = sorted[p];
+    const int j = sidx[e];
+    const int q = div_s(e);
+    unsigned f = SLOT ? static_cast<unsigned>(e - q * s) : snz[q];
+    if (!SLOT && f > static_cast<unsigned>(s)) f = s;
+    list[toff[j] + p] = make_uint2(static_cast<uint32_t>(t0 + q) | (f << 26), __float_as_uint(scoef[e]));
+  }
+}
+
+// ---- 4a. column j of B: B_j = sum a_ij x_i ---------------------------------------
+// One warp per segment (entries of one atom within one chunk of signals), four
+// entries at a time: eight lanes take an entry's row, lane l its dimensions l,
+// l + 8, .., in packed float-float registers, with the rows of 16 entries in
+// flight per warp.  The segments run chunk by chunk, so that the rows of the
+// chunks in flight (about 12 MB each) come from HBM once and stay in L2 for the
+// s entries that use them (0.7 GB of HBM reads at 3M instead of 5.7).  Bound by
+// those L2 gathers (208 bytes of sectors per entry) and the FP32 pipe together.
+constexpr int BQ = 6;  // dimensions per lane (48, 45 used)
+__global__ void __launch_bounds__(256, 4) accum_b_kernel(const float* __restrict__ X, int K, int P,
+                                                        const int* __restrict__ cstart,
+                                                        const int* __restrict__ atom_start,
+                                                        const int* __restrict__ segb_start, int segb,
+                                                        const uint2* __restrict__ list, double* __restrict__ Bp) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
+  const int seg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (seg >= segb_start[P * K]) return;
+  // the segment's (chunk, atom): the largest pj with segb_start[pj] <= seg
+  int lo = 0, hi = P * K - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (segb_start[mid] <= seg) lo = mid; else hi = mid - 1;
+  }
+  const int p = lo / K, j = lo - p * K;
+  const int q0 = cstart[lo] + (seg - segb_start[lo]) * segb;
+  const int end = p + 1 < P ? cstart[lo + K] : atom_start[j + 1];
+  const int q1 = q0 + segb < end ? q0 + segb : end;
+  const float* Xl = X + sub;
+  const int last = sub + 8 * (BQ - 1) < DLSH_D ? 8 * (BQ - 1) : 0;  // offset of the sixth dimension, if any
+  f2 h[BQ / 2], l[BQ / 2];
+#pragma unroll
+  for (int q = 0; q < BQ / 2; ++q) h[q] = l[q] = f2_make(0.f, 0.f);
+  constexpr int U = 4;  // steps of four entries whose loads are in flight
+  uint2 next = q0 + lane < q1 ? __ldg(list + q0 + lane) : make_uint2(0u, 0u);
+  for (int eb = q0; eb < q1; eb += 32) {
+    const uint2 rec = next;
+    if (eb + 32 + lane < q1) next = __ldg(list + eb + 32 + lane);
+    const bool whole = eb + 32 <= q1;
+#pragma unroll 1
+    for (int i0 = 0; i0 < 8; i0 += U) {
+      if (eb + 4 * i0 >= q1) break;
+      float x[U][BQ];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int src = 4 * (i0 + u) + grp;
+        const unsigned sig = __shfl_sync(FULL, rec.x, src) & 0x3FFFFFFu;
+        const float* xr = Xl + static_cast<size_t>(sig) * DLSH_D;
+        const bool on = whole || eb + src < q1;  // past the end: a = 0 and x = 0
+#pragma unroll
+        for (int q = 0; q < BQ; ++q) x[u][q] = on ? __ldg(xr + (q + 1 < BQ ? 8 * q : last)) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float a = __uint_as_float(__shfl_sync(FULL, rec.y, 4 * (i0 + u) + grp));
+        const f2 aa = f2_make(a, a), na = f2_make(-a, -a);
+#pragma unroll
+        for (int q = 0; q < BQ / 2; ++q) f2_acc(h[q], l[q], aa, na, f2_make(x[u][2 * q], x[u][2 * q + 1]));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < BQ / 2; ++q) f2_norm(h[q], l[q]);
+  }
+  double* out = Bp + static_cast<size_t>(seg) * RW;
+#pragma unroll
+  for (int q = 0; q < BQ; ++q) {
+    float h0, h1, l0, l1;
+    f2_get(h[q / 2], h0, h1);
+    f2_get(l[q / 2], l0, l1);
+    float vh = (q & 1) ? h1 : h0, vl = (q & 1) ? l1 : l0;
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+      const float h2 = __shfl_xor_sync(FULL, vh, o), l2 = __shfl_xor_sync(FULL, vl, o);
+      ff_add(vh, vl, h2, l2);
+    }
+    const int d = sub + 8 * q;
+    if (grp == 0) out[d] = d < DLSH_D ? static_cast<double>(vh) + static_cast<double>(vl) : 0.0;
+  }
+}
+
+// ---- 4b. row j of G (entries k >= j; k < j come from row k, mirrored later) --------
+// One CTA per segment (entries of one atom within a group of chunks, so that the
+// codes gathered meanwhile stay in L2), its warps on fixed slices.  Eight lanes
+// take one entry, lane t its code slots t, t + 8, ..: each adds a_ij a_ik into
+// the warp's float-float row in shared memory where k > j (the diagonal stays
+// in registers).  A signal's atoms are distinct, so two lanes seldom meet on one
+// k: any_shared finds out, and then they update it one after the other in lane
+// order.
+// Bound by the update's shared-memory latency at the warps that the rows leave
+// room for (28 per SM at K = 1024).  SG = slots per lane.
+template <int SG>
+__global__ void __launch_bounds__(128) accum_g_kernel(const uint16_t* __restrict__ idx, const float* __restrict__ coef,
+                                                     int s, int K, int P, int gc, int PG,
+                                                     const int* __restrict__ cstart, const int* __restrict__ atom_start,
+                                                     const int* __restrict__ segg_start,
+                                                     const uint2* __restrict__ list, double* __restrict__ Gp) {
+  extern __shared__ __align__(16) float2 grow[];  // [warps][K] (hi, lo)
+  const int seg = blockIdx.x;
+  if (seg >= segg_start[PG * K]) return;
   const int nw = blockDim.x >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned FULL = 0xffffffffu;
-  float* ghi = smf + static_cast<size_t>(warp) * 2 * K;
-  float* glo = ghi + K;
-  double* bpart = reinterpret_cast<double*>(smf + static_cast<size_t>(nw) * 2 * K) + warp * RW;
-  const int nseg = seg_start[PK];
-  for (int seg = blockIdx.x; seg < nseg; seg += gridDim.x) {
-    // the segment's (block, atom): the largest pj with seg_start[pj] <= seg
-    int pj = 0;
+  // the segment's (chunk group, atom): the largest pj with segg_start[pj] <= seg
+  int lo = 0, hi = PG * K - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (segg_start[mid] <= seg) lo = mid; else hi = mid - 1;
+  }
+  const int pg = lo / K, j = lo - pg * K;
+  float2* row = grow + static_cast<size_t>(warp) * K;
+  for (int k = j + lane; k < K; k += 32) row[k] = make_float2(0.f, 0.f);
+  __syncwarp();
+  const int e0 = cstart[static_cast<size_t>(pg) * gc * K + j] + (seg - segg_start[lo]) * SEGG;
+  const int end = (pg + 1) * gc < P ? cstart[static_cast<size_t>(pg + 1) * gc * K + j] : atom_start[j + 1];
+  const int len = (e0 + SEGG < end ? e0 + SEGG : end) - e0;
+  const int q0 = e0 + static_cast<int>(static_cast<long long>(len) * warp / nw);
+  const int q1 = e0 + static_cast<int>(static_cast<long long>(len) * (warp + 1) / nw);
+  const int sub = lane & 7, grp = lane >> 3;
+  float dh = 0.f, dl = 0.f;  // G[j][j]: each entry's a_ij^2 on the lane that loads its record
+  constexpr int U = SG == 1 ? 4 : 2;  // steps of four entries whose codes are in flight
+  // record of lane's entry in a block of 32, the next block's loaded ahead
+  uint2 next = q0 + lane < q1 ? __ldg(list + q0 + lane) : make_uint2(0u, 0u);
+  for (int eb = q0; eb < q1; eb += 32) {
+    const uint2 rec = next;
+    next = eb + 32 + lane < q1 ? __ldg(list + eb + 32 + lane) : make_uint2(0u, 0u);
     {
-      int lo = 0, hi = PK - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (seg_start[mid] <= seg) lo = mid; else hi = mid - 1;
-      }
-      pj = lo;
+      const float a = __uint_as_float(rec.y);
+      const float ph = __fmul_rn(a, a);
+      if (eb + lane < q1) ff_add(dh, dl, ph, __fmaf_rn(a, a, -ph));
     }
-    const int pb = pj / K, j = pj - pb * K;
-    for (int k = lane; k < K; k += 32) {
-      ghi[k] = 0.f;
-      glo[k] = 0.f;
-    }
-    __syncwarp();
-    int rlo, rhi;
-    block_range(off, atom_start, T, tpb, j, pb, rlo, rhi);
-    const int e0 = rlo + (seg - seg_start[pj]) * SEG;
-    const int e1 = e0 + SEG < rhi ? e0 + SEG : rhi;
-    const int len = e1 - e0;
-    const int q0 = e0 + static_cast<int>(static_cast<long long>(len) * warp / nw);
-    const int q1 = e0 + static_cast<int>(static_cast<long long>(len) * (warp + 1) / nw);
-    // lane pair (2p, 2p + 1) takes entry p of each step of 16: the even lane
-    // dimensions 0..22 and slots 0..SMAX/2-1, the odd lane the rest
-    const int sub = lane & 1, pe = lane >> 1;
-    const int d0 = sub * DH;
-    float bh[DH], bl[DH];
+#pragma unroll 1
+    for (int i0 = 0; i0 < 8; i0 += U) {
+      if (eb + 4 * i0 >= q1) break;
+      int kk[U][SG];
+      float cc[U][SG], aa[U];
 #pragma unroll
-    for (int d = 0; d < DH; ++d) {
-      bh[d] = 0.f;
-      bl[d] = 0.f;
-    }
-    float dh = 0.f, dl = 0.f;  // G[j][j]
-    constexpr int SH = SMAX / 2;
-    // the next step's list record is loaded one step ahead, and its signal row
-    // and code slots are prefetched into L2 while this step computes
-    uint2 rec_next = make_uint2(0u, 0u);
-    if (q0 + pe < q1) rec_next = list[q0 + pe];
-    for (int eb = q0; eb < q1; eb += 16) {
-      const int e = eb + pe;
-      const bool act = e < q1;
-      const uint2 rec = rec_next;
-      if (eb + 16 + pe < q1) {
-        rec_next = list[eb + 16 + pe];
-        const long long sn = static_cast<long long>(rec_next.x & 0x3FFFFFFu);
-        const char* xr = reinterpret_cast<const char*>(X + sn * DLSH_D);
-        if (sub == 0) {
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(xr));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(xr + 92));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(xr + 176));
-        } else {
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(idx + sn * s));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(coef + sn * s));
+      for (int u = 0; u < U; ++u) {
+        const int src = 4 * (i0 + u) + grp;
+        const unsigned rx = __shfl_sync(FULL, rec.x, src);
+        aa[u] = __uint_as_float(__shfl_sync(FULL, rec.y, src));
+        const int nz = eb + src < q1 ? static_cast<int>(rx >> 26) : 0;
+        const size_t c0 = static_cast<size_t>(rx & 0x3FFFFFFu) * s + sub;
+#pragma unroll
+        for (int g = 0; g < SG; ++g) {
+          const bool on = sub + 8 * g < nz;
+          kk[u][g] = on ? static_cast<int>(__ldg(idx + c0 + 8 * g)) : -1;
+          cc[u][g] = on ? __ldg(coef + c0 + 8 * g) : 0.f;
         }
       }
-      long long sig = 0;
-      int nz = 0;
-      float a = 0.f;
-      if (act) {
-        sig = static_cast<long long>(rec.x & 0x3FFFFFFu);
-        nz = static_cast<int>(rec.x >> 26);
-        a = __uint_as_float(rec.y);
-      }
-      int kk[SH];
-      float cc[SH];
-      {
-        const uint16_t* ir = idx + sig * s;
-        const float* cr = coef + sig * s;
 #pragma unroll
-        for (int u = 0; u < SH; ++u) {
-          const int t = sub * SH + u;
-          const bool on = act && t < nz;
-          kk[u] = on ? static_cast<int>(__ldg(ir + t)) : -1;
-          cc[u] = on ? __ldg(cr + t) : 0.f;
-        }
-      }
-      if (act) {
-        const float* xr = X + sig * DLSH_D + d0;
-        float xv[DH];
+      for (int u = 0; u < U; ++u) {
+        int selves = 0;  // slots that hold atom j, over the step's entries
 #pragma unroll
-        for (int d = 0; d < DH; ++d) xv[d] = (d0 + d < DLSH_D) ? __ldg(xr + d) : 0.f;
-#pragma unroll
-        for (int d = 0; d < DH; ++d) ff_fma(bh[d], bl[d], a, xv[d]);
-      }
-      const int mine = act ? (nz - sub * SH < 0 ? 0 : (nz - sub * SH > SH ? SH : nz - sub * SH)) : 0;
-      const int mx = __reduce_max_sync(FULL, mine);
-#pragma unroll
-      for (int u = 0; u < SH; ++u) {
-        if (u >= mx) break;  // uniform over the warp
-        const bool on = kk[u] >= 0;
-        const int k = kk[u];
-        const float c = cc[u];
-        if (on && k == j) ff_fma(dh, dl, a, c);
-        const bool upd = on && k > j && k < K;
-        const unsigned m = __ballot_sync(FULL, upd);
-        if (upd) {
-          const unsigned grp = __match_any_sync(m, k);
-          float ph = __fmul_rn(a, c);
-          float pl = __fmaf_rn(a, c, -ph);
-          const int first = __ffs(grp) - 1;
-          if (grp != (1u << lane)) {
-            // the group's products, summed in lane order on its first lane
-            unsigned rest = grp & ~(1u << first);
-            float sh = ph, sl = pl;
-            while (rest) {
-              const int src = __ffs(rest) - 1;
-              const float h2 = __shfl_sync(grp, ph, src);
-              const float l2 = __shfl_sync(grp, pl, src);
-              ff_add(sh, sl, h2, l2);
-              rest &= rest - 1;
+        for (int g = 0; g < SG; ++g) {
+          const int k = kk[u][g];
+          const float ph = __fmul_rn(aa[u], cc[u][g]);
+          const float pl = __fmaf_rn(aa[u], cc[u][g], -ph);
+          const bool upd = k > j && k < K;
+          float2* place = row + (upd ? k : j);
+          float2 r = *place;
+          const bool shared = any_shared<float>(&place->x, upd, __int_as_float(lane));
+          ff_add(r.x, r.y, ph, pl);
+          if (!shared) {
+            if (upd) *place = r;
+          } else {  // lanes that share a k, in lane order
+            const unsigned peers = __match_any_sync(FULL, upd ? k : -1 - lane);
+            const int rank = upd ? __popc(peers & ((1u << lane) - 1u)) : 0;
+            const int most = __reduce_max_sync(FULL, rank);
+            if (upd && rank == 0) *place = r;
+            for (int q = 1; q <= most; ++q) {
+              __syncwarp();
+              if (upd && rank == q) {
+                r = *place;
+                ff_add(r.x, r.y, ph, pl);
+                *place = r;
+              }
             }
-            ph = sh;
-            pl = sl;
           }
-          if (lane == first) {
-            float h = ghi[k], l = glo[k];
-            ff_add(h, l, ph, pl);
-            ghi[k] = h;
-            glo[k] = l;
+          __syncwarp();
+          selves += __popc(__ballot_sync(FULL, k == j));
+        }
+        // a code that names atom j more than once: the other slots' a_ij a_ij'
+        const int here = q1 - eb - 4 * (i0 + u);  // entries of this step
+        if (selves != (here < 4 ? (here > 0 ? here : 0) : 4)) {
+#pragma unroll
+          for (int g = 0; g < SG; ++g)
+            if (kk[u][g] == j) {
+              const float ph = __fmul_rn(aa[u], cc[u][g]);
+              ff_add(dh, dl, ph, __fmaf_rn(aa[u], cc[u][g], -ph));
+            }
+          if (sub == 0 && grp < here) {  // its own square is counted already
+            const float ph = __fmul_rn(-aa[u], aa[u]);
+            ff_add(dh, dl, ph, __fmaf_rn(-aa[u], aa[u], -ph));
           }
         }
-        __syncwarp();
       }
     }
-    // the lanes' sums: butterflies of two-sums, B over the lanes of equal
-    // parity (their dimensions agree), the diagonal over all lanes
+  }
 #pragma unroll
-    for (int d = 0; d < DH; ++d)
-#pragma unroll
-      for (int o = 16; o > 1; o >>= 1) {
-        const float h2 = __shfl_xor_sync(FULL, bh[d], o);
-        const float l2 = __shfl_xor_sync(FULL, bl[d], o);
-        ff_add(bh[d], bl[d], h2, l2);
-      }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float h2 = __shfl_xor_sync(FULL, dh, o);
-      const float l2 = __shfl_xor_sync(FULL, dl, o);
-      ff_add(dh, dl, h2, l2);
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h2 = __shfl_xor_sync(FULL, dh, o);
+    const float l2 = __shfl_xor_sync(FULL, dl, o);
+    ff_add(dh, dl, h2, l2);
+  }
+  if (lane == 0) row[j] = make_float2(dh, dl);
+  // the warps' rows in order, one conversion to FP64 per atom
+  __syncthreads();
+  for (int k = j + threadIdx.x; k < K; k += blockDim.x) {
+    float2 r = grow[k];
+    for (int w = 1; w < nw; ++w) {
+      const float2 o = grow[static_cast<size_t>(w) * K + k];
+      ff_add(r.x, r.y, o.x, o.y);
     }
-    if (lane == 0) {
-      float h = ghi[j], l = glo[j];
-      ff_add(h, l, dh, dl);
-      ghi[j] = h;
-      glo[j] = l;
-    }
-    {
-      // lanes 0 and 1 store the two halves.  Every index here is a constant:
-      // a lane-dependent pick of bh[d] would make the compiler keep bh and bl
-      // in local memory for the whole kernel.
-      if (pe == 0) {
-#pragma unroll
-        for (int d = 0; d < DH; ++d)
-          if (d0 + d < DLSH_D) bpart[d0 + d] = static_cast<double>(bh[d]) + static_cast<double>(bl[d]);
-      }
-      if (lane < RW - DLSH_D) bpart[DLSH_D + lane] = 0.0;
-    }
-    // sum the warps' partials in order, in float-float (FP64 arithmetic is
-    // slow on this part: one conversion pair and one add per atom instead of
-    // four)
-    __syncthreads();
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-      float h = smf[k], l = smf[K + k];
-      for (int w = 1; w < nw; ++w) {
-        const float* gh = smf + static_cast<size_t>(w) * 2 * K;
-        ff_add(h, l, gh[k], gh[K + k]);
-      }
-      Gp[static_cast<size_t>(seg) * K + k] = static_cast<double>(h) + static_cast<double>(l);
-    }
-    for (int q = threadIdx.x; q < RW; q += blockDim.x) {
-      double acc = 0.0;
-      for (int w = 0; w < nw; ++w)
-        acc += reinterpret_cast<const double*>(smf + static_cast<size_t>(nw) * 2 * K)[w * RW + q];
-      Bp[static_cast<size_t>(seg) * RW + q] = acc;
-    }
-    __syncthreads();  // shared partials are reused by the next segment
+    Gp[static_cast<size_t>(seg) * K + k] = static_cast<double>(r.x) + static_cast<double>(r.y);
   }
 }
 
@@ -609,58 +787,42 @@ __global__ void __launch_bounds__(MT * 8) mirror_kernel(double* __restrict__ M, 
   }
 }
 
-// Segment counts per (block p, atom j) (ceil(n_pj / SEG)) and their exclusive
-// scan, p-major.
-__global__ void seg_scan_kernel(const int* __restrict__ off, const int* __restrict__ atom_start,
-                                int T, int tpb, int K, int PK, int* __restrict__ seg_start) {
-  __shared__ int sm[1024];
-  __shared__ int carry_s;
-  int carry = 0;
-  for (int base = 0; base < PK; base += 1024) {
-    const int pj = base + threadIdx.x;
-    int v = 0;
-    if (pj < PK) {
-      const int p = pj / K, j = pj - p * K;
-      int lo, hi;
-      block_range(off, atom_start, T, tpb, j, p, lo, hi);
-      v = (hi - lo + SEG - 1) / SEG;
-    }
-    int tot = 0;
-    const int ex = block_exclusive_scan(v, sm, &tot);
-    if (pj < PK) seg_start[pj] = carry + ex;
-    if (threadIdx.x == 0) carry_s = carry + tot;
-    __syncthreads();
-    carry = carry_s;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) seg_start[PK] = carry;
-}
-
-// Row j of G and column j of B: the atom's segment partials summed in order.
-__global__ void seg_reduce_kernel(const int* __restrict__ seg_start, const double* __restrict__ Gp,
-                                  const double* __restrict__ Bp, int K, int P,
-                                  double* __restrict__ M, double* __restrict__ Z) {
+// Row j of G (entries k >= j) and column j of B: the atom's segment partials
+// summed in order, chunk (group) by chunk (group).
+__global__ void __launch_bounds__(256) seg_reduce_kernel(const int* __restrict__ segg_start, const int* __restrict__ segb_start,
+                                                        const double* __restrict__ Gp, const double* __restrict__ Bp,
+                                                        int K, int P, int PG, double* __restrict__ M,
+                                                        double* __restrict__ Z) {
   const int j = blockIdx.x;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+  for (int k = j + threadIdx.x; k < K; k += blockDim.x) {
     double acc = 0.0;
-    for (int p = 0; p < P; ++p)
-      for (int sg = seg_start[p * K + j]; sg < seg_start[p * K + j + 1]; ++sg)
-        acc += Gp[static_cast<size_t>(sg) * K + k];
+#pragma unroll 4
+    for (int p = 0; p < PG; ++p) {
+      const int g0 = segg_start[static_cast<size_t>(p) * K + j], g1 = segg_start[static_cast<size_t>(p) * K + j + 1];
+      for (int sg = g0; sg < g1; ++sg) acc += Gp[static_cast<size_t>(sg) * K + k];
+    }
     M[static_cast<size_t>(j) * K + k] = acc;
   }
-  for (int q = threadIdx.x; q < RW; q += blockDim.x) {
+  // B: four groups of threads take every fourth chunk, summed in group order
+  __shared__ double red[4][RW];
+  const int g = threadIdx.x >> 6, q = threadIdx.x & 63;
+  if (q < RW) {
     double acc = 0.0;
-    for (int p = 0; p < P; ++p)
-      for (int sg = seg_start[p * K + j]; sg < seg_start[p * K + j + 1]; ++sg)
+    for (int p = g; p < P; p += 4)
+      for (int sg = segb_start[static_cast<size_t>(p) * K + j]; sg < segb_start[static_cast<size_t>(p) * K + j + 1]; ++sg)
         acc += Bp[static_cast<size_t>(sg) * RW + q];
-    Z[static_cast<size_t>(j) * RW + q] = acc;
+    red[g][q] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x < RW) {
+    const int t = threadIdx.x;
+    Z[static_cast<size_t>(j) * RW + t] = ((red[0][t] + red[1][t]) + red[2][t]) + red[3][t];
   }
 }
 
-static int accum_warps(int K, int s, size_t* smem) {
-  (void)s;
+static int accum_warps(int K, size_t* smem) {
   for (int nw = 4; nw >= 1; --nw) {
-    const size_t b = static_cast<size_t>(nw) * 2 * K * 4 + static_cast<size_t>(nw) * RW * 8;
+    const size_t b = static_cast<size_t>(nw) * K * sizeof(float2);
     if (b <= static_cast<size_t>(SMEM_LIMIT)) {
       *smem = b;
       return nw;
@@ -1183,11 +1345,7 @@ constexpr int KS_V = DLSH_D + 1;   // reduced values: 45 of g R_i, then g^2
 
 struct KsWs {
   uint32_t* status;
-  int* cnt;
-  int* off;
-  int* atom_total;
-  int* atom_start;
-  uint2* list;
+  Sort so;         // records carry the entry's code slot
   float* R;        // N x 48 residual (45 used)
   float* part;     // grid x 48 per-CTA partial sums
   int* dead;
@@ -1198,13 +1356,8 @@ constexpr int KS_MAX_GRID = 1024;
 
 static size_t carve_ksvd(void* base, int K, int s, int64_t N, KsWs& w) {
   Carver c(base);
-  const int64_t T = (N + TS - 1) / TS > 0 ? (N + TS - 1) / TS : 1;
   w.status = c.take<uint32_t>(64);
-  w.cnt = c.take<int>(static_cast<size_t>(K) * T);
-  w.off = c.take<int>(static_cast<size_t>(K) * T);
-  w.atom_total = c.take<int>(K);
-  w.atom_start = c.take<int>(K + 1);
-  w.list = c.take<uint2>(static_cast<size_t>(N) * s + 1);
+  carve_sort(c, K, s, N, w.so);
   w.R = c.take<float>(static_cast<size_t>(N) * RROW);
   w.part = c.take<float>(static_cast<size_t>(KS_MAX_GRID) * 48);
   w.dead = c.take<int>(K);
@@ -1447,6 +1600,35 @@ size_t mod_ws_bytes(int K, int s, int64_t N) {
   return mod::carve(nullptr, K, s, N, w);
 }
 
+namespace mod {
+// Enqueues the counting sort: the atom-major list and its offsets.
+template <bool SLOT>
+static int sort_enqueue(const uint16_t* idx, const float* coef, const uint8_t* nnz, int s, int64_t N, int K,
+                        const Sort& so, uint32_t* status, cudaStream_t st, const char* call) {
+  if (N > 0) {
+    count_kernel<<<so.T, 256, (K + 1) / 2 * sizeof(unsigned), st>>>(idx, nnz, s, so.sdiv, N, K, so.ts, so.cnt, status);
+  } else {
+    DLSH_CUDA_TRY(cudaMemsetAsync(so.cnt, 0, sizeof(int) * K * so.T, st), call);
+  }
+  const dim3 g((K + 255) / 256, so.P);
+  chunk_sum_kernel<<<g, 256, 0, st>>>(so.cnt, so.T, K, so.segb, so.csum, so.segtot);
+  layout_kernel<<<1, 1024, 0, st>>>(so.csum, so.P, K, so.gc, so.PG, static_cast<int>(g.x * g.y), so.segtot, so.atom_start,
+                                    so.segg_start, so.segb_start + static_cast<size_t>(so.P) * K);
+  tile_offsets_kernel<<<g, 256, 0, st>>>(so.cnt, so.T, K, so.segb, so.csum, so.segtot, so.atom_start, so.cstart,
+                                         so.segb_start);
+  count_launches((N > 0 ? 1 : 0) + 3);
+  if (N > 0) {
+    const size_t smem = scatter_smem(K, s, so.ts, so.threads);
+    DLSH_CUDA_TRY(cudaFuncSetAttribute(scatter_kernel<SLOT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       SMEM_LIMIT - 512),
+                  call);
+    scatter_kernel<SLOT><<<so.T, so.threads, smem, st>>>(idx, coef, nnz, s, so.sdiv, N, K, so.ts, so.cnt, so.list);
+    count_launches(1);
+  }
+  return check_launch(call);
+}
+}  // namespace mod
+
 // Enqueues one MOD update (no host synchronisation; capturable).
 int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const float* coef,
                 const uint8_t* nnz, int s, const float* D_old, const float* resid,
@@ -1459,52 +1641,27 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
   carve(ws, K, s, N, w);
   if (status_out) *status_out = w.status;
   size_t acc_smem = 0;
-  const int acc_nw = accum_warps(K, s, &acc_smem);
+  const int acc_nw = accum_warps(K, &acc_smem);
   if (acc_nw == 0)
     return set_error(DLSH_ERR_UNSUPPORTED, "dlsh_mod_update: K=%d s=%d does not fit", K, s);
   DLSH_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(uint32_t), st), "dlsh_mod_update: reset");
-  const int T = static_cast<int>((N + TS - 1) / TS > 0 ? (N + TS - 1) / TS : 1);
   int launches = 0;
-  if (N > 0) {
-    count_kernel<<<T, 256, K * sizeof(int), st>>>(idx, nnz, s, N, K, T, w.cnt, w.status);
-  } else {
-    DLSH_CUDA_TRY(cudaMemsetAsync(w.cnt, 0, sizeof(int) * K * T, st), "dlsh_mod_update: cnt");
-  }
-  atom_total_kernel<<<K, 256, 0, st>>>(w.cnt, T, w.atom_total);
-  atom_scan_kernel<<<1, 1024, 0, st>>>(w.atom_total, K, w.atom_start);
-  tile_offsets_kernel<<<K, 256, 0, st>>>(w.cnt, T, w.atom_start, w.off);
-  launches += (N > 0 ? 1 : 0) + 3;
-  if (N > 0) {
-    const size_t sc_smem = scatter_smem(K, s);
-    DLSH_CUDA_TRY(cudaFuncSetAttribute(scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(sc_smem)),
-                  "dlsh_mod_update: attribute");
-    scatter_kernel<false><<<T, SC_T, sc_smem, st>>>(idx, coef, nnz, s, N, K, T, w.off, w.list);
-    ++launches;
-  }
-  void (*accum)(const float*, const uint16_t*, const float*, int, int, const int*, const int*, int, int, int,
-                const int*, const uint2*, double*, double*) =
-      s <= 8 ? accum_kernel<8> : (s <= 16 ? accum_kernel<16> : accum_kernel<32>);
-  DLSH_CUDA_TRY(cudaFuncSetAttribute(accum, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(acc_smem)),
-                "dlsh_mod_update: attribute");
-  const int P = static_cast<int>(n_blocks(N));
-  const int tpb = tiles_per_block(T);
-  seg_scan_kernel<<<1, 1024, 0, st>>>(w.off, w.atom_start, T, tpb, K, P * K, w.seg_start);
+  const Sort& so = w.so;
+  const int src = sort_enqueue<false>(idx, coef, nnz, s, N, K, so, w.status, st, "dlsh_mod_update: sort");
+  if (src) return src;
   {
-    int sms = device_sm_count();
-    if (sms <= 0) sms = 1;
-    int per_sm = 0;
-    DLSH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accum, acc_nw * 32, acc_smem),
-                  "dlsh_mod_update: occupancy");
-    if (per_sm < 1) per_sm = 1;
-    int64_t grid = static_cast<int64_t>(sms) * per_sm;
-    const int64_t ms = max_segments(K, s, N);
-    if (grid > ms) grid = ms;
-    accum<<<static_cast<int>(grid), acc_nw * 32, acc_smem, st>>>(X, idx, coef, s, K, w.atom_start, w.off, T, tpb,
-                                                                 P * K, w.seg_start, w.list, w.Gp, w.Bp);
+    const int64_t nb = (max_segb(so, K, s, N) + 7) / 8;
+    accum_b_kernel<<<static_cast<int>(nb > 0 ? nb : 1), 256, 0, st>>>(X, K, so.P, so.cstart, so.atom_start, so.segb_start,
+                                                                      so.segb, so.list, w.Bp);
+    void (*accum)(const uint16_t*, const float*, int, int, int, int, int, const int*, const int*, const int*,
+                  const uint2*, double*) =
+        s <= 8 ? accum_g_kernel<1> : (s <= 16 ? accum_g_kernel<2> : accum_g_kernel<4>);
+    DLSH_CUDA_TRY(cudaFuncSetAttribute(accum, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(acc_smem)),
+                  "dlsh_mod_update: attribute");
+    accum<<<static_cast<int>(max_segg(w.so, K, s, N)), acc_nw * 32, acc_smem, st>>>(
+        idx, coef, s, K, so.P, so.gc, so.PG, so.cstart, so.atom_start, so.segg_start, so.list, w.Gp);
   }
-  seg_reduce_kernel<<<K, 256, 0, st>>>(w.seg_start, w.Gp, w.Bp, K, P, w.M, w.Z);
+  seg_reduce_kernel<<<K, 256, 0, st>>>(so.segg_start, so.segb_start, w.Gp, w.Bp, K, so.P, so.PG, w.M, w.Z);
   {
     const int nb = (K + MT - 1) / MT;
     mirror_kernel<<<dim3(nb, nb), MT * 8, 0, st>>>(w.M, K);
@@ -1552,7 +1709,7 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
     trmm_kernel<true><<<tr_grid, 256, 0, st>>>(w.W32, K, w.Y32, nullptr, w.Xs, w.dsc, w.Xb);
     launches += 2;
   }
-  normalise_kernel<<<(K + 7) / 8, 256, 0, st>>>(w.Xb, w.atom_start, K, D_new, D_old, w.dead);
+  normalise_kernel<<<(K + 7) / 8, 256, 0, st>>>(w.Xb, so.atom_start, K, D_new, D_old, w.dead);
   ++launches;
   if (resid && N > 0) {
     refill_kernel<<<1, 1024, 0, st>>>(X, resid, N, K, w.dead, D_new);
@@ -1578,25 +1735,12 @@ int ksvd_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, float* c
   carve_ksvd(ws, K, s, N, w);
   if (status_out) *status_out = w.status;
   DLSH_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(uint32_t), st), "dlsh_ksvd_update: reset");
-  const int T = static_cast<int>((N + TS - 1) / TS > 0 ? (N + TS - 1) / TS : 1);
   int launches = 0;
+  const int src = sort_enqueue<true>(idx, coef, nnz, s, N, K, w.so, w.status, st, "dlsh_ksvd_update: sort");
+  if (src) return src;
   if (N > 0) {
-    count_kernel<<<T, 256, K * sizeof(int), st>>>(idx, nnz, s, N, K, T, w.cnt, w.status);
-  } else {
-    DLSH_CUDA_TRY(cudaMemsetAsync(w.cnt, 0, sizeof(int) * K * T, st), "dlsh_ksvd_update: cnt");
-  }
-  atom_total_kernel<<<K, 256, 0, st>>>(w.cnt, T, w.atom_total);
-  atom_scan_kernel<<<1, 1024, 0, st>>>(w.atom_total, K, w.atom_start);
-  tile_offsets_kernel<<<K, 256, 0, st>>>(w.cnt, T, w.atom_start, w.off);
-  launches += (N > 0 ? 1 : 0) + 3;
-  if (N > 0) {
-    const size_t sc_smem = scatter_smem(K, s);
-    DLSH_CUDA_TRY(cudaFuncSetAttribute(scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(sc_smem)),
-                  "dlsh_ksvd_update: attribute");
-    scatter_kernel<true><<<T, SC_T, sc_smem, st>>>(idx, coef, nnz, s, N, K, T, w.off, w.list);
     ksvd_resid_kernel<<<static_cast<int>((N + 7) / 8), 256, 0, st>>>(X, D_old, K, idx, coef, nnz, s, N, w.R);
-    launches += 2;
+    launches += 1;
   }
   {
     static PerDevice<int> coop;
@@ -1619,8 +1763,8 @@ int ksvd_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, float* c
     if (crc) return crc;
     const size_t smem = static_cast<size_t>(coop_grid) * 48 * sizeof(float);
     DLSH_CUDA_TRY(cudaMemsetAsync(w.gbar, 0, 2 * sizeof(unsigned), st), "dlsh_ksvd_update: barrier");
-    const int* as = w.atom_start;
-    const uint2* li = w.list;
+    const int* as = w.so.atom_start;
+    const uint2* li = w.so.list;
     int Kk = K, ss = s;
     float* cf = coef;
     const float* Do = D_old;

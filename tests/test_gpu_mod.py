@@ -37,6 +37,27 @@ def test_mod_matches_oracle(lib, N, K, s):
     np.testing.assert_allclose(got, ref, atol=3e-6, rtol=0)
 
 
+@pytest.mark.parametrize("N,K,s,skip", [(513, 40, 1, 0), (9000, 1500, 8, 0), (65537, 128, 17, 0), (33000, 96, 32, 2),
+                                        (330_000, 300, 3, 2), (311_297, 64, 8, 0)])
+def test_mod_on_random_codes(lib, N, K, s, skip):
+    """Uneven code lengths and codes that name an atom twice, at the edges of the
+    sort's tiles (512 and, from 311,296 signals on, 1024 signals), chunks and
+    segments; skip > 0 hands in arrays that start off 16-byte alignment.  Atoms
+    within 3e-6 as above (FP32 output of an FP64-accurate solve)."""
+    D = synth.hidden_dictionary(K, 11)
+    idx, coef, nnz = synth.random_codes(N + skip, K, s, 12)
+    X = np.einsum("ns,nsd->nd", coef.astype(np.float64), D[idx]) if N < 100_000 else sum(
+        coef[:, t, None].astype(np.float64) * D[idx[:, t]] for t in range(s))
+    X = (X + 0.05 * np.random.default_rng(13).standard_normal(X.shape)).astype(np.float32)
+    D0 = synth.hidden_dictionary(K, 14).astype(np.float32)
+    c = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()[skip:]  # noqa: E731
+    got = lib.mod_update(c(X), torch.from_numpy(D0).cuda(), c(idx.view(np.int16)), c(coef), c(nnz),
+                         sync=True).cpu().numpy()
+    ref, info = omod.mod_update(X[skip:].astype(np.float64), D0.astype(np.float64), idx[skip:].astype(np.int64),
+                                coef[skip:].astype(np.float64), nnz[skip:], np.zeros(N))
+    np.testing.assert_allclose(got, ref, atol=3e-6, rtol=0)
+
+
 def test_dead_atoms_refilled_in_order(lib):
     N, K, s = 4000, 64, 4
     X, D0, idx, coef, nnz, resid = _inputs(N, K, s, seed=5)
