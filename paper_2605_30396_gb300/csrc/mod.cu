@@ -30,8 +30,7 @@
 //      (right-looking steps over [A | I], a grid barrier between phases);
 //      each FP32 solve is then two triangular products with W = L^-1, and
 //      iterative refinement uses the residual of the scaled system computed
-//      in FP64 (GB300's FP64 rate is a small fraction of its FP32 rate, so
-//      FP64 is spent only there)
+//      in float-float
 //   6. normalise, then refill unused atoms (argmax passes over resid_sq)
 //
 // The same file holds the other reading of the D-step, the approximate K-SVD
@@ -54,7 +53,7 @@ constexpr int RW = 48;         // padded RHS width (45 used)
 constexpr int MAX_K = 4096;    // shared-memory G-row partials limit
 constexpr int SMEM_LIMIT = 232448;
 constexpr double RIDGE_REL = 1e-6;
-constexpr int kRefine = 3;     // FP32 solves (two FP64 residual corrections)
+constexpr int kRefine = 3;     // FP32 solves (two float-float residual corrections)
 
 // The counting sort of the codes by atom, shared by both dictionary updates.
 struct Sort {
@@ -113,18 +112,18 @@ inline int64_t max_segg(const Sort& so, int K, int s, int64_t N) {
 struct Ws {
   uint32_t* status;
   Sort so;         // the atom-major list
-  double* M;       // K x K: G + lambda I (FP64, kept for the refinement residuals)
-  double* Z;       // K x RW: B^T (lambda D_old is added where Z is read)
+  double* M;       // K x K: G (FP64, entries k >= j of row j)
+  double* Z;       // K x RW: B^T
   double* lam;     // [0] lambda
-  double* dsc;     // K: Jacobi scale 1 / sqrt(M_jj)
-  float* A32;      // K x K: S M S, then its FP32 Cholesky factor (lower)
+  double* dsc;     // K: Jacobi scale 1 / sqrt(M_jj + lambda)
+  float2* S;       // K x K: the scaled matrix, float-float
+  float* A32;      // K x K: the same in FP32 (lower), then its Cholesky factor
   float* W32;      // K x K: L^-1 (lower)
   float* Y32;      // K x RW: W r, between the two triangular products
   unsigned* gbar;  // grid barrier of the factorisation: arrivals, generation
-  double* Zs;      // K x RW: S Z
-  double* Xs;      // K x RW: solution of the scaled system (FP64 accumulation)
+  float2* Zs;      // K x RW: scaled right-hand side
+  float2* Xs;      // K x RW: solution of the scaled system
   float* R32;      // K x RW: current residual of the scaled system
-  double* Xb;      // K x RW: D~^T = S Xs, kept up to date with Xs
   int* dead;       // K
   double* Gp;      // G segments x K partial rows
   double* Bp;      // B segments x RW partial columns
@@ -138,14 +137,14 @@ static size_t carve(void* base, int K, int s, int64_t N, Ws& w) {
   w.Z = c.take<double>(static_cast<size_t>(K) * RW);
   w.lam = c.take<double>(4);
   w.dsc = c.take<double>(K);
+  w.S = c.take<float2>(static_cast<size_t>(K) * K);
   w.A32 = c.take<float>(static_cast<size_t>(K) * K);
   w.W32 = c.take<float>(static_cast<size_t>(K) * K);
   w.Y32 = c.take<float>(static_cast<size_t>(K) * RW);
   w.gbar = c.take<unsigned>(64);
-  w.Zs = c.take<double>(static_cast<size_t>(K) * RW);
-  w.Xs = c.take<double>(static_cast<size_t>(K) * RW);
+  w.Zs = c.take<float2>(static_cast<size_t>(K) * RW);
+  w.Xs = c.take<float2>(static_cast<size_t>(K) * RW);
   w.R32 = c.take<float>(static_cast<size_t>(K) * RW);
-  w.Xb = c.take<double>(static_cast<size_t>(K) * RW);
   w.dead = c.take<int>(K);
   w.Gp = c.take<double>(static_cast<size_t>(max_segg(w.so, K, s, N)) * K);
   w.Bp = c.take<double>(static_cast<size_t>(max_segb(w.so, K, s, N)) * RW);
@@ -765,28 +764,6 @@ __global__ void __launch_bounds__(128) accum_g_kernel(const uint16_t* __restrict
   }
 }
 
-// M's lower triangle from its upper one: row j of G holds the entries k >= j,
-// so M[k][j] = M[j][k] for k > j (32 x 32 tiles through shared memory; only
-// the tiles on or above the diagonal are read).
-constexpr int MT = 32;
-__global__ void __launch_bounds__(MT * 8) mirror_kernel(double* __restrict__ M, int K) {
-  __shared__ double t[MT][MT + 1];
-  const int rb = blockIdx.y, cb = blockIdx.x;  // source tile: rows rb, columns cb >= rb
-  if (cb < rb) return;
-  const int x = threadIdx.x % MT, y0 = threadIdx.x / MT;
-  for (int y = y0; y < MT; y += 8) {
-    const int r = rb * MT + y, c = cb * MT + x;
-    t[y][x] = (r < K && c < K) ? M[static_cast<size_t>(r) * K + c] : 0.0;
-  }
-  __syncthreads();
-  // destination: row cb*MT + y, column rb*MT + x, written where it lies below
-  // the diagonal
-  for (int y = y0; y < MT; y += 8) {
-    const int r = cb * MT + y, c = rb * MT + x;
-    if (r < K && c < K && r > c) M[static_cast<size_t>(r) * K + c] = t[x][y];
-  }
-}
-
 // Row j of G (entries k >= j) and column j of B: the atom's segment partials
 // summed in order, chunk (group) by chunk (group).
 __global__ void __launch_bounds__(256) seg_reduce_kernel(const int* __restrict__ segg_start, const int* __restrict__ segb_start,
@@ -831,8 +808,9 @@ static int accum_warps(int K, size_t* smem) {
   return 0;
 }
 
-// ---- 5a. lambda = 1e-6 trace(G)/K (applied where M and Z are read) ----------
-__global__ void ridge_kernel(const double* __restrict__ M, int K, double* lam_out) {
+// ---- 5a. lambda = 1e-6 trace(G)/K and the Jacobi scale 1 / sqrt(M_jj + lambda) ----
+__global__ void __launch_bounds__(1024) ridge_kernel(const double* __restrict__ M, int K, double* lam_out,
+                                                     double* __restrict__ dsc) {
   __shared__ double part[1024];
   double acc = 0.0;
   for (int j = threadIdx.x; j < K; j += blockDim.x) acc += M[static_cast<size_t>(j) * K + j];
@@ -842,40 +820,64 @@ __global__ void ridge_kernel(const double* __restrict__ M, int K, double* lam_ou
     if (static_cast<int>(threadIdx.x) < w) part[threadIdx.x] += part[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    const double tr = part[0];
-    *lam_out = tr > 0.0 ? RIDGE_REL * tr / K : RIDGE_REL;
-  }
+  const double tr = part[0];
+  const double lam = tr > 0.0 ? RIDGE_REL * tr / K : RIDGE_REL;
+  if (threadIdx.x == 0) *lam_out = lam;
+  for (int j = threadIdx.x; j < K; j += blockDim.x) dsc[j] = 1.0 / sqrt(M[static_cast<size_t>(j) * K + j] + lam);
 }
 
-// ---- 5b. Jacobi scaling: S = diag(M)^-1/2, A = S M S (FP32, lower), Zs = S Z --
-// One CTA per row j.  A has a unit diagonal, which keeps the FP32 factorisation
-// well scaled; the refinement below works on the same scaled system in FP64.
-// M and Z stay as accumulated; lambda enters here and in the residuals:
-// (M + lambda I) and (Z + lambda D_old).
-__global__ void scale_kernel(const double* __restrict__ M, const double* __restrict__ Z,
-                             const float* __restrict__ D_old, const double* __restrict__ lamp, int K,
-                             double* __restrict__ dsc, float* __restrict__ A,
-                             double* __restrict__ Zs, float* __restrict__ R32,
-                             double* __restrict__ Xs, double* __restrict__ Xb) {
-  const int j = blockIdx.x;
+// ---- 5b. the scaled system: S = diag(d) (M + lambda I) diag(d) from M's upper
+// triangle (row j of G holds the entries k >= j), whole, as float-float pairs for
+// the residuals, and its lower triangle in FP32 for the factorisation; right-hand
+// side Zs = d (Z + lambda D_old).  One CTA per 32 x 32 tile on or above the
+// diagonal, its mirror image written through shared memory.  S has a unit
+// diagonal, which keeps the FP32 factorisation well scaled.
+__device__ __forceinline__ float2 ff_split(double x) {
+  const float h = static_cast<float>(x);
+  return make_float2(h, static_cast<float>(x - static_cast<double>(h)));
+}
+constexpr int MT = 32;
+__global__ void __launch_bounds__(MT * 8) scale_kernel(const double* __restrict__ M, const double* __restrict__ Z,
+                                                       const float* __restrict__ D_old,
+                                                       const double* __restrict__ lamp,
+                                                       const double* __restrict__ dsc, int K, float2* __restrict__ S,
+                                                       float* __restrict__ A, float2* __restrict__ Zs,
+                                                       float* __restrict__ R32, float2* __restrict__ Xs) {
+  __shared__ float2 t[MT][MT + 1];
+  const int rb = blockIdx.y, cb = blockIdx.x;  // tile: rows rb, columns cb >= rb
+  if (cb < rb) return;
   const double lam = *lamp;
-  const double dj = 1.0 / sqrt(M[static_cast<size_t>(j) * K + j] + lam);
-  if (threadIdx.x == 0) dsc[j] = dj;
-  for (int k = threadIdx.x; k <= j; k += blockDim.x) {
-    const double dk = 1.0 / sqrt(M[static_cast<size_t>(k) * K + k] + lam);
-    const double m = M[static_cast<size_t>(j) * K + k] + (k == j ? lam : 0.0);
-    A[static_cast<size_t>(j) * K + k] = static_cast<float>(dj * m * dk);
+  const int x = threadIdx.x % MT, y0 = threadIdx.x / MT;
+  for (int y = y0; y < MT; y += 8) {
+    const int r = rb * MT + y, c = cb * MT + x;
+    float2 v = make_float2(0.f, 0.f);
+    if (r < K && c < K && r <= c) {
+      const double m = M[static_cast<size_t>(r) * K + c] + (r == c ? lam : 0.0);
+      v = ff_split(dsc[c] * m * dsc[r]);
+      S[static_cast<size_t>(r) * K + c] = v;
+    }
+    t[y][x] = v;
   }
-  for (int c = threadIdx.x; c < RW; c += blockDim.x) {
-    const double z = c < DLSH_D ? dj * (Z[static_cast<size_t>(j) * RW + c] +
-                                        lam * static_cast<double>(D_old[static_cast<size_t>(j) * DLSH_D + c]))
-                                : 0.0;
-    Zs[static_cast<size_t>(j) * RW + c] = z;
-    R32[static_cast<size_t>(j) * RW + c] = static_cast<float>(z);
-    Xs[static_cast<size_t>(j) * RW + c] = 0.0;
-    Xb[static_cast<size_t>(j) * RW + c] = 0.0;
+  __syncthreads();
+  for (int y = y0; y < MT; y += 8) {
+    const int r = cb * MT + y, c = rb * MT + x;
+    if (r < K && c < K && r >= c) {
+      const float2 v = t[x][y];
+      if (r > c) S[static_cast<size_t>(r) * K + c] = v;
+      A[static_cast<size_t>(r) * K + c] = v.x;
+    }
   }
+  if (rb == cb)
+    for (int f = threadIdx.x; f < MT * RW; f += MT * 8) {
+      const int r = rb * MT + f / RW, c = f % RW;
+      if (r >= K) break;
+      const size_t o = static_cast<size_t>(r) * RW + c;
+      const double z =
+          c < DLSH_D ? dsc[r] * (Z[o] + lam * static_cast<double>(D_old[static_cast<size_t>(r) * DLSH_D + c])) : 0.0;
+      Zs[o] = ff_split(z);
+      R32[o] = static_cast<float>(z);
+      Xs[o] = make_float2(0.f, 0.f);
+    }
 }
 
 // ---- 5c. FP32 Cholesky of A and the inverse of its factor, W = L^-1 ----------
@@ -897,7 +899,7 @@ constexpr int CH_TILE = 64;
 // the identity): L into Ls, L^-1 into Li (both lower, [32][33]).  Lane r holds
 // row r in registers; pivots and entries move by shuffles.  Every loop is
 // unrolled over the full block so that the rows stay in registers, and the
-// pivots use the hardware reciprocal square root: the FP64 refinement of the
+// pivots use the hardware reciprocal square root: the refinement of the
 // solve absorbs its last-bit error.
 __device__ void factor_diag(const float* __restrict__ A, int K, int k0, int nb, float (*Ls)[NB + 1],
                             float (*Li)[NB + 1], bool& bad) {
@@ -1088,136 +1090,146 @@ __global__ void __launch_bounds__(CH_T) chol_inv_kernel(float* __restrict__ A, f
   }
 }
 
-// ---- 5d. FP32 solve of (L L^T) c = r with W = L^-1: y = W r, then c = W^T y,
-// and X += c in FP64.  One warp per output row: the lanes split the inner index,
-// each keeps the row's 48 partial sums, and a butterfly adds them up.  No
-// shared memory and no block barriers: every row proceeds independently.
+// ---- 5d, 5e. products with the 48-column right-hand sides -------------------------
+// Eight output rows per CTA, their matrix entries staged in shared memory, the
+// inner index dealt to 16 warps; in a warp lane (row, g) = (lane / 4, lane % 4)
+// keeps the row's columns 12 g .. 12 g + 11, and the warps' sums are added in
+// order.  K / 8 CTAs: latency and the L2 reads of the right-hand side bound
+// them.  At K = 1024 a triangular product takes 15 us and a residual 44 (one warp
+// per row with 48 sums per lane: 33 to 46; the residual in FP64: 155 to 190, of
+// which its arithmetic alone 80).
+constexpr int PR = 8;              // rows per CTA
+constexpr int PT = 512;            // threads per CTA
+constexpr int PKC = 1024;          // inner indices staged at once
+constexpr int PS = PKC + 4;        // row stride of the stage: the rows start on different banks
+
+// FP32 solve of (L L^T) c = r with W = L^-1: y = W r (TRANS = false), then
+// c = W^T y and X += c in float-float.  W's upper triangle is zero.
 template <bool TRANS>
-__global__ void __launch_bounds__(256) trmm_kernel(const float* __restrict__ W, int K,
-                                                   const float* __restrict__ in, float* __restrict__ out,
-                                                   double* __restrict__ Xs, const double* __restrict__ dsc,
-                                                   double* __restrict__ Xb) {
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= K) return;
-  float acc[RW];
+__global__ void __launch_bounds__(PT) trmm_kernel(const float* __restrict__ W, int K, const float* __restrict__ in,
+                                                  float* __restrict__ out, float2* __restrict__ Xs) {
+  extern __shared__ __align__(16) float psm[];  // [PR][PS], then the warps' sums
+  const int j0 = blockIdx.x * PR;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = lane >> 2, c0 = (lane & 3) * 12;
+  const int kb = TRANS ? j0 : 0, ke = TRANS ? K : (j0 + PR < K ? j0 + PR : K);
+  float acc[12];
 #pragma unroll
-  for (int c = 0; c < RW; ++c) acc[c] = 0.f;
-  // W lower: y_i = sum_{j <= i} W_ij r_j;  W^T: c_j = sum_{i >= j} W_ij y_i
-  const int k_begin = TRANS ? row : 0;
-  const int k_end = TRANS ? K : row + 1;
-  for (int k = k_begin + lane; k < k_end; k += 32) {
-    const float w = TRANS ? W[static_cast<size_t>(k) * K + row] : W[static_cast<size_t>(row) * K + k];
-    const float4* v = reinterpret_cast<const float4*>(in + static_cast<size_t>(k) * RW);
-#pragma unroll
-    for (int q = 0; q < RW / 4; ++q) {
-      const float4 x = v[q];
-      acc[4 * q] = fmaf(w, x.x, acc[4 * q]);
-      acc[4 * q + 1] = fmaf(w, x.y, acc[4 * q + 1]);
-      acc[4 * q + 2] = fmaf(w, x.z, acc[4 * q + 2]);
-      acc[4 * q + 3] = fmaf(w, x.w, acc[4 * q + 3]);
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < RW; ++c)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-  // every lane holds every sum; lane l stores columns l and 32 + l
-  float v0 = 0.f, v1 = 0.f;
-#pragma unroll
-  for (int c = 0; c < 32; ++c) v0 = lane == c ? acc[c] : v0;
-#pragma unroll
-  for (int c = 32; c < RW; ++c) v1 = lane == c - 32 ? acc[c] : v1;
-  if (TRANS) {
-    // the solution and its unscaled form D~^T = S Xs, which the FP64 residual
-    // and the normalisation read
-    const size_t o = static_cast<size_t>(row) * RW;
-    const double dr = dsc[row];
-    const double x0 = Xs[o + lane] + static_cast<double>(v0);
-    Xs[o + lane] = x0;
-    Xb[o + lane] = dr * x0;
-    if (lane < DLSH_D - 32) {
-      const double x1 = Xs[o + 32 + lane] + static_cast<double>(v1);
-      Xs[o + 32 + lane] = x1;
-      Xb[o + 32 + lane] = dr * x1;
-    }
-  } else {
-    out[static_cast<size_t>(row) * RW + lane] = v0;
-    if (lane < RW - 32) out[static_cast<size_t>(row) * RW + 32 + lane] = v1;
-  }
-}
-
-// ---- 5e. FP64 residual of the scaled system: R = Zs - (S M S) X, as FP32 -----
-// 8 x 48 output tiles (K/8 CTAs, so the FP64 pipes of every SM take part);
-// thread (row tid / 24, columns tid % 24 and tid % 24 + 24); k in chunks of 32.
-constexpr int RS_ROWS = 8;
-constexpr int RS_T = 256;   // four groups of 64 threads split each k chunk
-__global__ void __launch_bounds__(RS_T) residual_kernel(const double* __restrict__ M,
-                                                        const double* __restrict__ lamp,
-                                                        const double* __restrict__ dsc, int K,
-                                                        const double* __restrict__ Zs,
-                                                        const double* __restrict__ Xb,
-                                                        float* __restrict__ R32) {
-  __shared__ double Ms[RS_ROWS][33];
-  __shared__ double Xt[32][RW + 1];
-  __shared__ double red[4][RS_ROWS][RW];
-  const int j0 = blockIdx.x * RS_ROWS;
-  const double lam = *lamp;
-  const int g = threadIdx.x >> 6, t = threadIdx.x & 63;
-  const int r0 = (t >> 4) * 2, c0 = (t & 15) * 3;  // 2 rows x 3 columns per thread
-  double acc[2][3] = {};
-  for (int k0 = 0; k0 < K; k0 += 32) {
-    {
-      const int r = threadIdx.x / 32, c = threadIdx.x % 32;
-      Ms[r][c] = (j0 + r < K && k0 + c < K)
-                     ? M[static_cast<size_t>(j0 + r) * K + k0 + c] + (j0 + r == k0 + c ? lam : 0.0)
-                     : 0.0;
-    }
-    for (int f = threadIdx.x; f < 32 * RW; f += RS_T) {
-      const int r = f / RW, c = f % RW;
-      Xt[r][c] = k0 + r < K ? Xb[static_cast<size_t>(k0 + r) * RW + c] : 0.0;
+  for (int c = 0; c < 12; ++c) acc[c] = 0.f;
+  for (int k0 = kb; k0 < ke; k0 += PKC) {
+    const int kn = ke - k0 < PKC ? ke - k0 : PKC;
+    __syncthreads();
+    for (int f = threadIdx.x; f < PR * kn; f += PT) {
+      const int r = TRANS ? f % PR : f / kn, k = TRANS ? f / PR : f % kn;
+      psm[r * PS + k] = j0 + r < K ? (TRANS ? W[static_cast<size_t>(k0 + k) * K + j0 + r]
+                                            : W[static_cast<size_t>(j0 + r) * K + k0 + k])
+                                   : 0.f;
     }
     __syncthreads();
+#pragma unroll 4
+    for (int k = warp; k < kn; k += PT / 32) {
+      const float w = psm[row * PS + k];
+      const float4* v = reinterpret_cast<const float4*>(in + static_cast<size_t>(k0 + k) * RW + c0);
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-      const int k = kk * 4 + g;
-      const double m0 = Ms[r0][k], m1 = Ms[r0 + 1][k];
-      const double x0 = Xt[k][c0], x1 = Xt[k][c0 + 1], x2 = Xt[k][c0 + 2];
-      acc[0][0] = fma(m0, x0, acc[0][0]);
-      acc[0][1] = fma(m0, x1, acc[0][1]);
-      acc[0][2] = fma(m0, x2, acc[0][2]);
-      acc[1][0] = fma(m1, x0, acc[1][0]);
-      acc[1][1] = fma(m1, x1, acc[1][1]);
-      acc[1][2] = fma(m1, x2, acc[1][2]);
+      for (int q = 0; q < 3; ++q) {
+        const float4 x = __ldg(v + q);
+        acc[4 * q] = fmaf(w, x.x, acc[4 * q]);
+        acc[4 * q + 1] = fmaf(w, x.y, acc[4 * q + 1]);
+        acc[4 * q + 2] = fmaf(w, x.z, acc[4 * q + 2]);
+        acc[4 * q + 3] = fmaf(w, x.w, acc[4 * q + 3]);
+      }
     }
-    __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int jj = 0; jj < 3; ++jj) red[g][r0 + i][c0 + jj] = acc[i][jj];
   __syncthreads();
-  // the four k groups in a fixed order
-  for (int f = threadIdx.x; f < RS_ROWS * RW; f += RS_T) {
-    const int r = f / RW, c = f % RW;
-    const int j = j0 + r;
-    if (j < K) {
-      const double sum = ((red[0][r][c] + red[1][r][c]) + red[2][r][c]) + red[3][r][c];
-      R32[static_cast<size_t>(j) * RW + c] = static_cast<float>(Zs[static_cast<size_t>(j) * RW + c] - dsc[j] * sum);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) psm[(warp * PR + row) * RW + c0 + c] = acc[c];
+  __syncthreads();
+  if (threadIdx.x < PR * RW && j0 + threadIdx.x / RW < K) {
+    float sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < PT / 32; ++w) sum += psm[w * PR * RW + threadIdx.x];
+    const size_t o = static_cast<size_t>(j0) * RW + threadIdx.x;
+    if (TRANS) {
+      float2 x = Xs[o];
+      ff_add(x.x, x.y, sum, 0.f);
+      Xs[o] = x;
+    } else {
+      out[o] = sum;
     }
   }
 }
 
+// Residual of the scaled system, R = Zs - S X, in float-float (products exact,
+// about 48 bits; FP64 runs at 1/64 of the FP32 rate here), as FP32.
+__global__ void __launch_bounds__(PT) residual_kernel(const float2* __restrict__ S, int K,
+                                                      const float2* __restrict__ Zs, const float2* __restrict__ Xs,
+                                                      float* __restrict__ R32) {
+  extern __shared__ __align__(16) float2 rsm[];  // [PR][PS], then the warps' sums
+  const int j0 = blockIdx.x * PR;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = lane >> 2, c0 = (lane & 3) * 12;
+  f2 h[6], l[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) h[c] = l[c] = f2_make(0.f, 0.f);
+  for (int k0 = 0; k0 < K; k0 += PKC) {
+    const int kn = K - k0 < PKC ? K - k0 : PKC;
+    __syncthreads();
+    for (int f = threadIdx.x; f < PR * kn; f += PT) {
+      const int r = f / kn, k = f % kn;
+      rsm[r * PS + k] = j0 + r < K ? S[static_cast<size_t>(j0 + r) * K + k0 + k] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int k = warp; k < kn; k += PT / 32) {
+      const float2 m = rsm[row * PS + k];
+      const f2 mh = f2_make(m.x, m.x), nmh = f2_make(-m.x, -m.x), ml = f2_make(m.y, m.y);
+      const float4* v = reinterpret_cast<const float4*>(Xs + static_cast<size_t>(k0 + k) * RW + c0);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const float4 x = __ldg(v + c);  // (hi, lo) of two columns
+        const f2 xh = f2_make(x.x, x.z);
+        f2_acc(h[c], l[c], mh, nmh, xh);
+        l[c] = f2_fma(mh, f2_make(x.y, x.w), f2_fma(ml, xh, l[c]));
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    f2_norm(h[c], l[c]);
+    float h0, h1, l0, l1;
+    f2_get(h[c], h0, h1);
+    f2_get(l[c], l0, l1);
+    rsm[(warp * PR + row) * RW + c0 + 2 * c] = make_float2(h0, l0);
+    rsm[(warp * PR + row) * RW + c0 + 2 * c + 1] = make_float2(h1, l1);
+  }
+  __syncthreads();
+  if (threadIdx.x < PR * RW && j0 + threadIdx.x / RW < K) {
+    const size_t o = static_cast<size_t>(j0) * RW + threadIdx.x;
+    float2 r = Zs[o];
+    for (int w = 0; w < PT / 32; ++w) {
+      const float2 p = rsm[w * PR * RW + threadIdx.x];
+      ff_add(r.x, r.y, -p.x, -p.y);
+    }
+    R32[o] = r.x;
+  }
+}
+constexpr int PSM32 = PR * PS * 4 > (PT / 32) * PR * RW * 4 ? PR * PS * 4 : (PT / 32) * PR * RW * 4;
+constexpr int PSM64 = 2 * PSM32;
 
 // ---- 6a. normalise; mark dead atoms ----------------------------------------------
-__global__ void normalise_kernel(const double* __restrict__ Z, const int* __restrict__ atom_start,
+__global__ void normalise_kernel(const float2* __restrict__ Xs, const double* __restrict__ dsc,
+                                 const int* __restrict__ atom_start,
                                  int K, float* __restrict__ D_new, const float* __restrict__ D_old,
                                  int* __restrict__ dead) {
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (j >= K) return;
-  const double z0 = Z[static_cast<size_t>(j) * RW + lane];
-  const double z1 = lane < DLSH_D - 32 ? Z[static_cast<size_t>(j) * RW + 32 + lane] : 0.0;
+  // D~^T = diag(d) Xs
+  const float2 x0 = Xs[static_cast<size_t>(j) * RW + lane];
+  const float2 x1 = lane < DLSH_D - 32 ? Xs[static_cast<size_t>(j) * RW + 32 + lane] : make_float2(0.f, 0.f);
+  const double z0 = dsc[j] * (static_cast<double>(x0.x) + static_cast<double>(x0.y));
+  const double z1 = dsc[j] * (static_cast<double>(x1.x) + static_cast<double>(x1.y));
   double n2 = z0 * z0 + z1 * z1;
   for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
   const bool unused = atom_start[j + 1] == atom_start[j];
@@ -1662,16 +1674,14 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
         idx, coef, s, K, so.P, so.gc, so.PG, so.cstart, so.atom_start, so.segg_start, so.list, w.Gp);
   }
   seg_reduce_kernel<<<K, 256, 0, st>>>(so.segg_start, so.segb_start, w.Gp, w.Bp, K, so.P, so.PG, w.M, w.Z);
+  ridge_kernel<<<1, 1024, 0, st>>>(w.M, K, w.lam, w.dsc);
+  // mixed-precision solve: FP32 Cholesky of the Jacobi-scaled matrix, then
+  // kRefine FP32 solves with float-float residuals in between
   {
     const int nb = (K + MT - 1) / MT;
-    mirror_kernel<<<dim3(nb, nb), MT * 8, 0, st>>>(w.M, K);
+    scale_kernel<<<dim3(nb, nb), MT * 8, 0, st>>>(w.M, w.Z, D_old, w.lam, w.dsc, K, w.S, w.A32, w.Zs, w.R32, w.Xs);
   }
-  ridge_kernel<<<1, 1024, 0, st>>>(w.M, K, w.lam);
   launches += 5;
-  // mixed-precision solve: FP32 Cholesky of the Jacobi-scaled matrix, then
-  // kRefine FP32 solves with FP64 residuals in between
-  scale_kernel<<<K, 256, 0, st>>>(w.M, w.Z, D_old, w.lam, K, w.dsc, w.A32, w.Zs, w.R32, w.Xs, w.Xb);
-  ++launches;
   {
     static PerDevice<int> coop;
     int coop_grid = 0;
@@ -1699,17 +1709,19 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
                   "dlsh_mod_update: factorisation");
     ++launches;
   }
-  const int tr_grid = (K + 7) / 8;
+  DLSH_CUDA_TRY(cudaFuncSetAttribute(residual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PSM64),
+                "dlsh_mod_update: attribute");
+  const int rows = (K + PR - 1) / PR;
   for (int it = 0; it < kRefine; ++it) {
     if (it > 0) {
-      residual_kernel<<<(K + RS_ROWS - 1) / RS_ROWS, RS_T, 0, st>>>(w.M, w.lam, w.dsc, K, w.Zs, w.Xb, w.R32);
+      residual_kernel<<<rows, PT, PSM64, st>>>(w.S, K, w.Zs, w.Xs, w.R32);
       ++launches;
     }
-    trmm_kernel<false><<<tr_grid, 256, 0, st>>>(w.W32, K, w.R32, w.Y32, nullptr, nullptr, nullptr);
-    trmm_kernel<true><<<tr_grid, 256, 0, st>>>(w.W32, K, w.Y32, nullptr, w.Xs, w.dsc, w.Xb);
+    trmm_kernel<false><<<rows, PT, PSM32, st>>>(w.W32, K, w.R32, w.Y32, nullptr);
+    trmm_kernel<true><<<rows, PT, PSM32, st>>>(w.W32, K, w.Y32, nullptr, w.Xs);
     launches += 2;
   }
-  normalise_kernel<<<(K + 7) / 8, 256, 0, st>>>(w.Xb, so.atom_start, K, D_new, D_old, w.dead);
+  normalise_kernel<<<(K + 7) / 8, 256, 0, st>>>(w.Xs, w.dsc, so.atom_start, K, D_new, D_old, w.dead);
   ++launches;
   if (resid && N > 0) {
     refill_kernel<<<1, 1024, 0, st>>>(X, resid, N, K, w.dead, D_new);
