@@ -115,6 +115,33 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, long long budget, ui
   return ok_s != 0;
 }
 
+// The same without a generation: *count (zeroed before the launch) only counts
+// arrivals, and the caller passes how many barriers it has reached, this one
+// included (1, 2, ..).  One reduction per CTA and a spin without sleeping.
+__device__ __forceinline__ bool grid_barrier_count(unsigned* count, unsigned reached, long long budget,
+                                                   uint32_t* status) {
+  __shared__ int ok_s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+    const unsigned want = reached * gridDim.x;
+    const long long t0 = clock64();
+    while (static_cast<int>(ld_acquire_u32(count) - want) < 0) {
+      if (clock64() - t0 > budget) {
+        flag_status(status, ST_TIMEOUT);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+    ok_s = ok;
+  }
+  __syncthreads();
+  return ok_s != 0;
+}
+
 // ---- proxy fences --------------------------------------------------------
 // Make generic-proxy shared-memory writes visible to the async proxy (TMA and
 // the tensor cores read shared memory through it).

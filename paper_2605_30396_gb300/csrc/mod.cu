@@ -27,7 +27,7 @@
 //   5. mixed-precision solve of (G + lambda I) D~^T = (B + lambda D_old)^T:
 //      Jacobi scaling S = diag^-1/2 (unit diagonal); one cooperative kernel
 //      factors S (G + lambda I) S = L L^T in FP32 and inverts L on the way
-//      (right-looking steps over [A | I], a grid barrier between phases);
+//      (right-looking steps over [A | I], one grid barrier per step);
 //      each FP32 solve is then two triangular products with W = L^-1, and
 //      iterative refinement uses the residual of the scaled system computed
 //      in float-float
@@ -117,8 +117,10 @@ struct Ws {
   double* lam;     // [0] lambda
   double* dsc;     // K: Jacobi scale 1 / sqrt(M_jj + lambda)
   float2* S;       // K x K: the scaled matrix, float-float
-  float* A32;      // K x K: the same in FP32 (lower), then its Cholesky factor
+  float* A32;      // K x K: the same in FP32 (lower), destroyed by the factorisation
+  float* Rh32;     // K x K: its right-hand sides
   float* W32;      // K x K: L^-1 (lower)
+  float* Yg;       // two 32 x 32 blocks: inverse of the factor's diagonal block
   float* Y32;      // K x RW: W r, between the two triangular products
   unsigned* gbar;  // grid barrier of the factorisation: arrivals, generation
   float2* Zs;      // K x RW: scaled right-hand side
@@ -139,6 +141,8 @@ static size_t carve(void* base, int K, int s, int64_t N, Ws& w) {
   w.dsc = c.take<double>(K);
   w.S = c.take<float2>(static_cast<size_t>(K) * K);
   w.A32 = c.take<float>(static_cast<size_t>(K) * K);
+  w.Rh32 = c.take<float>(static_cast<size_t>(K) * K);
+  w.Yg = c.take<float>(2 * NB * NB);
   w.W32 = c.take<float>(static_cast<size_t>(K) * K);
   w.Y32 = c.take<float>(static_cast<size_t>(K) * RW);
   w.gbar = c.take<unsigned>(64);
@@ -880,213 +884,269 @@ __global__ void __launch_bounds__(MT * 8) scale_kernel(const double* __restrict_
     }
 }
 
-// ---- 5c. FP32 Cholesky of A and the inverse of its factor, W = L^-1 ----------
+// ---- 5c. W = L^-1 of the FP32 Cholesky factor of A = L L^T -------------------------
 // One cooperative launch (every CTA resident) walks the 32-column steps of a
-// right-looking factorisation of the augmented matrix [A | I]:
-//   phase 1  each CTA factors the diagonal block in one warp (L_kk and its
-//            inverse); the grid computes the panel L_ik = A_ik L_kk^-T (i > k)
-//            and the rows W_k = L_kk^-1 R_k of the inverse
-//   phase 2  CTA 0 stores L_kk; trailing update A_ij -= L_ik L_jk^T (j <= i)
-//            and right-hand sides R_i -= L_ik W_k (i > k), on 64 x 64 tiles
-//            spread over the CTAs
-// with a grid barrier after each phase.  After the last step A holds L and W
-// holds L^-1 (lower; its upper triangle stays exactly zero), so every later
-// solve is two triangular products, parallel over the whole matrix.
+// right-looking factorisation of the augmented matrix [A | I]; a step needs only
+// Y_k = L_kk^-1, so that one grid barrier per step is enough:
+//   every CTA but 0  takes 64 x 64 tiles of the trailing matrix and of the
+//            right-hand sides, forms the panels it needs itself (P = A_ik Y_k^T,
+//            V = Y_k R_k) and applies A_ij -= P_i P_j^T and R_i -= P_i V; V is
+//            the finished row block of W
+//   CTA 0    meanwhile updates the next diagonal block, factors and inverts it
+//            and publishes Y_(k+1) before the barrier
+// L itself is not stored: every later solve is two triangular products with W.
+// Bound by the chain of CTA 0 and the barrier, 8 us a step (K = 1024: 32 steps,
+// 638 -> 253 us).  With the panel and the update as two phases, two barriers and the
+// block factored by every CTA before the panel, a step took 20 us.
 constexpr int CH_T = 256;   // threads per CTA
 constexpr int CH_TILE = 64;
 
-// One warp factors the nb x nb diagonal block at k0 (rows past K padded with
-// the identity): L into Ls, L^-1 into Li (both lower, [32][33]).  Lane r holds
-// row r in registers; pivots and entries move by shuffles.  Every loop is
-// unrolled over the full block so that the rows stay in registers, and the
-// pivots use the hardware reciprocal square root: the refinement of the
-// solve absorbs its last-bit error.
-__device__ void factor_diag(const float* __restrict__ A, int K, int k0, int nb, float (*Ls)[NB + 1],
-                            float (*Li)[NB + 1], bool& bad) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  float a[NB], il[NB];
+// The CTA inverts the factor of the 32 x 32 block B (symmetric, both triangles;
+// rows past the matrix padded with the identity): Y = L^-1, zeros above the
+// diagonal.  Thread (i, g) = (tid / 8, tid % 8) holds columns 4 g .. 4 g + 3 of
+// row i of [B | I], where column c of the right half takes the place of column c
+// of the left half once that is eliminated.  Per column, row c goes through
+// shared memory (buf, two rows in turn) and every other row i > c subtracts
+// b_ci / b_cc of it; by symmetry row c holds column c too.  Row i is scaled by
+// b_ii^-1/2 at the end.  About 120 cycles per column: one barrier, one
+// shared-memory read, one hardware reciprocal (the refinement of the solve
+// absorbs its last-bit error).  (One warp with the rows in registers and
+// shuffles took 340 to 500 cycles per column.)
+__device__ __forceinline__ bool factor_diag(const float (*B)[NB + 1], float (*Y)[NB + 1], float (*buf)[NB]) {
+  const int i = threadIdx.x >> 3, g = threadIdx.x & 7;
+  float a[4];
 #pragma unroll
-  for (int k = 0; k < NB; ++k)
-    a[k] = (lane < nb && k < nb) ? (k <= lane ? A[static_cast<size_t>(k0 + lane) * K + k0 + k] : 0.f)
-                                 : (k == lane ? 1.f : 0.f);
-  bad = false;
+  for (int m = 0; m < 4; ++m) a[m] = B[i][4 * g + m];
+  bool bad = false;
+  float di = 1.f;  // the row's own pivot
+#pragma unroll 1
+  for (int c4 = 0; c4 < NB; c4 += 4) {
 #pragma unroll
-  for (int c = 0; c < NB; ++c) {
-    float d = __shfl_sync(FULL, a[c], c);
-    if (!(d > 0.f)) {
-      bad = true;
-      d = 1e-30f;
-    }
-    const float r = rsqrtf(d);
-    il[c] = r;  // 1 / L[c][c]
-    a[c] = lane == c ? d * r : (lane > c ? a[c] * r : a[c]);  // L[lane][c]
+    for (int cc = 0; cc < 4; ++cc) {
+      const int c = c4 + cc;
+      float* row = buf[cc & 1];
+      if (i == c) *reinterpret_cast<float4*>(row + 4 * g) = make_float4(a[0], a[1], a[2], a[3]);
+      __syncthreads();
+      float d = row[c];
+      const float bi = row[i];
+      const float4 v = *reinterpret_cast<const float4*>(row + 4 * g);
+      if (!(d > 0.f)) {
+        bad = true;
+        d = 1e-30f;
+      }
+      const float f = i > c ? -bi * __fdividef(1.f, d) : 0.f;
+      di = i == c ? d : di;
+      const bool own = 4 * g == c4;  // this thread holds column c: its right half begins
+      const float x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      if (k > c) {
-        const float lkc = __shfl_sync(FULL, a[c], k);  // L[k][c]
-        a[k] = lane >= k ? fmaf(-a[c], lkc, a[k]) : a[k];
+      for (int m = 0; m < 4; ++m) {
+        if (m == cc && own) a[m] = i == c ? 1.f : (i > c ? f : 0.f);
+        else a[m] = fmaf(f, x[m], a[m]);
       }
     }
   }
+  const float r = rsqrtf(di);
 #pragma unroll
-  for (int k = 0; k < NB; ++k) Ls[lane][k] = k <= lane ? a[k] : 0.f;
-  // X = L^-1, one column per lane: X[r][c] = (delta_rc - sum_{k<r} L[r][k] X[k][c]) / L[r][r]
-  float x[NB];
-#pragma unroll
-  for (int r = 0; r < NB; ++r) {
-    float acc = r == lane ? 1.f : 0.f;
-#pragma unroll
-    for (int k = 0; k < NB; ++k)
-      if (k < r) acc = fmaf(-__shfl_sync(FULL, a[k], r), x[k], acc);
-    x[r] = r >= lane ? acc * il[r] : 0.f;
-  }
-#pragma unroll
-  for (int r = 0; r < NB; ++r) Li[r][lane] = x[r];
+  for (int m = 0; m < 4; ++m) Y[i][4 * g + m] = 4 * g + m <= i ? a[m] * r : 0.f;
+  return bad;
 }
 
-// C[64 x 64 tile] -= P Q^T over 32 k: P rows from pload(r, q), Q rows from
-// qload(c, q), both staged transposed; 4 x 4 outputs per thread, applied by
-// cupd(r, c, value).
-template <class PF, class QF, class CF>
-__device__ __forceinline__ void tile_update(float (*Ps)[CH_TILE + 1], float (*Qs)[CH_TILE + 1], PF pload,
-                                            QF qload, CF cupd) {
-  for (int f = threadIdx.x; f < CH_TILE * NB; f += CH_T) {
-    const int r = f / NB, q = f % NB;
-    Ps[q][r] = pload(r, q);
-    Qs[q][r] = qload(r, q);
+// The 64 x nb panel rows [r0, r0 + 64) of A's columns [k0, k0 + nb), transposed.
+__device__ __forceinline__ void stage_panel(const float* __restrict__ A, int K, int r0, int k0, int nb,
+                                            float (*raw)[CH_TILE + 1]) {
+#pragma unroll
+  for (int u = 0; u < CH_TILE * NB / CH_T; ++u) {
+    const int f = threadIdx.x + u * CH_T, r = f / NB, q = f % NB;
+    raw[q][r] = (r0 + r < K && q < nb) ? A[static_cast<size_t>(r0 + r) * K + k0 + q] : 0.f;
   }
-  __syncthreads();
-  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;  // rows tr + 16i, cols tc + 16j
-  float acc[4][4] = {};
+}
+
+// Pt[c][r] = sum_q Y[c][q] raw[q][r]: 32 x 64.
+__device__ __forceinline__ void times_y(const float (*Y)[NB + 1], const float (*raw)[CH_TILE + 1],
+                                        float (*Pt)[CH_TILE + 1]) {
+  const int tr = threadIdx.x % 16, tc = threadIdx.x / 16;  // columns tr + 16 i, rows tc, tc + 16
+  float acc[2][4] = {};
+#pragma unroll 8
+  for (int q = 0; q < NB; ++q) {
+    const float y0 = Y[tc][q], y1 = Y[tc + 16][q];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float v = raw[q][tr + 16 * i];
+      acc[0][i] = fmaf(v, y0, acc[0][i]);
+      acc[1][i] = fmaf(v, y1, acc[1][i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    Pt[tc][tr + 16 * i] = acc[0][i];
+    Pt[tc + 16][tr + 16 * i] = acc[1][i];
+  }
+}
+
+// acc[i][j] -= sum_q Pt[q][r] Qt[q][c] at r = tid / 16 + 16 i, c = tid % 16 + 16 j.
+__device__ __forceinline__ void tile_product(const float (*Pt)[CH_TILE + 1], const float (*Qt)[CH_TILE + 1],
+                                             float (&acc)[4][4]) {
+  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;
 #pragma unroll 8
   for (int q = 0; q < NB; ++q) {
     float pi[4], qj[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) pi[i] = Ps[q][tr + 16 * i];
+    for (int i = 0; i < 4; ++i) pi[i] = Pt[q][tr + 16 * i];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) qj[j] = Qs[q][tc + 16 * j];
+    for (int j = 0; j < 4; ++j) qj[j] = Qt[q][tc + 16 * j];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(pi[i], qj[j], acc[i][j]);
+      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(-pi[i], qj[j], acc[i][j]);
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) cupd(tr + 16 * i, tc + 16 * j, acc[i][j]);
-  __syncthreads();  // the staging tiles are reused by the next tile
 }
 
-__global__ void __launch_bounds__(CH_T) chol_inv_kernel(float* __restrict__ A, float* __restrict__ W, int K,
-                                                        unsigned* __restrict__ bar,
-                                                        uint32_t* __restrict__ status, long long budget) {
-  __shared__ float Ls[NB][NB + 1];
-  __shared__ float Li[NB][NB + 1];
-  __shared__ float Ps[NB][CH_TILE + 1];
-  __shared__ float Qs[NB][CH_TILE + 1];
+// A: the matrix (lower, destroyed).  R: K x K scratch, the right-hand sides below
+// the current step.  Yg: two 32 x 32 blocks, Y of the even and odd steps.
+__global__ void __launch_bounds__(CH_T) chol_inv_kernel(float* __restrict__ A, float* __restrict__ R,
+                                                        float* __restrict__ W, float* __restrict__ Yg, int K,
+                                                        unsigned* __restrict__ bar, uint32_t* __restrict__ status,
+                                                        long long budget) {
+  __shared__ float Y[NB][NB + 1];
+  __shared__ float Dg[NB][NB + 1];
+  __shared__ __align__(16) float buf[2][NB];
+  __shared__ float raw[2][NB][CH_TILE + 1];
+  __shared__ float Pt[NB][CH_TILE + 1];
+  __shared__ float Qt[NB][CH_TILE + 1];
   const int tid = threadIdx.x;
-  const long long gt = static_cast<long long>(blockIdx.x) * CH_T + tid;
-  const long long gstride = static_cast<long long>(gridDim.x) * CH_T;
-  // W = I (the augmented right-hand sides)
-  for (long long e = gt; e < static_cast<long long>(K) * K; e += gstride)
-    W[e] = (e / K == e % K) ? 1.f : 0.f;
-  if (!grid_barrier(bar, budget, status)) return;
   const int nblk = (K + NB - 1) / NB;
+  unsigned arrived = 0;  // barriers passed
+  // CTA 0: the diagonal block in Dg -> Y, published for step kb
+  auto publish = [&](int kb) {
+    __syncthreads();
+    if (factor_diag(Dg, Y, buf) && tid == 0) flag_status(status, ST_BAD_INPUT);
+    __syncthreads();
+    for (int f = tid; f < NB * NB; f += CH_T) Yg[(kb & 1) * NB * NB + f] = Y[f / NB][f % NB];
+  };
+  // entry (r, c) of the diagonal block at k0 (c <= r), identity past the matrix
+  auto diag_at = [&](int r, int c, int k0) {
+    return (k0 + r < K && k0 + c < K) ? A[static_cast<size_t>(k0 + r) * K + k0 + c] : (r == c ? 1.f : 0.f);
+  };
+  if (blockIdx.x == 0) {
+    for (int f = tid; f < NB * NB; f += CH_T) {
+      const int r = f / NB, c = f % NB;
+      Dg[r][c] = c <= r ? diag_at(r, c, 0) : diag_at(c, r, 0);
+    }
+    publish(0);
+  }
+  if (!grid_barrier_count(bar, ++arrived, budget, status)) return;
   for (int kb = 0; kb < nblk; ++kb) {
     const int k0 = kb * NB, nb = K - k0 < NB ? K - k0 : NB, k1 = k0 + nb;
-    // ---- phase 1 (the diagonal block is read by every CTA: nobody writes it here)
-    if (tid < 32) {
-      bool bad = false;
-      factor_diag(A, K, k0, nb, Ls, Li, bad);
-      if (bad && tid == 0 && blockIdx.x == 0) flag_status(status, ST_BAD_INPUT);
-    }
-    __syncthreads();
-    // Warp tasks over the whole grid: the panel rows (lane c, holding row c of
-    // L_kk^-1 in registers: L_ic = sum_q A_iq Li[c][q]) and 32-column tiles of
-    // the rows of W (one column per lane: W_qc = sum_p Li[q][p] R_pc).
-    {
-      const int lane = tid & 31;
-      float lr[NB];
-#pragma unroll
-      for (int q = 0; q < NB; ++q) lr[q] = Li[lane][q];
-      const int gw = blockIdx.x * (CH_T / 32) + (tid >> 5);
-      const int nwarps = gridDim.x * (CH_T / 32);
-      const int npanel = K - k1;
-      const int ntiles = (k1 + 31) / 32;
-      for (int task = gw; task < npanel + ntiles; task += nwarps) {
-        if (task < npanel) {
-          const int i = k1 + task;
-          float* ar = A + static_cast<size_t>(i) * K + k0;
-          const float v = lane < nb ? ar[lane] : 0.f;
-          float acc = 0.f;
-#pragma unroll
-          for (int q = 0; q < NB; ++q) acc = fmaf(__shfl_sync(0xffffffffu, v, q), lr[q], acc);
-          if (lane < nb) ar[lane] = acc;
-        } else {
-          // lane c: column c0 + c of R_k, y_q = sum_{p <= q} Li[q][p] R_pc
-          const int c = (task - npanel) * 32 + lane;
-          if (c < k1) {
-            float r[NB];
-#pragma unroll
-            for (int p = 0; p < NB; ++p) r[p] = p < nb ? W[static_cast<size_t>(k0 + p) * K + c] : 0.f;
-#pragma unroll
-            for (int q = 0; q < NB; ++q) {
-              if (q < nb) {
-                float acc = 0.f;
-#pragma unroll
-                for (int p = 0; p <= q; ++p) acc = fmaf(Li[q][p], r[p], acc);
-                W[static_cast<size_t>(k0 + q) * K + c] = acc;
-              }
-            }
-          }
-        }
-      }
-    }
-    if (!grid_barrier(bar, budget, status)) return;
-    // ---- phase 2: the factored diagonal block, the trailing update of A
-    // (lower tiles) and of the right-hand sides
-    if (blockIdx.x == 0 && tid < nb)
-      for (int k = 0; k < nb; ++k) A[static_cast<size_t>(k0 + tid) * K + k0 + k] = Ls[tid][k];
+    for (int f = tid; f < NB * NB; f += CH_T) Y[f / NB][f % NB] = Yg[(kb & 1) * NB * NB + f];
     const int rest = K - k1;  // > 0 only when nb = NB (a partial block is the last)
-    if (rest > 0) {
-      const int T1 = (rest + CH_TILE - 1) / CH_TILE;
-      const int T2 = (k1 + CH_TILE - 1) / CH_TILE;
-      const int nsyrk = T1 * (T1 + 1) / 2;
-      const int total = nsyrk + T1 * T2;
-      for (int t = blockIdx.x; t < total; t += gridDim.x) {
+    if (blockIdx.x == 0 && rest > 0) {
+      // the next diagonal block: D - P P^T over its 32 rows
+      float dv[NB * NB / CH_T];
+#pragma unroll
+      for (int u = 0; u < NB * NB / CH_T; ++u) {
+        const int f = tid + u * CH_T, r = f / NB, c = f % NB;
+        dv[u] = c <= r ? diag_at(r, c, k1) : diag_at(c, r, k1);
+      }
+      stage_panel(A, K, k1, k0, nb, raw[0]);
+      __syncthreads();
+      times_y(Y, raw[0], Pt);
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < NB * NB / CH_T; ++u) {
+        const int f = tid + u * CH_T, r = f / NB, c = f % NB;
+        float acc = 0.f;
+#pragma unroll
+        for (int q = 0; q < NB; ++q) acc = fmaf(Pt[q][r], Pt[q][c], acc);  // rows past the matrix are zero
+        Dg[r][c] = dv[u] - acc;
+      }
+      publish(kb + 1);
+      __syncthreads();
+      if (gridDim.x == 1)
+        for (int f = tid; f < NB * NB; f += CH_T) Y[f / NB][f % NB] = Yg[(kb & 1) * NB * NB + f];
+    }
+    const int T1 = (rest + CH_TILE - 1) / CH_TILE;
+    const int T2 = (k1 + CH_TILE - 1) / CH_TILE;
+    const int nsyrk = T1 * (T1 + 1) / 2;
+    const int total = nsyrk + (T1 > 0 ? T1 : 1) * T2;
+    const int workers = gridDim.x > 1 ? gridDim.x - 1 : 1;
+    const int first = gridDim.x > 1 ? static_cast<int>(blockIdx.x) - 1 : 0;
+    const int tr = tid / 16, tc = tid % 16;
+    if (first >= 0)
+      for (int t = first; t < total; t += workers) {
+        // the tile's values are loaded first: their latency hides behind the panels
+        float acc[4][4];
+        __syncthreads();  // Y is there, and the previous tile's panels are consumed
         if (t < nsyrk) {
           int bi = static_cast<int>((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
           while (bi * (bi + 1) / 2 > t) --bi;
           while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
           const int bj = t - bi * (bi + 1) / 2;
           const int r0 = k1 + bi * CH_TILE, c0 = k1 + bj * CH_TILE;
-          tile_update(
-              Ps, Qs,
-              [&](int r, int q) { return r0 + r < K ? A[static_cast<size_t>(r0 + r) * K + k0 + q] : 0.f; },
-              [&](int r, int q) { return c0 + r < K ? A[static_cast<size_t>(c0 + r) * K + k0 + q] : 0.f; },
-              [&](int r, int c, float v) {
-                const int gr = r0 + r, gc = c0 + c;
-                if (gr < K && gc <= gr) A[static_cast<size_t>(gr) * K + gc] -= v;
-              });
+          // (the next diagonal block is CTA 0's, and is not read again)
+          auto mine = [&](int gr, int gc) { return gr < K && gc <= gr && !(gr < k1 + NB && gc < k1 + NB); };
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int gr = r0 + tr + 16 * i, gc = c0 + tc + 16 * j;
+              acc[i][j] = mine(gr, gc) ? A[static_cast<size_t>(gr) * K + gc] : 0.f;
+            }
+          stage_panel(A, K, r0, k0, nb, raw[0]);
+          if (bi != bj) stage_panel(A, K, c0, k0, nb, raw[1]);
+          __syncthreads();
+          times_y(Y, raw[0], Pt);
+          if (bi != bj) times_y(Y, raw[1], Qt);
+          __syncthreads();
+          tile_product(Pt, bi != bj ? Qt : Pt, acc);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int gr = r0 + tr + 16 * i, gc = c0 + tc + 16 * j;
+              if (mine(gr, gc)) A[static_cast<size_t>(gr) * K + gc] = acc[i][j];
+            }
         } else {
           const int u = t - nsyrk;
           const int bi = u / T2, bc = u % T2;
           const int r0 = k1 + bi * CH_TILE, c0 = bc * CH_TILE;
-          tile_update(
-              Ps, Qs,
-              [&](int r, int q) { return r0 + r < K ? A[static_cast<size_t>(r0 + r) * K + k0 + q] : 0.f; },
-              [&](int c, int q) {
-                return (c0 + c < k1 && q < nb) ? W[static_cast<size_t>(k0 + q) * K + c0 + c] : 0.f;
-              },
-              [&](int r, int c, float v) {
-                const int gr = r0 + r, gc = c0 + c;
-                if (gr < K && gc < k1) W[static_cast<size_t>(gr) * K + gc] -= v;
-              });
+          // this step's own columns start from zero
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int gr = r0 + tr + 16 * i, gc = c0 + tc + 16 * j;
+              acc[i][j] = gr < K && gc < k0 ? R[static_cast<size_t>(gr) * K + gc] : 0.f;
+            }
+          // R_k (32 x 64 columns; the identity in its own columns) and the panel
+#pragma unroll
+          for (int v = 0; v < NB * CH_TILE / CH_T; ++v) {
+            const int f = tid + v * CH_T, p = f / CH_TILE, c = f % CH_TILE, gc = c0 + c;
+            raw[1][p][c] = (p < nb && gc < k0) ? R[static_cast<size_t>(k0 + p) * K + gc] : (gc == k0 + p ? 1.f : 0.f);
+          }
+          if (rest > 0) stage_panel(A, K, r0, k0, nb, raw[0]);
+          __syncthreads();
+          times_y(Y, raw[1], Qt);  // V = Y R_k: the finished rows of W
+          if (rest > 0) times_y(Y, raw[0], Pt);
+          __syncthreads();
+          if (bi == 0)
+#pragma unroll
+            for (int v = 0; v < NB * CH_TILE / CH_T; ++v) {
+              const int f = tid + v * CH_T, q = f / CH_TILE, c = f % CH_TILE;
+              if (q < nb && c0 + c < k1) W[static_cast<size_t>(k0 + q) * K + c0 + c] = Qt[q][c];
+            }
+          if (rest > 0) {
+            tile_product(Pt, Qt, acc);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const int gr = r0 + tr + 16 * i, gc = c0 + tc + 16 * j;
+                if (gr < K && gc < k1) R[static_cast<size_t>(gr) * K + gc] = acc[i][j];
+              }
+          }
         }
       }
-    }
-    if (!grid_barrier(bar, budget, status)) return;
+    if (kb + 1 < nblk && !grid_barrier_count(bar, ++arrived, budget, status)) return;
   }
 }
 
@@ -1698,12 +1758,14 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
     if (crc) return crc;
     DLSH_CUDA_TRY(cudaMemsetAsync(w.gbar, 0, 2 * sizeof(unsigned), st), "dlsh_mod_update: barrier");
     float* A32 = w.A32;
+    float* Rh32 = w.Rh32;
     float* W32 = w.W32;
+    float* Yg = w.Yg;
     int Kk = K;
     unsigned* gb = w.gbar;
     uint32_t* stw = w.status;
     long long budget = kWaitBudget;
-    void* args[] = {&A32, &W32, &Kk, &gb, &stw, &budget};
+    void* args[] = {&A32, &Rh32, &W32, &Yg, &Kk, &gb, &stw, &budget};
     DLSH_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(chol_inv_kernel), dim3(coop_grid),
                                               dim3(CH_T), args, 0, st),
                   "dlsh_mod_update: factorisation");
