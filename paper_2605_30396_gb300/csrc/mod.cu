@@ -1403,25 +1403,36 @@ __global__ void __launch_bounds__(1024)
 //   E = R_w + g d_j^T (R = X - D A, kept current),  d = E^T g / ||E^T g||,
 //   g' = E d,  R_w <- E - g' d^T,  d_j <- d,  A[j, w] <- g'.
 // R lives in the workspace, rows padded to 48 floats (16-byte loads).  One
-// cooperative kernel runs the sweep: per atom, every thread takes list entries
-// lo + tid, lo + tid + (grid threads), ...; phase 1 sums g R_i and g^2 (per
-// thread, then a transposing butterfly per warp, then the warps and the CTAs
-// in a fixed order: the result does not depend on timing); a grid barrier;
-// phase 2 forms d in every CTA and updates R, the coefficients and the atom; a
-// second grid barrier before the next atom reads R.  The atom-major list
-// records each entry's code slot, so the coefficient is written directly.
-constexpr int KS_T = 256;          // threads per sweep CTA
-constexpr int KS_W = KS_T / 32;
+// cooperative kernel runs the sweep.  A CTA owns a range of signals (whole tiles
+// of the counting sort), so that the rows it reads and writes are its own and
+// atom after atom needs no barrier for them; per atom the CTAs only exchange
+// their sums of g R_i and g^2:
+//   phase 1  sixteen lanes take one entry of the CTA's part of the list (a
+//            float4 of its row each); the sums go through shared memory to 16
+//            words of 16 bytes, three values and the atom's number in each,
+//            written and read by single 128-bit accesses, so that a word's
+//            arrival is its own flag
+//   phase 2  every CTA sums all words in the same order, forms d, and updates
+//            its rows (up to KS_KEEP passes still in registers), coefficients
+//            and, on CTA 0, the atom
+// Two sets of words alternate: a CTA writes an atom's words only after it has
+// read all of the previous atom's, so no word is overwritten before its readers
+// are through.  Every sum runs in a fixed order.  Bound by latency: the row
+// gather, one L2 round trip of the words and the reductions, 3.4 us per
+// atom (N = 400k, K = 512, s = 8; with two grid barriers per atom and one
+// thread per entry 12.4 us).
+constexpr int KS_T = 512;          // threads per sweep CTA
+constexpr int KS_E = KS_T / 16;    // entries per pass
+constexpr int KS_KEEP = 5;         // passes kept in registers between the phases
+constexpr int KS_WORDS = 16;       // 16-byte words of a CTA's sums: 45 of g R_i, then g^2
 constexpr int RROW = 48;           // residual row stride in floats
-constexpr int KS_V = DLSH_D + 1;   // reduced values: 45 of g R_i, then g^2
 
 struct KsWs {
   uint32_t* status;
   Sort so;         // records carry the entry's code slot
   float* R;        // N x 48 residual (45 used)
-  float* part;     // grid x 48 per-CTA partial sums
+  uint4* part;     // 2 x grid x KS_WORDS: the CTAs' sums
   int* dead;
-  unsigned* gbar;
 };
 
 constexpr int KS_MAX_GRID = 1024;
@@ -1431,9 +1442,8 @@ static size_t carve_ksvd(void* base, int K, int s, int64_t N, KsWs& w) {
   w.status = c.take<uint32_t>(64);
   carve_sort(c, K, s, N, w.so);
   w.R = c.take<float>(static_cast<size_t>(N) * RROW);
-  w.part = c.take<float>(static_cast<size_t>(KS_MAX_GRID) * 48);
+  w.part = c.take<uint4>(static_cast<size_t>(2) * KS_MAX_GRID * KS_WORDS);
   w.dead = c.take<int>(K);
-  w.gbar = c.take<unsigned>(64);
   return c.size();
 }
 
@@ -1466,202 +1476,237 @@ __global__ void __launch_bounds__(256) ksvd_resid_kernel(const float* __restrict
   if (lane < RROW - 32) R[i * RROW + 32 + lane] = r1;
 }
 
-__global__ void __launch_bounds__(KS_T) ksvd_sweep_kernel(const int* __restrict__ atom_start,
-                                                          const uint2* __restrict__ list, int K, int s,
-                                                          float* __restrict__ coef, const float* __restrict__ D_old,
-                                                          float* __restrict__ D_new, float* __restrict__ R,
-                                                          float* __restrict__ part, int* __restrict__ dead,
-                                                          unsigned* gbar, uint32_t* status, long long budget) {
-  extern __shared__ float pall[];  // [gridDim.x][48] the CTAs' partial sums, phase 2
-  __shared__ float wsum[KS_W][64];
-  __shared__ __align__(16) float dj[RROW], dn[RROW];
-  __shared__ float tot[48];
-  __shared__ float dd_s;
-  __shared__ int skip_s;
+__device__ __forceinline__ void st_word(uint4* p, float a, float b, float c, unsigned tag) {
+  const unsigned long long lo = static_cast<unsigned long long>(__float_as_uint(b)) << 32 | __float_as_uint(a);
+  const unsigned long long hi = static_cast<unsigned long long>(tag) << 32 | __float_as_uint(c);
+  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+               "l"(lo), "l"(hi)
+               : "memory");
+}
+__device__ __forceinline__ uint4 ld_word(const uint4* p) {
+  unsigned long long lo, hi;
+  asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+               : "=l"(lo), "=l"(hi)
+               : "l"(p)
+               : "memory");
+  return make_uint4(static_cast<unsigned>(lo), static_cast<unsigned>(lo >> 32), static_cast<unsigned>(hi),
+                    static_cast<unsigned>(hi >> 32));
+}
+
+__global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restrict__ off, int T,
+                                                             const int* __restrict__ atom_start,
+                                                             const uint2* __restrict__ list, int K, int s,
+                                                             float* __restrict__ coef, const float* __restrict__ D_old,
+                                                             float* __restrict__ D_new, float* __restrict__ R,
+                                                             uint4* __restrict__ part, int* __restrict__ dead,
+                                                             uint32_t* status, long long budget) {
+  __shared__ float4 wsum[KS_T / 32][16];
+  __shared__ float tsum[KS_T / 32][3 * KS_WORDS];
+  __shared__ __align__(16) float dsm[KS_T / 32][RROW];
+  const unsigned FULL = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t gthreads = static_cast<int64_t>(gridDim.x) * KS_T;
-  const int64_t gtid = static_cast<int64_t>(blockIdx.x) * KS_T + tid;
+  const int l = tid & 15, slot = tid >> 4;  // the thread's float4 of a row, its entry in a pass
   const int G = gridDim.x;
-  // The list is read-only during the sweep: the next atom's bounds and this
-  // thread's first record of it are loaded ahead, while the current atom is
-  // being processed.  A thread's first entry of the current atom (record and
-  // residual row) stays in registers from phase 1 to phase 2.
-  int lo = atom_start[0], hi = K > 0 ? atom_start[1] : 0;
-  uint2 rec_next = lo + gtid < hi ? list[lo + gtid] : make_uint2(0u, 0u);
+  const int t0 = static_cast<int>(static_cast<long long>(T) * blockIdx.x / G);
+  const int t1 = static_cast<int>(static_cast<long long>(T) * (blockIdx.x + 1) / G);
+  const bool rl = l < RROW / 4;
+  // what is read ahead of the next atom: the CTA's range of its list, the
+  // thread's first record, and its part of the atom
+  auto lo_of = [&](int j) { return off[static_cast<size_t>(t0) * K + j]; };
+  auto hi_of = [&](int j) { return t1 < T ? off[static_cast<size_t>(t1) * K + j] : atom_start[j + 1]; };
+  auto old_of = [&](int j) {
+    const float* d = D_old + static_cast<size_t>(j) * DLSH_D + 4 * l;
+    return make_float4(4 * l < DLSH_D ? __ldg(d) : 0.f, 4 * l + 1 < DLSH_D ? __ldg(d + 1) : 0.f,
+                       4 * l + 2 < DLSH_D ? __ldg(d + 2) : 0.f, 4 * l + 3 < DLSH_D ? __ldg(d + 3) : 0.f);
+  };
+  int a0 = atom_start[0], a1 = atom_start[1];
+  int lo = lo_of(0), hi = hi_of(0);
+  uint2 first = lo + slot < hi ? list[lo + slot] : make_uint2(0u, 0u);
+  float4 dj = rl ? old_of(0) : make_float4(0.f, 0.f, 0.f, 0.f);
   for (int j = 0; j < K; ++j) {
-    const uint2 rec0 = rec_next;
-    const int nlo = hi;
-    const int nhi = j + 2 <= K ? atom_start[j + 2] : hi;
-    if (blockIdx.x == 0 && tid == 0) dead[j] = hi == lo ? 1 : 0;
-    if (hi == lo) {
-      if (blockIdx.x == 0 && tid < DLSH_D)
-        D_new[static_cast<size_t>(j) * DLSH_D + tid] = D_old[static_cast<size_t>(j) * DLSH_D + tid];
-      rec_next = nlo + gtid < nhi ? list[nlo + gtid] : make_uint2(0u, 0u);
-      lo = nlo;
-      hi = nhi;
-      continue;  // the same decision in every CTA
-    }
-    if (tid < RROW) dj[tid] = tid < DLSH_D ? D_old[static_cast<size_t>(j) * DLSH_D + tid] : 0.f;
-    // ---- phase 1: sum g R_i and g^2 over this thread's entries
-    float v[64];
+    const bool used = a1 > a0;  // the same decision in every CTA
+    const int clo = lo, chi = hi;
+    const uint2 rec0 = first;
+    const float4 d = dj;
+    if (blockIdx.x == 0 && tid == 0) dead[j] = used ? 0 : 1;
+    uint2 rec[KS_KEEP];
+    float4 r[KS_KEEP];
+    if (used) {
+      // ---- phase 1: sum g R_i (lanes 0..11) and g^2 (lane 12) over the CTA's entries
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int d = 0; d < 64; ++d) v[d] = 0.f;
-    const bool has0 = lo + gtid < hi;
-    const int64_t i0 = rec0.x & 0x3FFFFFFu;
-    const float g0 = __uint_as_float(rec0.y);
-    float4 r0[RROW / 4];
-    if (has0) {
-      const float4* r4 = reinterpret_cast<const float4*>(R + i0 * RROW);
-#pragma unroll
-      for (int q = 0; q < RROW / 4; ++q) r0[q] = __ldcg(r4 + q);
-#pragma unroll
-      for (int q = 0; q < RROW / 4; ++q) {
-        if (4 * q + 0 < DLSH_D) v[4 * q + 0] = g0 * r0[q].x;
-        if (4 * q + 1 < DLSH_D) v[4 * q + 1] = g0 * r0[q].y;
-        if (4 * q + 2 < DLSH_D) v[4 * q + 2] = g0 * r0[q].z;
-        if (4 * q + 3 < DLSH_D) v[4 * q + 3] = g0 * r0[q].w;
+      for (int p = 0; p < KS_KEEP; ++p) {
+        const int e = clo + p * KS_E + slot;
+        rec[p] = p == 0 ? rec0 : (e < chi ? __ldg(list + e) : make_uint2(0u, 0u));
       }
-      v[DLSH_D] = g0 * g0;  // after the row: slot 45 of the row is padding
-    } else {
 #pragma unroll
-      for (int q = 0; q < RROW / 4; ++q) r0[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (int64_t e = lo + gtid + gthreads; e < hi; e += gthreads) {
-      const uint2 rec = list[e];
-      const int64_t i = rec.x & 0x3FFFFFFu;
-      const float g = __uint_as_float(rec.y);
-      v[DLSH_D] = fmaf(g, g, v[DLSH_D]);
-      const float4* r4 = reinterpret_cast<const float4*>(R + i * RROW);
-#pragma unroll
-      for (int q = 0; q < RROW / 4; ++q) {
-        const float4 x = __ldcg(r4 + q);
-        v[4 * q + 0] = fmaf(g, x.x, v[4 * q + 0]);
-        v[4 * q + 1] = fmaf(g, x.y, v[4 * q + 1]);
-        v[4 * q + 2] = fmaf(g, x.z, v[4 * q + 2]);
-        if (4 * q + 3 < DLSH_D) v[4 * q + 3] = fmaf(g, x.w, v[4 * q + 3]);
+      for (int p = 0; p < KS_KEEP; ++p) {
+        r[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (rl && clo + p * KS_E + slot < chi)
+          r[p] = __ldcg(reinterpret_cast<const float4*>(R + static_cast<size_t>(rec[p].x & 0x3FFFFFFu) * RROW) + l);
       }
-    }
-    // transposing butterfly: after it, lane l holds the warp's sums of values
-    // 2l and 2l + 1 in v[0], v[1]
+      auto add = [&](float g, float4 x) {
+        if (l == RROW / 4) x.x = g;
+        v.x = fmaf(g, x.x, v.x);
+        v.y = fmaf(g, x.y, v.y);
+        v.z = fmaf(g, x.z, v.z);
+        v.w = fmaf(g, x.w, v.w);
+      };
 #pragma unroll
-    for (int m = 64, o = 16; o > 0; m >>= 1, o >>= 1) {
-      const bool up = (lane & o) != 0;
+      for (int p = 0; p < KS_KEEP; ++p) add(__uint_as_float(rec[p].y), r[p]);  // no entry: g = 0, r = 0
+      for (int e = clo + KS_KEEP * KS_E + slot; e < chi; e += KS_E) {
+        const uint2 q = __ldg(list + e);
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (rl) x = __ldcg(reinterpret_cast<const float4*>(R + static_cast<size_t>(q.x & 0x3FFFFFFu) * RROW) + l);
+        add(__uint_as_float(q.y), x);
+      }
+      v.x += __shfl_xor_sync(FULL, v.x, 16);
+      v.y += __shfl_xor_sync(FULL, v.y, 16);
+      v.z += __shfl_xor_sync(FULL, v.z, 16);
+      v.w += __shfl_xor_sync(FULL, v.w, 16);
+      if (lane < 16) wsum[warp][lane] = v;
+      __syncthreads();
+      // the warps' sums in order; word w carries values 3 w .. 3 w + 2 (45 of
+      // g R_i, then g^2, which sits at value 48 of wsum)
+      if (tid < KS_WORDS) {
+        float t3[3];
 #pragma unroll
-      for (int k = 0; k < m / 2; ++k) {
-        const float send = up ? v[k] : v[k + m / 2];
-        const float keep = up ? v[k + m / 2] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        for (int q = 0; q < 3; ++q) {
+          const int val = 3 * tid + q < DLSH_D ? 3 * tid + q : (3 * tid + q == DLSH_D ? RROW : RROW + 1);
+          float sum = 0.f;
+#pragma unroll
+          for (int w = 0; w < KS_T / 32; ++w) sum += reinterpret_cast<const float*>(&wsum[w][0])[val];
+          t3[q] = sum;
+        }
+        st_word(part + (static_cast<size_t>(j & 1) * G + blockIdx.x) * KS_WORDS + tid, t3[0], t3[1], t3[2],
+                static_cast<unsigned>(j) + 1u);
       }
     }
-    wsum[warp][2 * lane] = v[0];
-    wsum[warp][2 * lane + 1] = v[1];
-    __syncthreads();
-    if (tid < KS_V) {
-      float sum = 0.f;
-#pragma unroll
-      for (int w = 0; w < KS_W; ++w) sum += wsum[w][tid];
-      __stcg(part + static_cast<size_t>(blockIdx.x) * 48 + tid, sum);
+    // ---- the next atom's reads, while the words travel
+    a0 = a1;
+    if (j + 1 < K) {
+      a1 = atom_start[j + 2 <= K ? j + 2 : K];
+      lo = lo_of(j + 1);
+      hi = hi_of(j + 1);
+      first = lo + slot < hi ? list[lo + slot] : make_uint2(0u, 0u);
+      if (rl) dj = old_of(j + 1);
     }
-    if (!grid_barrier(gbar, budget, status)) return;
-    rec_next = nlo + gtid < nhi ? list[nlo + gtid] : make_uint2(0u, 0u);
-    // ---- phase 2: d = E^T g = sum g R_i + d_j sum g^2, in every CTA
-    for (int f = tid; f < G * 48; f += KS_T) pall[f] = __ldcg(part + f);
-    __syncthreads();
-    if (tid < KS_V) {
-      float sum = 0.f;
-#pragma unroll 8
-      for (int c = 0; c < G; ++c) sum += pall[c * 48 + tid];
-      tot[tid] = sum;
-    }
-    __syncthreads();
-    if (tid < 32) {
-      const float v0 = fmaf(dj[tid], tot[DLSH_D], tot[tid]);
-      const float v1 = tid < DLSH_D - 32 ? fmaf(dj[32 + tid], tot[DLSH_D], tot[32 + tid]) : 0.f;
-      float n2 = fmaf(v0, v0, v1 * v1);
+    if (!used) {
+      if (blockIdx.x == 0 && warp == 0 && rl && lane < 16) {
+        const float x[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        for (int q = 0; q < 4; ++q)
+          if (4 * l + q < DLSH_D) D_new[static_cast<size_t>(j) * DLSH_D + 4 * l + q] = x[q];
+      }
+      continue;
+    }
+    // ---- every CTA's words, summed CTA by CTA within a slot, then slot by slot
+    {
+      float t3[3] = {0.f, 0.f, 0.f};
+      bool ok = true;
+      const uint4* base = part + static_cast<size_t>(j & 1) * G * KS_WORDS + (tid & 15);
+      const unsigned want = static_cast<unsigned>(j) + 1u;
+      constexpr int B = 5;  // words in flight per thread: all of 152 CTAs' in one go
+      for (int c0 = slot; c0 < G; c0 += B * KS_E) {
+        uint4 w[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+          if (c0 + b * KS_E < G) w[b] = ld_word(base + static_cast<size_t>(c0 + b * KS_E) * KS_WORDS);
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+          if (c0 + b * KS_E >= G) break;
+          if (w[b].w != want) {
+            const long long tw = clock64();
+            do {
+              if (clock64() - tw > budget) {
+                flag_status(status, ST_TIMEOUT);
+                ok = false;
+                break;
+              }
+              w[b] = ld_word(base + static_cast<size_t>(c0 + b * KS_E) * KS_WORDS);
+            } while (w[b].w != want);
+          }
+          t3[0] += __uint_as_float(w[b].x);
+          t3[1] += __uint_as_float(w[b].y);
+          t3[2] += __uint_as_float(w[b].z);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) t3[q] += __shfl_xor_sync(FULL, t3[q], 16);
+      if (lane < 16)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) tsum[warp][3 * lane + q] = t3[q];
+      if (__syncthreads_or(!ok)) return;
+    }
+    // ---- phase 2, every warp for itself: d = E^T g = sum g R_i + d_j sum g^2
+    float u0 = 0.f, u1 = 0.f, gg = 0.f;
+#pragma unroll
+    for (int w = 0; w < KS_T / 32; ++w) {
+      u0 += tsum[w][lane];
+      if (lane < RROW - 32) u1 += tsum[w][32 + lane];
+      gg += tsum[w][DLSH_D];
+    }
+    {
+      // d_j in the lanes' order (dimension lane and 32 + lane)
+      if (lane < 16 && rl) *reinterpret_cast<float4*>(&dsm[warp][4 * l]) = d;
+      __syncwarp();
+      const float o0 = dsm[warp][lane], o1 = lane < DLSH_D - 32 ? dsm[warp][32 + lane] : 0.f;
+      const float v0 = fmaf(o0, gg, u0);
+      const float v1 = lane < DLSH_D - 32 ? fmaf(o1, gg, u1) : 0.f;
+      float n2 = fmaf(v0, v0, v1 * v1), dot = fmaf(o0, v0, o1 * v1);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        n2 += __shfl_xor_sync(FULL, n2, o);
+        dot += __shfl_xor_sync(FULL, dot, o);
+      }
       const bool zero = !(n2 > 0.f);
       const float inv = zero ? 0.f : rsqrtf(n2);
-      const float u0 = v0 * inv, u1 = v1 * inv;
-      dn[tid] = u0;
-      if (tid < RROW - 32) dn[32 + tid] = u1;
-      float dd = fmaf(dj[tid], u0, tid < DLSH_D - 32 ? dj[32 + tid] * u1 : 0.f);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(0xffffffffu, dd, o);
-      if (tid == 0) {
-        dd_s = dd;
-        skip_s = zero ? 1 : 0;
-      }
-      if (blockIdx.x == 0) {
+      u0 = v0 * inv;
+      u1 = v1 * inv;
+      if (blockIdx.x == 0 && warp == 0) {
         float* out = D_new + static_cast<size_t>(j) * DLSH_D;
-        out[tid] = zero ? dj[tid] : u0;
-        if (tid < DLSH_D - 32) out[32 + tid] = zero ? dj[32 + tid] : u1;
+        out[lane] = zero ? o0 : u0;
+        if (lane < DLSH_D - 32) out[32 + lane] = zero ? o1 : u1;
+      }
+      __syncwarp();
+      dsm[warp][lane] = u0;
+      if (lane < RROW - 32) dsm[warp][32 + lane] = lane < DLSH_D - 32 ? u1 : 0.f;
+      __syncwarp();
+      if (!zero) {
+        const float dd = dot * inv;  // d_j . d
+        const float4 u = rl ? *reinterpret_cast<const float4*>(&dsm[warp][4 * l]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        // E_i . d = R_i . d + g (d_j . d); R_i <- R_i + g d_j - g' d
+        auto refit = [&](uint2 q, float4 x, bool on) {
+          const float g = __uint_as_float(q.y);
+          float e = fmaf(x.x, u.x, fmaf(x.y, u.y, fmaf(x.z, u.z, x.w * u.w)));
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) e += __shfl_xor_sync(FULL, e, o);
+          const float gn = fmaf(g, dd, e);
+          if (!on) return;
+          const size_t i = q.x & 0x3FFFFFFu;
+          if (rl) {
+            float4 y;
+            y.x = fmaf(-gn, u.x, fmaf(g, d.x, x.x));
+            y.y = fmaf(-gn, u.y, fmaf(g, d.y, x.y));
+            y.z = fmaf(-gn, u.z, fmaf(g, d.z, x.z));
+            y.w = fmaf(-gn, u.w, fmaf(g, d.w, x.w));
+            __stcg(reinterpret_cast<float4*>(R + i * RROW) + l, y);
+          }
+          if (l == RROW / 4) coef[i * s + static_cast<int>(q.x >> 26)] = gn;
+        };
+#pragma unroll
+        for (int p = 0; p < KS_KEEP; ++p)
+          if (clo + p * KS_E + 2 * warp < chi) refit(rec[p], r[p], clo + p * KS_E + slot < chi);  // uniform per warp
+        for (int e = clo + KS_KEEP * KS_E + 2 * warp; e < chi; e += KS_E) {
+          const bool on = e + (lane >> 4) < chi;
+          const uint2 q = on ? __ldg(list + e + (lane >> 4)) : make_uint2(0u, 0u);
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (rl && on) x = __ldcg(reinterpret_cast<const float4*>(R + static_cast<size_t>(q.x & 0x3FFFFFFu) * RROW) + l);
+          refit(q, x, on);
+        }
       }
     }
-    __syncthreads();
-    if (!skip_s) {
-      const float dd = dd_s;
-      const float4* dn4 = reinterpret_cast<const float4*>(dn);
-      const float4* dj4 = reinterpret_cast<const float4*>(dj);
-      if (has0) {
-        // the first entry: record and row still in registers
-        float e_dot = 0.f;
-#pragma unroll
-        for (int q = 0; q < RROW / 4; ++q) {
-          const float4 u = dn4[q];
-          e_dot = fmaf(r0[q].x, u.x, e_dot);
-          e_dot = fmaf(r0[q].y, u.y, e_dot);
-          e_dot = fmaf(r0[q].z, u.z, e_dot);
-          e_dot = fmaf(r0[q].w, u.w, e_dot);
-        }
-        const float gn = fmaf(g0, dd, e_dot);
-        float4* r4 = reinterpret_cast<float4*>(R + i0 * RROW);
-#pragma unroll
-        for (int q = 0; q < RROW / 4; ++q) {
-          const float4 u = dn4[q], o = dj4[q];
-          float4 y;
-          y.x = fmaf(-gn, u.x, fmaf(g0, o.x, r0[q].x));
-          y.y = fmaf(-gn, u.y, fmaf(g0, o.y, r0[q].y));
-          y.z = fmaf(-gn, u.z, fmaf(g0, o.z, r0[q].z));
-          y.w = fmaf(-gn, u.w, fmaf(g0, o.w, r0[q].w));
-          __stcg(r4 + q, y);
-        }
-        coef[i0 * s + static_cast<int>(rec0.x >> 26)] = gn;
-      }
-      for (int64_t e = lo + gtid + gthreads; e < hi; e += gthreads) {
-        const uint2 rec = list[e];
-        const int64_t i = rec.x & 0x3FFFFFFu;
-        const int slot = static_cast<int>(rec.x >> 26);
-        const float g = __uint_as_float(rec.y);
-        float4* r4 = reinterpret_cast<float4*>(R + i * RROW);
-        float4 r[RROW / 4];
-        float e_dot = 0.f;
-#pragma unroll
-        for (int q = 0; q < RROW / 4; ++q) {
-          r[q] = __ldcg(r4 + q);
-          const float4 u = dn4[q];
-          e_dot = fmaf(r[q].x, u.x, e_dot);
-          e_dot = fmaf(r[q].y, u.y, e_dot);
-          e_dot = fmaf(r[q].z, u.z, e_dot);
-          e_dot = fmaf(r[q].w, u.w, e_dot);  // padding: r = 0, u = 0
-        }
-        const float gn = fmaf(g, dd, e_dot);  // E_i . d = R_i . d + g (d_j . d)
-#pragma unroll
-        for (int q = 0; q < RROW / 4; ++q) {
-          const float4 u = dn4[q], o = dj4[q];
-          float4 y;
-          y.x = fmaf(-gn, u.x, fmaf(g, o.x, r[q].x));
-          y.y = fmaf(-gn, u.y, fmaf(g, o.y, r[q].y));
-          y.z = fmaf(-gn, u.z, fmaf(g, o.z, r[q].z));
-          y.w = fmaf(-gn, u.w, fmaf(g, o.w, r[q].w));
-          __stcg(r4 + q, y);
-        }
-        coef[i * s + slot] = gn;
-      }
-    }
-    if (!grid_barrier(gbar, budget, status)) return;
-    lo = nlo;
-    hi = nhi;
+    __syncthreads();  // the rows are written before the next atom's phase 1 reads them
   }
 }
 
@@ -1823,20 +1868,17 @@ int ksvd_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, float* c
       int per_sm = 0;
       int sms = device_sm_count();
       if (sms <= 0) sms = 1;
-      const int g = sms < KS_MAX_GRID ? sms : KS_MAX_GRID;  // one CTA per SM
-      const size_t sm_need = static_cast<size_t>(g) * 48 * sizeof(float);
-      DLSH_CUDA_TRY(cudaFuncSetAttribute(ksvd_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(sm_need)),
-                    "dlsh_ksvd_update: attribute");
-      DLSH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ksvd_sweep_kernel, KS_T, sm_need),
+      DLSH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ksvd_sweep_kernel, KS_T, 0),
                     "dlsh_ksvd_update: occupancy");
       if (per_sm < 1) return set_error(DLSH_ERR_CUDA, "dlsh_ksvd_update: sweep kernel does not fit");
-      grid = g;
+      grid = sms < KS_MAX_GRID ? sms : KS_MAX_GRID;  // one CTA per SM
       return DLSH_OK;
     });
     if (crc) return crc;
-    const size_t smem = static_cast<size_t>(coop_grid) * 48 * sizeof(float);
-    DLSH_CUDA_TRY(cudaMemsetAsync(w.gbar, 0, 2 * sizeof(unsigned), st), "dlsh_ksvd_update: barrier");
+    if (coop_grid > w.so.T) coop_grid = w.so.T;  // each CTA owns at least a tile
+    DLSH_CUDA_TRY(cudaMemsetAsync(w.part, 0, sizeof(uint4) * 2 * coop_grid * KS_WORDS, st), "dlsh_ksvd_update: words");
+    const int* of = w.so.cnt;
+    int T = w.so.T;
     const int* as = w.so.atom_start;
     const uint2* li = w.so.list;
     int Kk = K, ss = s;
@@ -1844,14 +1886,13 @@ int ksvd_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, float* c
     const float* Do = D_old;
     float* Dn = D_new;
     float* Rr = w.R;
-    float* pt = w.part;
+    uint4* pt = w.part;
     int* dd = w.dead;
-    unsigned* gb = w.gbar;
     uint32_t* stw = w.status;
     long long budget = kWaitBudget;
-    void* args[] = {&as, &li, &Kk, &ss, &cf, &Do, &Dn, &Rr, &pt, &dd, &gb, &stw, &budget};
+    void* args[] = {&of, &T, &as, &li, &Kk, &ss, &cf, &Do, &Dn, &Rr, &pt, &dd, &stw, &budget};
     DLSH_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(ksvd_sweep_kernel), dim3(coop_grid),
-                                              dim3(KS_T), args, smem, st),
+                                              dim3(KS_T), args, 0, st),
                   "dlsh_ksvd_update: sweep");
     ++launches;
   }

@@ -49,6 +49,34 @@ def test_ksvd_matches_oracle(lib, N, K, s):
     assert obj_g <= info["objective"][0]
 
 
+@pytest.mark.parametrize("N,K,s", [(513, 16, 3), (60_000, 8, 4), (320_000, 24, 2), (100, 4, 4)])
+def test_ksvd_on_uneven_codes(lib, N, K, s):
+    """Codes of 0 to s distinct atoms near a planted dictionary, at the edges of
+    the sweep's split: two tiles, more entries of an atom per CTA than its
+    threads keep in registers (60,000 x 4 / 8 over 118 CTAs), tiles of 1024
+    signals, one partial tile.  The file's relative tolerance (1e-4)."""
+    rng = np.random.default_rng(70 + N)
+    D = synth.hidden_dictionary(K, 71)
+    idx = np.argsort(rng.random((N, K)), axis=1)[:, :s]
+    nnz = rng.integers(0, s + 1, N).astype(np.uint8)
+    coef = (0.5 + rng.exponential(1.0, (N, s))) * rng.choice([-1.0, 1.0], (N, s))
+    pad = np.arange(s)[None, :] >= nnz[:, None]
+    idx[pad], coef[pad] = 0, 0.0
+    X = (np.einsum("ns,nsd->nd", coef, D[idx]) + 0.05 * rng.standard_normal((N, 45))).astype(np.float32)
+    D0 = D + 0.1 * rng.standard_normal(D.shape)
+    D0 = (D0 / np.linalg.norm(D0, axis=1, keepdims=True)).astype(np.float32)
+    args = (X, D0, idx.astype(np.uint16), coef.astype(np.float32), nnz, None)
+    Dg, cg = _gpu(lib, *args)
+    Do, co, _ = oks.ksvd_update(X.astype(np.float64), D0.astype(np.float64), idx, args[3].astype(np.float64),
+                                nnz.astype(np.int64), np.zeros(N))
+    ok, worst = close_rel(Dg, Do)
+    assert ok, ("D", worst)
+    ok, worst = close_rel(cg, co)
+    assert ok, ("coef", worst)
+    again = _gpu(lib, *args)
+    assert (again[0] == Dg).all() and (again[1] == cg).all()
+
+
 def _recon(D, idx, coef, nnz):
     out = np.zeros((idx.shape[0], 45))
     for t in range(idx.shape[1]):
