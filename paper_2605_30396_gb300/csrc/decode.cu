@@ -18,9 +18,11 @@
 //    (128 bytes), lane q reading bases 2q and 2q+1 of all three channels in
 //    one 16-byte word; its three channel sums are reduced over the eight lanes
 //    in four shuffles (a transposing butterfly).
-// Results are staged and written back coalesced.  For dictionaries too large
-// for shared memory the FP32 rows are read through the read-only cache, with
-// the FP16 path's lane mapping.
+// Results are staged and written back coalesced.  An FP32 dictionary of which
+// only one channel plane fits in shared memory (about 1150 to 3100 atoms) is
+// decoded channel by channel, each by its own CTAs (decode_channel_kernel);
+// beyond that the FP32 rows are read through the read-only cache, with the FP16
+// path's lane mapping.
 #include <cuda_fp16.h>
 #include <math.h>
 #include <stdio.h>
@@ -32,7 +34,8 @@
 namespace dlsh {
 namespace dec {
 
-enum : int { FM_F32 = 0, FM_GLOBAL = 1, FM_C8 = 2, FM_C16 = 3 };
+// FM_PLANE: the FP32 table, one channel plane per CTA
+enum : int { FM_F32 = 0, FM_GLOBAL = 1, FM_C8 = 2, FM_C16 = 3, FM_PLANE = 4 };
 
 constexpr int YS = 16;          // basis values per Gaussian slot (15 and a zero)
 // A slot is four 16-byte words; word k of slot g sits at word k ^ ((g >> 1) & 3),
@@ -56,7 +59,9 @@ inline int staged_slots(int s) {
 }
 // Per-warp shared memory: basis slots, staged rgb, codes, nnz.
 __host__ __device__ constexpr int warp_floats(int sp, int gb) { return gb * YS + gb * 3 + gb * sp * 2 + gb; }
-__host__ __device__ constexpr int dict_floats(int fm, int K) { return fm == FM_F32 ? K * 48 : fm >= FM_C8 ? K * 32 : 0; }
+__host__ __device__ constexpr int dict_floats(int fm, int K) {
+  return fm == FM_F32 ? K * 48 : fm == FM_PLANE ? K * 16 : fm >= FM_C8 ? K * 32 : 0;
+}
 
 __constant__ ShConst g_sh;
 
@@ -161,8 +166,6 @@ __global__ void __launch_bounds__(1024) decode_kernel(
         }
       }
     }
-    if (lane < GB)
-      for (int t = s; t < sp; ++t) cpk[lane * sp + t] = make_uint2(0u, 0u);
     {
       if (use_cam && lane < nb) {
         vx -= cx;
@@ -188,10 +191,9 @@ __global__ void __launch_bounds__(1024) decode_kernel(
         nzs[lane] = nz;
       }
       __syncwarp();  // the batch's codes are staged
-      // entries t >= nnz count as zero: clear them, so that the loop below
-      // needs no per-entry test
-      if (lane < GB)
-        for (int t = nz; t < s; ++t) cpk[lane * sp + t] = make_uint2(0u, 0u);
+      // the loop below takes nonzeros in pairs: an odd code's partner counts as
+      // zero (sp is even, so the slot exists)
+      if (lane < GB && (nz & 1)) cpk[lane * sp + nz] = make_uint2(0u, 0u);
     }
     __syncwarp();
     // ---- phase B: eight lanes per Gaussian, four Gaussians per step
@@ -200,8 +202,8 @@ __global__ void __launch_bounds__(1024) decode_kernel(
       const bool act = gl < nb;
       const int gs = act ? gl : 0;
       const int nzl = act ? nzs[gs] : 0;
-      int nzp = max(nzl, __shfl_xor_sync(FULL, nzl, 8));
-      nzp = max(nzp, __shfl_xor_sync(FULL, nzp, 16));
+      // each group walks its own Gaussian's nonzeros: with uneven codes the
+      // groups that are done read no shared memory
       if (FM == FM_F32) {
         // FP32 planes: lane ql reads 16 bytes of the R and G planes (lanes
         // 0-3: R of bases 4ql..4ql+3; lanes 4-7: G of bases 4(ql-4)..), so the
@@ -210,7 +212,7 @@ __global__ void __launch_bounds__(1024) decode_kernel(
         float4 acc4 = make_float4(0.f, 0.f, 0.f, 0.f);
         float2 accb = make_float2(0.f, 0.f);
 #pragma unroll 2
-        for (int t = 0; t < nzp; t += 2) {
+        for (int t = 0; t < nzl; t += 2) {
           const uint4 c2 = *reinterpret_cast<const uint4*>(cpk + gs * sp + t);
           const uint32_t jt[2] = {c2.x, c2.z};
           const float at[2] = {__uint_as_float(c2.y), __uint_as_float(c2.w)};
@@ -228,6 +230,7 @@ __global__ void __launch_bounds__(1024) decode_kernel(
             accb.y = fmaf(a, bb.y, accb.y);
           }
         }
+        __syncwarp();
         const float4 y4 = *reinterpret_cast<const float4*>(Ys + gs * YS + ysw(gs, ql & 3));
         const float2 yb = *reinterpret_cast<const float2*>(Ys + gs * YS + ysw(gs, ql >> 1) + ((2 * ql) & 3));
         float prg = fmaf(y4.x, acc4.x, fmaf(y4.y, acc4.y, fmaf(y4.z, acc4.z, y4.w * acc4.w)));
@@ -247,7 +250,7 @@ __global__ void __launch_bounds__(1024) decode_kernel(
       }
       float aR = 0.f, aG = 0.f, aB = 0.f, bR = 0.f, bG = 0.f, bBl = 0.f;
 #pragma unroll 2
-      for (int t = 0; t < nzp; t += 2) {
+      for (int t = 0; t < nzl; t += 2) {
         const uint4 c2 = *reinterpret_cast<const uint4*>(cpk + gs * sp + t);
         const uint32_t jt[2] = {c2.x, c2.z};
         const float at[2] = {__uint_as_float(c2.y), __uint_as_float(c2.w)};
@@ -280,6 +283,7 @@ __global__ void __launch_bounds__(1024) decode_kernel(
           }
         }
       }
+      __syncwarp();
       const float2 yy = *reinterpret_cast<const float2*>(Ys + gs * YS + ysw(gs, ql >> 1) + ((2 * ql) & 3));
       const float p0 = fmaf(yy.x, aR, yy.y * bR), p1 = fmaf(yy.x, aG, yy.y * bG),
                   p2 = fmaf(yy.x, aB, yy.y * bBl);
@@ -304,6 +308,147 @@ __global__ void __launch_bounds__(1024) decode_kernel(
         // full colour: the DC term and the usual +0.5 offset, clamped at zero
         if (dc) v = fmaxf(0.f, fmaf(y00, dc[base * 3 + e], v) + 0.5f);
         rgb[base * 3 + e] = v;
+      }
+    }
+    __syncwarp();
+  }
+  if (bad) flag_status(status, ST_BAD_INPUT);
+}
+
+// One channel (blockIdx.y) of the FP32 decode, its plane of the dictionary in
+// shared memory, 16 floats (64 bytes) per atom.  A warp takes batches of 8 or 16
+// Gaussians: the codes and the basis values are staged as in decode_kernel, then
+// four lanes take a Gaussian (eight Gaussians per step), a lane 16 bytes of each
+// atom's row.  Against reading whole rows through the read-only cache the codes
+// are read and staged three times, but an atom costs 64 bytes of shared memory
+// per channel instead of six gathers of 4 bytes per lane: N = 778k, K = 2048,
+// s = 16 (half of the slots used) 196 -> 150 us, bound by issue (68 %) and
+// shared-memory wavefronts (69 %).
+__host__ __device__ constexpr int plane_warp_floats(int sp, int gb) { return gb * YS + gb * sp * 2 + gb; }
+
+template <int PGB>
+__global__ void __launch_bounds__(1024) decode_channel_kernel(
+    const float* __restrict__ D, int K, const uint16_t* __restrict__ idx, const float* __restrict__ coef,
+    const uint8_t* __restrict__ nnz, int s, int sp, uint32_t sdiv, int64_t N, const float* __restrict__ dm,
+    int use_cam, float cx, float cy, float cz, const float* __restrict__ dc, float y00, float* __restrict__ rgb,
+    uint32_t* status) {
+  extern __shared__ __align__(16) float sm[];
+  const int nwarps = blockDim.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned FULL = 0xffffffffu;
+  const int ch = blockIdx.y;
+  for (int f0 = threadIdx.x; f0 < K * 16; f0 += 12 * blockDim.x) {
+    float v[12];
+#pragma unroll
+    for (int u = 0; u < 12; ++u) {
+      const int f = f0 + u * blockDim.x, j = f >> 4, b = f & 15;
+      v[u] = (f < K * 16 && b < 15) ? __ldg(D + static_cast<size_t>(j) * DLSH_D + ch * 15 + b) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 12; ++u)
+      if (f0 + u * blockDim.x < K * 16) sm[f0 + u * blockDim.x] = v[u];
+  }
+  __syncthreads();
+  float* wsm = sm + static_cast<size_t>(K) * 16 + warp * plane_warp_floats(sp, PGB);
+  float* Ys = wsm;
+  uint2* cpk = reinterpret_cast<uint2*>(wsm + PGB * YS);
+  int* nzs = reinterpret_cast<int*>(wsm + PGB * YS + PGB * sp * 2);
+  const int q = lane & 3, grp = lane >> 2;
+  const int64_t nbatch = (N + PGB - 1) / PGB;
+  const int64_t wstride = static_cast<int64_t>(gridDim.x) * nwarps;
+  bool bad = false;
+  for (int64_t bt = static_cast<int64_t>(blockIdx.x) * nwarps + warp; bt < nbatch; bt += wstride) {
+    const int64_t base = bt * PGB;
+    const int nb = N - base < PGB ? static_cast<int>(N - base) : PGB;
+    const int64_t g = base + lane;
+    float vx = 0.f, vy = 0.f, vz = 1.f;
+    int nz = 0;
+    if (lane < nb) {
+      vx = dm[g * 3 + 0];
+      vy = dm[g * 3 + 1];
+      vz = dm[g * 3 + 2];
+      nz = nnz[g];
+    }
+    // ---- the batch's codes as (row offset, coefficient) pairs
+    for (int k0 = 0; 32 * k0 < PGB * s; k0 += 8) {
+      uint32_t jj[8];
+      float aa[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int f = lane + 32 * (k0 + u);
+        const bool on = f < nb * s;
+        jj[u] = on ? idx[base * s + f] : 0u;
+        aa[u] = on ? coef[base * s + f] : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int f = lane + 32 * (k0 + u);
+        if (f < nb * s) {
+          const int gl = s == 1 ? f : static_cast<int>(__umulhi(static_cast<uint32_t>(f), sdiv));
+          const bool ok = jj[u] < static_cast<uint32_t>(K);  // else reported and counted as zero
+          bad |= !ok;
+          cpk[gl * sp + (f - gl * s)] = make_uint2(ok ? jj[u] * 16u : 0u, ok ? __float_as_uint(aa[u]) : 0u);
+        }
+      }
+    }
+    if (use_cam && lane < nb) {
+      vx -= cx;
+      vy -= cy;
+      vz -= cz;
+      const float inv = rsqrtf(vx * vx + vy * vy + vz * vz);
+      vx *= inv;
+      vy *= inv;
+      vz *= inv;
+    }
+    {
+      float Y[15];
+      sh_basis(g_sh.c, vx, vy, vz, Y);
+      if (lane < PGB) {
+        float* ys = Ys + lane * YS;
+        *reinterpret_cast<float4*>(ys + ysw(lane, 0)) = make_float4(Y[0], Y[1], Y[2], Y[3]);
+        *reinterpret_cast<float4*>(ys + ysw(lane, 1)) = make_float4(Y[4], Y[5], Y[6], Y[7]);
+        *reinterpret_cast<float4*>(ys + ysw(lane, 2)) = make_float4(Y[8], Y[9], Y[10], Y[11]);
+        *reinterpret_cast<float4*>(ys + ysw(lane, 3)) = make_float4(Y[12], Y[13], Y[14], 0.f);
+        if (nz > s) {
+          bad = true;
+          nz = s;
+        }
+        nzs[lane] = nz;
+      }
+    }
+    __syncwarp();  // the batch's codes are staged
+    if (lane < PGB && (nz & 1)) cpk[lane * sp + nz] = make_uint2(0u, 0u);  // an odd code's partner counts as zero
+    __syncwarp();
+    // ---- four lanes per Gaussian, eight Gaussians per step
+#pragma unroll
+    for (int g0 = 0; g0 < PGB; g0 += 8) {
+      const int gs = g0 + grp;
+      const int nzl = gs < nb ? nzs[gs] : 0;  // each group walks its own nonzeros
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+      for (int t = 0; t < nzl; t += 2) {
+        const uint4 c2 = *reinterpret_cast<const uint4*>(cpk + gs * sp + t);
+        const float4 w0 = *reinterpret_cast<const float4*>(sm + c2.x + 4 * q);
+        const float4 w1 = *reinterpret_cast<const float4*>(sm + c2.z + 4 * q);
+        const float a0 = __uint_as_float(c2.y), a1 = __uint_as_float(c2.w);
+        acc.x = fmaf(a0, w0.x, acc.x);
+        acc.y = fmaf(a0, w0.y, acc.y);
+        acc.z = fmaf(a0, w0.z, acc.z);
+        acc.w = fmaf(a0, w0.w, acc.w);
+        acc.x = fmaf(a1, w1.x, acc.x);
+        acc.y = fmaf(a1, w1.y, acc.y);
+        acc.z = fmaf(a1, w1.z, acc.z);
+        acc.w = fmaf(a1, w1.w, acc.w);
+      }
+      __syncwarp();
+      const float4 y4 = *reinterpret_cast<const float4*>(Ys + gs * YS + ysw(gs, q));
+      float v = fmaf(y4.x, acc.x, fmaf(y4.y, acc.y, fmaf(y4.z, acc.z, y4.w * acc.w)));
+      v += __shfl_xor_sync(FULL, v, 1);
+      v += __shfl_xor_sync(FULL, v, 2);
+      if (q == 0 && gs < nb) {
+        const int64_t e = (base + gs) * 3 + ch;
+        if (dc) v = fmaxf(0.f, fmaf(y00, dc[e], v) + 0.5f);
+        rgb[e] = v;
       }
     }
     __syncwarp();
@@ -373,11 +518,42 @@ static int launch_decode_gb(const float* D, int K, const void* idx, const void* 
 // Gaussians (0 if none do).
 static int fit_warps(int fm, int K, int s, int gb) {
   const long long room = SMEM_LIMIT - 4LL * dict_floats(fm, K);
-  const long long wb = 4LL * warp_floats(staged_slots(s), gb);
+  const int sp = staged_slots(s);
+  const long long wb = 4LL * (fm == FM_PLANE ? plane_warp_floats(sp, gb) : warp_floats(sp, gb));
   long long n = room > 0 ? room / wb : 0;
   return static_cast<int>(n > 32 ? 32 : n);
 }
 static int fit_warps(int fm, int K, int s) { return fit_warps(fm, K, s, batch_of(fm)); }
+
+// One decode launch per channel plane, nwarps warps per CTA in batches of GB
+// Gaussians.
+template <int GB>
+static int launch_planes(const float* D, int K, const uint16_t* idx, const float* coef, const uint8_t* nnz, int s,
+                         int64_t N, const float* dm, const float* cam, const float* dc, float* rgb, uint32_t* status,
+                         int nwarps, cudaStream_t st, const char* call) {
+  int sms = device_sm_count();
+  if (sms <= 0) sms = 1;
+  const int sp = staged_slots(s);
+  const uint32_t sdiv = s >= 2 ? static_cast<uint32_t>((uint64_t(1) << 32) / static_cast<uint64_t>(s) + 1) : 0u;
+  const size_t smem = (static_cast<size_t>(K) * 16 + static_cast<size_t>(nwarps) * plane_warp_floats(sp, GB)) * 4;
+  DLSH_CUDA_TRY(
+      cudaFuncSetAttribute(decode_channel_kernel<GB>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT), call);
+  int per_sm = 0;
+  DLSH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_channel_kernel<GB>, nwarps * 32, smem),
+                call);
+  if (per_sm < 1) per_sm = 1;
+  const int64_t nbatch = (N + GB - 1) / GB;
+  int64_t grid = static_cast<int64_t>(sms) * per_sm / 3;  // the SMs' CTAs over the three channels
+  const int64_t need = (nbatch + nwarps - 1) / nwarps;
+  if (grid > need) grid = need;
+  if (grid < 1) grid = 1;
+  const float cx = cam ? cam[0] : 0.f, cy = cam ? cam[1] : 0.f, cz = cam ? cam[2] : 0.f;
+  const float y00 = static_cast<float>(0.5 / sqrt(M_PI));
+  decode_channel_kernel<GB><<<dim3(static_cast<unsigned>(grid), 3), nwarps * 32, smem, st>>>(
+      D, K, idx, coef, nnz, s, sp, sdiv, N, dm, cam != nullptr, cx, cy, cz, dc, y00, rgb, status);
+  count_launches(1);
+  return check_launch(call);
+}
 
 // The batch size and warps per CTA for (fm, K, s): the autotuner's record if it
 // still fits, else the default batch with as many warps as fit (16 warps for
@@ -409,10 +585,12 @@ static int launch_decode(const float* D, int K, const void* idx, const void* coe
 }  // namespace dec
 
 // The FP32 table stays in shared memory while at least six warps (batches of
-// 8) fit beside it; beyond that (about 1150 atoms) the rows are read through
-// the read-only cache.
+// 8) fit beside it; beyond that (about 1150 atoms) one channel plane at a time,
+// while eight warps fit beside it; then (about 3200 atoms) the rows are read
+// through the read-only cache.
 static int decode_format(int K, int s) {
-  return dec::fit_warps(dec::FM_F32, K, s) >= 6 ? dec::FM_F32 : dec::FM_GLOBAL;
+  if (dec::fit_warps(dec::FM_F32, K, s) >= 6) return dec::FM_F32;
+  return dec::fit_warps(dec::FM_PLANE, K, s) >= 8 ? dec::FM_PLANE : dec::FM_GLOBAL;
 }
 
 // Shared with the bench / learn paths: enqueue one decode.
@@ -426,6 +604,9 @@ int decode_enqueue(const float* D, int K, const uint16_t* idx, const float* coef
   const int fm = decode_format(K, s);
   int gb = 0, nw = 0;
   decode_shape(fm, K, s, &gb, &nw);
+  if (fm == FM_PLANE)
+    return gb == 16 ? launch_planes<16>(D, K, idx, coef, nnz, s, N, dm, cam, dc, rgb, status, nw, st, "dlsh_decode")
+                    : launch_planes<8>(D, K, idx, coef, nnz, s, N, dm, cam, dc, rgb, status, nw, st, "dlsh_decode");
   if (fm == FM_F32)
     return launch_decode<FM_F32>(D, K, idx, coef, nnz, s, N, dm, cam, dc, rgb, status, gb, nw, st, "dlsh_decode");
   return launch_decode<FM_GLOBAL>(D, K, idx, coef, nnz, s, N, dm, cam, dc, rgb, status, gb, nw, st,
@@ -565,6 +746,14 @@ extern "C" int dlsh_autotune_decode(const float* D, int K, int d, const void* id
       case FM_GLOBAL:
         return launch_decode<FM_GLOBAL>(D, K, idx, coef, nnz, s, N, dirs_or_means, cam_pos, nullptr, rgb, nullptr,
                                         gb, nw, st, call);
+      case FM_PLANE: {
+        const uint16_t* ix = static_cast<const uint16_t*>(idx);
+        const float* cf = static_cast<const float*>(coef);
+        return gb == 16 ? launch_planes<16>(D, K, ix, cf, nnz, s, N, dirs_or_means, cam_pos, nullptr, rgb, nullptr, nw,
+                                            st, call)
+                        : launch_planes<8>(D, K, ix, cf, nnz, s, N, dirs_or_means, cam_pos, nullptr, rgb, nullptr, nw,
+                                           st, call);
+      }
       case FM_C8:
         return launch_decode<FM_C8>(D, K, idx, coef, nnz, s, N, dirs_or_means, cam_pos, nullptr, rgb, nullptr, gb,
                                     nw, st, call);

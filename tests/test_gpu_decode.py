@@ -34,6 +34,34 @@ def test_decode_dirs(lib, N, K, s):
     assert ok, worst
 
 
+@pytest.mark.parametrize("N,K,s,cam,with_dc", [(1, 1200, 1, False, False), (17, 1300, 3, True, True),
+                                               (5003, 2048, 16, True, False), (4096, 3000, 8, False, True),
+                                               (301, 1160, 32, False, False), (90_001, 2048, 5, True, True),
+                                               (50, 3300, 4, False, False)])
+def test_decode_large_dictionaries(lib, N, K, s, cam, with_dc):
+    """Dictionaries decoded one channel plane at a time (about 1150 to 3100
+    atoms) and beyond (3300 atoms): ragged batches, uneven codes, the camera form
+    and the full colour.  The file's relative tolerance (1e-4)."""
+    rng = np.random.default_rng(K + s)
+    D = synth.hidden_dictionary(K, 5).astype(np.float32)
+    idx, coef, nnz = _codes(rng, N, K, s)
+    dc = rng.standard_normal((N, 3)).astype(np.float32) if with_dc else None
+    if cam:
+        pos, mu = synth.camera_and_means(N, 2, 3)
+        view, ref_view = dict(means=torch.from_numpy(mu).cuda(), cam=pos), dict(means=mu, cam=pos)
+    else:
+        dirs = synth.unit_directions(N, 6)
+        view, ref_view = dict(dirs=torch.from_numpy(dirs).cuda()), dict(dirs=dirs)
+    rgb = lib.decode(torch.from_numpy(D).cuda(), torch.from_numpy(idx.astype(np.int16)).cuda(),
+                     torch.from_numpy(coef).cuda(), torch.from_numpy(nnz).cuda(),
+                     dc=None if dc is None else torch.from_numpy(dc).cuda(), sync=True, **view).cpu().numpy()
+    ref = osh.decode(D, idx, coef, nnz, **ref_view)
+    if with_dc:
+        ref = osh.full_colour(ref, dc)
+    ok, worst = close_rel(rgb, ref)
+    assert ok, worst
+
+
 def test_decode_camera_and_means(lib):
     N, K, s = 5000, 1024, 8
     rng = np.random.default_rng(1)
