@@ -1,5 +1,5 @@
-// Host side of the encoder: plans, dictionary preparation (prep_kernel,
-// gram_kernel), the correlation-only kernel, kernel choice, the C ABI entry
+// Host side of the encoder: plans, dictionary preparation
+// (prepare_kernel), the correlation-only kernel, kernel choice, the C ABI entry
 // points, the autotuner and the multi-scene call.  The encoder kernels are in
 // encode_core.cuh.
 #include "encode_core.cuh"
@@ -9,23 +9,21 @@ namespace enc {
 
 // ---------------------------------------------------------------------------
 // Dictionary preparation: padded FP32 copy, FP8 scales and the packed operand
-// image, one block of 64 threads per (padded) atom.
+// image, 64 threads per (padded) atom.
 // ---------------------------------------------------------------------------
-__global__ void prep_kernel(const float* __restrict__ D, int K, int Kp, int BN, int prec,
-                            float* __restrict__ D32p, uint8_t* __restrict__ img,
-                            float* __restrict__ sigma, uint32_t chunk_bytes) {
-  const int j = blockIdx.x;
-  const int k = threadIdx.x;
+__device__ __forceinline__ void prep_atom(const float* __restrict__ D, int K, int j, int k, int BN, int prec,
+                                          float* __restrict__ D32p, uint8_t* __restrict__ img,
+                                          float* __restrict__ sigma, uint32_t chunk_bytes, float* pair_max) {
   const float v = (j < K && k < DLSH_D) ? D[static_cast<size_t>(j) * DLSH_D + k] : 0.f;
   if (k < DPAD) D32p[static_cast<size_t>(j) * DPAD + k] = v;
-  __shared__ float red[64];
-  red[k] = fabsf(v);
+  // the atom's largest |value|, over its two warps
+  float mx = fabsf(v);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((k & 31) == 0) pair_max[k >> 5] = mx;
   __syncthreads();
-  for (int w = 32; w > 0; w >>= 1) {
-    if (k < w) red[k] = fmaxf(red[k], red[k + w]);
-    __syncthreads();
-  }
-  const float sj = red[0] > 0.f ? red[0] / FP8_MAX : 1.f;
+  mx = fmaxf(pair_max[0], pair_max[1]);
+  const float sj = mx > 0.f ? mx / FP8_MAX : 1.f;
   if (k == 0 && sigma) sigma[j] = sj;
   const int c = j / BN, n = j % BN;
   uint8_t* base = img + static_cast<size_t>(c) * chunk_bytes;
@@ -63,16 +61,29 @@ __global__ void prep_kernel(const float* __restrict__ D, int K, int Kp, int BN, 
   }
 }
 
-// G = D D^T (FP32), 32 x 32 output tiles.
-__global__ void gram_kernel(const float* __restrict__ D32p, int K, float* __restrict__ G) {
+// The whole preparation in one launch: the first nprep blocks take four padded
+// atoms each, the others a 32 x 32 tile of G = D D^T (FP32) straight from D;
+// block 0 also clears the status word.
+__global__ void __launch_bounds__(256) prepare_kernel(const float* __restrict__ D, int K, int Kp, int BN, int prec,
+                                                      float* __restrict__ D32p, uint8_t* __restrict__ img,
+                                                      float* __restrict__ sigma, uint32_t chunk_bytes, int nprep,
+                                                      float* __restrict__ G, uint32_t* __restrict__ status) {
   __shared__ float ta[32][DPAD + 1];
   __shared__ float tb[32][DPAD + 1];
-  const int j0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  for (int f = ty * 32 + tx; f < 32 * DPAD; f += 256) {
-    const int r = f / DPAD, c = f % DPAD;
-    ta[r][c] = (j0 + r < K) ? D32p[static_cast<size_t>(j0 + r) * DPAD + c] : 0.f;
-    tb[r][c] = (k0 + r < K) ? D32p[static_cast<size_t>(k0 + r) * DPAD + c] : 0.f;
+  const int b = static_cast<int>(blockIdx.x), tid = threadIdx.x;
+  if (b == 0 && tid == 0) *status = 0u;
+  if (b < nprep) {  // Kp is a multiple of 64
+    prep_atom(D, K, 4 * b + (tid >> 6), tid & 63, BN, prec, D32p, img, sigma, chunk_bytes, &ta[tid >> 6][0]);
+    return;
+  }
+  const int nt = (K + 31) / 32, tile = b - nprep;
+  const int j0 = tile / nt * 32, k0 = tile % nt * 32;
+  const int tx = tid % 32, ty = tid / 32;  // 32 x 8
+#pragma unroll
+  for (int f = tid; f < 32 * DLSH_D; f += 256) {
+    const int r = f / DLSH_D, c = f % DLSH_D;
+    ta[r][c] = (j0 + r < K) ? D[static_cast<size_t>(j0 + r) * DLSH_D + c] : 0.f;
+    tb[r][c] = (k0 + r < K) ? D[static_cast<size_t>(k0 + r) * DLSH_D + c] : 0.f;
   }
   __syncthreads();
   for (int r = ty; r < 32; r += 8) {
@@ -241,19 +252,11 @@ static int launch_correlate(const float* R, int64_t M, const Plan& p, const Ws& 
 
 // Launches the dictionary preparation (padded copy, Gram, operand image).
 static int prepare(const float* D, const Plan& p, const Ws& w, bool gram, cudaStream_t st) {
-  DLSH_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(uint32_t), st), "dlsh: status reset");
-  prep_kernel<<<p.Kp, 64, 0, st>>>(D, p.K, p.Kp, p.BN, p.prec, w.D32p, w.img, w.sigma,
-                                   p.chunk_bytes);
+  const int nt = gram ? (p.K + 31) / 32 : 0;
+  prepare_kernel<<<p.Kp / 4 + nt * nt, 256, 0, st>>>(D, p.K, p.Kp, p.BN, p.prec, w.D32p, w.img, w.sigma, p.chunk_bytes,
+                                                     p.Kp / 4, w.G, w.status);
   count_launches(1);
-  int rc = check_launch("dlsh: prep_kernel");
-  if (rc) return rc;
-  if (gram) {
-    dim3 g((p.K + 31) / 32, (p.K + 31) / 32);
-    gram_kernel<<<g, dim3(32, 8), 0, st>>>(w.D32p, p.K, w.G);
-    count_launches(1);
-    rc = check_launch("dlsh: gram_kernel");
-  }
-  return rc;
+  return check_launch("dlsh: prepare_kernel");
 }
 
 }  // namespace enc
@@ -367,8 +370,15 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
       SplitArgs a{};
       fill(a);
       a.p = choice == 6 ? sp16x3 : (choice == 5 ? sp16 : sp);
-      if (choice == 6) return launch_split<true, 3>(a, grid, st);
-      return choice == 5 ? launch_split<true, 2>(a, grid, st) : launch_split<false, 2>(a, grid, st);
+      if (choice == 6) return launch_split<true, 3, 128>(a, grid, st);
+      if (choice == 4) return launch_split<false, 2, 128>(a, grid, st);
+      // up to one tile per SM: tiles of 64 signals, one or two per CTA (N = 10,000,
+      // K = 256, s = 8: 99 us a call on 40 CTAs with two tiles of 128 each, 61 so)
+      if (!n_dev && ntiles <= sms) {
+        const int64_t half = (N + 63) / 64;
+        return launch_split<true, 2, 64>(a, static_cast<int>(half < sms ? half : sms), st);
+      }
+      return launch_split<true, 2, 128>(a, grid, st);
     }
     AltArgs a{};
     fill(a);

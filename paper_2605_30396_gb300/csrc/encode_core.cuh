@@ -1188,12 +1188,12 @@ int launch_pair(const PairArgs& a, int grid, cudaStream_t st) {
 // One launch of the alternating two-tile encoder (defined in enc_split.cu).
 int launch_alt(const AltArgs& a, int grid, cudaStream_t st);
 
-template <bool F16, int NS>
+template <bool F16, int NS, int TR>
 int launch_split(const SplitArgs& a, int grid, cudaStream_t st) {
-  DLSH_CUDA_TRY(cudaFuncSetAttribute(encode_split_kernel<F16, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  DLSH_CUDA_TRY(cudaFuncSetAttribute(encode_split_kernel<F16, NS, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      SMEM_LIMIT),
                 "dlsh_encode: cudaFuncSetAttribute");
-  encode_split_kernel<F16, NS><<<grid, NTHREADS, a.p.smem, st>>>(a);
+  encode_split_kernel<F16, NS, TR><<<grid, NTHREADS, a.p.smem, st>>>(a);
   count_launches(1);
   return check_launch("dlsh_encode: launch");
 }
@@ -1212,9 +1212,10 @@ extern template int launch_pair<1, false>(const PairArgs&, int, cudaStream_t);
 extern template int launch_pair<1, true>(const PairArgs&, int, cudaStream_t);
 extern template int launch_pair<2, false>(const PairArgs&, int, cudaStream_t);
 extern template int launch_pair<2, true>(const PairArgs&, int, cudaStream_t);
-extern template int launch_split<false, 2>(const SplitArgs&, int, cudaStream_t);
-extern template int launch_split<true, 2>(const SplitArgs&, int, cudaStream_t);
-extern template int launch_split<true, 3>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<false, 2, 128>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 2, 128>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 2, 64>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 3, 128>(const SplitArgs&, int, cudaStream_t);
 
 }  // namespace enc
 }  // namespace dlsh

@@ -106,7 +106,10 @@ inline int make_split_plan(int K, int s, int code, SplitPlan& p, bool f16, int n
   return DLSH_OK;
 }
 
-template <bool F16, int NSL>
+// TR: signals per tile, 128, or 64 where whole tiles would leave SMs idle (the
+// solver then makes one pass per job instead of two, on twice the CTAs; the
+// operand's other 64 rows are not looked at).
+template <bool F16, int NSL, int TR>
 __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_constant__ SplitArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr uint32_t ACC0 = 128;
@@ -116,7 +119,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
   constexpr bool XC = F16 && NSL == 2;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long NS = a.n_dev ? *a.n_dev : a.N;
-  const int ntiles = static_cast<int>((NS + TILE_M - 1) / TILE_M);
+  constexpr int NPASS = TR / 64;
+  static_assert(TR == TILE_M || TR == 64, "whole or half tiles");
+  const int ntiles = static_cast<int>((NS + TR - 1) / TR);
   const int Gd = static_cast<int>(gridDim.x), bidx = static_cast<int>(blockIdx.x);
   const int s = p.s;
   // rounds k in which tile slot t has a tile (tiles b + (NSL k + t) Gd); the
@@ -147,8 +152,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
     return r;
   };
   auto rows_of = [&](long long tl) -> int {
-    const long long g0 = tl * TILE_M;
-    return static_cast<int>(NS - g0 < TILE_M ? NS - g0 : TILE_M);
+    const long long g0 = tl * TR;
+    return static_cast<int>(NS - g0 < TR ? NS - g0 : TR);
   };
 
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
@@ -251,6 +256,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
             if (prof_on) pcs[0] += clock64() - W0;
             tc_fence_after();
             __syncwarp();
+            if (TR < TILE_M && 32 * wq >= TR) {  // no signals in this lane quarter
+              tc_fence_before();
+              if (lane == 0) mbar_arrive(&bar_empty[buf]);
+              continue;
+            }
             uint32_t r0[32], r1[32];
             tmem_ld32_issue(trow + static_cast<uint32_t>(buf * ABN), r0);
             tmem_ld32_issue(trow + static_cast<uint32_t>(buf * ABN + 32), r1);
@@ -349,7 +359,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
     auto st_inv = [&](int t) { return reinterpret_cast<float*>(smem + p.off_row[t]) + 3 * TILE_M; };
     // row r of tile `tl` (slot t) into the staging area; its ||x||^2
     auto stage_x = [&](int t, long long tl, int r) -> float {
-      const int64_t tg0 = tl * TILE_M;
+      const int64_t tg0 = tl * TR;
       const bool tin = r < rows_of(tl);
       const float* txr = a.X + (tg0 + r) * DLSH_D;
       float x[12];
@@ -372,7 +382,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
       if (rounds_of(t) > 0 && ok) {
         if (!wait_staging(job_index(t, 0, 0))) ok = false;
         if (ok)
-          for (int ps = 0; ps < 2; ++ps) {
+          for (int ps = 0; ps < NPASS; ++ps) {
             const int r = row_of(ps);
             st_rn2(t)[r] = stage_x(t, tile_of(t, 0), r);
           }
@@ -385,7 +395,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
       const int nk = slots_in(k);
       for (int t = 0; t < nk; ++t) {
         const int rows = rows_of(tile_of(t, k));
-        for (int ps = 0; ps < 2; ++ps) {
+        for (int ps = 0; ps < NPASS; ++ps) {
           const int r = row_of(ps);
           st_xn(t)[r] = sqrtf(st_rn2(t)[r]);
           st_tc(t)[r] = r < rows ? 0 : 0x100;
@@ -422,10 +432,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
           int* sel = reinterpret_cast<int*>(smem + p.off_sel[t]);
           float* ys = reinterpret_cast<float*>(smem + p.off_y[t]);
           const long long tl = tile_of(t, k);
-          const int64_t g0 = tl * TILE_M;
+          const int64_t g0 = tl * TR;
           const int rows = rows_of(tl);
 #pragma unroll 1
-          for (int ps = 0; ps < 2; ++ps) {
+          for (int ps = 0; ps < NPASS; ++ps) {
             const int R2 = row_of(ps);
 #define LS(rr, cc2) Ls[(((rr) * ((rr) + 1)) / 2 + (cc2)) * TILE_M + R2]
 #define IDG(rr) LS(rr, rr)

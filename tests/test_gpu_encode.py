@@ -242,3 +242,19 @@ def test_multi_tile_fp32_encoders_over_several_rounds(lib, variant):
     np.testing.assert_array_equal(nnz[sep], ref["nnz"][sep])
     r = resid.cpu().numpy().astype(np.float64)
     np.testing.assert_allclose(r[sep], ref["resid_sq"][sep], rtol=2e-4, atol=1e-9)
+
+
+@pytest.mark.parametrize("K,s", [(256, 8), (1024, 4), (130, 1)])
+def test_small_calls_match_large_ones(lib, K, s):
+    """Up to one tile per SM the encoder takes tiles of 64 signals instead of
+    128: a signal's code does not depend on the tiling, so the first N signals
+    alone give bitwise the codes they have in a call of 20,000 (152 SMs: 64-signal
+    tiles up to 19,456)."""
+    n = 20_000
+    D = torch.from_numpy(synth.hidden_dictionary(K, 1).astype(np.float32)).cuda()
+    X = torch.from_numpy(synth.signals(n, synth.hidden_dictionary(K, 2), min(s, 4), 3)).cuda()
+    whole = lib.encode(D, X, s, sync=True)
+    for N in (1, 63, 64, 65, 129, 9728, 9729, 19_456, 19_457):
+        part = lib.encode(D, X[:N].contiguous(), s, sync=True)
+        for a, b in zip(part, whole):
+            assert torch.equal(a, b[:N]), N
