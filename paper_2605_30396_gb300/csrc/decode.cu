@@ -73,6 +73,12 @@ __global__ void __launch_bounds__(1024) decode_kernel(
     const float* __restrict__ dc, float y00, float* __restrict__ rgb, uint32_t* status) {
   extern __shared__ __align__(16) float sm[];
   static_assert(GB == 8 || GB == 16, "batches of 8 or 16 Gaussians");
+  // FP32 table: each group of lanes walks its own Gaussian's nonzeros, so that
+  // with uneven codes the groups that are done read no shared memory, which
+  // bounds this format.  The others are bound by issue, and the common loop of
+  // the step's longest code is the cheaper one (146 against 152 us, compact
+  // codes of 0 to 4 atoms, N = 2.3M).
+  constexpr bool OWN = FM == FM_F32;
   const int nwarps = blockDim.x >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned FULL = 0xffffffffu;
@@ -166,6 +172,8 @@ __global__ void __launch_bounds__(1024) decode_kernel(
         }
       }
     }
+    if (!OWN && lane < GB)
+      for (int t = s; t < sp; ++t) cpk[lane * sp + t] = make_uint2(0u, 0u);
     {
       if (use_cam && lane < nb) {
         vx -= cx;
@@ -191,9 +199,17 @@ __global__ void __launch_bounds__(1024) decode_kernel(
         nzs[lane] = nz;
       }
       __syncwarp();  // the batch's codes are staged
-      // the loop below takes nonzeros in pairs: an odd code's partner counts as
-      // zero (sp is even, so the slot exists)
-      if (lane < GB && (nz & 1)) cpk[lane * sp + nz] = make_uint2(0u, 0u);
+      if (lane < GB) {
+        if (OWN) {
+          // the loop below takes nonzeros in pairs: an odd code's partner counts
+          // as zero (sp is even, so the slot exists)
+          if (nz & 1) cpk[lane * sp + nz] = make_uint2(0u, 0u);
+        } else {
+          // entries t >= nnz count as zero: clear them, so that the loop below
+          // needs no per-entry test
+          for (int t = nz; t < s; ++t) cpk[lane * sp + t] = make_uint2(0u, 0u);
+        }
+      }
     }
     __syncwarp();
     // ---- phase B: eight lanes per Gaussian, four Gaussians per step
@@ -201,9 +217,11 @@ __global__ void __launch_bounds__(1024) decode_kernel(
       const int gl = g0 + grp;
       const bool act = gl < nb;
       const int gs = act ? gl : 0;
-      const int nzl = act ? nzs[gs] : 0;
-      // each group walks its own Gaussian's nonzeros: with uneven codes the
-      // groups that are done read no shared memory
+      int nzl = act ? nzs[gs] : 0;
+      if (!OWN) {  // the step's longest code
+        nzl = max(nzl, __shfl_xor_sync(FULL, nzl, 8));
+        nzl = max(nzl, __shfl_xor_sync(FULL, nzl, 16));
+      }
       if (FM == FM_F32) {
         // FP32 planes: lane ql reads 16 bytes of the R and G planes (lanes
         // 0-3: R of bases 4ql..4ql+3; lanes 4-7: G of bases 4(ql-4)..), so the
@@ -283,7 +301,6 @@ __global__ void __launch_bounds__(1024) decode_kernel(
           }
         }
       }
-      __syncwarp();
       const float2 yy = *reinterpret_cast<const float2*>(Ys + gs * YS + ysw(gs, ql >> 1) + ((2 * ql) & 3));
       const float p0 = fmaf(yy.x, aR, yy.y * bR), p1 = fmaf(yy.x, aG, yy.y * bG),
                   p2 = fmaf(yy.x, aB, yy.y * bBl);
@@ -601,7 +618,11 @@ int decode_enqueue(const float* D, int K, const uint16_t* idx, const float* coef
   int rc = upload_constants(st);
   if (rc) return rc;
   if (N == 0) return DLSH_OK;
-  const int fm = decode_format(K, s);
+  int fm = decode_format(K, s);
+  // staging three planes on every SM takes about 28 us: short calls read the rows
+  // through the read-only cache instead (K = 2048, us: N = 262k, s = 4 33 by
+  // planes, 31 so; N = 131k, s = 16 35 and 55)
+  if (fm == FM_PLANE && N * s < 1500000) fm = FM_GLOBAL;
   int gb = 0, nw = 0;
   decode_shape(fm, K, s, &gb, &nw);
   if (fm == FM_PLANE)

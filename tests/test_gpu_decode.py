@@ -34,13 +34,13 @@ def test_decode_dirs(lib, N, K, s):
     assert ok, worst
 
 
-@pytest.mark.parametrize("N,K,s,cam,with_dc", [(1, 1200, 1, False, False), (17, 1300, 3, True, True),
-                                               (5003, 2048, 16, True, False), (4096, 3000, 8, False, True),
-                                               (301, 1160, 32, False, False), (90_001, 2048, 5, True, True),
+@pytest.mark.parametrize("N,K,s,cam,with_dc", [(17, 1300, 3, True, True), (5003, 2048, 16, True, False),
+                                               (1_500_001, 1160, 1, False, False), (300_007, 2048, 5, True, True),
+                                               (187_500, 3000, 8, False, True), (46_877, 1200, 32, False, False),
                                                (50, 3300, 4, False, False)])
 def test_decode_large_dictionaries(lib, N, K, s, cam, with_dc):
     """Dictionaries decoded one channel plane at a time (about 1150 to 3100
-    atoms) and beyond (3300 atoms): ragged batches, uneven codes, the camera form
+    atoms, from 1.5 million code slots on), shorter calls and larger dictionaries: ragged batches, uneven codes, the camera form
     and the full colour.  The file's relative tolerance (1e-4)."""
     rng = np.random.default_rng(K + s)
     D = synth.hidden_dictionary(K, 5).astype(np.float32)
