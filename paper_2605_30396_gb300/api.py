@@ -122,7 +122,7 @@ def encode(D, X, s: int, eps: float = 0.0, precision="fp32", sync: bool = False,
 ENCODE_VARIANTS = {1: "encode_kernel (one tile per CTA)", 2: "encode_pair_kernel",
                    3: "encode_alt_kernel", 4: "encode_split_kernel (TF32 parts)",
                    5: "encode_split_kernel (FP16 parts)", 6: "encode_split_kernel (FP16 parts, three tiles)",
-                   7: "encode_kernel (one tile per CTA, FP16 parts)"}
+                   7: "FP16 parts: encode_kernel (one tile per CTA) up to s = 8, encode_split_kernel above"}
 
 
 def encode_variant(K: int, s: int, precision="fp32") -> int:
@@ -153,7 +153,7 @@ def encode_profile(D, X, s: int, eps: float = 0.0, precision="fp32"):
     if variant == 3:  # two tiles served in turn by all warps (see dlsh.h)
         names = ("sel_wait_mma", "selection", "solver", "solver_wait_staging", "tile_iterations",
                  "unused", "mma_wait_a", "mma_wait_chunk", "mma_wait_tmem", "mma_wait_copy")
-    elif variant in (4, 5, 6):  # selection and solver warps (TF32 / FP16 products, 2 or 3 tiles)
+    elif variant in (4, 5, 6, 7):  # selection and solver warps (TF32 / FP16 products, 2 or 3 tiles)
         names = ("sel_wait_mma", "selection", "solver", "solver_wait_staging", "jobs",
                  "solver_wait_cand", "mma_wait_a", "mma_wait_chunk", "mma_wait_tmem", "mma_wait_copy",
                  "sel_wait_solver")

@@ -14,10 +14,10 @@ int launch_alt(const AltArgs& a, int grid, cudaStream_t st) {
   return check_launch("dlsh_encode: launch");
 }
 
-template int launch_split<false, 2, 128>(const SplitArgs&, int, cudaStream_t);
-template int launch_split<true, 2, 128>(const SplitArgs&, int, cudaStream_t);
-template int launch_split<true, 2, 64>(const SplitArgs&, int, cudaStream_t);
-template int launch_split<true, 3, 128>(const SplitArgs&, int, cudaStream_t);
+template int launch_split<false, 2, 128, 8>(const SplitArgs&, int, cudaStream_t);
+template int launch_split<true, 2, 128, 8>(const SplitArgs&, int, cudaStream_t);
+template int launch_split<true, 2, 64, 8>(const SplitArgs&, int, cudaStream_t);
+template int launch_split<true, 3, 128, 8>(const SplitArgs&, int, cudaStream_t);
 
 }  // namespace enc
 }  // namespace dlsh

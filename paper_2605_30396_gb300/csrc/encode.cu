@@ -327,17 +327,20 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
   cap_ring(sp, cap, 2);
   cap_ring(sp16, cap, 2);
   cap_ring(sp16x3, cap, 2);
-  if (choice >= 3 && choice <= 6) {
+  SplitPlan deep;
+  const bool use_deep = choice == 7 && s > 8 && make_split_plan(K, s, prec, deep, true, 2, SMEM_LIMIT, true) == DLSH_OK;
+  if ((choice >= 3 && choice <= 6) || use_deep) {
     Plan p;  // the one-tile encoder's 128-atom FP32 operand image
-    if (make_plan(K, s, prec, p, 128) != DLSH_OK || p.BN != 128)
+    if (use_deep) p = p16;
+    else if (make_plan(K, s, prec, p, 128) != DLSH_OK || p.BN != 128)
       return set_error(DLSH_ERR_UNSUPPORTED, "dlsh_encode: K=%d s=%d does not fit", K, s);
     Ws w;
     carve(ws, p, w);
     if (status_out) *status_out = w.status;
     Plan pi = p;  // the operand image: TF32 hi / lo, or FP16 hi / lo (half the bytes)
-    if (choice == 5 || choice == 6) {
+    if (choice >= 5) {
       pi.prec = OPF16X2;
-      pi.chunk_bytes = sp16.chunk_bytes;
+      pi.chunk_bytes = use_deep ? deep.chunk_bytes : (choice == 6 ? sp16x3 : sp16).chunk_bytes;
     }
     int rc = prepare(D, pi, w, true, st);
     if (rc) return rc;
@@ -369,16 +372,17 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
     if (choice >= 4) {
       SplitArgs a{};
       fill(a);
-      a.p = choice == 6 ? sp16x3 : (choice == 5 ? sp16 : sp);
-      if (choice == 6) return launch_split<true, 3, 128>(a, grid, st);
-      if (choice == 4) return launch_split<false, 2, 128>(a, grid, st);
+      a.p = use_deep ? deep : (choice == 6 ? sp16x3 : (choice == 5 ? sp16 : sp));
+      if (choice == 6) return launch_split<true, 3, 128, 8>(a, grid, st);
+      if (choice == 4) return launch_split<false, 2, 128, 8>(a, grid, st);
       // up to one tile per SM: tiles of 64 signals, one or two per CTA (N = 10,000,
       // K = 256, s = 8: 99 us a call on 40 CTAs with two tiles of 128 each, 61 so)
       if (!n_dev && ntiles <= sms) {
         const int64_t half = (N + 63) / 64;
-        return launch_split<true, 2, 64>(a, static_cast<int>(half < sms ? half : sms), st);
+        const int hgrid = static_cast<int>(half < sms ? half : sms);
+        return use_deep ? launch_split<true, 2, 64, 16>(a, hgrid, st) : launch_split<true, 2, 64, 8>(a, hgrid, st);
       }
-      return launch_split<true, 2, 128>(a, grid, st);
+      return use_deep ? launch_split<true, 2, 128, 16>(a, grid, st) : launch_split<true, 2, 128, 8>(a, grid, st);
     }
     AltArgs a{};
     fill(a);

@@ -36,6 +36,7 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "host.hpp"
@@ -1167,7 +1168,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_kernel(const __grid_consta
 
 template <int PREC, int BN, bool T4 = false>
 int launch_encode(const Args& a, int grid, cudaStream_t st) {
-  auto fn = a.p.s <= 8 ? encode_kernel<PREC, BN, 8, T4> : encode_kernel<PREC, BN, 16, T4>;
+  auto fn = encode_kernel<PREC, BN, 8, T4>;
+  if constexpr (PREC != OPF16X2)  // (FP16 parts with s > 8: the split kernel)
+    if (a.p.s > 8) fn = encode_kernel<PREC, BN, 16, T4>;
   DLSH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT),
                 "dlsh_encode: cudaFuncSetAttribute");
   fn<<<grid, NTHREADS, a.p.smem, st>>>(a);
@@ -1188,12 +1191,12 @@ int launch_pair(const PairArgs& a, int grid, cudaStream_t st) {
 // One launch of the alternating two-tile encoder (defined in enc_split.cu).
 int launch_alt(const AltArgs& a, int grid, cudaStream_t st);
 
-template <bool F16, int NS, int TR>
+template <bool F16, int NS, int TR, int SM>
 int launch_split(const SplitArgs& a, int grid, cudaStream_t st) {
-  DLSH_CUDA_TRY(cudaFuncSetAttribute(encode_split_kernel<F16, NS, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  DLSH_CUDA_TRY(cudaFuncSetAttribute(encode_split_kernel<F16, NS, TR, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      SMEM_LIMIT),
                 "dlsh_encode: cudaFuncSetAttribute");
-  encode_split_kernel<F16, NS, TR><<<grid, NTHREADS, a.p.smem, st>>>(a);
+  encode_split_kernel<F16, NS, TR, SM><<<grid, NTHREADS, a.p.smem, st>>>(a);
   count_launches(1);
   return check_launch("dlsh_encode: launch");
 }
@@ -1212,10 +1215,12 @@ extern template int launch_pair<1, false>(const PairArgs&, int, cudaStream_t);
 extern template int launch_pair<1, true>(const PairArgs&, int, cudaStream_t);
 extern template int launch_pair<2, false>(const PairArgs&, int, cudaStream_t);
 extern template int launch_pair<2, true>(const PairArgs&, int, cudaStream_t);
-extern template int launch_split<false, 2, 128>(const SplitArgs&, int, cudaStream_t);
-extern template int launch_split<true, 2, 128>(const SplitArgs&, int, cudaStream_t);
-extern template int launch_split<true, 2, 64>(const SplitArgs&, int, cudaStream_t);
-extern template int launch_split<true, 3, 128>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<false, 2, 128, 8>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 2, 128, 8>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 2, 64, 8>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 3, 128, 8>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 2, 128, 16>(const SplitArgs&, int, cudaStream_t);
+extern template int launch_split<true, 2, 64, 16>(const SplitArgs&, int, cudaStream_t);
 
 }  // namespace enc
 }  // namespace dlsh

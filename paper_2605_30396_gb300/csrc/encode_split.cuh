@@ -1,4 +1,5 @@
-// Batch-OMP, FP32 correlations (three TF32 or three FP16 products), s <= 8:
+// Batch-OMP, FP32 correlations (three TF32 or three FP16 products; s up to 16
+// with two tiles and FP16 products, else 8):
 // two or three tiles per CTA with the warps split by task (Sec. 2.1: OMP against the dictionary, one greedy atom at
 // a time, least-squares re-fit).
 //
@@ -67,11 +68,17 @@ struct SplitArgs {
 // f16: the correlations as three FP16 products (the operand split into FP16 hi
 // and lo parts of a power-of-two scaled copy) instead of three TF32 products;
 // nslots: tiles per CTA in flight (2 or 3).
+// deep (two slots, FP16 parts): up to 16 atoms per row.  Two such factors leave room
+// for the operand and two ring stages only because what the last step would
+// write and nobody reads (row 15 of the factor, y_15) has no place, and the
+// support is kept in 16 bits.
+constexpr int DEEP = 16;
 inline int make_split_plan(int K, int s, int code, SplitPlan& p, bool f16, int nslots = 2,
-                           int smem_limit = SMEM_LIMIT) {
+                           int smem_limit = SMEM_LIMIT, bool deep = false) {
   int top4 = 0;
-  if (s > 8 || operand_precision(code, &top4) != 0 || nslots < 2 || nslots > SMAXSLOT)
+  if (s > (deep ? DEEP : 8) || operand_precision(code, &top4) != 0 || nslots < 2 || nslots > SMAXSLOT)
     return DLSH_ERR_UNSUPPORTED;
+  if (deep && (!f16 || nslots != 2)) return DLSH_ERR_UNSUPPORTED;
   p.K = K;
   p.s = s;
   p.nslots = nslots;
@@ -87,12 +94,12 @@ inline int make_split_plan(int K, int s, int code, SplitPlan& p, bool f16, int n
   };
   p.off_stage = take(p.a_bytes);
   for (int t = 0; t < nslots; ++t) {
-    p.off_L[t] = take(36 * TILE_M * 4);
-    p.off_sel[t] = take(8 * TILE_M * 4);
-    p.off_y[t] = take(8 * TILE_M * 4);
+    p.off_L[t] = take((deep ? DEEP * (DEEP - 1) / 2 : 36) * TILE_M * 4);
+    p.off_sel[t] = take(deep ? DEEP * TILE_M * 2 : 8 * TILE_M * 4);
+    p.off_y[t] = take((deep ? DEEP - 1 : 8) * TILE_M * 4);
     p.off_row[t] = take(4 * TILE_M * 4);
     p.off_cand[t] = take(2 * TILE_M * 8);
-    p.off_x[t] = (f16 && nslots == 2) ? take(12 * 4 * TILE_M * 4) : 0u;
+    p.off_x[t] = (f16 && nslots == 2 && !deep) ? take(12 * 4 * TILE_M * 4) : 0u;
   }
   p.off_bar = take(1024);
   const uint32_t fixed = (off + 1023u) & ~1023u;
@@ -109,14 +116,22 @@ inline int make_split_plan(int K, int s, int code, SplitPlan& p, bool f16, int n
 // TR: signals per tile, 128, or 64 where whole tiles would leave SMs idle (the
 // solver then makes one pass per job instead of two, on twice the CTAs; the
 // operand's other 64 rows are not looked at).
-template <bool F16, int NSL, int TR>
+// SM: atoms per row at most (8 or 16).  With 16 a row's sub-lane owns dimensions
+// 12 u .. 12 u + 11, as in the one-tile kernel that used to serve these s: the
+// sums, and so the codes, are bitwise that kernel's.  (N = 400k, K = 2048, s = 16
+// with a tolerance: 7490 us on one tile per CTA, whose selection and solver take
+// turns, 4709 here.)
+template <bool F16, int NSL, int TR, int SM>
 __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_constant__ SplitArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr uint32_t ACC0 = 128;
   const SplitPlan& p = a.p;
   // the signals stay in shared memory across a tile's iterations (only the
-  // two-slot FP16 layout has room for them)
-  constexpr bool XC = F16 && NSL == 2;
+  // two-slot FP16 layout with 8 atoms per row has room for them)
+  constexpr bool XC = F16 && NSL == 2 && SM == 8;
+  constexpr bool CD = SM > 8;  // contiguous dimensions per sub-lane
+  auto dim_of = [](int u, int q) { return CD ? 12 * u + q : alt_dim(u, q); };
+  using SelT = std::conditional_t<CD, uint16_t, int>;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long NS = a.n_dev ? *a.n_dev : a.N;
   constexpr int NPASS = TR / 64;
@@ -344,7 +359,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
         for (int q = 0; q < 12; ++q) mx = fmaxf(mx, fabsf(v[q]));
         float rinv;
         const float sc = pow2_scale(quad_max(mx), rinv);
-        write_a_f16(A, r, u, v, sc);
+        if constexpr (CD) write_a_part<OPF16X2>(A, r, u, v, sc);
+        else write_a_f16(A, r, u, v, sc);
         return rinv;
       } else {
         write_a_alt(A, r, u, v);
@@ -364,7 +380,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
       const float* txr = a.X + (tg0 + r) * DLSH_D;
       float x[12];
 #pragma unroll
-      for (int q = 0; q < 12; ++q) x[q] = (tin && alt_dim(u, q) < DLSH_D) ? __ldg(txr + alt_dim(u, q)) : 0.f;
+      for (int q = 0; q < 12; ++q) x[q] = (tin && dim_of(u, q) < DLSH_D) ? __ldg(txr + dim_of(u, q)) : 0.f;
       float part = 0.f;
 #pragma unroll
       for (int q = 0; q < 12; ++q) part = fmaf(x[q], x[q], part);
@@ -429,7 +445,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
           __syncwarp();
           if (lane == 0) mbar_arrive(&cand_empty[t]);
           float* Ls = reinterpret_cast<float*>(smem + p.off_L[t]);
-          int* sel = reinterpret_cast<int*>(smem + p.off_sel[t]);
+          SelT* sel = reinterpret_cast<SelT*>(smem + p.off_sel[t]);
           float* ys = reinterpret_cast<float*>(smem + p.off_y[t]);
           const long long tl = tile_of(t, k);
           const int64_t g0 = tl * TR;
@@ -449,12 +465,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
             const int stc = st_tc(t)[R2];
             const float inv_sc = st_inv(t)[R2];
             int tcc = stc & 0xff;
-            bool act = (stc & 0x100) == 0 && rn2c > eps2;
+            bool act = (stc & 0x100) == 0 && (CD ? !(rn2c <= eps2) : rn2c > eps2);
             if (act) {
               // the step for a support of T atoms, compiled once per T
               auto step = [&](auto tag) {
                 constexpr int T = decltype(tag)::value;
                 constexpr int TA = T > 0 ? T : 1;
+                constexpr bool LAST = CD && T == SM - 1;  // its factor row and y are not kept
+                // 16 atoms: y, the new factor row and the support are read back
+                // from shared memory where they are used (registers)
+                constexpr bool REG = !CD;
                 float x[12], r[12];
                 if constexpr (XC) {
                   const float* xs = reinterpret_cast<const float*>(smem + p.off_x[t]);
@@ -463,7 +483,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
                 } else {
 #pragma unroll
                   for (int q = 0; q < 12; ++q)
-                    x[q] = (in_tile && alt_dim(u, q) < DLSH_D) ? __ldg(xr + alt_dim(u, q)) : 0.f;
+                    x[q] = (in_tile && dim_of(u, q) < DLSH_D) ? __ldg(xr + dim_of(u, q)) : 0.f;
                 }
                 int sl[TA];
 #pragma unroll
@@ -494,9 +514,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
                 const float gjj = __ldg(Grow + js);
                 float4 dj[3];
                 {
-                  const float4* dr = reinterpret_cast<const float4*>(a.D32p + static_cast<size_t>(js) * DPAD + 4 * u);
+                  const float4* dr =
+                      reinterpret_cast<const float4*>(a.D32p + static_cast<size_t>(js) * DPAD + (CD ? 12 : 4) * u);
 #pragma unroll
-                  for (int w4 = 0; w4 < 3; ++w4) dj[w4] = __ldg(dr + 4 * w4);
+                  for (int w4 = 0; w4 < 3; ++w4) dj[w4] = __ldg(dr + (CD ? 1 : 4) * w4);
                 }
                 float w[TA];
                 float wn2 = 0.f;
@@ -516,8 +537,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
                 const float ell = sqrtf(ell2);
                 const float iell = 1.f / ell;
 #pragma unroll
-                for (int m = 0; m < T; ++m) LS(T, m) = w[m];
-                IDG(T) = iell;  // the diagonal holds 1 / L(t, t)
+                for (int m = 0; m < T; ++m)
+                  if constexpr (!LAST) LS(T, m) = w[m];
+                if constexpr (!LAST) IDG(T) = iell;  // the diagonal holds 1 / L(t, t)
                 float bp = 0.f;
 #pragma unroll
                 for (int w4 = 0; w4 < 3; ++w4) {
@@ -526,23 +548,33 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
                   bp = fmaf(dj[w4].z, x[4 * w4 + 2], bp);
                   bp = fmaf(dj[w4].w, x[4 * w4 + 3], bp);
                 }
-                float yv[TA];
+                float yv[REG ? TA : 1];
+                if constexpr (REG) {
 #pragma unroll
-                for (int m = 0; m < T; ++m) yv[m] = ys[m * TILE_M + R2];
+                  for (int m = 0; m < T; ++m) yv[m] = ys[m * TILE_M + R2];
+                }
+                auto y_at = [&](int m) -> float {
+                  if constexpr (REG) return yv[m];
+                  else return ys[m * TILE_M + R2];
+                };
+                auto w_at = [&](int m) -> float {
+                  if constexpr (REG || LAST) return w[m];
+                  else return LS(T, m);
+                };
                 float yt = quad_sum(bp);
 #pragma unroll
-                for (int m = 0; m < T; ++m) yt = fmaf(-w[m], yv[m], yt);
+                for (int m = 0; m < T; ++m) yt = fmaf(-w_at(m), y_at(m), yt);
                 yt *= iell;
-                ys[T * TILE_M + R2] = yt;
-                sel[T * TILE_M + R2] = js;
+                if constexpr (!LAST) ys[T * TILE_M + R2] = yt;
+                sel[T * TILE_M + R2] = static_cast<SelT>(js);
                 const float gt = yt * iell;
                 float gam[TA];
 #pragma unroll
                 for (int m = T - 1; m >= 0; --m) {
-                  float acc = yv[m];
+                  float acc = y_at(m);
 #pragma unroll
                   for (int q = m + 1; q < T; ++q) acc = fmaf(-LS(q, m), gam[q], acc);
-                  acc = fmaf(-w[m], gt, acc);
+                  acc = fmaf(-w_at(m), gt, acc);
                   gam[m] = acc * IDG(m);
                 }
                 // the row's coefficients so far (sub-lane u writes slots u, u+4)
@@ -563,10 +595,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
 #pragma unroll
                   for (int mm = 0; mm < 4; ++mm)
                     if (m0 + mm < T) {
+                      const int sm = REG ? sl[m0 + mm] : static_cast<int>(sel[(m0 + mm) * TILE_M + R2]);
                       const float4* da =
-                          reinterpret_cast<const float4*>(a.D32p + static_cast<size_t>(sl[m0 + mm]) * DPAD + 4 * u);
+                          reinterpret_cast<const float4*>(a.D32p + static_cast<size_t>(sm) * DPAD + (CD ? 12 : 4) * u);
 #pragma unroll
-                      for (int w4 = 0; w4 < 3; ++w4) dv[mm][w4] = __ldg(da + 4 * w4);
+                      for (int w4 = 0; w4 < 3; ++w4) dv[mm][w4] = __ldg(da + (CD ? 1 : 4) * w4);
                     }
 #pragma unroll
                   for (int mm = 0; mm < 4; ++mm)
@@ -602,8 +635,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
                   if (prof_on) pcs[3] += clock64() - W5;
                 }
               };
-              if (tcc < 8)
-                with_t<8>(tcc, step);
+              if (tcc < SM)
+                with_t<SM>(tcc, step);
               else
                 act = false;
             }
@@ -651,7 +684,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
   __syncthreads();
   if (prof_any && tid == 0) {
     for (int q = 0; q < 11; ++q) atomicAdd(a.prof + q, pcs[q]);
-    if (blockIdx.x == 0) a.prof[11] = F16 ? (NSL == 3 ? 6 : 5) : 4;  // the variant that ran
+    if (blockIdx.x == 0) a.prof[11] = SM > 8 ? 7 : (F16 ? (NSL == 3 ? 6 : 5) : 4);  // the variant that ran
   }
   if (warp == 0) {
     tc_fence_after();
