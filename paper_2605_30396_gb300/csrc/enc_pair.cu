@@ -1,4 +1,5 @@
-// The two-tile encoder kernels on two warp groups (FP32, BF16, FP8).
+// The two-tile encoder kernels of 64-atom chunks: FP32 on two warp groups,
+// BF16 and FP8 on selection and solver warps.
 #include "encode_core.cuh"
 
 namespace dlsh {

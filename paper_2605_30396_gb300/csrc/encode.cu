@@ -279,8 +279,8 @@ static void cap_ring(enc::Plan& p, int cap) {
 
 // The built-in encoder choice among the kernels whose plans fit: 5 (FP32 on
 // selection and solver warps, FP16 parts), else 7 (FP32, one tile, FP16
-// parts), else 3 (FP32, two tiles in turn), else 2 (BF16/FP8 on two warp
-// groups), else 0 (one tile; the chunk width from choose_bn).
+// parts), else 3 (FP32, two tiles in turn), else 2 (BF16/FP8 on
+// selection and solver warps), else 0 (one tile; the chunk width from choose_bn).
 static int default_variant(bool split16_ok, bool alt_ok, bool pair_lowp_ok, bool one16_ok) {
   return split16_ok ? 5 : (one16_ok ? 7 : (alt_ok ? 3 : (pair_lowp_ok ? 2 : 0)));
 }
@@ -291,7 +291,8 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
                    cudaStream_t st, uint32_t** status_out, unsigned long long* prof,
                    const long long* n_dev, int bn) {
   using namespace enc;
-  // kernel variant (s <= 8): 2 = two tiles in flight on two warp groups,
+  // kernel variant (s <= 8): 2 = two tiles in flight (FP32 on two warp
+  // groups, BF16/FP8 on selection and solver warps),
   // 3 = two tiles served in turn by all warps (FP32), 4 / 5 = two tiles with
   // the warps split into selection and solver groups (FP32 as three TF32 / three
   // FP16 products), 6 = the same with three tiles and FP16 products, 7 = one
@@ -312,7 +313,7 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
   Plan p16;
   const bool one16_ok = prec == 0 && make_plan(K, s, prec, p16, 128, SMEM_LIMIT, true) == DLSH_OK;
   // default (measured at N = 3M, K = 1024): BF16/FP8, bound by selection and
-  // solver, on two warp groups (1.2-1.3x faster than one tile); FP32 on
+  // solver, on selection and solver warps (1.3x faster than one tile); FP32 on
   // selection and solver warps with three FP16 products (1.9x faster than one
   // tile at s = 8)
   if (choice == 0) choice = default_variant(split16_ok, alt_ok, pair_ok && pp.prec != 0, one16_ok);
@@ -417,9 +418,10 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
     const int ntiles = static_cast<int>((N + TILE_M - 1) / TILE_M);
     int sms = device_sm_count();
     if (sms <= 0) sms = 1;
-    // two tiles per CTA: enough CTAs for every SM, fewer when the tiles run out
-    // (a count read on the device takes every SM)
-    const int grid = (!n_dev && (ntiles + 1) / 2 < sms) ? ((ntiles + 1) / 2 > 0 ? (ntiles + 1) / 2 : 1) : sms;
+    // two tiles in flight per CTA; a tile of its own for each SM while they last
+    // (FP32's two warp groups are made for two tiles: half as many CTAs)
+    const int want = pp.prec == 0 ? (ntiles + 1) / 2 : ntiles;
+    const int grid = (!n_dev && want < sms) ? (want > 0 ? want : 1) : sms;
     if (pp.prec == 0) return launch_pair<0, false>(a, grid, st);
     if (pp.prec == 1) return pp.top4 ? launch_pair<1, true>(a, grid, st) : launch_pair<1, false>(a, grid, st);
     return pp.top4 ? launch_pair<2, true>(a, grid, st) : launch_pair<2, false>(a, grid, st);

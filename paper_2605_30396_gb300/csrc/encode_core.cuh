@@ -1165,6 +1165,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_kernel(const __grid_consta
 #include "encode_pair.cuh"
 #include "encode_alt.cuh"
 #include "encode_split.cuh"
+#include "encode_lowp.cuh"
 
 template <int PREC, int BN, bool T4 = false>
 int launch_encode(const Args& a, int grid, cudaStream_t st) {
@@ -1180,7 +1181,9 @@ int launch_encode(const Args& a, int grid, cudaStream_t st) {
 
 template <int PREC, bool T4>
 int launch_pair(const PairArgs& a, int grid, cudaStream_t st) {
-  auto fn = encode_pair_kernel<PREC, T4>;
+  void (*fn)(const PairArgs) = nullptr;
+  if constexpr (PREC == 0) fn = encode_pair_kernel<PREC>;
+  else fn = encode_lowp_kernel<PREC, T4>;
   DLSH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT),
                 "dlsh_encode: cudaFuncSetAttribute");
   fn<<<grid, NTHREADS, a.p.smem, st>>>(a);
