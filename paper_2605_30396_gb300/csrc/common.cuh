@@ -389,6 +389,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
 }
 
+// c + a b with FP16 a and b (the low 16 bits given) and FP32 c, one rounding: the
+// value of fmaf on the converted operands, without the conversions.
+__device__ __forceinline__ float fma_f16(uint32_t a, uint32_t b, float c) {
+  float d;
+  asm("{\n\t.reg .b16 x, y;\n\tcvt.u16.u32 x, %1;\n\tcvt.u16.u32 y, %2;\n\tfma.rn.f32.f16 %0, x, y, %3;\n\t}"
+      : "=f"(d)
+      : "r"(a), "r"(b), "f"(c));
+  return d;
+}
+
 // ---- number conversions ----------------------------------------------------
 __device__ __forceinline__ float to_tf32(float x) {
   uint32_t r;

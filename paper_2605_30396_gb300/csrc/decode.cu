@@ -27,6 +27,7 @@
 #include <math.h>
 #include <stdio.h>
 
+#include "codes.cuh"
 #include "common.cuh"
 #include "host.hpp"
 #include "sh.cuh"
@@ -124,6 +125,8 @@ __global__ void __launch_bounds__(1024) decode_kernel(
   const int ql = lane & 7, grp = lane >> 3;
   const int64_t nbatch = (N + GB - 1) / GB;
   const int64_t wstride = static_cast<int64_t>(gridDim.x) * nwarps;
+  // batches of 16 fill the lanes with groups of four slots
+  const bool quads = GB == 16 && codes_in_quads<FM == FM_C8, FM >= FM_C8>(idxv, coefv, s);
   bool bad = false;
   for (int64_t bt = static_cast<int64_t>(blockIdx.x) * nwarps + warp; bt < nbatch; bt += wstride) {
     const int64_t base = bt * GB;
@@ -140,6 +143,9 @@ __global__ void __launch_bounds__(1024) decode_kernel(
     }
     // ---- phase A: the batch's codes as (index, coefficient) pairs, element
     // f = lane + 32 k (k < s/2 rounded up), four loads in flight per lane
+    if (quads) {
+      bad |= stage_quads<FM == FM_C8, FM >= FM_C8>(idxv, coefv, base * s, nb * s, s, sp, sdiv, K, cpk);
+    } else
     for (int k0 = 0; 32 * k0 < GB * s; k0 += 4) {
       uint32_t jj[4];
       float aa[4];
@@ -156,7 +162,7 @@ __global__ void __launch_bounds__(1024) decode_kernel(
           } else {
             jj[u] = FM == FM_C8 ? static_cast<uint32_t>(static_cast<const uint8_t*>(idxv)[e])
                                 : static_cast<uint32_t>(static_cast<const uint16_t*>(idxv)[e]);
-            aa[u] = __half2float(static_cast<const __half*>(coefv)[e]);
+            aa[u] = __uint_as_float(static_cast<const uint16_t*>(coefv)[e]);  // FP16 bits
           }
         }
       }
@@ -288,16 +294,13 @@ __global__ void __launch_bounds__(1024) decode_kernel(
             }
           } else {
             const uint4 w = reinterpret_cast<const uint4*>(sm)[jt[u] * 8 + ql];
-            const float2 rg = __half22float2(*reinterpret_cast<const __half2*>(&w.x));
-            const float2 bz = __half22float2(*reinterpret_cast<const __half2*>(&w.y));
-            const float2 rh = __half22float2(*reinterpret_cast<const __half2*>(&w.z));
-            const float2 bh = __half22float2(*reinterpret_cast<const __half2*>(&w.w));
-            aR = fmaf(a, rg.x, aR);
-            aG = fmaf(a, rg.y, aG);
-            aB = fmaf(a, bz.x, aB);
-            bR = fmaf(a, rh.x, bR);
-            bG = fmaf(a, rh.y, bG);
-            bBl = fmaf(a, bh.x, bBl);
+            const uint32_t h = __float_as_uint(a);  // the coefficient's FP16 bits
+            aR = fma_f16(h, w.x, aR);
+            aG = fma_f16(h, w.x >> 16, aG);
+            aB = fma_f16(h, w.y, aB);
+            bR = fma_f16(h, w.z, bR);
+            bG = fma_f16(h, w.z >> 16, bG);
+            bBl = fma_f16(h, w.w, bBl);
           }
         }
       }
@@ -373,6 +376,7 @@ __global__ void __launch_bounds__(1024) decode_channel_kernel(
   const int q = lane & 3, grp = lane >> 2;
   const int64_t nbatch = (N + PGB - 1) / PGB;
   const int64_t wstride = static_cast<int64_t>(gridDim.x) * nwarps;
+  const bool quads = PGB == 16 && codes_in_quads<false, false>(idx, coef, s);
   bool bad = false;
   for (int64_t bt = static_cast<int64_t>(blockIdx.x) * nwarps + warp; bt < nbatch; bt += wstride) {
     const int64_t base = bt * PGB;
@@ -387,6 +391,9 @@ __global__ void __launch_bounds__(1024) decode_channel_kernel(
       nz = nnz[g];
     }
     // ---- the batch's codes as (row offset, coefficient) pairs
+    if (quads) {
+      bad |= stage_quads<false, false, 16>(idx, coef, base * s, nb * s, s, sp, sdiv, K, cpk);
+    } else
     for (int k0 = 0; 32 * k0 < PGB * s; k0 += 8) {
       uint32_t jj[8];
       float aa[8];

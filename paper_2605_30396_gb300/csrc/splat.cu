@@ -32,6 +32,7 @@
 #include <cuda_fp16.h>
 #include <math.h>
 
+#include "codes.cuh"
 #include "common.cuh"
 #include "host.hpp"
 #include "sh.cuh"
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(1024) preprocess_kernel(const __grid_constant_
   const int64_t N = p.N;
   const int64_t nbatch = (N + GB - 1) / GB;
   const int64_t wstride = static_cast<int64_t>(gridDim.x) * nwarps;
+  const bool quads = CM != CM_SH && codes_in_quads<CM == CM_C8, CM != CM_F32>(p.idx, p.coef, s);
   for (int64_t bt = static_cast<int64_t>(blockIdx.x) * nwarps + warp; bt < nbatch; bt += wstride) {
     const int64_t base = bt * GB;
     const int nb = N - base < GB ? static_cast<int>(N - base) : GB;
@@ -179,6 +181,9 @@ __global__ void __launch_bounds__(1024) preprocess_kernel(const __grid_constant_
     }
     // codes of the whole batch, staged as (index, coefficient bits) pairs
     if (CM != CM_SH) {
+      if (quads) {
+        stage_quads<CM == CM_C8, CM != CM_F32>(p.idx, p.coef, base * s, nb * s, s, sp, p.sdiv, K, cpk);
+      } else
       // element f = lane + 32 k of the batch (k < s); four loads in flight per lane
       for (int k0 = 0; k0 < s; k0 += 4) {
         uint32_t jj[4];
@@ -196,7 +201,7 @@ __global__ void __launch_bounds__(1024) preprocess_kernel(const __grid_constant_
             } else {
               jj[u] = CM == CM_C8 ? static_cast<uint32_t>(static_cast<const uint8_t*>(p.idx)[e])
                                   : static_cast<uint32_t>(static_cast<const uint16_t*>(p.idx)[e]);
-              aa[u] = __half2float(static_cast<const __half*>(p.coef)[e]);
+              aa[u] = __uint_as_float(static_cast<const uint16_t*>(p.coef)[e]);  // FP16 bits
             }
           }
         }
@@ -382,26 +387,19 @@ __global__ void __launch_bounds__(1024) preprocess_kernel(const __grid_constant_
             // (R, G) and (B, 0) of basis 2ql, then of basis 2ql + 1
             const uint4* D4 = reinterpret_cast<const uint4*>(sm);
             const uint4 w0 = D4[j0 * 8 + ql], w1 = D4[j1 * 8 + ql];
-            const float2 rg0 = __half22float2(*reinterpret_cast<const __half2*>(&w0.x));
-            const float2 bz0 = __half22float2(*reinterpret_cast<const __half2*>(&w0.y));
-            const float2 rh0 = __half22float2(*reinterpret_cast<const __half2*>(&w0.z));
-            const float2 bh0 = __half22float2(*reinterpret_cast<const __half2*>(&w0.w));
-            const float2 rg1 = __half22float2(*reinterpret_cast<const __half2*>(&w1.x));
-            const float2 bz1 = __half22float2(*reinterpret_cast<const __half2*>(&w1.y));
-            const float2 rh1 = __half22float2(*reinterpret_cast<const __half2*>(&w1.z));
-            const float2 bh1 = __half22float2(*reinterpret_cast<const __half2*>(&w1.w));
-            aR = fmaf(a0, rg0.x, aR);
-            aG = fmaf(a0, rg0.y, aG);
-            aB = fmaf(a0, bz0.x, aB);
-            bR = fmaf(a0, rh0.x, bR);
-            bG = fmaf(a0, rh0.y, bG);
-            bBl = fmaf(a0, bh0.x, bBl);
-            aR = fmaf(a1, rg1.x, aR);
-            aG = fmaf(a1, rg1.y, aG);
-            aB = fmaf(a1, bz1.x, aB);
-            bR = fmaf(a1, rh1.x, bR);
-            bG = fmaf(a1, rh1.y, bG);
-            bBl = fmaf(a1, bh1.x, bBl);
+            const uint32_t h0 = c2.y, h1 = c2.w;  // the coefficients' FP16 bits
+            aR = fma_f16(h0, w0.x, aR);
+            aG = fma_f16(h0, w0.x >> 16, aG);
+            aB = fma_f16(h0, w0.y, aB);
+            bR = fma_f16(h0, w0.z, bR);
+            bG = fma_f16(h0, w0.z >> 16, bG);
+            bBl = fma_f16(h0, w0.w, bBl);
+            aR = fma_f16(h1, w1.x, aR);
+            aG = fma_f16(h1, w1.x >> 16, aG);
+            aB = fma_f16(h1, w1.y, aB);
+            bR = fma_f16(h1, w1.z, bR);
+            bG = fma_f16(h1, w1.z >> 16, bG);
+            bBl = fma_f16(h1, w1.w, bBl);
           }
         }
         const float yA = Ys[gl * YS + bA], yB = Ys[gl * YS + bB];
