@@ -22,6 +22,17 @@ __device__ __forceinline__ void flag_status(uint32_t* status, uint32_t bits) {
   if (status) atomicOr(status, bits);
 }
 
+// ---- programmatic dependent launch -------------------------------------------
+// A kernel launched by launch_dependent (host.hpp) may start while the kernel
+// before it in the stream still runs.  depend() lets the next kernel start as
+// soon as every CTA of this one has, then waits until the kernels before this
+// one are complete and their writes visible: it comes before the first access
+// to global memory.
+__device__ __forceinline__ void depend() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---- shared-memory addresses -------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));

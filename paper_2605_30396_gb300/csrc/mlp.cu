@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
     tmem_alloc(tslot, GN);
     tmem_relinquish();
   }
+  depend();  // nothing above touches global memory
   constexpr uint32_t idesc =
       umma_idesc(1, 1, GM, GN) | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u);  // bits 15, 16: MN-major
   if (XA) {
@@ -410,6 +411,7 @@ struct ReduceArgs {
 
 template <bool ADAM>
 __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ ReduceArgs a) {
+  depend();
   if (blockIdx.x == gridDim.x - 1) {  // the last block: the mean loss, a fixed-order sum
     __shared__ double red[256];
     double acc = 0.0;
@@ -585,7 +587,7 @@ static int launch_gemm_ns(const GemmArgs& g, int tiles, int splits, cudaStream_t
     return DLSH_OK;
   });
   if (arc) return arc;
-  train_gemm_kernel<EPI, AMN, BMN, XA, NS><<<dim3(tiles, splits), GT, gemm_smem(NS), st>>>(g);
+  launch_dependent(train_gemm_kernel<EPI, AMN, BMN, XA, NS>, dim3(tiles, splits), GT, gemm_smem(NS), st, g);
   count_launches(1);
   return check_launch("dlsh_mlp: gemm");
 }
@@ -724,7 +726,7 @@ static int gradients(Plan& t, int K, const float* X, long long B, const uint16_t
   if (rc) return rc;
   ReduceArgs a = reduce_args(K, B, w, loss);
   a.G = grads;
-  reduce_kernel<false><<<static_cast<int>((a.L.n + 255) / 256) + 1, 256, 0, st>>>(a);
+  launch_dependent(reduce_kernel<false>, static_cast<int>((a.L.n + 255) / 256) + 1, 256, 0, st, a);
   count_launches(1);
   return check_launch("dlsh_mlp: reduce");
 }
@@ -742,7 +744,7 @@ static int train_step(Plan& t, const Blob& b, int K, const float* X, long long B
   a.eps = 1e-8f;
   a.bc1 = static_cast<float>(1.0 - pow(0.9, static_cast<double>(step)));
   a.bc2 = static_cast<float>(1.0 - pow(0.999, static_cast<double>(step)));
-  reduce_kernel<true><<<static_cast<int>((a.L.n + 255) / 256) + 1, 256, 0, st>>>(a);
+  launch_dependent(reduce_kernel<true>, static_cast<int>((a.L.n + 255) / 256) + 1, 256, 0, st, a);
   count_launches(1);
   return check_launch("dlsh_mlp: adam");
 }

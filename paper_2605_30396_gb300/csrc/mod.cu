@@ -235,6 +235,7 @@ __device__ __forceinline__ bool any_shared(T* place, bool active, T tag) {
 __global__ void __launch_bounds__(256) count_kernel(const uint16_t* __restrict__ idx, const uint8_t* __restrict__ nnz,
                                                    int s, uint32_t sdiv, int64_t N, int K, int ts,
                                                    int* __restrict__ cnt, uint32_t* status) {
+  depend();
   extern __shared__ unsigned hist[];  // [(K + 1) / 2]
   const int nw = (K + 1) / 2;
   for (int j = threadIdx.x; j < nw; j += blockDim.x) hist[j] = 0;
@@ -307,6 +308,7 @@ __device__ __forceinline__ int block_scan(int v, int* sm, int& total) {
 
 __global__ void __launch_bounds__(256) chunk_sum_kernel(const int* __restrict__ cnt, int T, int K, int segb,
                                                        int* __restrict__ csum, int* __restrict__ segtot) {
+  depend();
   __shared__ int sm[32];
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int t0 = blockIdx.y * CH, t1 = t0 + CH < T ? t0 + CH : T;
@@ -324,6 +326,7 @@ __global__ void __launch_bounds__(256) chunk_sum_kernel(const int* __restrict__ 
 __global__ void __launch_bounds__(1024) layout_kernel(const int* __restrict__ csum, int P, int K, int gc, int PG,
                                                       int nseg, int* __restrict__ segtot, int* __restrict__ atom_start,
                                                       int* __restrict__ segg_start, int* __restrict__ segb_end) {
+  depend();
   __shared__ int sm[32];
   int carry = 0;
   for (int base = 0; base < K; base += 1024) {
@@ -377,6 +380,7 @@ __global__ void __launch_bounds__(256) tile_offsets_kernel(int* __restrict__ cnt
                                                           const int* __restrict__ csum, const int* __restrict__ segtot,
                                                           const int* __restrict__ atom_start, int* __restrict__ cstart,
                                                           int* __restrict__ segb_start) {
+  depend();
   __shared__ int sm[32];
   const int j = blockIdx.x * blockDim.x + threadIdx.x, p = blockIdx.y;
   const int n = j < K ? csum[static_cast<size_t>(p) * K + j] : 0;
@@ -422,6 +426,7 @@ __global__ void __launch_bounds__(512) scatter_kernel(const uint16_t* __restrict
                                                       const uint8_t* __restrict__ nnz, int s, uint32_t sdiv, int64_t N,
                                                       int K, int ts, const int* __restrict__ off,
                                                       uint2* __restrict__ list) {
+  depend();
   extern __shared__ __align__(16) uint8_t scb[];
   const int ncap = ts * s;
   const int kp = (K + 1) / 2 * 2;
@@ -565,6 +570,7 @@ __global__ void __launch_bounds__(256, 4) accum_b_kernel(const float* __restrict
                                                         const int* __restrict__ atom_start,
                                                         const int* __restrict__ segb_start, int segb,
                                                         const uint2* __restrict__ list, double* __restrict__ Bp) {
+  depend();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
   const int seg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -647,6 +653,7 @@ __global__ void __launch_bounds__(128) accum_g_kernel(const uint16_t* __restrict
                                                      const int* __restrict__ cstart, const int* __restrict__ atom_start,
                                                      const int* __restrict__ segg_start,
                                                      const uint2* __restrict__ list, double* __restrict__ Gp) {
+  depend();
   extern __shared__ __align__(16) float2 grow[];  // [warps][K] (hi, lo)
   const int seg = blockIdx.x;
   if (seg >= segg_start[PG * K]) return;
@@ -774,6 +781,7 @@ __global__ void __launch_bounds__(256) seg_reduce_kernel(const int* __restrict__
                                                         const double* __restrict__ Gp, const double* __restrict__ Bp,
                                                         int K, int P, int PG, double* __restrict__ M,
                                                         double* __restrict__ Z) {
+  depend();
   const int j = blockIdx.x;
   for (int k = j + threadIdx.x; k < K; k += blockDim.x) {
     double acc = 0.0;
@@ -815,6 +823,7 @@ static int accum_warps(int K, size_t* smem) {
 // ---- 5a. lambda = 1e-6 trace(G)/K and the Jacobi scale 1 / sqrt(M_jj + lambda) ----
 __global__ void __launch_bounds__(1024) ridge_kernel(const double* __restrict__ M, int K, double* lam_out,
                                                      double* __restrict__ dsc) {
+  depend();
   __shared__ double part[1024];
   double acc = 0.0;
   for (int j = threadIdx.x; j < K; j += blockDim.x) acc += M[static_cast<size_t>(j) * K + j];
@@ -847,6 +856,7 @@ __global__ void __launch_bounds__(MT * 8) scale_kernel(const double* __restrict_
                                                        const double* __restrict__ dsc, int K, float2* __restrict__ S,
                                                        float* __restrict__ A, float2* __restrict__ Zs,
                                                        float* __restrict__ R32, float2* __restrict__ Xs) {
+  depend();
   __shared__ float2 t[MT][MT + 1];
   const int rb = blockIdx.y, cb = blockIdx.x;  // tile: rows rb, columns cb >= rb
   if (cb < rb) return;
@@ -1168,6 +1178,7 @@ constexpr int PS = PKC + 4;        // row stride of the stage: the rows start on
 template <bool TRANS>
 __global__ void __launch_bounds__(PT) trmm_kernel(const float* __restrict__ W, int K, const float* __restrict__ in,
                                                   float* __restrict__ out, float2* __restrict__ Xs) {
+  depend();
   extern __shared__ __align__(16) float psm[];  // [PR][PS], then the warps' sums
   const int j0 = blockIdx.x * PR;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1224,6 +1235,7 @@ __global__ void __launch_bounds__(PT) trmm_kernel(const float* __restrict__ W, i
 __global__ void __launch_bounds__(PT) residual_kernel(const float2* __restrict__ S, int K,
                                                       const float2* __restrict__ Zs, const float2* __restrict__ Xs,
                                                       float* __restrict__ R32) {
+  depend();
   extern __shared__ __align__(16) float2 rsm[];  // [PR][PS], then the warps' sums
   const int j0 = blockIdx.x * PR;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1282,6 +1294,7 @@ __global__ void normalise_kernel(const float2* __restrict__ Xs, const double* __
                                  const int* __restrict__ atom_start,
                                  int K, float* __restrict__ D_new, const float* __restrict__ D_old,
                                  int* __restrict__ dead) {
+  depend();
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (j >= K) return;
@@ -1308,6 +1321,7 @@ __global__ void normalise_kernel(const float2* __restrict__ Xs, const double* __
 __global__ void __launch_bounds__(1024)
     refill_kernel(const float* __restrict__ X, const float* __restrict__ resid, int64_t N, int K,
                   const int* __restrict__ dead, float* __restrict__ D_new) {
+  depend();
   __shared__ float bv[1024];
   __shared__ long long bi[1024];
   __shared__ int dl[MAX_K];   // the dead atoms, increasing
@@ -1454,6 +1468,7 @@ __global__ void __launch_bounds__(256) ksvd_resid_kernel(const float* __restrict
                                                          const float* __restrict__ coef,
                                                          const uint8_t* __restrict__ nnz, int s, int64_t N,
                                                          float* __restrict__ R) {
+  depend();
   const int lane = threadIdx.x & 31;
   const int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= N) return;
@@ -1723,23 +1738,25 @@ template <bool SLOT>
 static int sort_enqueue(const uint16_t* idx, const float* coef, const uint8_t* nnz, int s, int64_t N, int K,
                         const Sort& so, uint32_t* status, cudaStream_t st, const char* call) {
   if (N > 0) {
-    count_kernel<<<so.T, 256, (K + 1) / 2 * sizeof(unsigned), st>>>(idx, nnz, s, so.sdiv, N, K, so.ts, so.cnt, status);
+    launch_dependent(count_kernel, so.T, 256, (K + 1) / 2 * sizeof(unsigned), st, idx, nnz, s, so.sdiv, N, K, so.ts,
+                     so.cnt, status);
   } else {
     DLSH_CUDA_TRY(cudaMemsetAsync(so.cnt, 0, sizeof(int) * K * so.T, st), call);
   }
   const dim3 g((K + 255) / 256, so.P);
-  chunk_sum_kernel<<<g, 256, 0, st>>>(so.cnt, so.T, K, so.segb, so.csum, so.segtot);
-  layout_kernel<<<1, 1024, 0, st>>>(so.csum, so.P, K, so.gc, so.PG, static_cast<int>(g.x * g.y), so.segtot, so.atom_start,
-                                    so.segg_start, so.segb_start + static_cast<size_t>(so.P) * K);
-  tile_offsets_kernel<<<g, 256, 0, st>>>(so.cnt, so.T, K, so.segb, so.csum, so.segtot, so.atom_start, so.cstart,
-                                         so.segb_start);
+  launch_dependent(chunk_sum_kernel, g, 256, 0, st, so.cnt, so.T, K, so.segb, so.csum, so.segtot);
+  launch_dependent(layout_kernel, 1, 1024, 0, st, so.csum, so.P, K, so.gc, so.PG, static_cast<int>(g.x * g.y),
+                   so.segtot, so.atom_start, so.segg_start, so.segb_start + static_cast<size_t>(so.P) * K);
+  launch_dependent(tile_offsets_kernel, g, 256, 0, st, so.cnt, so.T, K, so.segb, so.csum, so.segtot, so.atom_start,
+                   so.cstart, so.segb_start);
   count_launches((N > 0 ? 1 : 0) + 3);
   if (N > 0) {
     const size_t smem = scatter_smem(K, s, so.ts, so.threads);
     DLSH_CUDA_TRY(cudaFuncSetAttribute(scatter_kernel<SLOT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        SMEM_LIMIT - 512),
                   call);
-    scatter_kernel<SLOT><<<so.T, so.threads, smem, st>>>(idx, coef, nnz, s, so.sdiv, N, K, so.ts, so.cnt, so.list);
+    launch_dependent(scatter_kernel<SLOT>, so.T, so.threads, smem, st, idx, coef, nnz, s, so.sdiv, N, K, so.ts,
+                     so.cnt, so.list);
     count_launches(1);
   }
   return check_launch(call);
@@ -1768,8 +1785,11 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
   if (src) return src;
   {
     const int64_t nb = (max_segb(so, K, s, N) + 7) / 8;
-    accum_b_kernel<<<static_cast<int>(nb > 0 ? nb : 1), 256, 0, st>>>(X, K, so.P, so.cstart, so.atom_start, so.segb_start,
-                                                                      so.segb, so.list, w.Bp);
+    // (launched normally: started early, these two lose more than a launch. With
+    // accum_b beside the scatter's last CTAs the update of 3M signals takes 2360 us
+    // instead of 2040, with accum_g beside accum_b that of 10,000 220 instead of 201)
+    accum_b_kernel<<<static_cast<int>(nb > 0 ? nb : 1), 256, 0, st>>>(X, K, so.P, so.cstart, so.atom_start,
+                                                                      so.segb_start, so.segb, so.list, w.Bp);
     void (*accum)(const uint16_t*, const float*, int, int, int, int, int, const int*, const int*, const int*,
                   const uint2*, double*) =
         s <= 8 ? accum_g_kernel<1> : (s <= 16 ? accum_g_kernel<2> : accum_g_kernel<4>);
@@ -1778,13 +1798,15 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
     accum<<<static_cast<int>(max_segg(w.so, K, s, N)), acc_nw * 32, acc_smem, st>>>(
         idx, coef, s, K, so.P, so.gc, so.PG, so.cstart, so.atom_start, so.segg_start, so.list, w.Gp);
   }
-  seg_reduce_kernel<<<K, 256, 0, st>>>(so.segg_start, so.segb_start, w.Gp, w.Bp, K, so.P, so.PG, w.M, w.Z);
-  ridge_kernel<<<1, 1024, 0, st>>>(w.M, K, w.lam, w.dsc);
+  launch_dependent(seg_reduce_kernel, K, 256, 0, st, so.segg_start, so.segb_start, w.Gp, w.Bp, K, so.P, so.PG, w.M,
+                   w.Z);
+  launch_dependent(ridge_kernel, 1, 1024, 0, st, w.M, K, w.lam, w.dsc);
   // mixed-precision solve: FP32 Cholesky of the Jacobi-scaled matrix, then
   // kRefine FP32 solves with float-float residuals in between
   {
     const int nb = (K + MT - 1) / MT;
-    scale_kernel<<<dim3(nb, nb), MT * 8, 0, st>>>(w.M, w.Z, D_old, w.lam, w.dsc, K, w.S, w.A32, w.Zs, w.R32, w.Xs);
+    launch_dependent(scale_kernel, dim3(nb, nb), MT * 8, 0, st, w.M, w.Z, D_old, w.lam, w.dsc, K, w.S, w.A32, w.Zs,
+                     w.R32, w.Xs);
   }
   launches += 5;
   {
@@ -1821,17 +1843,17 @@ int mod_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, const flo
   const int rows = (K + PR - 1) / PR;
   for (int it = 0; it < kRefine; ++it) {
     if (it > 0) {
-      residual_kernel<<<rows, PT, PSM64, st>>>(w.S, K, w.Zs, w.Xs, w.R32);
+      launch_dependent(residual_kernel, rows, PT, PSM64, st, w.S, K, w.Zs, w.Xs, w.R32);
       ++launches;
     }
-    trmm_kernel<false><<<rows, PT, PSM32, st>>>(w.W32, K, w.R32, w.Y32, nullptr);
-    trmm_kernel<true><<<rows, PT, PSM32, st>>>(w.W32, K, w.Y32, nullptr, w.Xs);
+    launch_dependent(trmm_kernel<false>, rows, PT, PSM32, st, w.W32, K, w.R32, w.Y32, nullptr);
+    launch_dependent(trmm_kernel<true>, rows, PT, PSM32, st, w.W32, K, w.Y32, nullptr, w.Xs);
     launches += 2;
   }
-  normalise_kernel<<<(K + 7) / 8, 256, 0, st>>>(w.Xs, w.dsc, so.atom_start, K, D_new, D_old, w.dead);
+  launch_dependent(normalise_kernel, (K + 7) / 8, 256, 0, st, w.Xs, w.dsc, so.atom_start, K, D_new, D_old, w.dead);
   ++launches;
   if (resid && N > 0) {
-    refill_kernel<<<1, 1024, 0, st>>>(X, resid, N, K, w.dead, D_new);
+    launch_dependent(refill_kernel, 1, 1024, 0, st, X, resid, N, K, w.dead, D_new);
     ++launches;
   }
   count_launches(launches);
@@ -1858,7 +1880,8 @@ int ksvd_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, float* c
   const int src = sort_enqueue<true>(idx, coef, nnz, s, N, K, w.so, w.status, st, "dlsh_ksvd_update: sort");
   if (src) return src;
   if (N > 0) {
-    ksvd_resid_kernel<<<static_cast<int>((N + 7) / 8), 256, 0, st>>>(X, D_old, K, idx, coef, nnz, s, N, w.R);
+    launch_dependent(ksvd_resid_kernel, static_cast<int>((N + 7) / 8), 256, 0, st, X, D_old, K, idx, coef, nnz, s, N,
+                     w.R);
     launches += 1;
   }
   {
@@ -1897,7 +1920,7 @@ int ksvd_enqueue(const float* X, int64_t N, int K, const uint16_t* idx, float* c
     ++launches;
   }
   if (resid && N > 0) {
-    refill_kernel<<<1, 1024, 0, st>>>(X, resid, N, K, w.dead, D_new);
+    launch_dependent(refill_kernel, 1, 1024, 0, st, X, resid, N, K, w.dead, D_new);
     ++launches;
   }
   count_launches(launches);
