@@ -187,6 +187,25 @@ def test_fused_propose_ties_and_many_tiles(lib):
     assert both.any()
 
 
+@pytest.mark.parametrize("K,N,m", [(1024, 300, 2), (1024, 300, 16), (1000, 513, 32), (512, 128, 8), (128, 257, 16),
+                                   (2048, 200, 32)])
+def test_fused_propose_full_queues(lib, K, N, m):
+    """Rows whose candidates crowd into the columns of one thread (the queue
+    holds 21 or 30: the rest goes through the thread's list) and rows that tie
+    throughout (zero signals under zero biases).  The candidates are the top m of
+    the forward pass's logits exactly, ties to the smaller index."""
+    p = _params(K, 60 + K)
+    crowd = np.isin(np.arange(K) % 64, [5, 6, 7, 8])
+    p["W3"] = np.where(crowd[:, None], 8.0 * p["W3"], p["W3"])
+    X = synth.signals(N, synth.hidden_dictionary(K, 61), 4, 62)
+    X[::9] = 0.0
+    for bias in (p["b3"], np.zeros(K)):
+        net = lib.MLP(K, dict(p, b3=bias))
+        z = net.forward(torch.from_numpy(X)).cpu().numpy()
+        cand = net.propose(torch.from_numpy(X), m).cpu().numpy().view(np.uint16).astype(np.int64)
+        np.testing.assert_array_equal(cand, _top_m(z, m))
+
+
 @pytest.mark.parametrize("m,s,K", [(16, 8, 256), (8, 4, 1024), (32, 16, 512), (32, 8, 32)])
 def test_restricted_omp_matches_oracle(lib, m, s, K):
     N = 2000
