@@ -209,8 +209,9 @@ int dlsh_decode(const float* D, int K, int d, const uint16_t* idx,
  * minimisation of Eq. 1), read as MOD:
  *   G = A A^T, B = X A^T, lambda = 1e-6 trace(G)/K (1e-6 if trace is 0),
  *   D~ = (B + lambda D_old)(G + lambda I)^-1, solved on the device with an FP32
- *   Cholesky factor of the Jacobi-scaled matrix and FP64 iterative refinement
- *   (G and B accumulated in float-float: about FP64 accuracy),
+ *   Cholesky factor of the Jacobi-scaled matrix and iterative refinement with
+ *   float-float residuals (G and B too are accumulated in float-float: about
+ *   FP64 accuracy),
  *   d_j = d~_j / ||d~_j||; atoms with no nonzero in A (or d~_j = 0) are
  *   refilled in increasing j with the normalised signals of largest resid_sq
  *   (decreasing order, ties to the smallest index, zero signals skipped).
@@ -453,7 +454,8 @@ int dlsh_csc_from_ell(const uint16_t* idx, const float* coef,
  * code must be distinct (as the encoder writes them).  D_new [K*d] must not
  * alias D_old.  Every sum runs in a fixed order: results are bitwise
  * reproducible.  Limits: K <= 4096, N < 2^26, N*s < 2^31.  The sweep is one
- * cooperative launch with two bounded grid barriers per used atom.
+ * cooperative launch in which the CTAs exchange partial sums per used atom; its
+ * waits are bounded.
  * Workspace: dlsh_ksvd_workspace_size(K, d, s, N) (it holds R: N*45 floats).
  */
 size_t dlsh_ksvd_workspace_size(int K, int d, int s, int64_t N);

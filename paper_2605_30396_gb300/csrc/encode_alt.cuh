@@ -2,7 +2,7 @@
 // the same sixteen warps in alternation (Sec. 2.1: OMP against the dictionary,
 // one greedy atom at a time, least-squares re-fit).
 //
-// Included by encode.cu inside namespace dlsh::enc, after encode_pair.cuh
+// Included by encode_core.cuh inside namespace dlsh::enc, after encode_pair.cuh
 // (it shares that file's staging protocol and MMA helpers).
 //
 // The warps select for tile A while the tensor pipe computes A's correlations,

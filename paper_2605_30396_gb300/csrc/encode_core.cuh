@@ -72,7 +72,7 @@ __device__ __forceinline__ void with_t(int t, F&& f) {
   }
 }
 constexpr float FP8_MAX = 448.f;
-// Operand-image code of the FP16-split FP32 format (prep_kernel): hi and lo
+// Operand-image code of the FP16-split FP32 format (prepare_kernel): hi and lo
 // FP16 parts of 256 * D, 6 K blocks of 8 elements each
 constexpr int OPF16X2 = 3;
 

@@ -3,7 +3,7 @@
 // FP32 kernel on two warp groups (3xTF32), and the plan and operand packing that
 // the BF16/FP8 kernel of encode_lowp.cuh shares.
 //
-// Included by encode.cu inside namespace dlsh::enc (it uses that file's
+// Included by encode_core.cuh inside namespace dlsh::enc (it uses that file's
 // operand packing, key networks and constants).
 //
 // Each CTA runs two groups of eight warps; group g owns its own tiles of 128

@@ -3,7 +3,7 @@
 // two or three tiles per CTA with the warps split by task (Sec. 2.1: OMP against the dictionary, one greedy atom at
 // a time, least-squares re-fit).
 //
-// Included by encode.cu inside namespace dlsh::enc, after encode_alt.cuh (it
+// Included by encode_core.cuh inside namespace dlsh::enc, after encode_alt.cuh (it
 // uses that file's dictionary producer, MMA issuer, A-operand layout and the
 // staging protocol).
 //
