@@ -285,6 +285,25 @@ static int default_variant(bool split16_ok, bool alt_ok, bool pair_lowp_ok, bool
   return split16_ok ? 5 : (one16_ok ? 7 : (alt_ok ? 3 : (pair_lowp_ok ? 2 : 0)));
 }
 
+// With 9 to 16 atoms (FP16 parts): whether two tiles per CTA on selection and
+// solver warps beat one tile per CTA on warps that do both.  Eight solver warps
+// take about twice as long over a tile as sixteen; that pays where the other
+// eight have enough chunks to select from meanwhile.  Measured, one tile / two:
+//   tiles of 64 fill no SM twice (N = 3000, s = 16): K = 98 110 / 92 us, K = 2048
+//   409 / 311: always two;
+//   tiles of 128 fill no SM twice (N = 18,000): a tile of 128 per SM competes with
+//   two of 64.  K = 256 138 / 150, K = 512 195 / 174, K = 2048 406 / 450 (s = 16),
+//   K = 1024 137 / 141 (s = 9): between 256 and 1024;
+//   more (N = 200,000): K = 256 1369 / 1485, K = 512 1939 / 1605, K = 2048 3933 / 2534
+//   (s = 16), K = 256 606 / 640, K = 512 823 / 693 (s = 9): from three chunks on.
+static bool deep_pays(int K, int s, int64_t N, const long long* n_dev) {
+  if (s <= 8) return false;
+  const int sms = device_sm_count();
+  if (!n_dev && N <= static_cast<int64_t>(64) * sms) return true;
+  if (!n_dev && N <= static_cast<int64_t>(enc::TILE_M) * sms) return K > 256 && K < 1024;
+  return K > 256;
+}
+
 // Entry points shared with the learning loop (learn.cu).
 int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, float eps, int prec,
                    uint16_t* idx, float* coef, uint8_t* nnz, float* resid_sq, void* ws,
@@ -329,7 +348,8 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
   cap_ring(sp16, cap, 2);
   cap_ring(sp16x3, cap, 2);
   SplitPlan deep;
-  const bool use_deep = choice == 7 && s > 8 && make_split_plan(K, s, prec, deep, true, 2, SMEM_LIMIT, true) == DLSH_OK;
+  const bool use_deep =
+      choice == 7 && deep_pays(K, s, N, n_dev) && make_split_plan(K, s, prec, deep, true, 2, SMEM_LIMIT, true) == DLSH_OK;
   if ((choice >= 3 && choice <= 6) || use_deep) {
     Plan p;  // the one-tile encoder's 128-atom FP32 operand image
     if (use_deep) p = p16;

@@ -1169,9 +1169,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_kernel(const __grid_consta
 
 template <int PREC, int BN, bool T4 = false>
 int launch_encode(const Args& a, int grid, cudaStream_t st) {
-  auto fn = encode_kernel<PREC, BN, 8, T4>;
-  if constexpr (PREC != OPF16X2)  // (FP16 parts with s > 8: the split kernel)
-    if (a.p.s > 8) fn = encode_kernel<PREC, BN, 16, T4>;
+  auto fn = a.p.s <= 8 ? encode_kernel<PREC, BN, 8, T4> : encode_kernel<PREC, BN, 16, T4>;
   DLSH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT),
                 "dlsh_encode: cudaFuncSetAttribute");
   fn<<<grid, NTHREADS, a.p.smem, st>>>(a);

@@ -245,13 +245,15 @@ def test_multi_tile_fp32_encoders_over_several_rounds(lib, variant):
 
 
 @pytest.mark.parametrize("K,s,prec", [(256, 8, "fp32"), (1024, 4, "fp32"), (130, 1, "fp32"), (512, 16, "fp32"),
-                                      (300, 9, "fp32"), (256, 8, "bf16"), (500, 5, "fp8"), (130, 3, "bf16_qw"),
+                                      (300, 9, "fp32"), (200, 12, "fp32"), (1100, 10, "fp32"), (256, 8, "bf16"),
+                                      (500, 5, "fp8"), (130, 3, "bf16_qw"),
                                       (256, 8, "fp8_qw")])
 def test_small_calls_match_large_ones(lib, K, s, prec):
     """Up to one tile per SM the FP32 encoder takes tiles of 64 signals instead of
-    128, and BF16/FP8 give each CTA one tile instead of two: a signal's code does not depend on the tiling, so the first N signals
-    alone give bitwise the codes they have in a call of 20,000 (152 SMs: 64-signal
-    tiles up to 19,456)."""
+    128, BF16/FP8 give each CTA one tile instead of two, and with s > 8 the kernel
+    itself depends on K and N: a signal's code does not depend on any of it, so the
+    first N signals alone give bitwise the codes they have in a call of 20,000 (152
+    SMs: 64-signal tiles up to 19,456)."""
     n = 20_000
     D = torch.from_numpy(synth.hidden_dictionary(K, 1).astype(np.float32)).cuda()
     X = torch.from_numpy(synth.signals(n, synth.hidden_dictionary(K, 2), min(s, 4), 3)).cuda()
