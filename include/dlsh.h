@@ -115,9 +115,9 @@ int dlsh_encode(const float* D, int K, int d, const float* X, int64_t N, int s,
 /*
  * The encoder kernel dlsh_encode runs for (K, s, precision) with the built-in
  * choice (no tuning record): 1 one tile per CTA, 2 two tiles on two warp
- * groups (FP32) or on selection and solver warps (BF16/FP8), 3 two tiles served
- * in turn, 4 / 5 two tiles with selection and solver warps (TF32 / FP16 parts),
- * 6 three such tiles (FP16 parts), 7 FP16 parts on one tile per CTA or, for
+ * groups (FP32; BF16/FP8 with few atoms) or on selection and solver warps
+ * (BF16/FP8), 3 two tiles served in turn, 4 / 5 two tiles with selection and
+ * solver warps (TF32 / FP16 parts), 6 three such tiles (FP16 parts), 7 FP16 parts on one tile per CTA or, for
  * s > 8 and where K and N make it the faster one, on two tiles as in 5; 0 if the
  * configuration is unsupported.  A record from dlsh_autotune_encode overrides
  * this choice.

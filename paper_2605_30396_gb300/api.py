@@ -119,7 +119,7 @@ def encode(D, X, s: int, eps: float = 0.0, precision="fp32", sync: bool = False,
     return idx, coef, nnz, resid
 
 
-ENCODE_VARIANTS = {1: "encode_kernel (one tile per CTA)", 2: "encode_pair_kernel (FP32), encode_lowp_kernel (BF16, FP8)",
+ENCODE_VARIANTS = {1: "encode_kernel (one tile per CTA)", 2: "encode_pair_kernel (FP32, or few atoms), encode_lowp_kernel (BF16, FP8)",
                    3: "encode_alt_kernel", 4: "encode_split_kernel (TF32 parts)",
                    5: "encode_split_kernel (FP16 parts)", 6: "encode_split_kernel (FP16 parts, three tiles)",
                    7: "FP16 parts: encode_kernel (one tile per CTA); above s = 8 encode_split_kernel where it is faster"}

@@ -310,8 +310,8 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
                    cudaStream_t st, uint32_t** status_out, unsigned long long* prof,
                    const long long* n_dev, int bn) {
   using namespace enc;
-  // kernel variant (s <= 8): 2 = two tiles in flight (FP32 on two warp
-  // groups, BF16/FP8 on selection and solver warps),
+  // kernel variant (s <= 8): 2 = two tiles in flight (on two warp groups,
+  // or BF16/FP8 on selection and solver warps),
   // 3 = two tiles served in turn by all warps (FP32), 4 / 5 = two tiles with
   // the warps split into selection and solver groups (FP32 as three TF32 / three
   // FP16 products), 6 = the same with three tiles and FP16 products, 7 = one
@@ -438,13 +438,20 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
     const int ntiles = static_cast<int>((N + TILE_M - 1) / TILE_M);
     int sms = device_sm_count();
     if (sms <= 0) sms = 1;
-    // two tiles in flight per CTA; a tile of its own for each SM while they last
-    // (FP32's two warp groups are made for two tiles: half as many CTAs)
-    const int want = pp.prec == 0 ? (ntiles + 1) / 2 : ntiles;
+    // two warp groups, or (BF16/FP8) selection and solver warps: the solver warps
+    // take twice as long over a tile as a group does with all of them at work, which
+    // pays with at least four chunks to select from, or with a tile per SM at most
+    // (200,000 signals, BF16, s = 4, groups / split: K = 98 297 / 313 us, K = 192 335 /
+    // 340, K = 256 354 / 350; 1M, K = 98, s = 2 618 / 719; 18,000, K = 98, s = 2 44 / 40)
+    const bool groups = pp.prec == 0 || (pp.nchunks < 4 && (n_dev || ntiles > sms));
+    // two tiles in flight per CTA; split, a tile of its own for each SM while they
+    // last (the groups are made for two tiles: half as many CTAs)
+    const int want = groups ? (ntiles + 1) / 2 : ntiles;
     const int grid = (!n_dev && want < sms) ? (want > 0 ? want : 1) : sms;
-    if (pp.prec == 0) return launch_pair<0, false>(a, grid, st);
-    if (pp.prec == 1) return pp.top4 ? launch_pair<1, true>(a, grid, st) : launch_pair<1, false>(a, grid, st);
-    return pp.top4 ? launch_pair<2, true>(a, grid, st) : launch_pair<2, false>(a, grid, st);
+    if (pp.prec == 0) return launch_pair<0, false>(a, groups, grid, st);
+    if (pp.prec == 1)
+      return pp.top4 ? launch_pair<1, true>(a, groups, grid, st) : launch_pair<1, false>(a, groups, grid, st);
+    return pp.top4 ? launch_pair<2, true>(a, groups, grid, st) : launch_pair<2, false>(a, groups, grid, st);
   }
   Plan p;
   if (make_plan(K, s, prec, p, (choice >= 2 && choice <= 7) ? 0 : choice, SMEM_LIMIT, choice == 7) != DLSH_OK)

@@ -1178,10 +1178,10 @@ int launch_encode(const Args& a, int grid, cudaStream_t st) {
 }
 
 template <int PREC, bool T4>
-int launch_pair(const PairArgs& a, int grid, cudaStream_t st) {
-  void (*fn)(const PairArgs) = nullptr;
-  if constexpr (PREC == 0) fn = encode_pair_kernel<PREC>;
-  else fn = encode_lowp_kernel<PREC, T4>;
+int launch_pair(const PairArgs& a, bool groups, int grid, cudaStream_t st) {
+  auto fn = encode_pair_kernel<PREC, T4>;
+  if constexpr (PREC != 0)
+    if (!groups) fn = encode_lowp_kernel<PREC, T4>;
   DLSH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT),
                 "dlsh_encode: cudaFuncSetAttribute");
   fn<<<grid, NTHREADS, a.p.smem, st>>>(a);
@@ -1211,11 +1211,11 @@ extern template int launch_encode<1, 128, false>(const Args&, int, cudaStream_t)
 extern template int launch_encode<1, 128, true>(const Args&, int, cudaStream_t);
 extern template int launch_encode<2, 128, false>(const Args&, int, cudaStream_t);
 extern template int launch_encode<2, 128, true>(const Args&, int, cudaStream_t);
-extern template int launch_pair<0, false>(const PairArgs&, int, cudaStream_t);
-extern template int launch_pair<1, false>(const PairArgs&, int, cudaStream_t);
-extern template int launch_pair<1, true>(const PairArgs&, int, cudaStream_t);
-extern template int launch_pair<2, false>(const PairArgs&, int, cudaStream_t);
-extern template int launch_pair<2, true>(const PairArgs&, int, cudaStream_t);
+extern template int launch_pair<0, false>(const PairArgs&, bool, int, cudaStream_t);
+extern template int launch_pair<1, false>(const PairArgs&, bool, int, cudaStream_t);
+extern template int launch_pair<1, true>(const PairArgs&, bool, int, cudaStream_t);
+extern template int launch_pair<2, false>(const PairArgs&, bool, int, cudaStream_t);
+extern template int launch_pair<2, true>(const PairArgs&, bool, int, cudaStream_t);
 extern template int launch_split<false, 2, 128, 8>(const SplitArgs&, int, cudaStream_t);
 extern template int launch_split<true, 2, 128, 8>(const SplitArgs&, int, cudaStream_t);
 extern template int launch_split<true, 2, 64, 8>(const SplitArgs&, int, cudaStream_t);

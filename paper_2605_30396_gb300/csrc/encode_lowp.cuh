@@ -3,10 +3,10 @@
 //
 // Included by encode_core.cuh after encode_pair.cuh, whose plan, chunk width (64
 // atoms), candidate keys and arithmetic it shares: the codes are bitwise those
-// of the two-group kernel that used to serve these precisions.  There each group
-// of eight warps selected and then solved its own tile, so that the ALU-bound
-// top-4 network and the load-bound solver of a tile took turns (23,000 cycles
-// per tile and iteration on an SM).  Here
+// of the two-group kernel, which serves these precisions where there are fewer
+// than four chunks.  There each group of eight warps selects and then solves its
+// own tile, so that the ALU-bound top-4 network and the load-bound solver of a
+// tile take turns (23,000 cycles per tile and iteration on an SM at K = 1024).  Here
 //   warps 0-7   select: warp w reads tensor-memory lane quarter w & 3 and the
 //               column half w >> 2 of every chunk, one job ahead of the solver;
 //   warps 8-15  re-score the candidates in FP32 and solve, two lanes per row;

@@ -1,7 +1,5 @@
 // Batch-OMP with two tiles in flight per CTA (Sec. 2.1: OMP against the
-// dictionary, one greedy atom at a time, least-squares re-fit), for s <= 8: the
-// FP32 kernel on two warp groups (3xTF32), and the plan and operand packing that
-// the BF16/FP8 kernel of encode_lowp.cuh shares.
+// dictionary, one greedy atom at a time, least-squares re-fit), for s <= 8.
 //
 // Included by encode_core.cuh inside namespace dlsh::enc (it uses that file's
 // operand packing, key networks and constants).
@@ -13,16 +11,18 @@
 //   warp 17  TMA producer: streams 64-atom chunks of the packed dictionary
 //            through a ring, in the order the MMA warp consumes them.
 //   warp 16  MMA issuer: serves the groups' OMP iterations alternately
-//            (group 0 iteration it, group 1 iteration it, ...): the
+//            (group 0 iteration it, group 1 iteration it, ...).  FP32: the
 //            group's residual, staged in shared memory as TF32 hi/lo parts,
 //            is first copied into the group's tensor-memory A columns
-//            (tcgen05.cp), and the 3xTF32 MMAs read A from tensor memory.
+//            (tcgen05.cp), and the 3xTF32 MMAs read A from tensor memory;
+//            BF16/FP8: A stays in shared memory (one region per group).
 //   warps 0-15  two groups of eight.  Selection: thread (lane, warp w of the
 //            group) reads TMEM lane 32 (w % 4) + lane, i.e. one row, over the
 //            column half w / 4 of every chunk.  Solver: two sub-lanes per
 //            signal, each owning 24 of the 48 padded dimensions.
-// Tensor memory: 256 columns per group: A hi at columns 0..47, A lo at 48..95,
-// two 64-column accumulator buffers at 128..255.
+// Tensor memory: 256 columns per group.  FP32: A hi at columns 0..47, A lo at
+// 48..95, two 64-column accumulator buffers at 128..255.  BF16/FP8: four
+// 64-column accumulator buffers.
 
 constexpr int PBN = 64;   // atoms per chunk
 constexpr int PQC = 32;   // chunk columns read by one selection thread
@@ -148,31 +148,36 @@ __device__ __forceinline__ void write_a_part24(uint8_t* A, int row, int u, const
   }
 }
 
-// One chunk of MMAs for the pair kernel: D[tmem] = A . B^T over K = 48, N = 64,
-// A (hi, lo) from tensor memory at a_tmem.
-__device__ __forceinline__ void issue_pair_chunk(uint32_t tmem_d, uint32_t a_tmem, uint32_t b_addr) {
-  constexpr uint32_t idesc = umma_idesc(2, 2, TILE_M, PBN);
-  constexpr uint32_t B_LBO = PBN * 16, SBO = 128, B_PART = PBN * 12 * 16;
+// One chunk of MMAs for the pair kernel: D[tmem] = A . B^T over K = 48 (64 for
+// FP8), N = 64.  FP32: A (hi, lo) from tensor memory at a_tmem; else A from
+// shared memory at a_addr.
+template <int PREC>
+__device__ __forceinline__ void issue_pair_chunk(uint32_t tmem_d, uint32_t a_tmem, uint32_t a_addr,
+                                                 uint32_t b_addr) {
+  if constexpr (PREC == 0) {
+    constexpr uint32_t idesc = umma_idesc(2, 2, TILE_M, PBN);
+    constexpr uint32_t B_LBO = PBN * 16, SBO = 128, B_PART = PBN * 12 * 16;
 #pragma unroll
-  for (int pass = 0; pass < 3; ++pass) {
-    const uint32_t ao = pass == 2 ? 48u : 0u;    // lo(r) . hi(D)
-    const uint32_t bo = pass == 1 ? B_PART : 0u;  // hi(r) . lo(D)
+    for (int pass = 0; pass < 3; ++pass) {
+      const uint32_t ao = pass == 2 ? 48u : 0u;    // lo(r) . hi(D)
+      const uint32_t bo = pass == 1 ? B_PART : 0u;  // hi(r) . lo(D)
 #pragma unroll
-    for (int ks = 0; ks < 6; ++ks) {
-      const uint64_t bd = umma_smem_desc(b_addr + bo + ks * 2 * B_LBO, B_LBO, SBO);
-      umma_tf32_tmem_a(tmem_d, a_tmem + ao + ks * 8, bd, idesc, (pass | ks) != 0);
+      for (int ks = 0; ks < 6; ++ks) {
+        const uint64_t bd = umma_smem_desc(b_addr + bo + ks * 2 * B_LBO, B_LBO, SBO);
+        umma_tf32_tmem_a(tmem_d, a_tmem + ao + ks * 8, bd, idesc, (pass | ks) != 0);
+      }
     }
+  } else {
+    issue_chunk<PREC, PBN>(tmem_d, a_addr, b_addr);
   }
 }
 
-// (A template so that only enc_pair.cu compiles it.)
-template <int PREC>
+template <int PREC, bool T4>
 __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_constant__ PairArgs a) {
-  static_assert(PREC == 0, "FP32; BF16 and FP8 run encode_lowp_kernel");
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int SMAX = 8;
-  constexpr int NBUF = 2;
-  constexpr uint32_t BUF0 = 128u;
+  constexpr int NBUF = PREC == 0 ? 2 : 4;
+  constexpr uint32_t BUF0 = PREC == 0 ? 128u : 0u;
   const PairPlan& p = a.p;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long NS = a.n_dev ? *a.n_dev : a.N;
@@ -269,23 +274,25 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
             aph[g] ^= 1u;
             tc_fence_after();
             const uint32_t tg = tmem_base + static_cast<uint32_t>(g) * 256u;
-            // staged residual (TF32 hi, lo) -> this group's A columns; the
-            // staging area is free again once the copies complete
-            constexpr uint32_t LBO = TILE_M * 16, SBO = 128, PART = TILE_M * 12 * 16;
-            const uint32_t sa = smem_u32(smem + p.off_a[0]);
+            if constexpr (PREC == 0) {
+              // staged residual (TF32 hi, lo) -> this group's A columns; the
+              // staging area is free again once the copies complete
+              constexpr uint32_t LBO = TILE_M * 16, SBO = 128, PART = TILE_M * 12 * 16;
+              const uint32_t sa = smem_u32(smem + p.off_a[0]);
 #pragma unroll
-            for (int part = 0; part < 2; ++part)
+              for (int part = 0; part < 2; ++part)
 #pragma unroll
-              for (int kk = 0; kk < 6; ++kk)
-                tmem_cp_128x256b(tg + part * 48 + kk * 8,
-                                 umma_smem_desc(sa + part * PART + kk * 2 * LBO, LBO, SBO));
-            tc_commit(bar_stage);
-            if (!mbar_wait(bar_stage, static_cast<uint32_t>(job & 1), a.budget)) {
-              flag_status(a.status, ST_TIMEOUT);
-              ok = false;
-              break;
+                for (int kk = 0; kk < 6; ++kk)
+                  tmem_cp_128x256b(tg + part * 48 + kk * 8,
+                                   umma_smem_desc(sa + part * PART + kk * 2 * LBO, LBO, SBO));
+              tc_commit(bar_stage);
+              if (!mbar_wait(bar_stage, static_cast<uint32_t>(job & 1), a.budget)) {
+                flag_status(a.status, ST_TIMEOUT);
+                ok = false;
+                break;
+              }
+              *stage_done = job;
             }
-            *stage_done = job;
             for (int c = 0; c < p.nchunks; ++c, ++ring, ++cc[g]) {
               const int st = static_cast<int>(ring % p.stages);
               const uint32_t dpar = static_cast<uint32_t>((ring / p.stages) & 1);
@@ -298,8 +305,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
                 break;
               }
               tc_fence_after();
-              issue_pair_chunk(tg + BUF0 + static_cast<uint32_t>(buf) * PBN, tg,
-                               ring_addr + static_cast<uint32_t>(st) * p.chunk_bytes);
+              issue_pair_chunk<PREC>(tg + BUF0 + static_cast<uint32_t>(buf) * PBN, tg,
+                                     smem_u32(smem + p.off_a[g]),
+                                     ring_addr + static_cast<uint32_t>(st) * p.chunk_bytes);
               tc_commit(&bar_full[g * 4 + buf]);
               tc_commit(&bar_dempty[st]);
             }
@@ -317,6 +325,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
     float* idg = reinterpret_cast<float*>(smem + p.off_idg[g]);
     float* cv = reinterpret_cast<float*>(smem + p.off_cand[g]);       // [128][2]
     int* cj = reinterpret_cast<int*>(smem + p.off_cand[g] + TILE_M * 2 * 4);
+    uint32_t* ckeys = reinterpret_cast<uint32_t*>(smem + p.off_cand[g]);  // T4: [128][2][4]
+    float* rsm = reinterpret_cast<float*>(smem + p.off_r[g]);  // [24][256]
+    float* sig = reinterpret_cast<float*>(smem + p.off_sig);
+    if constexpr (PREC == 2) {
+      for (int j = tid; j < p.Kp; j += 2 * PGT) sig[j] = a.sigma[j];
+      // FP8 rows hold 64 bytes: bytes 48..63 are zero padding, written once
+      for (int row = gtid; row < TILE_M; row += PGT)
+        *reinterpret_cast<uint4*>(A + 3 * TILE_M * 16 + row * 16) = make_uint4(0, 0, 0, 0);
+      named_bar_sync(3, 2 * PGT);
+    }
     const int R1 = 32 * (gw & 3) + lane, h = gw >> 2;
     const int R2 = 16 * gw + (lane >> 1), u = lane & 1;
     const uint32_t trow = tmem_base + (static_cast<uint32_t>(32 * (gw & 3)) << 16) +
@@ -328,11 +346,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
     // FP32: the staging area may be written for job J once the copy of job
     // J - 1 into TMEM has completed (published by the MMA warp)
     auto wait_staging = [&](long long J) -> bool {
-      const long long t0 = clock64();
-      while (*stage_done < J - 1) {
-        if (clock64() - t0 > a.budget) {
-          flag_status(a.status, ST_TIMEOUT);
-          return false;
+      if constexpr (PREC == 0) {
+        const long long t0 = clock64();
+        while (*stage_done < J - 1) {
+          if (clock64() - t0 > a.budget) {
+            flag_status(a.status, ST_TIMEOUT);
+            return false;
+          }
         }
       }
       return true;
@@ -359,10 +379,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
 #pragma unroll
         for (int q = 0; q < 24; ++q) part = fmaf(x[q], x[q], part);
         float inv = 1.f;
+        if constexpr (PREC == 2) {
+          float mx = 0.f;
+#pragma unroll
+          for (int q = 0; q < 24; ++q) mx = fmaxf(mx, fabsf(x[q]));
+          mx = pair_max(mx);
+          inv = mx > 0.f ? FP8_MAX / mx : 1.f;
+        }
         if (wait_staging(job_index(g, k, 0)))
-          write_a_part24<0>(A, R2, u, x, inv);
+          write_a_part24<PREC>(A, R2, u, x, inv);
         else
           ok = false;
+        if constexpr (PREC != 0) {
+#pragma unroll
+          for (int q = 0; q < 24; ++q) rsm[q * PGT + gtid] = x[q];
+        }
         rn2 = pair_sum(part);
       }
       fence_proxy_async_smem();
@@ -380,6 +411,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
         {
           uint32_t best = 0;
           int bestc = 0;
+          const uint32_t vmask = 0x7fffffffu & ~((1u << p.ib) - 1u);
+          uint32_t run[4] = {0u, 0u, 0u, 0u};
           for (int c = 0; c < nchunks; ++c, ++ccg) {
             const int buf = static_cast<int>(ccg % NBUF);
             if (!mbar_wait(&bar_full[g * 4 + buf], static_cast<uint32_t>((ccg / NBUF) & 1), a.budget)) {
@@ -395,20 +428,47 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_empty[g * 4 + buf]);
-            uint32_t m0 = 0, m1 = 0;
+            if constexpr (PREC == 2) {
+              const int j0 = c * PBN + h * PQC;
 #pragma unroll
-            for (int q = 0; q < PQC; q += 2) {
-              m0 = max(m0, (rr[q] & 0x7fffffe0u) | static_cast<uint32_t>(31 - q));
-              m1 = max(m1, (rr[q + 1] & 0x7fffffe0u) | static_cast<uint32_t>(30 - q));
+              for (int q = 0; q < PQC; ++q) rr[q] = __float_as_uint(__uint_as_float(rr[q]) * sig[j0 + q]);
             }
-            const uint32_t m = max(m0, m1);
-            if ((m & ~31u) > (best & ~31u)) {
-              best = m;
-              bestc = c;
+            if constexpr (T4) {
+#pragma unroll
+              for (int q = 0; q < PQC; ++q) rr[q] = (rr[q] & vmask) | static_cast<uint32_t>(31 - q);
+              uint32_t ct[4];
+              top4_of8(rr, ct);
+#pragma unroll
+              for (int o = 8; o < PQC; o += 8) {
+                uint32_t t8[4];
+                top4_of8(rr + o, t8);
+                merge_top4(ct, t8);
+              }
+              const uint32_t cf = ((1u << p.ib) - 32u) - static_cast<uint32_t>(c) * 32u;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) ct[i] |= cf;
+              merge_top4(run, ct);
+            } else {
+              uint32_t m0 = 0, m1 = 0;
+#pragma unroll
+              for (int q = 0; q < PQC; q += 2) {
+                m0 = max(m0, (rr[q] & 0x7fffffe0u) | static_cast<uint32_t>(31 - q));
+                m1 = max(m1, (rr[q + 1] & 0x7fffffe0u) | static_cast<uint32_t>(30 - q));
+              }
+              const uint32_t m = max(m0, m1);
+              if ((m & ~31u) > (best & ~31u)) {
+                best = m;
+                bestc = c;
+              }
             }
           }
-          cv[R1 * 2 + h] = __uint_as_float(best & ~31u);
-          cj[R1 * 2 + h] = bestc * PBN + h * PQC + 31 - static_cast<int>(best & 31u);
+          if constexpr (T4) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ckeys[(R1 * 2 + h) * 4 + i] = run[i];
+          } else {
+            cv[R1 * 2 + h] = __uint_as_float(best & ~31u);
+            cj[R1 * 2 + h] = bestc * PBN + h * PQC + 31 - static_cast<int>(best & 31u);
+          }
         }
         if (named_bar_or(gbar, PGT, !ok)) {
           ok = false;
@@ -423,13 +483,68 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
           for (int m = 0; m < SMAX; ++m) sl[m] = m < t ? sel[m * TILE_M + R2] : 0;
           int js = -1;
           float best = -1.f;
+          if constexpr (PREC == 0) {
 #pragma unroll
-          for (int qq = 0; qq < 2; ++qq) {
-            const float v = cv[R2 * 2 + qq];
-            const int j = cj[R2 * 2 + qq];
-            if (j < K && (v > best || (v == best && j < js))) {
-              best = v;
-              js = j;
+            for (int qq = 0; qq < 2; ++qq) {
+              const float v = cv[R2 * 2 + qq];
+              const int j = cj[R2 * 2 + qq];
+              if (j < K && (v > best || (v == best && j < js))) {
+                best = v;
+                js = j;
+              }
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < 24; ++q) r[q] = rsm[q * PGT + gtid];
+            // candidates: T4, the row's exact low-precision top 4 (sub-lane u
+            // reads half u's list, one butterfly round); else the winner of
+            // each column half
+            int cjr[4];
+            if constexpr (T4) {
+              const uint32_t imask = (1u << p.ib) - 1u;
+              unsigned long long lst[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const uint32_t key = ckeys[(R2 * 2 + u) * 4 + i];
+                const uint32_t col = imask - (key & imask);
+                const uint32_t j = (col >> 5) * PBN + static_cast<uint32_t>(u * PQC) + (col & 31u);
+                lst[i] = key == 0u ? 0ull
+                                   : (static_cast<unsigned long long>(key & ~imask & 0x7fffffffu) << 32) |
+                                         static_cast<unsigned long long>(0xFFFFFFFFu - j);
+              }
+              unsigned long long oth[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) oth[i] = __shfl_xor_sync(pair_mask(), lst[i], 1);
+              merge_top4(lst, oth);
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                cjr[i] = lst[i] == 0ull ? 0x7fffffff
+                                        : static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(lst[i]));
+            } else {
+              cjr[0] = cj[R2 * 2 + 0];
+              cjr[1] = cj[R2 * 2 + 1];
+              cjr[2] = cjr[3] = 0x7fffffff;
+            }
+#pragma unroll
+            for (int qq = 0; qq < 4; ++qq) {
+              const int j = cjr[qq];
+              float c0 = 0.f;
+              if (j < K) {
+                const float4* dr = reinterpret_cast<const float4*>(a.D32p + static_cast<size_t>(j) * DPAD + 24 * u);
+#pragma unroll
+                for (int w4 = 0; w4 < 6; ++w4) {
+                  const float4 dv = __ldg(dr + w4);
+                  c0 = fmaf(r[4 * w4 + 0], dv.x, c0);
+                  c0 = fmaf(r[4 * w4 + 1], dv.y, c0);
+                  c0 = fmaf(r[4 * w4 + 2], dv.z, c0);
+                  c0 = fmaf(r[4 * w4 + 3], dv.w, c0);
+                }
+              }
+              c0 = fabsf(pair_sum(c0));
+              if (j < K && (c0 > best || (c0 == best && j < js))) {
+                best = c0;
+                js = j;
+              }
             }
           }
           {
@@ -551,10 +666,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_pair_kernel(const __grid_c
               rn2 = pair_sum(pr);
               if (it + 1 < s) {
                 float inv = 1.f;
+                if constexpr (PREC == 2) {
+                  float mx = 0.f;
+#pragma unroll
+                  for (int q = 0; q < 24; ++q) mx = fmaxf(mx, fabsf(r[q]));
+                  mx = pair_max(mx);
+                  inv = mx > 0.f ? FP8_MAX / mx : 1.f;
+                }
                 if (wait_staging(job_index(g, k, it + 1)))
-                  write_a_part24<0>(A, R2, u, r, inv);
+                  write_a_part24<PREC>(A, R2, u, r, inv);
                 else
                   ok = false;
+              }
+              if constexpr (PREC != 0) {
+#pragma unroll
+                for (int q = 0; q < 24; ++q) rsm[q * PGT + gtid] = r[q];
               }
             };
             if (t < 8)

@@ -246,7 +246,7 @@ def test_multi_tile_fp32_encoders_over_several_rounds(lib, variant):
 
 @pytest.mark.parametrize("K,s,prec", [(256, 8, "fp32"), (1024, 4, "fp32"), (130, 1, "fp32"), (512, 16, "fp32"),
                                       (300, 9, "fp32"), (200, 12, "fp32"), (1100, 10, "fp32"), (256, 8, "bf16"),
-                                      (500, 5, "fp8"), (130, 3, "bf16_qw"),
+                                      (500, 5, "fp8"), (130, 3, "bf16_qw"), (100, 4, "bf16"), (130, 3, "fp8"),
                                       (256, 8, "fp8_qw")])
 def test_small_calls_match_large_ones(lib, K, s, prec):
     """Up to one tile per SM the FP32 encoder takes tiles of 64 signals instead of
