@@ -19,7 +19,7 @@
 //    one 16-byte word; its three channel sums are reduced over the eight lanes
 //    in four shuffles (a transposing butterfly).
 // Results are staged and written back coalesced.  An FP32 dictionary of which
-// only one channel plane fits in shared memory (about 1150 to 3100 atoms) is
+// only one channel plane fits in shared memory (about 1150 to 2500 atoms, s >= 8) is
 // decoded channel by channel, each by its own CTAs (decode_channel_kernel);
 // beyond that the FP32 rows are read through the read-only cache, with the FP16
 // path's lane mapping.
@@ -609,12 +609,16 @@ static int launch_decode(const float* D, int K, const void* idx, const void* coe
 }  // namespace dec
 
 // The FP32 table stays in shared memory while at least six warps (batches of
-// 8) fit beside it; beyond that (about 1150 atoms) one channel plane at a time,
-// while eight warps fit beside it; then (about 3200 atoms) the rows are read
-// through the read-only cache.
+// 8) fit beside it; beyond that (about 1150 atoms) one channel plane at a time, up
+// to 2500 atoms and from 8 slots per code on; else the rows are read through the
+// read-only cache.  Three walks over the codes cost more than they save on short
+// codes, and so do the few warps beside a larger plane (1M Gaussians, rows / planes:
+// K = 2048, s = 3 89 / 105 us, s = 4 102 / 100 and with uneven codes 90 / 117, s = 8
+// 182 / 137 and 142 / 136; K = 2500, s = 8 182 / 142 and 143 / 142; K = 3100, s = 8
+// 182 / 238).
 static int decode_format(int K, int s) {
   if (dec::fit_warps(dec::FM_F32, K, s) >= 6) return dec::FM_F32;
-  return dec::fit_warps(dec::FM_PLANE, K, s) >= 8 ? dec::FM_PLANE : dec::FM_GLOBAL;
+  return s >= 8 && K <= 2500 && dec::fit_warps(dec::FM_PLANE, K, s) >= 8 ? dec::FM_PLANE : dec::FM_GLOBAL;
 }
 
 // Shared with the bench / learn paths: enqueue one decode.

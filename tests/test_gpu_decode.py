@@ -37,10 +37,12 @@ def test_decode_dirs(lib, N, K, s):
 @pytest.mark.parametrize("N,K,s,cam,with_dc", [(17, 1300, 3, True, True), (5003, 2048, 16, True, False),
                                                (1_500_001, 1160, 1, False, False), (300_007, 2048, 5, True, True),
                                                (187_500, 3000, 8, False, True), (46_877, 1200, 32, False, False),
+                                               (187_501, 2500, 8, False, True), (100_003, 2048, 16, True, True),
                                                (50, 3300, 4, False, False)])
 def test_decode_large_dictionaries(lib, N, K, s, cam, with_dc):
-    """Dictionaries decoded one channel plane at a time (about 1150 to 3100
-    atoms, from 1.5 million code slots on), shorter calls and larger dictionaries: ragged batches, uneven codes, the camera form
+    """Dictionaries decoded one channel plane at a time (about 1150 to 2500
+    atoms, from 8 slots per code and 1.5 million code slots on), shorter codes and
+    calls and larger dictionaries: ragged batches, uneven codes, the camera form
     and the full colour.  The file's relative tolerance (1e-4)."""
     rng = np.random.default_rng(K + s)
     D = synth.hidden_dictionary(K, 5).astype(np.float32)
