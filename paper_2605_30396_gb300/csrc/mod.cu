@@ -1423,15 +1423,18 @@ __global__ void __launch_bounds__(1024)
 // their sums of g R_i and g^2:
 //   phase 1  sixteen lanes take one entry of the CTA's part of the list (a
 //            float4 of its row each); the sums go through shared memory to 16
-//            words of 16 bytes, three values and the atom's number in each,
-//            written and read by single 128-bit accesses, so that a word's
-//            arrival is its own flag
+//            words of 16 bytes, three values and the exchange's number in
+//            each, written and read by single 128-bit accesses, so that a
+//            word's arrival is its own flag
 //   phase 2  every CTA sums all words in the same order, forms d, and updates
 //            its rows (up to KS_KEEP passes still in registers), coefficients
 //            and, on CTA 0, the atom
-// Two sets of words alternate: a CTA writes an atom's words only after it has
-// read all of the previous atom's, so no word is overwritten before its readers
-// are through.  Every sum runs in a fixed order.  Bound by latency: the row
+// Two sets of words alternate from one exchange to the next (an unused atom has
+// none, so they go by the exchanges done, not by the atom's number): a CTA writes
+// the words of an exchange only after it has read all of the previous one's, which
+// the others write only after they have read the one before, so no word is
+// overwritten before its readers are through.  Every sum runs in a fixed order.
+// Bound by latency: the row
 // gather, one L2 round trip of the words and the reductions, 3.4 us per
 // atom (N = 400k, K = 512, s = 8; with two grid barriers per atom and one
 // thread per entry 12.4 us).
@@ -1538,6 +1541,7 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
   int lo = lo_of(0), hi = hi_of(0);
   uint2 first = lo + slot < hi ? list[lo + slot] : make_uint2(0u, 0u);
   float4 dj = rl ? old_of(0) : make_float4(0.f, 0.f, 0.f, 0.f);
+  unsigned turn = 0;  // exchanges begun, the same in every CTA; the words' tag
   for (int j = 0; j < K; ++j) {
     const bool used = a1 > a0;  // the same decision in every CTA
     const int clo = lo, chi = hi;
@@ -1547,6 +1551,7 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
     uint2 rec[KS_KEEP];
     float4 r[KS_KEEP];
     if (used) {
+      ++turn;
       // ---- phase 1: sum g R_i (lanes 0..11) and g^2 (lane 12) over the CTA's entries
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -1593,8 +1598,7 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
           for (int w = 0; w < KS_T / 32; ++w) sum += reinterpret_cast<const float*>(&wsum[w][0])[val];
           t3[q] = sum;
         }
-        st_word(part + (static_cast<size_t>(j & 1) * G + blockIdx.x) * KS_WORDS + tid, t3[0], t3[1], t3[2],
-                static_cast<unsigned>(j) + 1u);
+        st_word(part + (static_cast<size_t>(turn & 1u) * G + blockIdx.x) * KS_WORDS + tid, t3[0], t3[1], t3[2], turn);
       }
     }
     // ---- the next atom's reads, while the words travel
@@ -1619,10 +1623,9 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
     {
       float t3[3] = {0.f, 0.f, 0.f};
       bool ok = true;
-      const uint4* base = part + static_cast<size_t>(j & 1) * G * KS_WORDS + (tid & 15);
-      const unsigned want = static_cast<unsigned>(j) + 1u;
+      const uint4* base = part + static_cast<size_t>(turn & 1u) * G * KS_WORDS + (tid & 15);
       constexpr int B = 5;  // words in flight per thread: all of 152 CTAs' in one go
-      for (int c0 = slot; c0 < G; c0 += B * KS_E) {
+      for (int c0 = slot; c0 < G && ok; c0 += B * KS_E) {
         uint4 w[B];
 #pragma unroll
         for (int b = 0; b < B; ++b)
@@ -1630,7 +1633,7 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
 #pragma unroll
         for (int b = 0; b < B; ++b) {
           if (c0 + b * KS_E >= G) break;
-          if (w[b].w != want) {
+          if (w[b].w != turn) {
             const long long tw = clock64();
             do {
               if (clock64() - tw > budget) {
@@ -1639,7 +1642,8 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
                 break;
               }
               w[b] = ld_word(base + static_cast<size_t>(c0 + b * KS_E) * KS_WORDS);
-            } while (w[b].w != want);
+            } while (w[b].w != turn);
+            if (!ok) break;  // one budget per thread, whatever else is missing
           }
           t3[0] += __uint_as_float(w[b].x);
           t3[1] += __uint_as_float(w[b].y);

@@ -77,6 +77,56 @@ def test_ksvd_on_uneven_codes(lib, N, K, s):
     assert (again[0] == Dg).all() and (again[1] == cg).all()
 
 
+@pytest.mark.parametrize("gaps", ["even", "odd", "two", "mixed"])
+def test_ksvd_skips_unused_atoms_between_used_ones(lib, gaps):
+    """Unused atoms between used ones (and before the first, and after the last):
+    one in two, two between each, and runs of one to three, with about ten entries
+    per used atom spread over 152 CTAs, so that a CTA is through with an atom while
+    others still wait for its sums.  Atoms without entries stay as they were, and
+    every run gives the same bits.  The file's relative tolerance (1e-4)."""
+    N, K, s = 160_000, 512, 2
+    rng = np.random.default_rng(90)
+    if gaps == "mixed":
+        used, j = [], 2
+        while j < K - 1:
+            used.append(j)
+            j += int(rng.integers(1, 5))
+        used = np.array(used)
+    else:
+        used = {"even": np.arange(0, K, 2), "odd": np.arange(1, K, 2), "two": np.arange(2, K, 3)}[gaps]
+    U, M = len(used), 5 * len(used)  # M signals with codes, U used atoms
+    D = synth.hidden_dictionary(K, 91)
+    rows = np.sort(rng.choice(N, M, replace=False))
+    idx = np.zeros((N, s), dtype=np.int64)
+    coef = np.zeros((N, s))
+    nnz = np.zeros(N, dtype=np.uint8)
+    first = np.tile(np.arange(U), 5)
+    rng.shuffle(first)
+    idx[rows, 0] = used[first]
+    idx[rows, 1] = used[(first + 1 + rng.integers(0, U - 1, M)) % U]
+    coef[rows] = (0.5 + rng.exponential(1.0, (M, s))) * rng.choice([-1.0, 1.0], (M, s))
+    nnz[rows] = s
+    X = rng.standard_normal((N, 45)) * 0.05
+    X[rows] += np.einsum("ns,nsd->nd", coef[rows], D[idx[rows]])
+    X = X.astype(np.float32)
+    D0 = D + 0.1 * rng.standard_normal(D.shape)
+    D0 = (D0 / np.linalg.norm(D0, axis=1, keepdims=True)).astype(np.float32)
+    args = (X, D0, idx.astype(np.uint16), coef.astype(np.float32), nnz, None)
+    Dg, cg = _gpu(lib, *args)
+    Do, co, info = oks.ksvd_update(X.astype(np.float64), D0.astype(np.float64), idx, args[3].astype(np.float64),
+                                   nnz.astype(np.int64), np.zeros(N))
+    unused = np.setdiff1d(np.arange(K), used)
+    assert list(info["unused"]) == list(unused)
+    np.testing.assert_array_equal(Dg[unused], D0[unused])
+    ok, worst = close_rel(Dg[used], Do[used])
+    assert ok, ("D", worst)
+    ok, worst = close_rel(cg, co)
+    assert ok, ("coef", worst)
+    for _ in range(20):
+        again = _gpu(lib, *args)
+        assert (again[0] == Dg).all() and (again[1] == cg).all()
+
+
 def _recon(D, idx, coef, nnz):
     out = np.zeros((idx.shape[0], 45))
     for t in range(idx.shape[1]):
