@@ -529,11 +529,12 @@ size_t dlsh_preprocess_max_k(int s, int compact);
 
 /* ---- self-test of the bounded device waits --------------------------------
  * Not part of the method (the paper has no counterpart): every pipelined kernel
- * here waits on mbarriers or a grid barrier with a cycle budget, so that a lost
- * arrival ends in DLSH_ERR_TIMEOUT instead of a hung GPU.  This call makes such
- * a wait run out on purpose, with nothing else in flight: kind 0 waits on an
- * mbarrier nobody arrives on; kind 1 is a cooperative launch in which one CTA
- * skips the grid barrier.  budget_cycles (1 .. 4e9 SM cycles) bounds the wait.
+ * here waits on mbarriers, a grid barrier or other CTAs' words with a cycle budget,
+ * so that a lost arrival ends in DLSH_ERR_TIMEOUT instead of a hung GPU.  This call
+ * makes such a wait run out on purpose, with nothing else in flight: kind 0 waits
+ * on an mbarrier nobody arrives on; kind 1 is two cooperative launches, in which
+ * one CTA skips the grid barrier and does not write its tagged word (both waits
+ * have to run out; words 1 and 2 of ws hold their status).  budget_cycles (1 .. 4e9 SM cycles) bounds the wait.
  * Returns DLSH_ERR_TIMEOUT when the wait gave up as designed; the CUDA context
  * stays usable.  ws: dlsh_selftest_workspace_size() bytes of device memory,
  * 256-byte aligned.  Synchronises the stream. */

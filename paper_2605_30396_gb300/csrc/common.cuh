@@ -87,48 +87,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
   return true;
 }
 
-// ---- grid barrier (cooperative launches only) --------------------------------
+// ---- waits of cooperative launches (every CTA resident) -----------------------
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
 
-// Grid-wide barrier of a cooperative launch: bar[0] counts arrivals, bar[1] is
-// the generation.  The wait is bounded: on timeout it records ST_TIMEOUT and
-// returns false, and the caller leaves the kernel.
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, long long budget, uint32_t* status) {
-  __shared__ int ok_s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    const unsigned g = ld_acquire_u32(bar + 1);
-    __threadfence();
-    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (ld_acquire_u32(bar + 1) == g) {
-        if (clock64() - t0 > budget) {
-          flag_status(status, ST_TIMEOUT);
-          ok = 0;
-          break;
-        }
-        __nanosleep(64);
-      }
-    }
-    __threadfence();
-    ok_s = ok;
-  }
-  __syncthreads();
-  return ok_s != 0;
-}
-
-// The same without a generation: *count (zeroed before the launch) only counts
-// arrivals, and the caller passes how many barriers it has reached, this one
-// included (1, 2, ..).  One reduction per CTA and a spin without sleeping.
+// Grid-wide barrier: *count (zeroed before the launch) counts arrivals, and the
+// caller passes how many barriers it has reached, this one included (1, 2, ..).
+// One reduction per CTA and a spin without sleeping.  The wait is bounded: on
+// timeout it records ST_TIMEOUT and returns false, and the caller leaves the
+// kernel.
 __device__ __forceinline__ bool grid_barrier_count(unsigned* count, unsigned reached, long long budget,
                                                    uint32_t* status) {
   __shared__ int ok_s;
@@ -151,6 +121,48 @@ __device__ __forceinline__ bool grid_barrier_count(unsigned* count, unsigned rea
   }
   __syncthreads();
   return ok_s != 0;
+}
+
+// 16-byte words of three values and a tag, written and read by single 128-bit
+// accesses, so that a word's arrival is its own flag.
+__device__ __forceinline__ void st_word(uint4* p, float a, float b, float c, unsigned tag) {
+  const unsigned long long lo = static_cast<unsigned long long>(__float_as_uint(b)) << 32 | __float_as_uint(a);
+  const unsigned long long hi = static_cast<unsigned long long>(tag) << 32 | __float_as_uint(c);
+  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+               "l"(lo), "l"(hi)
+               : "memory");
+}
+__device__ __forceinline__ uint4 ld_word(const uint4* p) {
+  unsigned long long lo, hi;
+  asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+               : "=l"(lo), "=l"(hi)
+               : "l"(p)
+               : "memory");
+  return make_uint4(static_cast<unsigned>(lo), static_cast<unsigned>(lo >> 32), static_cast<unsigned>(hi),
+                    static_cast<unsigned>(hi >> 32));
+}
+// Reads the words p, p + step, .. (n of them, at most B) into w until each carries
+// the tag (not 0): all that are missing at once, so that a late word costs the
+// others no further round trip.  Bounded as above.
+template <int B>
+__device__ __forceinline__ bool wait_words(const uint4* p, size_t step, int n, unsigned tag, uint4 (&w)[B],
+                                           long long budget, uint32_t* status) {
+#pragma unroll
+  for (int b = 0; b < B; ++b) w[b] = make_uint4(0u, 0u, 0u, 0u);
+  const long long t0 = clock64();
+  for (;;) {
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+      if (b < n && w[b].w != tag) w[b] = ld_word(p + b * step);
+    bool missing = false;
+#pragma unroll
+    for (int b = 0; b < B; ++b) missing |= b < n && w[b].w != tag;
+    if (!missing) return true;
+    if (clock64() - t0 > budget) {
+      flag_status(status, ST_TIMEOUT);
+      return false;
+    }
+  }
 }
 
 // ---- proxy fences --------------------------------------------------------

@@ -1494,23 +1494,6 @@ __global__ void __launch_bounds__(256) ksvd_resid_kernel(const float* __restrict
   if (lane < RROW - 32) R[i * RROW + 32 + lane] = r1;
 }
 
-__device__ __forceinline__ void st_word(uint4* p, float a, float b, float c, unsigned tag) {
-  const unsigned long long lo = static_cast<unsigned long long>(__float_as_uint(b)) << 32 | __float_as_uint(a);
-  const unsigned long long hi = static_cast<unsigned long long>(tag) << 32 | __float_as_uint(c);
-  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
-               "l"(lo), "l"(hi)
-               : "memory");
-}
-__device__ __forceinline__ uint4 ld_word(const uint4* p) {
-  unsigned long long lo, hi;
-  asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
-               : "=l"(lo), "=l"(hi)
-               : "l"(p)
-               : "memory");
-  return make_uint4(static_cast<unsigned>(lo), static_cast<unsigned>(lo >> 32), static_cast<unsigned>(hi),
-                    static_cast<unsigned>(hi >> 32));
-}
-
 __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restrict__ off, int T,
                                                              const int* __restrict__ atom_start,
                                                              const uint2* __restrict__ list, int K, int s,
@@ -1626,25 +1609,11 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
       const uint4* base = part + static_cast<size_t>(turn & 1u) * G * KS_WORDS + (tid & 15);
       constexpr int B = 5;  // words in flight per thread: all of 152 CTAs' in one go
       for (int c0 = slot; c0 < G && ok; c0 += B * KS_E) {
-        uint4 w[B];
-#pragma unroll
-        for (int b = 0; b < B; ++b)
-          if (c0 + b * KS_E < G) w[b] = ld_word(base + static_cast<size_t>(c0 + b * KS_E) * KS_WORDS);
+        uint4 w[B];  // zeros past the last CTA
+        ok = wait_words(base + static_cast<size_t>(c0) * KS_WORDS, KS_E * KS_WORDS, (G - c0 + KS_E - 1) / KS_E, turn, w,
+                        budget, status);
 #pragma unroll
         for (int b = 0; b < B; ++b) {
-          if (c0 + b * KS_E >= G) break;
-          if (w[b].w != turn) {
-            const long long tw = clock64();
-            do {
-              if (clock64() - tw > budget) {
-                flag_status(status, ST_TIMEOUT);
-                ok = false;
-                break;
-              }
-              w[b] = ld_word(base + static_cast<size_t>(c0 + b * KS_E) * KS_WORDS);
-            } while (w[b].w != turn);
-            if (!ok) break;  // one budget per thread, whatever else is missing
-          }
           t3[0] += __uint_as_float(w[b].x);
           t3[1] += __uint_as_float(w[b].y);
           t3[2] += __uint_as_float(w[b].z);

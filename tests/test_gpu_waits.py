@@ -34,6 +34,16 @@ def test_lost_arrival_times_out_and_context_survives(lib, kind):
     assert abs(rg - ro) <= 1e-4 * ro
 
 
+def test_both_grid_wide_waits_run_out(lib):
+    """Kind 1 runs the waits that the cooperative kernels use, the counting grid
+    barrier and the tagged word, and each records its own time-out (words 1 and 2)."""
+    L = _lib.lib()
+    ws = torch.empty(L.dlsh_selftest_workspace_size(), dtype=torch.uint8, device="cuda")
+    rc = L.dlsh_selftest_bounded_wait(1, 2_000_000, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
+    assert rc == DLSH_ERR_TIMEOUT, (rc, L.dlsh_last_error())
+    assert ws.view(torch.int32)[:3].tolist() == [1, 1, 1]
+
+
 def test_bad_arguments_rejected(lib):
     L = _lib.lib()
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
