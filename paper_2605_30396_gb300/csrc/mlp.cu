@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
   double* lsum = reinterpret_cast<double*>(smem + 4 * GN * 4);
   if (ok) {
     unsigned long long tgt = 0;  // EPI_BCE: bit c = column n0 + 64 h + c is a target of the row
-    float lh = 0.f, ll = 0.f;    // the row's loss, float-float
+    double loss = 0.0;           // EPI_BCE: the row's, over the thread's columns
     if (EPI == EPI_BCE && row < g.M) {
       int nz = g.nnz[row];
       nz = nz > g.s ? g.s : nz;
@@ -316,16 +316,18 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
       if (EPI == EPI_BCE) {
         // BCE(z, y) = max(y ? -z : z, 0) + log(1 + e^-|z|); the group's logs are
         // taken once, of the float-float product of its 1 + e^-|z| (at most
-        // 2^32), each 1 + e^-|z| exact as a pair.  1 / (1 + e^-z) is the
-        // hardware reciprocal after one Newton step.
+        // 2^32), each 1 + e^-|z| exact as a pair, and the max terms are summed in
+        // float-float.  1 / (1 + e^-z) is the hardware reciprocal after one Newton
+        // step (__frcp_rn gives the same gradients and takes 5 % longer over the
+        // call).  A NaN logit leaves a NaN in the gradient and in the loss.
         const unsigned y32 = static_cast<unsigned>(tgt >> (32 * cg));
-        float ph = 1.f, pl = 0.f;
+        float ph = 1.f, pl = 0.f, lh = 0.f, ll = 0.f;
         auto elem = [&](int k, float bias) {
           const float z = add_bias(v[k], bias);
           const bool y = (y32 >> k) & 1u;
-          const float e = expf(-z), d = fminf(1.f + e, 1e37f);
-          float r = rcp_approx(d);
-          r = fmaf(r, fmaf(-d, r, 1.f), r);
+          const float e = expf(-z), d = 1.f + e, r0 = rcp_approx(d);
+          // (an infinite d keeps the 0, a NaN the NaN)
+          const float r = d < 1e37f ? fmaf(r0, fmaf(-d, r0, 1.f), r0) : r0;
           v[k] = (r - (y ? 1.f : 0.f)) * g.inv_bk;
           const float q = z < 0.f ? rcp_approx(e) : e;  // e^-|z|
           const float f = 1.f + q, fl = q - (f - 1.f);
@@ -347,7 +349,25 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
             else v[k] = 0.f;
           }
         }
-        ll += logf(ph) + __fdividef(pl, ph);
+        const float logs = logf(ph) + __fdividef(pl, ph);
+        double sum = static_cast<double>(lh) + static_cast<double>(ll + logs);
+        // infinite logits, or a sum beyond FP32's range: from the accumulators again, in FP64
+        if (__any_sync(0xffffffffu, !(lh < INFINITY))) {
+          double lin = 0.0;
+#pragma unroll 1
+          for (int c0 = 0; c0 < 32; c0 += 16) {
+            float w[16];
+            tmem_ld16(tmem + (static_cast<uint32_t>(q4 * 32) << 16) + cb + c0, w);
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+              if (row < g.M && col + c0 + k < P.N) {
+                const float z = add_bias(w[k], __ldg(g.bias + col + c0 + k));
+                lin += fmaxf((y32 >> (c0 + k)) & 1u ? -z : z, 0.f);
+              }
+          }
+          if (!(lh < INFINITY)) sum = lin + static_cast<double>(logs);
+        }
+        loss += sum;
       } else {
         float4 z4[8];
 #pragma unroll
@@ -366,7 +386,7 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
       csum[q4 * GN + cb + lane] = col_sums(v);
     }
     if (EPI == EPI_BCE) {
-      double l = static_cast<double>(lh) + static_cast<double>(ll);
+      double l = loss;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
       if (lane == 0) lsum[warp] = l;

@@ -114,6 +114,57 @@ def test_gradients_ragged_shapes(lib, B, K, s):
     assert np.abs(gd["W1"][:, 45:]).max() == 0.0
 
 
+@pytest.mark.parametrize("bias", ["nan", "inf", "-inf", "huge"])
+def test_gradients_of_logits_beyond_the_finite(lib, bias):
+    """Biases that make whole columns of logits NaN, infinite, or so large that 32 of
+    them leave FP32's range: a NaN stays one in its bias and weight gradients and in
+    the loss, an infinite logit saturates (sigmoid 0 or 1) and makes the loss
+    infinite only where it misses its target, and large ones keep the FP64 mean."""
+    B, K, s = 200, 100, 3
+    p = _params(K, 80)
+    X = synth.signals(B, synth.hidden_dictionary(K, 81), 4, 82)
+    rng = np.random.default_rng(83)
+    idx = 64 + synth.distinct_supports(rng, B, K - 64, s)  # atoms below 64 are never targets
+    hit = 64
+    b3 = np.array(p["b3"], dtype=np.float64)
+    cols = {"nan": [7], "inf": [3, 40], "-inf": [5, hit], "huge": list(range(64))}[bias]
+    b3[cols] = {"nan": np.nan, "inf": np.inf, "-inf": -np.inf, "huge": 2e38}[bias]
+    assert (idx == hit).any()
+    net = lib.MLP(K, {**p, "b3": b3.astype(np.float32)})
+    g, loss = net.gradients(torch.from_numpy(X), torch.from_numpy(idx.astype(np.int16)).cuda(),
+                            torch.full((B,), s, dtype=torch.uint8, device="cuda"))
+    gd = lib.mlp_unpack(g, K)
+    db3, dW3 = np.asarray(gd["b3"]), np.asarray(gd["W3"])
+    other = np.setdiff1d(np.arange(K), cols)
+    assert np.isfinite(db3[other]).all() and np.isfinite(dW3[other]).all()
+    if bias == "nan":
+        assert np.isnan(db3[cols]).all() and np.isnan(dW3[cols]).all() and np.isnan(loss)
+    elif bias == "huge":
+        # sigmoid 1 for 64 of 100 columns; the rest of the loss is below its rounding
+        np.testing.assert_allclose(db3[cols], 1.0 / K, rtol=1e-5)
+        np.testing.assert_allclose(loss, 0.64 * float(np.float32(2e38)), rtol=1e-6)
+    elif bias == "inf":
+        np.testing.assert_allclose(db3[cols], 1.0 / K, rtol=1e-5)
+        assert loss == np.inf
+    else:
+        np.testing.assert_allclose(db3[cols], [0.0, -(idx == hit).sum() / (B * K)], rtol=1e-5)
+        assert loss == np.inf
+
+
+def test_sigmoid_of_the_gradient_is_rounded_as_a_division(lib):
+    """Zero weights and one signal: the logits are the biases, and K db3 the sigmoids
+    (K = 2048, a power of two).  1 / (1 + exp(-z)) in FP32 with CUDA's bounds of 2 ulp
+    for expf, half for the sum and 1 for the reciprocal: 3.5 ulp relative to FP64."""
+    K = 2048
+    b3 = np.linspace(-80.0, 80.0, K).astype(np.float32)
+    p = {k: np.zeros_like(v) for k, v in _params(K, 1).items()}
+    net = lib.MLP(K, {**p, "b3": b3})
+    g, _ = net.gradients(torch.ones((1, 45)), torch.zeros((1, 1), dtype=torch.int16, device="cuda"),
+                         torch.zeros(1, dtype=torch.uint8, device="cuda"))
+    got = np.asarray(lib.mlp_unpack(g, K)["b3"], dtype=np.float64) * K
+    np.testing.assert_allclose(got, 1.0 / (1.0 + np.exp(-b3.astype(np.float64))), rtol=3.5 * 2.0**-23)
+
+
 def test_adam_step_matches_oracle(lib):
     K, B, s = 128, 512, 4
     p = _params(K, 8)
