@@ -464,8 +464,20 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Red
     n = a.tiles;
   }
   float g = 0.f;
+  if (stride == a.zstride) {
 #pragma unroll 8
-  for (int z = 0; z < n; ++z) g += src[z * stride];
+    for (int z = 0; z < n; ++z) g += src[z * stride];
+  } else {  // eight sums side by side: a hundred tiles in a row would cost a bias gradient a bit
+    float p[8] = {};
+    int z = 0;
+    for (; z + 8 <= n; z += 8)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) p[u] += src[(z + u) * stride];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (z + u < n) p[u] += src[(z + u) * stride];
+    g = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+  }
   if (!ADAM) {
     a.G[i] = g;
     return;

@@ -151,6 +151,23 @@ def test_gradients_of_logits_beyond_the_finite(lib, bias):
         assert loss == np.inf
 
 
+def test_bias_gradient_of_a_large_batch(lib):
+    """db3 over 16,384 rows against FP64 sums of the kernel's own logits.  Tiles of 128
+    rows are summed in seven levels (rounding errors that average out over 128
+    tiles), and the tiles' sums in eight sequences of 16 and three levels: 2^-23 in
+    the norm, where one FP32 sequence of the 128 tiles has 1.7e-7."""
+    B, K, s = 16_384, 2048, 8
+    p = _params(K, 0, 3.0)
+    X = torch.from_numpy(synth.signals(B, synth.hidden_dictionary(K, 0), 4, 1)).cuda()
+    idx = torch.from_numpy(synth.distinct_supports(np.random.default_rng(0), B, K, s).astype(np.int64)).cuda()
+    net = lib.MLP(K, p)
+    g, _ = net.gradients(X, idx.to(torch.int16), torch.full((B,), s, dtype=torch.uint8, device="cuda"))
+    dz = torch.sigmoid(net.forward(X).double())
+    dz.scatter_add_(1, idx, torch.full(idx.shape, -1.0, dtype=torch.float64, device="cuda"))
+    ref = dz.sum(dim=0) / (B * K)
+    assert float((g[-K:].double() - ref).norm() / ref.norm()) < 2.0**-23
+
+
 def test_sigmoid_of_the_gradient_is_rounded_as_a_division(lib):
     """Zero weights and one signal: the logits are the biases, and K db3 the sigmoids
     (K = 2048, a power of two).  1 / (1 + exp(-z)) in FP32 with CUDA's bounds of 2 ulp
