@@ -409,7 +409,10 @@ int dlsh_decode_compact(const float* D, int K, int d, const void* idx, int idx_b
  * fit beside the shared-memory dictionary, three quarters and half of that;
  * 32, 24 and 16 where rows are read through the read-only cache), and records
  * the fastest for (format, K, s); later dlsh_decode / dlsh_decode_compact calls
- * of that shape use it.  The colours do not depend on the choice.
+ * of that shape use it.  The colours do not depend on the choice.  (FP32 codes
+ * with about 1150 < K <= 2500 and s >= 8: calls of 1.5 million code slots or more
+ * run another kernel than shorter ones, and a sample tunes the one that a call of
+ * its size runs.)
  *   format 0: dlsh_decode's codes (idx uint16, coef FP32);
  *          1 / 2: compact codes with 8- / 16-bit indices and FP16 coef.
  * rgb (N x 3, device) is scratch; the DC term is not applied.  *best_batch and
@@ -425,6 +428,8 @@ int dlsh_autotune_decode(const float* D, int K, int d, const void* idx, const vo
  * dlsh_autotune_decode: returns 1 and sets *batch and *warps (host, may be
  * NULL) if one is recorded, else 0 (also for arguments out of range).  A
  * record that no longer fits beside the dictionary is ignored by the decode.
+ * Where long and short calls run different kernels, the long ones' record if
+ * there is one, else the short ones'.
  * Host only (no GPU work). */
 int dlsh_tuned_decode(int format, int K, int s, int* batch, int* warps);
 

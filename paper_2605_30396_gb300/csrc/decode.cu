@@ -615,10 +615,15 @@ static int launch_decode(const float* D, int K, const void* idx, const void* coe
 // codes, and so do the few warps beside a larger plane (1M Gaussians, rows / planes:
 // K = 2048, s = 3 89 / 105 us, s = 4 102 / 100 and with uneven codes 90 / 117, s = 8
 // 182 / 137 and 142 / 136; K = 2500, s = 8 182 / 142 and 143 / 142; K = 3100, s = 8
-// 182 / 238).
-static int decode_format(int K, int s) {
+// 182 / 238).  Staging three planes on every SM takes about 28 us, so that short
+// calls read the rows through the read-only cache too (K = 2048, rows / planes: N =
+// 262k, s = 4 31 / 33; N = 131k, s = 16 55 / 35).  At 1.5 million code slots the
+// planes are the faster ones from K = 1160 to 2490 and s = 8 to 16, by 1.02 (N =
+// 300k, K = 2490, s = 8, uneven codes: 46 / 45) to 1.7.
+static int decode_format(int K, int s, int64_t N) {
   if (dec::fit_warps(dec::FM_F32, K, s) >= 6) return dec::FM_F32;
-  return s >= 8 && K <= 2500 && dec::fit_warps(dec::FM_PLANE, K, s) >= 8 ? dec::FM_PLANE : dec::FM_GLOBAL;
+  return s >= 8 && K <= 2500 && N * s >= 1500000 && dec::fit_warps(dec::FM_PLANE, K, s) >= 8 ? dec::FM_PLANE
+                                                                                            : dec::FM_GLOBAL;
 }
 
 // Shared with the bench / learn paths: enqueue one decode.
@@ -629,11 +634,7 @@ int decode_enqueue(const float* D, int K, const uint16_t* idx, const float* coef
   int rc = upload_constants(st);
   if (rc) return rc;
   if (N == 0) return DLSH_OK;
-  int fm = decode_format(K, s);
-  // staging three planes on every SM takes about 28 us: short calls read the rows
-  // through the read-only cache instead (K = 2048, us: N = 262k, s = 4 33 by
-  // planes, 31 so; N = 131k, s = 16 35 and 55)
-  if (fm == FM_PLANE && N * s < 1500000) fm = FM_GLOBAL;
+  const int fm = decode_format(K, s, N);
   int gb = 0, nw = 0;
   decode_shape(fm, K, s, &gb, &nw);
   if (fm == FM_PLANE)
@@ -738,11 +739,17 @@ extern "C" int dlsh_tuned_decode(int format, int K, int s, int* batch, int* warp
   using namespace dlsh;
   using namespace dlsh::dec;
   if (format < 0 || format > 2 || K < 1 || K > DLSH_MAX_K || s < 1 || s > DLSH_MAX_S) return 0;
-  const int fm = format == 0 ? decode_format(K, s) : (format == 1 ? FM_C8 : FM_C16);
-  char key[64];
-  snprintf(key, sizeof(key), "decode f=%d K=%d s=%d", fm, K, s);
+  // FP32 codes: long and short calls may run different kernels; the long ones' record first
+  const int64_t sizes[2] = {INT64_MAX / DLSH_MAX_S, 1};
   int v[2] = {0, 0};
-  if (!tune_get(key, v, 2)) return 0;
+  bool found = false;
+  for (int i = 0; i < 2 && !found; ++i) {
+    const int fm = format == 0 ? decode_format(K, s, sizes[i]) : (format == 1 ? FM_C8 : FM_C16);
+    char key[64];
+    snprintf(key, sizeof(key), "decode f=%d K=%d s=%d", fm, K, s);
+    found = tune_get(key, v, 2);
+  }
+  if (!found) return 0;
   if (batch) *batch = v[0];
   if (warps) *warps = v[1];
   return 1;
@@ -768,7 +775,7 @@ extern "C" int dlsh_autotune_decode(const float* D, int K, int d, const void* id
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = upload_constants(st);
   if (rc) return rc;
-  const int fm = format == 0 ? decode_format(K, s) : (format == 1 ? FM_C8 : FM_C16);
+  const int fm = format == 0 ? decode_format(K, s, N) : (format == 1 ? FM_C8 : FM_C16);
   const char* call = "dlsh_autotune_decode";
   auto run = [&](int gb, int nw) -> int {
     switch (fm) {

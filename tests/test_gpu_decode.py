@@ -1,4 +1,9 @@
 """Step a6: radiance from sparse codes vs the oracle's dense SH evaluation of D alpha."""
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -8,6 +13,7 @@ from oracle import sh as osh
 from paper_2605_30396_gb300 import synth
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _codes(rng, N, K, s, ragged=True):
@@ -169,6 +175,29 @@ def test_decode_full_colour_with_dc(lib, compact):
     assert (ref == 0).any() and (ref > 0).any()
     ok, worst = close_rel(rgb, ref)
     assert ok, worst
+
+
+def test_decode_autotune_tunes_the_kernel_that_runs(lib, tmp_path):
+    """K = 1500, s = 16 on both sides of 1.5 million code slots: a short sample tunes
+    the rows (internal format 1: up to 32 warps, whatever fits beside a plane), a long
+    one the planes (format 4), each with colours bitwise as before."""
+    cache = tmp_path / "tune.jsonl"
+    cache.write_text("")
+    code = ["import sys, numpy as np, torch", "sys.path[:0] = [%r, %r]" % (ROOT, ROOT + "/tests"),
+            "from paper_2605_30396_gb300 import api, synth", "from test_gpu_decode import _codes",
+            "D = torch.from_numpy(synth.hidden_dictionary(1500, 5).astype(np.float32)).cuda()",
+            "for N in (5000, 94000):",
+            "    idx, coef, nnz = _codes(np.random.default_rng(N), N, 1500, 16)",
+            "    a = [torch.from_numpy(x).cuda() for x in (idx.astype(np.int16), coef, nnz)]",
+            "    v = torch.from_numpy(synth.unit_directions(N, 6)).cuda()",
+            "    before = api.decode(D, *a, dirs=v, sync=True)",
+            "    api.autotune_decode(D, *a, dirs=v)",
+            "    assert torch.equal(api.decode(D, *a, dirs=v, sync=True), before)"]
+    out = subprocess.run([sys.executable, "-c", "\n".join(code)], env=dict(os.environ, DLSH_AUTOTUNE_CACHE=str(cache)),
+                         capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr
+    keys = {json.loads(line)["key"] for line in cache.read_text().splitlines() if line.strip()}
+    assert keys == {"decode f=1 K=1500 s=16", "decode f=4 K=1500 s=16"}
 
 
 @pytest.mark.parametrize("K,s,compact", [(1024, 8, False), (2048, 8, False), (1024, 8, True), (200, 4, True)])

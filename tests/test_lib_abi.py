@@ -189,6 +189,33 @@ def test_tuning_table_read_from_the_cache_file(tmp_path):
     assert got[4:] == [1, 16, 14, 1, 8, 21, 0, 0], got
 
 
+def test_tuned_decode_where_long_and_short_calls_differ(tmp_path):
+    """FP32 codes at K = 2048 and s >= 8: long calls decode by channel planes, short
+    ones by rows.  The query reports the rows' record if there is no other, and the
+    planes' before it; elsewhere there is one kernel.  In a child process, as above."""
+    import subprocess
+    import sys
+    cache = tmp_path / "tune.jsonl"
+    cache.write_text('{"key": "decode f=1 K=2048 s=16", "values": [8, 24]}\n'
+                     '{"key": "decode f=1 K=2048 s=8", "values": [8, 32]}\n'
+                     '{"key": "decode f=4 K=2048 s=8", "values": [16, 9]}\n'
+                     '{"key": "decode f=1 K=4000 s=8", "values": [16, 30]}\n')
+    code = (
+        "import ctypes, sys\n"
+        "sys.path.insert(0, %r)\n"
+        "from paper_2605_30396_gb300 import _lib\n"
+        "L = _lib.lib()\n"
+        "b, w, r = ctypes.c_int(0), ctypes.c_int(0), []\n"
+        "for K, s in ((2048, 16), (2048, 8), (4000, 8), (2048, 12)):\n"
+        "    ok = L.dlsh_tuned_decode(0, K, s, ctypes.byref(b), ctypes.byref(w))\n"
+        "    r.append((ok, b.value, w.value) if ok else 0)\n"
+        "print(r)\n" % ROOT)
+    env = dict(os.environ, DLSH_AUTOTUNE_CACHE=str(cache))
+    out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr
+    assert eval(out.stdout.strip().splitlines()[-1]) == [(1, 8, 24), (1, 16, 9), (1, 16, 30), 0]
+
+
 def test_binding_refuses_host_tensors_for_device_arguments():
     import torch
 
