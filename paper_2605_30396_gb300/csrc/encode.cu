@@ -291,16 +291,20 @@ static int default_variant(bool split16_ok, bool alt_ok, bool pair_lowp_ok, bool
 // eight have enough chunks to select from meanwhile.  Measured, one tile / two:
 //   tiles of 64 fill no SM twice (N = 3000, s = 16): K = 98 110 / 92 us, K = 2048
 //   409 / 311: always two;
-//   tiles of 128 fill no SM twice (N = 18,000): a tile of 128 per SM competes with
-//   two of 64.  K = 256 138 / 150, K = 512 195 / 174, K = 2048 406 / 450 (s = 16),
-//   K = 1024 137 / 141 (s = 9): between 256 and 1024;
+//   tiles of 128 fill no SM twice (N = 14,000): a tile of 128 per SM competes with
+//   two of 64, which pays for long codes and neither the smallest nor the largest
+//   dictionaries.  s = 16: K = 256 131 / 150, 300 166 / 160, 512 187 / 175, 700 224 /
+//   204, 1024 260 / 245, 1200 291 / 291, 2048 400 / 449; s = 13: K = 300 115 / 120,
+//   512 140 / 132, 700 170 / 160, 1024 200 / 199, 1200 225 / 238; s = 12: K = 300 104 /
+//   108, 512 117 / 119, 700 154 / 147, 1000 181 / 184; s = 10: K = 300 82 / 86, 700 121 /
+//   123, 1000 148 / 156;
 //   more (N = 200,000): K = 256 1369 / 1485, K = 512 1939 / 1605, K = 2048 3933 / 2534
 //   (s = 16), K = 256 606 / 640, K = 512 823 / 693 (s = 9): from three chunks on.
 static bool deep_pays(int K, int s, int64_t N, const long long* n_dev) {
   if (s <= 8) return false;
   const int sms = device_sm_count();
   if (!n_dev && N <= static_cast<int64_t>(64) * sms) return true;
-  if (!n_dev && N <= static_cast<int64_t>(enc::TILE_M) * sms) return K > 256 && K < 1024;
+  if (!n_dev && N <= static_cast<int64_t>(enc::TILE_M) * sms) return K > 256 && (s > 12 ? K <= 1024 : s == 12 && K < 1024);
   return K > 256;
 }
 
