@@ -308,6 +308,11 @@ static bool deep_pays(int K, int s, int64_t N, const long long* n_dev) {
   return K > 256;
 }
 
+// The two-tile plan of variant 7, if that is what runs for these sizes.
+static bool deep_plan(int K, int s, int prec, int64_t N, const long long* n_dev, enc::SplitPlan& p) {
+  return deep_pays(K, s, N, n_dev) && enc::make_split_plan(K, s, prec, p, true, 2, enc::SMEM_LIMIT, true) == DLSH_OK;
+}
+
 // Entry points shared with the learning loop (learn.cu).
 int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, float eps, int prec,
                    uint16_t* idx, float* coef, uint8_t* nnz, float* resid_sq, void* ws,
@@ -352,8 +357,8 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
   cap_ring(sp16, cap, 2);
   cap_ring(sp16x3, cap, 2);
   SplitPlan deep;
-  const bool use_deep =
-      choice == 7 && deep_pays(K, s, N, n_dev) && make_split_plan(K, s, prec, deep, true, 2, SMEM_LIMIT, true) == DLSH_OK;
+  const bool use_deep = choice == 7 && deep_plan(K, s, prec, N, n_dev, deep);
+  if (use_deep) cap_ring(deep, cap, 2);
   if ((choice >= 3 && choice <= 6) || use_deep) {
     Plan p;  // the one-tile encoder's 128-atom FP32 operand image
     if (use_deep) p = p16;
@@ -742,7 +747,9 @@ extern "C" int dlsh_autotune_encode(const float* D, int K, int d, const float* X
     if (best == 0 || ms < best_ms) {
       best = bn;
       best_ms = ms;
-      best_stages = bn == 2 ? pp.stages : bn == 3 ? ap.stages : (bn >= 4 && bn <= 6) ? sp.stages : p.stages;
+      // (variant 7 on two tiles has a ring of its own, of the two stages that fit)
+      if (bn == 7 && deep_plan(K, s, precision, N, nullptr, sp)) best_stages = sp.stages;
+      else best_stages = bn == 2 ? pp.stages : bn == 3 ? ap.stages : (bn >= 4 && bn <= 6) ? sp.stages : p.stages;
       min_stages = bn == 2 ? 3 : 2;
     }
   }

@@ -80,3 +80,19 @@ def test_ring_stage_cap_keeps_codes(lib, prec, v, cap, K):
     got = lib.encode_multi([sc], precision=prec, bn=v + 256 * cap, sync=True)[0]
     for a, b in zip(got, ref):
         np.testing.assert_array_equal(a.cpu().numpy(), b.cpu().numpy())
+
+
+def test_ring_of_long_codes(lib):
+    """s = 16: variant 7 runs on two tiles per CTA at N = 5003, K = 1024, whose ring has
+    two stages whatever the cap, and on one tile at K = 200, N = 12,000.  The codes are
+    bitwise those of the full ring, and a sample that runs on two tiles records no
+    cap (there is no shallower ring to time)."""
+    for N, K in ((5003, 1024), (12_000, 200)):
+        sc = _scene(22, N, K, 16)
+        ref = lib.encode_multi([sc], bn=7, sync=True)[0]
+        got = lib.encode_multi([sc], bn=7 + 256 * 2, sync=True)[0]
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b), (N, K)
+    sc = _scene(23, 5003, 1000, 16)
+    bn = lib.autotune_encode(sc["D"], sc["X"], 16)
+    assert bn & 255 != 7 or bn >> 8 == 0, bn
