@@ -452,7 +452,7 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
     // pays with at least four chunks to select from, or with a tile per SM at most
     // (200,000 signals, BF16, s = 4, groups / split: K = 98 297 / 313 us, K = 192 335 /
     // 340, K = 256 354 / 350; 1M, K = 98, s = 2 618 / 719; 18,000, K = 98, s = 2 44 / 40)
-    const bool groups = pp.prec == 0 || (pp.nchunks < 4 && (n_dev || ntiles > sms));
+    const bool groups = pp.prec == 0 || pp.off_row[0] == 0 || (pp.nchunks < 4 && (n_dev || ntiles > sms));
     // two tiles in flight per CTA; split, a tile of its own for each SM while they
     // last (the groups are made for two tiles: half as many CTAs)
     const int want = groups ? (ntiles + 1) / 2 : ntiles;

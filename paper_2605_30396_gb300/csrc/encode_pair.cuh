@@ -32,7 +32,7 @@ struct PairPlan {
   int prec, top4, ib, K, Kp, nchunks, stages, s;
   uint32_t chunk_bytes, a_bytes;
   uint32_t off_a[2], off_L[2], off_sel[2], off_y[2], off_g[2], off_idg[2], off_cand[2], off_r[2];
-  uint32_t off_row[2];  // encode_lowp_kernel: per-row state of the two tile slots
+  uint32_t off_row[2];  // encode_lowp_kernel: per-row state of the two tile slots (0: no room, two groups only)
   uint32_t off_sig, off_ring, off_bar, smem;
 };
 
@@ -54,7 +54,9 @@ struct PairArgs {
   PairPlan p;
 };
 
-inline int make_pair_plan(int K, int s, int code, PairPlan& p, int smem_limit = SMEM_LIMIT) {
+// row_state: with room for encode_lowp_kernel's per-row state.  Without it FP8
+// plans reach 1024 atoms further (K = 18,944), on the two-group kernel.
+inline int make_pair_plan(int K, int s, int code, PairPlan& p, int smem_limit = SMEM_LIMIT, bool row_state = true) {
   if (s > 8) return DLSH_ERR_UNSUPPORTED;
   const int prec = operand_precision(code, &p.top4);
   p.prec = prec;
@@ -83,15 +85,15 @@ inline int make_pair_plan(int K, int s, int code, PairPlan& p, int smem_limit = 
     p.off_idg[g] = take(8 * TILE_M * 4);
     p.off_cand[g] = take(p.top4 ? TILE_M * 2 * 4 * 4 : TILE_M * 2 * 8);
     p.off_r[g] = take(prec == 0 ? 0 : PGT * 24 * 4);
-    p.off_row[g] = take(prec == 0 ? 0 : 3 * TILE_M * 4);
+    p.off_row[g] = prec == 0 || !row_state ? 0 : take(3 * TILE_M * 4);
   }
   p.off_sig = take(prec == 2 ? p.Kp * 4 : 0);
   p.off_bar = take(1024);
   const uint32_t fixed = (off + 1023u) & ~1023u;
-  if (fixed >= static_cast<uint32_t>(smem_limit)) return DLSH_ERR_UNSUPPORTED;
-  int fit = static_cast<int>((smem_limit - fixed) / p.chunk_bytes);
+  int fit = fixed < static_cast<uint32_t>(smem_limit) ? static_cast<int>((smem_limit - fixed) / p.chunk_bytes) : 0;
   if (fit > 32) fit = 32;
-  if (fit < 3) return DLSH_ERR_UNSUPPORTED;
+  if (fit < 3)
+    return prec != 0 && row_state ? make_pair_plan(K, s, code, p, smem_limit, false) : DLSH_ERR_UNSUPPORTED;
   p.stages = fit;
   p.off_ring = fixed;
   p.smem = fixed + p.stages * p.chunk_bytes;

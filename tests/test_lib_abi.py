@@ -241,3 +241,12 @@ def test_encode_variant_choice(L):
     assert L.dlsh_encode_variant(0, 8, 0) == 0
     assert L.dlsh_encode_variant(1024, 0, 0) == 0
     assert L.dlsh_encode_variant(1024, 8, 5) == 0
+
+
+def test_encode_variant_of_the_largest_fp8_dictionaries(L):
+    """FP8 on two tiles per CTA up to K = 18,944 (19,968 with one candidate per half row):
+    beyond 17,920 (18,944) only the two-group kernel has room, and it serves them."""
+    for prec, k_rows, k_last in ((2, 17_920, 18_944), (4, 18_944, 19_968)):
+        for K in (k_rows, k_rows + 1, k_last):
+            assert L.dlsh_encode_variant(K, 8, prec) == 2, (prec, K)
+        assert L.dlsh_encode_variant(k_last + 1, 8, prec) == 1
