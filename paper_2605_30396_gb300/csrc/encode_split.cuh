@@ -303,11 +303,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) encode_split_kernel(const __grid_
             }
           }
           if (!ok) break;
-          // this thread's candidate: the better group, ties to the smaller column
+          // this thread's candidate: the better group, ties to the smaller column (with
+          // more than 8 atoms, a group whose largest key is a NaN gives way, as one of
+          // the four quarters does in the one-tile kernel)
           const float v0 = __uint_as_float(b0 & ~31u), v1 = __uint_as_float(b1 & ~31u);
           const int j0 = c0 * ABN + h * 64 + 31 - static_cast<int>(b0 & 31u);
           const int j1 = c1 * ABN + h * 64 + 32 + 31 - static_cast<int>(b1 & 31u);
-          const bool second = v1 > v0 || (v1 == v0 && j1 < j0);
+          const bool second = v1 > v0 || (v1 == v0 && j1 < j0) || (CD && v0 != v0);
           const long long W1 = prof_on ? clock64() : 0;
           if (!mbar_wait(&cand_empty[t], (epar >> t) & 1u, a.budget)) {
             flag_status(a.status, ST_TIMEOUT);

@@ -264,6 +264,32 @@ def test_small_calls_match_large_ones(lib, K, s, prec):
             assert torch.equal(a, b[:N]), N
 
 
+@pytest.mark.parametrize("K,s", [(200, 12), (64, 16)])
+def test_long_codes_around_atoms_without_a_correlation(lib, K, s):
+    """s > 8 with atoms that hold a NaN, an infinity, or values beyond the FP16 parts
+    (each takes its 32 columns out of the selection): a call of half tiles, two per
+    CTA, and one of a whole tile per CTA on the one-tile kernel give the same bits,
+    and most signals still get codes."""
+    D = synth.hidden_dictionary(K, 1).astype(np.float32)
+    D[3], D[5, 2], D[7, 1], D[9] = 0.0, np.nan, np.inf, D[9] * 1e30
+    Dt = torch.from_numpy(D).cuda()
+    X = torch.from_numpy(synth.signals(14_000, synth.hidden_dictionary(K, 2), 8, 3)).cuda()
+    whole = lib.encode(Dt, X, s, sync=True)
+    part = lib.encode(Dt, X[:3000].contiguous(), s, sync=True)
+    for a, b in zip(part, whole):
+        a, b = a.cpu().numpy(), b[:3000].cpu().numpy()
+        np.testing.assert_array_equal(a, b)
+    assert (part[2].cpu().numpy() > 0).mean() > 0.9
+
+
+@pytest.mark.parametrize("N,K,s,eps", [(100_003, 300, 12, 0.2), (45_000, 1024, 9, 0.0), (79_000, 640, 16, 0.3)])
+def test_long_codes_over_several_rounds(lib, N, K, s, eps):
+    """s > 8 on whole tiles, two per CTA, K > 256 and more than 256 signals per SM (one to
+    three rounds per CTA, ragged last tiles, tolerance stops), with the bounds of the
+    test below."""
+    test_codes_of_nine_to_sixteen_atoms(lib, N, K, s, eps)
+
+
 @pytest.mark.parametrize("N,K,s,eps", [(40_000, 129, 9, 0.0), (2500, 640, 13, 0.3), (300, 2048, 16, 0.0),
                                        (20_100, 64, 16, 0.05)])
 def test_codes_of_nine_to_sixteen_atoms(lib, N, K, s, eps):
