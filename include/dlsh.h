@@ -198,7 +198,8 @@ int dlsh_correlate(const float* D, int K, int d, const float* R, int64_t M,
  * the output is the view-dependent part only (the DC term is not part of the
  * dictionary); with dc [N*3] (device, the DC SH coefficient of each channel)
  * it is the full colour max(0, Y00 dc + view-dependent part + 0.5),
- * Y00 = 1/(2 sqrt(pi)).  No workspace.
+ * Y00 = 1/(2 sqrt(pi)).  rgb may be dirs_or_means or dc itself (written in
+ * place).  No workspace.
  */
 int dlsh_decode(const float* D, int K, int d, const uint16_t* idx,
                 const float* coef, const uint8_t* nnz, int s, int64_t N,

@@ -634,7 +634,12 @@ int decode_enqueue(const float* D, int K, const uint16_t* idx, const float* coef
   int rc = upload_constants(st);
   if (rc) return rc;
   if (N == 0) return DLSH_OK;
-  const int fm = decode_format(K, s, N);
+  int fm = decode_format(K, s, N);
+  // colours written over the directions: a warp of the other kernels has read all of
+  // its batch before it writes, but a plane's CTAs read what two other channels' write
+  const uintptr_t in = reinterpret_cast<uintptr_t>(dm), out = reinterpret_cast<uintptr_t>(rgb);
+  const uintptr_t bytes = static_cast<uintptr_t>(N) * 3 * sizeof(float);
+  if (fm == FM_PLANE && in < out + bytes && out < in + bytes) fm = FM_GLOBAL;
   int gb = 0, nw = 0;
   decode_shape(fm, K, s, &gb, &nw);
   if (fm == FM_PLANE)

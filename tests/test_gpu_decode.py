@@ -177,6 +177,26 @@ def test_decode_full_colour_with_dc(lib, compact):
     assert ok, worst
 
 
+@pytest.mark.parametrize("N,K,s", [(3001, 256, 8), (3001, 2048, 8), (120_000, 2048, 16), (200_003, 1500, 8)])
+def test_decode_in_place(lib, N, K, s):
+    """Colours over the directions, and over the DC colours, by the table in shared
+    memory, by rows, and at sizes that decode by channel planes: as into a buffer of
+    their own (up to the order of the sums, with the file's relative tolerance)."""
+    D = torch.from_numpy(synth.hidden_dictionary(K, 5).astype(np.float32)).cuda()
+    codes = [torch.from_numpy(a).cuda() for a in _codes(np.random.default_rng(N), N, K, s)]
+    codes[0] = codes[0].to(torch.int16)
+    dirs = torch.from_numpy(synth.unit_directions(N, 6).astype(np.float32)).cuda()
+    dc = torch.from_numpy(np.random.default_rng(8).standard_normal((N, 3)).astype(np.float32)).cuda()
+    for inputs in ({"dirs": dirs}, {"dirs": dirs, "dc": dc}):
+        ref = lib.decode(D, *codes, **inputs, sync=True).cpu().numpy()
+        for name in inputs:
+            mine = {k: v.clone() for k, v in inputs.items()}
+            got = lib.decode(D, *codes, **mine, out=mine[name], sync=True)
+            assert got.data_ptr() == mine[name].data_ptr()
+            ok, worst = close_rel(got.cpu().numpy(), ref)
+            assert ok, (name, worst)
+
+
 def test_decode_autotune_tunes_the_kernel_that_runs(lib, tmp_path):
     """K = 1500, s = 16 on both sides of 1.5 million code slots: a short sample tunes
     the rows (internal format 1: up to 32 warps, whatever fits beside a plane), a long
