@@ -27,7 +27,10 @@ __device__ __forceinline__ void flag_status(uint32_t* status, uint32_t bits) {
 // before it in the stream still runs.  depend() lets the next kernel start as
 // soon as every CTA of this one has, then waits until the kernels before this
 // one are complete and their writes visible: it comes before the first access
-// to global memory.
+// to global memory.  Such a kernel begins before what it reads is written, so that
+// it reads by plain loads through pointers without __restrict__: the read-only path
+// (__ldg, const __restrict__) is for data that does not change while a kernel
+// lives, and its loads may be moved above the wait.
 __device__ __forceinline__ void depend() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

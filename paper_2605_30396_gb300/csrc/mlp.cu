@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
       }
       if (EPI == EPI_GELU) {
 #pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = add_bias(v[k], __ldg(g.bias + col + k));
+        for (int k = 0; k < 32; ++k) v[k] = add_bias(v[k], g.bias[col + k]);
         if (row < g.M) {
           store_f32(P.C + static_cast<size_t>(row) * P.ldc + col, v);
 #pragma unroll
@@ -341,11 +341,11 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
         };
         if (row < g.M && col + 32 <= P.N) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k) elem(k, __ldg(g.bias + col + k));
+          for (int k = 0; k < 32; ++k) elem(k, g.bias[col + k]);
         } else {
 #pragma unroll
           for (int k = 0; k < 32; ++k) {
-            if (row < g.M && col + k < P.N) elem(k, __ldg(g.bias + col + k));
+            if (row < g.M && col + k < P.N) elem(k, g.bias[col + k]);
             else v[k] = 0.f;
           }
         }
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
 #pragma unroll
             for (int k = 0; k < 16; ++k)
               if (row < g.M && col + c0 + k < P.N) {
-                const float z = add_bias(w[k], __ldg(g.bias + col + c0 + k));
+                const float z = add_bias(w[k], g.bias[col + c0 + k]);
                 lin += fmaxf((y32 >> (c0 + k)) & 1u ? -z : z, 0.f);
               }
           }

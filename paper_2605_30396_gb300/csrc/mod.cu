@@ -232,7 +232,7 @@ __device__ __forceinline__ bool any_shared(T* place, bool active, T tag) {
 // ---- 1. per-tile histograms, cnt[tile][atom] -----------------------------------
 // Two 16-bit counters per word (a tile has fewer than 65,536 entries), integer
 // atomics in shared memory.
-__global__ void __launch_bounds__(256) count_kernel(const uint16_t* __restrict__ idx, const uint8_t* __restrict__ nnz,
+__global__ void __launch_bounds__(256) count_kernel(const uint16_t* idx, const uint8_t* nnz,
                                                    int s, uint32_t sdiv, int64_t N, int K, int ts,
                                                    int* __restrict__ cnt, uint32_t* status) {
   depend();
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(256) count_kernel(const uint16_t* __restrict__
   if ((reinterpret_cast<uintptr_t>(tidx) & 15u) == 0) {  // eight indices per load
     const int nv = ne / 8;
     for (int v = threadIdx.x; v < nv; v += blockDim.x) {
-      const uint4 w = __ldg(reinterpret_cast<const uint4*>(tidx) + v);
+      const uint4 w = reinterpret_cast<const uint4*>(tidx)[v];
       const unsigned u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -306,7 +306,7 @@ __device__ __forceinline__ int block_scan(int v, int* sm, int& total) {
   return before + x - v;
 }
 
-__global__ void __launch_bounds__(256) chunk_sum_kernel(const int* __restrict__ cnt, int T, int K, int segb,
+__global__ void __launch_bounds__(256) chunk_sum_kernel(const int* cnt, int T, int K, int segb,
                                                        int* __restrict__ csum, int* __restrict__ segtot) {
   depend();
   __shared__ int sm[32];
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(256) chunk_sum_kernel(const int* __restrict__ 
   if (threadIdx.x == 0) segtot[blockIdx.y * gridDim.x + blockIdx.x] = all;
 }
 
-__global__ void __launch_bounds__(1024) layout_kernel(const int* __restrict__ csum, int P, int K, int gc, int PG,
+__global__ void __launch_bounds__(1024) layout_kernel(const int* csum, int P, int K, int gc, int PG,
                                                       int nseg, int* __restrict__ segtot, int* __restrict__ atom_start,
                                                       int* __restrict__ segg_start, int* __restrict__ segb_end) {
   depend();
@@ -377,8 +377,8 @@ __global__ void __launch_bounds__(1024) layout_kernel(const int* __restrict__ cs
 }
 
 __global__ void __launch_bounds__(256) tile_offsets_kernel(int* __restrict__ cnt, int T, int K, int segb,
-                                                          const int* __restrict__ csum, const int* __restrict__ segtot,
-                                                          const int* __restrict__ atom_start, int* __restrict__ cstart,
+                                                          const int* csum, const int* segtot,
+                                                          const int* atom_start, int* __restrict__ cstart,
                                                           int* __restrict__ segb_start) {
   depend();
   __shared__ int sm[32];
@@ -422,9 +422,9 @@ inline size_t scatter_smem(int K, int s, int ts, int threads) {
   return ne * 8 + ts + 16 + kp * 2 * (threads / 32) + static_cast<size_t>(K) * 4 + 128;
 }
 template <bool SLOT>
-__global__ void __launch_bounds__(512) scatter_kernel(const uint16_t* __restrict__ idx, const float* __restrict__ coef,
-                                                      const uint8_t* __restrict__ nnz, int s, uint32_t sdiv, int64_t N,
-                                                      int K, int ts, const int* __restrict__ off,
+__global__ void __launch_bounds__(512) scatter_kernel(const uint16_t* idx, const float* coef,
+                                                      const uint8_t* nnz, int s, uint32_t sdiv, int64_t N,
+                                                      int K, int ts, const int* off,
                                                       uint2* __restrict__ list) {
   depend();
   extern __shared__ __align__(16) uint8_t scb[];
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(512) scatter_kernel(const uint16_t* __restrict
     if ((reinterpret_cast<uintptr_t>(cs) & 15u) == 0) {
       const int nv = ne / 4;
       for (int v = tid; v < nv; v += nthr)
-        reinterpret_cast<float4*>(scoef)[v] = __ldg(reinterpret_cast<const float4*>(cs) + v);
+        reinterpret_cast<float4*>(scoef)[v] = reinterpret_cast<const float4*>(cs)[v];
       done = nv * 4;
     }
     for (int e = done + tid; e < ne; e += nthr) scoef[e] = cs[e];
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(512) scatter_kernel(const uint16_t* __restrict
     if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
       const int nv = ne / 8;
       for (int v = tid; v < nv; v += nthr) {
-        const uint4 w = __ldg(reinterpret_cast<const uint4*>(src) + v);
+        const uint4 w = reinterpret_cast<const uint4*>(src)[v];
         unsigned u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -777,8 +777,8 @@ __global__ void __launch_bounds__(128) accum_g_kernel(const uint16_t* __restrict
 
 // Row j of G (entries k >= j) and column j of B: the atom's segment partials
 // summed in order, chunk (group) by chunk (group).
-__global__ void __launch_bounds__(256) seg_reduce_kernel(const int* __restrict__ segg_start, const int* __restrict__ segb_start,
-                                                        const double* __restrict__ Gp, const double* __restrict__ Bp,
+__global__ void __launch_bounds__(256) seg_reduce_kernel(const int* segg_start, const int* segb_start,
+                                                        const double* Gp, const double* Bp,
                                                         int K, int P, int PG, double* __restrict__ M,
                                                         double* __restrict__ Z) {
   depend();
@@ -821,7 +821,7 @@ static int accum_warps(int K, size_t* smem) {
 }
 
 // ---- 5a. lambda = 1e-6 trace(G)/K and the Jacobi scale 1 / sqrt(M_jj + lambda) ----
-__global__ void __launch_bounds__(1024) ridge_kernel(const double* __restrict__ M, int K, double* lam_out,
+__global__ void __launch_bounds__(1024) ridge_kernel(const double* M, int K, double* lam_out,
                                                      double* __restrict__ dsc) {
   depend();
   __shared__ double part[1024];
@@ -850,10 +850,10 @@ __device__ __forceinline__ float2 ff_split(double x) {
   return make_float2(h, static_cast<float>(x - static_cast<double>(h)));
 }
 constexpr int MT = 32;
-__global__ void __launch_bounds__(MT * 8) scale_kernel(const double* __restrict__ M, const double* __restrict__ Z,
-                                                       const float* __restrict__ D_old,
-                                                       const double* __restrict__ lamp,
-                                                       const double* __restrict__ dsc, int K, float2* __restrict__ S,
+__global__ void __launch_bounds__(MT * 8) scale_kernel(const double* M, const double* Z,
+                                                       const float* D_old,
+                                                       const double* lamp,
+                                                       const double* dsc, int K, float2* __restrict__ S,
                                                        float* __restrict__ A, float2* __restrict__ Zs,
                                                        float* __restrict__ R32, float2* __restrict__ Xs) {
   depend();
@@ -1176,7 +1176,7 @@ constexpr int PS = PKC + 4;        // row stride of the stage: the rows start on
 // FP32 solve of (L L^T) c = r with W = L^-1: y = W r (TRANS = false), then
 // c = W^T y and X += c in float-float.  W's upper triangle is zero.
 template <bool TRANS>
-__global__ void __launch_bounds__(PT) trmm_kernel(const float* __restrict__ W, int K, const float* __restrict__ in,
+__global__ void __launch_bounds__(PT) trmm_kernel(const float* W, int K, const float* in,
                                                   float* __restrict__ out, float2* __restrict__ Xs) {
   depend();
   extern __shared__ __align__(16) float psm[];  // [PR][PS], then the warps' sums
@@ -1203,7 +1203,7 @@ __global__ void __launch_bounds__(PT) trmm_kernel(const float* __restrict__ W, i
       const float4* v = reinterpret_cast<const float4*>(in + static_cast<size_t>(k0 + k) * RW + c0);
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const float4 x = __ldg(v + q);
+        const float4 x = v[q];
         acc[4 * q] = fmaf(w, x.x, acc[4 * q]);
         acc[4 * q + 1] = fmaf(w, x.y, acc[4 * q + 1]);
         acc[4 * q + 2] = fmaf(w, x.z, acc[4 * q + 2]);
@@ -1232,8 +1232,8 @@ __global__ void __launch_bounds__(PT) trmm_kernel(const float* __restrict__ W, i
 
 // Residual of the scaled system, R = Zs - S X, in float-float (products exact,
 // about 48 bits; FP64 runs at 1/64 of the FP32 rate here), as FP32.
-__global__ void __launch_bounds__(PT) residual_kernel(const float2* __restrict__ S, int K,
-                                                      const float2* __restrict__ Zs, const float2* __restrict__ Xs,
+__global__ void __launch_bounds__(PT) residual_kernel(const float2* S, int K,
+                                                      const float2* Zs, const float2* Xs,
                                                       float* __restrict__ R32) {
   depend();
   extern __shared__ __align__(16) float2 rsm[];  // [PR][PS], then the warps' sums
@@ -1258,7 +1258,7 @@ __global__ void __launch_bounds__(PT) residual_kernel(const float2* __restrict__
       const float4* v = reinterpret_cast<const float4*>(Xs + static_cast<size_t>(k0 + k) * RW + c0);
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        const float4 x = __ldg(v + c);  // (hi, lo) of two columns
+        const float4 x = v[c];  // (hi, lo) of two columns
         const f2 xh = f2_make(x.x, x.z);
         f2_acc(h[c], l[c], mh, nmh, xh);
         l[c] = f2_fma(mh, f2_make(x.y, x.w), f2_fma(ml, xh, l[c]));
@@ -1290,9 +1290,9 @@ constexpr int PSM32 = PR * PS * 4 > (PT / 32) * PR * RW * 4 ? PR * PS * 4 : (PT 
 constexpr int PSM64 = 2 * PSM32;
 
 // ---- 6a. normalise; mark dead atoms ----------------------------------------------
-__global__ void normalise_kernel(const float2* __restrict__ Xs, const double* __restrict__ dsc,
-                                 const int* __restrict__ atom_start,
-                                 int K, float* __restrict__ D_new, const float* __restrict__ D_old,
+__global__ void normalise_kernel(const float2* Xs, const double* dsc,
+                                 const int* atom_start,
+                                 int K, float* __restrict__ D_new, const float* D_old,
                                  int* __restrict__ dead) {
   depend();
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1319,8 +1319,8 @@ __global__ void normalise_kernel(const float2* __restrict__ Xs, const double* __
 // Picks come in the order (resid desc, index asc); each pass takes the best key
 // strictly after the previous pick.  Signals with x = 0 are skipped.
 __global__ void __launch_bounds__(1024)
-    refill_kernel(const float* __restrict__ X, const float* __restrict__ resid, int64_t N, int K,
-                  const int* __restrict__ dead, float* __restrict__ D_new) {
+    refill_kernel(const float* X, const float* resid, int64_t N, int K,
+                  const int* dead, float* __restrict__ D_new) {
   depend();
   __shared__ float bv[1024];
   __shared__ long long bi[1024];
@@ -1466,10 +1466,10 @@ static size_t carve_ksvd(void* base, int K, int s, int64_t N, KsWs& w) {
 
 // R = X - D A with the input codes; one warp per signal, lane d owning
 // dimensions d and d + 32 (and the zero padding 45..47).
-__global__ void __launch_bounds__(256) ksvd_resid_kernel(const float* __restrict__ X, const float* __restrict__ D,
-                                                         int K, const uint16_t* __restrict__ idx,
-                                                         const float* __restrict__ coef,
-                                                         const uint8_t* __restrict__ nnz, int s, int64_t N,
+__global__ void __launch_bounds__(256) ksvd_resid_kernel(const float* X, const float* D,
+                                                         int K, const uint16_t* idx,
+                                                         const float* coef,
+                                                         const uint8_t* nnz, int s, int64_t N,
                                                          float* __restrict__ R) {
   depend();
   const int lane = threadIdx.x & 31;

@@ -250,3 +250,21 @@ def test_encode_variant_of_the_largest_fp8_dictionaries(L):
         for K in (k_rows, k_rows + 1, k_last):
             assert L.dlsh_encode_variant(K, 8, prec) == 2, (prec, K)
         assert L.dlsh_encode_variant(k_last + 1, 8, prec) == 1
+
+
+def test_kernels_that_start_early_read_by_coherent_loads():
+    """Kernels launched by launch_dependent begin before the kernel ahead of them ends:
+    no load of theirs may take the read-only path (__ldg, const __restrict__)."""
+    import glob
+    import re
+    src = {f: open(f).read() for f in glob.glob(os.path.join(ROOT, "paper_2605_30396_gb300", "csrc", "*.cu"))}
+    names = {n for t in src.values() for n in re.findall(r"launch_dependent\((\w+)", t)}
+    assert len(names) >= 15
+    for n in sorted(names):
+        defs = [m.group(0) for t in src.values()
+                for m in re.finditer(r"__global__ [^;{]*?\b%s\(.*?\n}\n" % n, t, re.S)]
+        assert len(defs) == 1, n
+        params, body = defs[0].split(") {\n", 1)
+        assert "__ldg(" not in body, n
+        assert not re.search(r"const \w+\* __restrict__", params), n
+        assert "depend();" in body, n
