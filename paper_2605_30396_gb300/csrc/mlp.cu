@@ -277,7 +277,8 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
   double* lsum = reinterpret_cast<double*>(smem + 4 * GN * 4);
   if (ok) {
     unsigned long long tgt = 0;  // EPI_BCE: bit c = column n0 + 64 h + c is a target of the row
-    double loss = 0.0;           // EPI_BCE: the row's, over the thread's columns
+    float lh = 0.f, ll = 0.f;    // the row's loss, float-float
+    double big = 0.0;            // and the part of it that FP32 cannot hold
     if (EPI == EPI_BCE && row < g.M) {
       int nz = g.nnz[row];
       nz = nz > g.s ? g.s : nz;
@@ -321,13 +322,14 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
         // step (__frcp_rn gives the same gradients and takes 5 % longer over the
         // call).  A NaN logit leaves a NaN in the gradient and in the loss.
         const unsigned y32 = static_cast<unsigned>(tgt >> (32 * cg));
-        float ph = 1.f, pl = 0.f, lh = 0.f, ll = 0.f;
+        float ph = 1.f, pl = 0.f;
+        const float lh0 = lh, ll0 = ll;
         auto elem = [&](int k, float bias) {
           const float z = add_bias(v[k], bias);
           const bool y = (y32 >> k) & 1u;
           const float e = expf(-z), d = 1.f + e, r0 = rcp_approx(d);
-          // (an infinite d keeps the 0, a NaN the NaN)
-          const float r = d < 1e37f ? fmaf(r0, fmaf(-d, r0, 1.f), r0) : r0;
+          // (an infinite d keeps its reciprocal 0; a NaN is one in r0)
+          const float r = fmaf(r0, fmaf(-fminf(d, 3.402823466e38f), r0, 1.f), r0);
           v[k] = (r - (y ? 1.f : 0.f)) * g.inv_bk;
           const float q = z < 0.f ? rcp_approx(e) : e;  // e^-|z|
           const float f = 1.f + q, fl = q - (f - 1.f);
@@ -349,9 +351,8 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
             else v[k] = 0.f;
           }
         }
-        const float logs = logf(ph) + __fdividef(pl, ph);
-        double sum = static_cast<double>(lh) + static_cast<double>(ll + logs);
-        // infinite logits, or a sum beyond FP32's range: from the accumulators again, in FP64
+        // infinite logits, or a sum beyond FP32's range: the max terms from the accumulators
+        // again, in FP64
         if (__any_sync(0xffffffffu, !(lh < INFINITY))) {
           double lin = 0.0;
 #pragma unroll 1
@@ -365,9 +366,13 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
                 lin += fmaxf((y32 >> (c0 + k)) & 1u ? -z : z, 0.f);
               }
           }
-          if (!(lh < INFINITY)) sum = lin + static_cast<double>(logs);
+          if (!(lh < INFINITY)) {
+            big += lin;
+            lh = lh0;
+            ll = ll0;
+          }
         }
-        loss += sum;
+        ll += logf(ph) + __fdividef(pl, ph);
       } else {
         float4 z4[8];
 #pragma unroll
@@ -386,7 +391,8 @@ __global__ void __launch_bounds__(GT, NS > 3 ? 1 : 2) train_gemm_kernel(const __
       csum[q4 * GN + cb + lane] = col_sums(v);
     }
     if (EPI == EPI_BCE) {
-      double l = loss;
+      double l = static_cast<double>(lh) + static_cast<double>(ll);
+      if (big != 0.0) l += big;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
       if (lane == 0) lsum[warp] = l;
@@ -432,7 +438,9 @@ struct ReduceArgs {
 template <bool ADAM>
 __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ ReduceArgs a) {
   depend();
-  if (blockIdx.x == gridDim.x - 1) {  // the last block: the mean loss, a fixed-order sum
+  // The first block takes the mean loss (a fixed-order sum), the others the
+  // parameters from the last on, so that the longest sums (b3) begin first.
+  if (blockIdx.x == 0) {
     __shared__ double red[256];
     double acc = 0.0;
     for (int q = threadIdx.x; q < a.nloss; q += 256) acc += a.loss_part[q];
@@ -445,7 +453,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Red
     if (threadIdx.x == 0 && a.loss) *a.loss = static_cast<float>(red[0] * a.inv_bk);
     return;
   }
-  const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
+  const long long i = static_cast<long long>(gridDim.x - 1 - blockIdx.x) * 256 + threadIdx.x;
   if (i >= a.L.n) return;
   const float* src = a.part + i;
   long long stride = a.zstride;
@@ -463,30 +471,36 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Red
     stride = HID;
     n = a.tiles;
   }
+  float m = 0.f, v = 0.f, p = 0.f;  // Adam's operands, in flight beside the partials
+  if (ADAM) {
+    m = a.b.m1[i];
+    v = a.b.m2[i];
+    p = a.b.P[i];
+  }
   float g = 0.f;
   if (stride == a.zstride) {
 #pragma unroll 8
     for (int z = 0; z < n; ++z) g += src[z * stride];
   } else {  // eight sums side by side: a hundred tiles in a row would cost a bias gradient a bit
-    float p[8] = {};
+    float c[8] = {};
     int z = 0;
     for (; z + 8 <= n; z += 8)
 #pragma unroll
-      for (int u = 0; u < 8; ++u) p[u] += src[(z + u) * stride];
+      for (int u = 0; u < 8; ++u) c[u] += src[(z + u) * stride];
 #pragma unroll
     for (int u = 0; u < 8; ++u)
-      if (z + u < n) p[u] += src[(z + u) * stride];
-    g = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+      if (z + u < n) c[u] += src[(z + u) * stride];
+    g = ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
   }
   if (!ADAM) {
     a.G[i] = g;
     return;
   }
-  const float m = a.beta1 * a.b.m1[i] + (1.f - a.beta1) * g;
-  const float v = a.beta2 * a.b.m2[i] + (1.f - a.beta2) * g * g;
+  m = a.beta1 * m + (1.f - a.beta1) * g;
+  v = a.beta2 * v + (1.f - a.beta2) * g * g;
   a.b.m1[i] = m;
   a.b.m2[i] = v;
-  const float p = a.b.P[i] - a.lr * (m / a.bc1) / (sqrtf(v / a.bc2) + a.eps);
+  p = p - a.lr * (m / a.bc1) / (sqrtf(v / a.bc2) + a.eps);
   a.b.P[i] = p;
   a.b.Pb[i] = __float2bfloat16(p);
 }
