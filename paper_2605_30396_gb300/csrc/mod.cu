@@ -1641,16 +1641,16 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
       const float o0 = dsm[warp][lane], o1 = lane < DLSH_D - 32 ? dsm[warp][32 + lane] : 0.f;
       const float v0 = fmaf(o0, gg, u0);
       const float v1 = lane < DLSH_D - 32 ? fmaf(o1, gg, u1) : 0.f;
-      float n2 = fmaf(v0, v0, v1 * v1), dot = fmaf(o0, v0, o1 * v1);
+      float n2 = fmaf(v0, v0, v1 * v1);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        n2 += __shfl_xor_sync(FULL, n2, o);
-        dot += __shfl_xor_sync(FULL, dot, o);
-      }
+      for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(FULL, n2, o);
       const bool zero = !(n2 > 0.f);
       const float inv = zero ? 0.f : rsqrtf(n2);
       u0 = v0 * inv;
       u1 = v1 * inv;
+      float dd = fmaf(o0, u0, o1 * u1);  // d_j . d, of the atom as it is rounded
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(FULL, dd, o);
       if (blockIdx.x == 0 && warp == 0) {
         float* out = D_new + static_cast<size_t>(j) * DLSH_D;
         out[lane] = zero ? o0 : u0;
@@ -1661,7 +1661,6 @@ __global__ void __launch_bounds__(KS_T, 1) ksvd_sweep_kernel(const int* __restri
       if (lane < RROW - 32) dsm[warp][32 + lane] = lane < DLSH_D - 32 ? u1 : 0.f;
       __syncwarp();
       if (!zero) {
-        const float dd = dot * inv;  // d_j . d
         const float4 u = rl ? *reinterpret_cast<const float4*>(&dsm[warp][4 * l]) : make_float4(0.f, 0.f, 0.f, 0.f);
         // E_i . d = R_i . d + g (d_j . d); R_i <- R_i + g d_j - g' d
         auto refit = [&](uint2 q, float4 x, bool on) {
