@@ -37,6 +37,24 @@ def test_mod_matches_oracle(lib, N, K, s):
     np.testing.assert_allclose(got, ref, atol=3e-6, rtol=0)
 
 
+def test_mod_on_nearly_dependent_atoms(lib):
+    """K = 1024 with the atoms in pairs that are always used together, with coefficients
+    1 % apart (the scaled Gram matrix has a condition of 6e4): the refined solution is
+    FP64's rounded to FP32, below 2^-24 in the norm."""
+    N, K, s = 60_000, 1024, 8
+    rng = np.random.default_rng(21)
+    h = synth.distinct_supports(rng, N, K // 2, s // 2)
+    idx = np.stack([2 * h, 2 * h + 1], axis=2).reshape(N, s)
+    c = rng.laplace(0, 1, h.shape)
+    coef = np.stack([c, c * (1 + 1e-2 * rng.standard_normal(c.shape))], axis=2).reshape(N, s).astype(np.float32)
+    X = synth.signals(N, synth.hidden_dictionary(K, 22), 4, 23)
+    D0 = synth.hidden_dictionary(K, 24).astype(np.float32)
+    nnz = np.full(N, s, dtype=np.uint8)
+    got = _gpu(lib, X, D0, idx.astype(np.uint16), coef, nnz, None)
+    ref, _ = omod.mod_update(X.astype(np.float64), D0.astype(np.float64), idx, coef.astype(np.float64), nnz)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 2.0**-24
+
+
 @pytest.mark.parametrize("N,K,s,skip", [(513, 40, 1, 0), (9000, 1500, 8, 0), (65537, 128, 17, 0), (33000, 96, 32, 2),
                                         (330_000, 300, 3, 2), (311_297, 64, 8, 0)])
 def test_mod_on_random_codes(lib, N, K, s, skip):
