@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(1024) decode_kernel(
 // atom's row.  Against reading whole rows through the read-only cache the codes
 // are read and staged three times, but an atom costs 64 bytes of shared memory
 // per channel instead of six gathers of 4 bytes per lane: N = 778k, K = 2048,
-// s = 16 (half of the slots used) 196 -> 150 us, bound by issue (68 %) and
+// s = 16 (half of the slots used) 196 -> 143 us, bound by issue (68 %) and
 // shared-memory wavefronts (69 %).
 __host__ __device__ constexpr int plane_warp_floats(int sp, int gb) { return gb * YS + gb * sp * 2 + gb; }
 

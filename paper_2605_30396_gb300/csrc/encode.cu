@@ -406,7 +406,8 @@ int encode_enqueue(const float* D, int K, const float* X, int64_t N, int s, floa
       if (choice == 6) return launch_split<true, 3, 128, 8>(a, grid, st);
       if (choice == 4) return launch_split<false, 2, 128, 8>(a, grid, st);
       // up to one tile per SM: tiles of 64 signals, one or two per CTA (N = 10,000,
-      // K = 256, s = 8: 99 us a call on 40 CTAs with two tiles of 128 each, 61 so)
+      // K = 256, s = 8: 99 us a call on 40 CTAs with two tiles of 128 each, 53 so, the
+      // preparation in one launch included)
       if (!n_dev && ntiles <= sms) {
         const int64_t half = (N + 63) / 64;
         const int hgrid = static_cast<int>(half < sms ? half : sms);

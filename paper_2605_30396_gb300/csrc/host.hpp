@@ -63,7 +63,7 @@ int device_sm_count();
 // Launches a kernel that opens with depend() (common.cuh): its launch overlaps
 // the end of the kernel before it in the stream.  In a chain of short dependent
 // kernels this hides most of each launch (a MOD update of 10,000 signals, 20
-// launches: 231 -> 201 us; the network's gradients at batch 8192, 8 launches: 101 ->
+// launches: 231 -> 201 us; the network's gradients at batch 8192, 7 launches: 101 ->
 // 90 us on the device).  Errors are left to check_launch.
 template <class... P, class... A>
 inline void launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {

@@ -8,17 +8,16 @@
 //                   TMEM, 128 x 128 tiles.  An operand is read in place by
 //                   TMA, K-major or MN-major (the transposed activations and
 //                   weights of the backward pass need no copies).  Each epilogue
-//                   does the
-//                   element-wise work that follows the product: bias + GELU,
-//                   BCE gradient + loss + column sums, GELU backward + column
-//                   sums, or the FP32 partial of a weight gradient.
-//   weight gradients  one launch for all three layers, split over the batch
-//                   Batch 8192, K = 1024 (us of device time): logits with the
-//                   BCE work 34 + 67 -> 31, dH2 with the GELU backward 103 ->
-//                   15, weight gradients 479 -> 12, the whole gradient call 810
-//                   -> 163 of which about 95 are kernels.
+//                   does the element-wise work that follows the product: bias +
+//                   GELU, BCE gradient + loss + column sums, GELU backward +
+//                   column sums, or the FP32 partial of a weight gradient.  The
+//                   weight gradients of all three layers are one launch, split
+//                   over the batch.
 //   reduce_kernel   adds the split partials and the column sums in a fixed
 //                   order (gradients), and applies Adam in a training step
+// Batch 8192, K = 1024 (us of device time): logits with the BCE work 34 + 67 -> 29,
+// dH2 with the GELU backward 103 -> 15, weight gradients 479 -> 12; the whole
+// gradient call 810 -> 157, of which about 90 are the seven launches.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>

@@ -1,5 +1,5 @@
-// Definitions shared by the proposal network's kernels (mlp.cu: training and
-// the layer-by-layer forward; propose.cu: the fused inference kernel).  The
+// Definitions shared by the proposal network's kernels (mlp.cu: training, layer by
+// layer; propose.cu: the fused inference kernel).  The
 // element-wise arithmetic lives here once, written with explicit rounding
 // intrinsics, so that both paths produce bit-identical activations and logits.
 #pragma once

@@ -122,7 +122,7 @@ struct Ws {
   float* W32;      // K x K: L^-1 (lower)
   float* Yg;       // two 32 x 32 blocks: inverse of the factor's diagonal block
   float* Y32;      // K x RW: W r, between the two triangular products
-  unsigned* gbar;  // grid barrier of the factorisation: arrivals, generation
+  unsigned* gbar;  // grid barrier of the factorisation: arrivals
   float2* Zs;      // K x RW: scaled right-hand side
   float2* Xs;      // K x RW: solution of the scaled system
   float* R32;      // K x RW: current residual of the scaled system
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(256, 4) accum_b_kernel(const float* __restrict
         const int src = 4 * (i0 + u) + grp;
         const unsigned sig = __shfl_sync(FULL, rec.x, src) & 0x3FFFFFFu;
         const float* xr = Xl + static_cast<size_t>(sig) * DLSH_D;
-        const bool on = whole || eb + src < q1;  // past the end: a = 0 and x = 0
+        const bool on = whole || eb + src < q1;  // past the end: x = 0
 #pragma unroll
         for (int q = 0; q < BQ; ++q) x[u][q] = on ? __ldg(xr + (q + 1 < BQ ? 8 * q : last)) : 0.f;
       }
@@ -1443,10 +1443,10 @@ __global__ void __launch_bounds__(1024)
 // the words of an exchange only after it has read all of the previous one's, which
 // the others write only after they have read the one before, so no word is
 // overwritten before its readers are through.  Every sum runs in a fixed order.
-// Bound by latency: the row
-// gather, one L2 round trip of the words and the reductions, 3.4 us per
-// atom (N = 400k, K = 512, s = 8; with two grid barriers per atom and one
-// thread per entry 12.4 us).
+// Bound by latency: the row gather, one L2 round trip of the words and the
+// reductions, 3.0 us per atom (N = 400k, K = 512, s = 8; with two grid barriers per
+// atom and one thread per entry 12.4 us; with the words waited for one after the
+// other 3.4).
 constexpr int KS_T = 512;          // threads per sweep CTA
 constexpr int KS_E = KS_T / 16;    // entries per pass
 constexpr int KS_KEEP = 5;         // passes kept in registers between the phases
