@@ -481,14 +481,15 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Red
 #pragma unroll 8
     for (int z = 0; z < n; ++z) g += src[z * stride];
   } else {  // eight sums side by side: a hundred tiles in a row would cost a bias gradient a bit
+    // (32 of them in flight: the chain of loads is what this kernel takes)
     float c[8] = {};
-    int z = 0;
-    for (; z + 8 <= n; z += 8)
+    for (int z = 0; z < n; z += 32) {
+      float x[32];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) c[u] += src[(z + u) * stride];
+      for (int u = 0; u < 32; ++u) x[u] = z + u < n ? src[(z + u) * stride] : 0.f;
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (z + u < n) c[u] += src[(z + u) * stride];
+      for (int u = 0; u < 32; ++u) c[u & 7] += x[u];
+    }
     g = ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
   }
   if (!ADAM) {
